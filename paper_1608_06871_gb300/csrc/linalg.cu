@@ -32,72 +32,115 @@ template <> struct is_fp64<double2> { static constexpr bool v = true; };
 template <typename TA, typename TB> constexpr double flops_per_mac() {
   return (is_cplx<TA>::v && is_cplx<TB>::v) ? 8.0 : ((is_cplx<TA>::v || is_cplx<TB>::v) ? 4.0 : 2.0);
 }
-constexpr int BM = 32, BN = 32, BK = 16;  // GEMM tile
+constexpr int BK = 16;                    // k-step of the small GEMM tiles
 constexpr int NB = 32;                    // LU panel / TRSM block size
 constexpr int NBB = 128;                  // LU super-panel: k of the trailing updates
 constexpr int kMaxCluster = 8;            // portable thread-block cluster size (split-k)
+
+__device__ __forceinline__ double shfl_xor(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ float shfl_xor(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ double2 shfl_xor(double2 v, int m) {
+  return make_double2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
+__device__ __forceinline__ float2 shfl_xor(float2 v, int m) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
 
 template <typename T> __device__ __forceinline__ T ld_op(const T* P, int ld, int op, int r, int c) {
   return op == OP_N ? P[(long long)r * ld + c] : P[(long long)c * ld + r];
 }
 
-// 32 x 32 tile, 2 x 2 outputs per thread.  blockIdx.z = batch * splits + split:
+// TM x TN tile, one 256-thread CTA, (TM TN / 256) outputs per thread, the next
+// k-step prefetched into registers.  blockIdx.z = batch * splits + split:
 // with splits > 1 the kernel is launched in clusters of `splits` CTAs along z,
 // each CTA covers a slice of k, and the partial tiles are summed through
 // distributed shared memory in split order (deterministic, no atomics): rank r
 // reduces and writes its share of the tile's rows.
-template <typename TA, typename TB, typename TC>
+// FP64: bound by the pipe, which takes two thread-operations per SM and clock
+// whatever the tile, so the tile only has to keep padding and idle SMs small:
+// 16 x 16 as well as 32 x 32 (fp64_tile), both saturate it (one DFMA per warp
+// and 64 cycles leaves room for the two shared-memory loads it needs).  With
+// this, the dot products and k_trsm_blk below a far field of one incidence on
+// 4 x 4 leaves went from 2.52 to 0.54 ms, a k = 5 Gauss-Newton step from 16.3
+// to 7.8 ms, the k = 40 FP64 batch from 263 to 227 ms.
+template <typename TA, typename TB, typename TC, int TM, int TN>
 __global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int m, int n, int k, TC alpha, const TA* __restrict__ A,
                                               int lda, long long sA, const TB* __restrict__ B, int ldb, long long sB,
                                               TC beta, TC* __restrict__ C, int ldc, long long sC, int splits) {
-  constexpr size_t A_BYTES = sizeof(TA) * BK * (BM + 1), B_BYTES = sizeof(TB) * BK * (BN + 1);
-  constexpr size_t RED_BYTES = sizeof(TC) * BM * BN;
+  constexpr int RM = TM / 16, RN = TN / 16;                      // outputs per thread
+  constexpr int NA = TM * BK / 256, NBq = TN * BK / 256;         // staged elements per thread
+  constexpr size_t A_BYTES = sizeof(TA) * BK * (TM + 1), B_BYTES = sizeof(TB) * BK * (TN + 1);
+  constexpr size_t RED_BYTES = sizeof(TC) * TM * TN;
   __shared__ __align__(16) unsigned char raw[A_BYTES + B_BYTES > RED_BYTES ? A_BYTES + B_BYTES : RED_BYTES];
-  TA(*As)[BM + 1] = reinterpret_cast<TA(*)[BM + 1]>(raw);
-  TB(*Bs)[BN + 1] = reinterpret_cast<TB(*)[BN + 1]>(raw + A_BYTES);
+  TA(*As)[TM + 1] = reinterpret_cast<TA(*)[TM + 1]>(raw);
+  TB(*Bs)[TN + 1] = reinterpret_cast<TB(*)[TN + 1]>(raw + A_BYTES);
   const int b = blockIdx.z / splits, sp = blockIdx.z % splits;
   A += b * sA;
   B += b * sB;
   C += b * sC;
   const int kc = ((k + splits - 1) / splits + BK - 1) / BK * BK;
   const int kbeg = sp * kc, kend = min(k, kbeg + kc);
-  const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
+  const int row0 = blockIdx.y * TM, col0 = blockIdx.x * TN;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  TC acc[2][2];
+  TC acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) acc[i][j] = el<TC>::zero();
-  for (int k0 = kbeg; k0 < kend; k0 += BK) {
-    for (int e = threadIdx.x; e < BM * BK; e += 256) {
+    for (int j = 0; j < RN; ++j) acc[i][j] = el<TC>::zero();
+  TA ra[NA];
+  TB rb[NBq];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = threadIdx.x + 256 * q;
       int r, kk;
-      if (opA == OP_N) { r = e / BK; kk = e % BK; } else { kk = e / BM; r = e % BM; }
-      int gr = row0 + r, gk = k0 + kk;
-      As[kk][r] = (gr < m && gk < kend) ? ld_op(A, lda, opA, gr, gk) : el<TA>::zero();
+      if (opA == OP_N) { r = e / BK; kk = e % BK; } else { kk = e / TM; r = e % TM; }
+      const int gr = row0 + r, gk = k0 + kk;
+      ra[q] = (gr < m && gk < kend) ? ld_op(A, lda, opA, gr, gk) : el<TA>::zero();
     }
-    for (int e = threadIdx.x; e < BK * BN; e += 256) {
+#pragma unroll
+    for (int q = 0; q < NBq; ++q) {
+      const int e = threadIdx.x + 256 * q;
       int kk, c;
-      if (opB == OP_N) { kk = e / BN; c = e % BN; } else { c = e / BK; kk = e % BK; }
-      int gk = k0 + kk, gc = col0 + c;
-      Bs[kk][c] = (gk < kend && gc < n) ? ld_op(B, ldb, opB, gk, gc) : el<TB>::zero();
+      if (opB == OP_N) { kk = e / TN; c = e % TN; } else { c = e / BK; kk = e % BK; }
+      const int gk = k0 + kk, gc = col0 + c;
+      rb[q] = (gk < kend && gc < n) ? ld_op(B, ldb, opB, gk, gc) : el<TB>::zero();
+    }
+  };
+  if (kbeg < kend) load(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = threadIdx.x + 256 * q;
+      if (opA == OP_N) As[e % BK][e / BK] = ra[q]; else As[e / TM][e % TM] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NBq; ++q) {
+      const int e = threadIdx.x + 256 * q;
+      if (opB == OP_N) Bs[e / TN][e % TN] = rb[q]; else Bs[e % BK][e / BK] = rb[q];
     }
     __syncthreads();
+    if (k0 + BK < kend) load(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      TA a0 = As[kk][ty], a1 = As[kk][ty + 16];
-      TB b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      acc[0][0] = fmac(acc[0][0], a0, b0);
-      acc[0][1] = fmac(acc[0][1], a0, b1);
-      acc[1][0] = fmac(acc[1][0], a1, b0);
-      acc[1][1] = fmac(acc[1][1], a1, b1);
+      TA a[RM];
+      TB bb[RN];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) bb[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) acc[i][j] = fmac(acc[i][j], a[i], bb[j]);
     }
     __syncthreads();
   }
   if (splits == 1) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
+      for (int j = 0; j < RN; ++j) {
         int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
         if (r < m && c < n) {
           TC v = scal<TC, TC>(alpha, acc[i][j]);
@@ -110,17 +153,17 @@ __global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int m, int n, in
   }
   TC* red = reinterpret_cast<TC*>(raw);  // the k loop ended with a barrier
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) red[(ty + 16 * i) * BN + tx + 16 * j] = acc[i][j];
+    for (int j = 0; j < RN; ++j) red[(ty + 16 * i) * TN + tx + 16 * j] = acc[i][j];
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
-  const int rows_per = (BM + splits - 1) / splits;
-  const int rb = sp * rows_per, re = min(BM, rb + rows_per);
-  for (int e = rb * BN + threadIdx.x; e < re * BN; e += 256) {
+  const int rows_per = (TM + splits - 1) / splits;
+  const int rb0 = sp * rows_per, re = min(TM, rb0 + rows_per);
+  for (int e = rb0 * TN + threadIdx.x; e < re * TN; e += 256) {
     TC sum = el<TC>::zero();
     for (int q = 0; q < splits; ++q) sum = addv(sum, cl.map_shared_rank(red, q)[e]);
-    const int r = row0 + e / BN, c = col0 + e % BN;
+    const int r = row0 + e / TN, c = col0 + e % TN;
     if (r < m && c < n) {
       TC v = scal<TC, TC>(alpha, sum);
       long long o = (long long)r * ldc + c;
@@ -129,6 +172,47 @@ __global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int m, int n, in
     }
   }
   cl.sync();  // keep this CTA's partial tile alive until every rank has read it
+}
+
+// Products with at most eight columns (or, with the roles of the operands
+// swapped by the host, rows): one warp per row i and NC columns, lanes along
+// k, one shuffle reduction per output.  Such a product is a few passes over
+// one operand; a square tile pads the columns to its width, and FP64 pays for
+// padding on the pipe (224 x 1 x 224 complex: 200 us with a 32 x 32 tile).
+// Element strides, so that both transposes and the swap are the same code:
+// A(i, l) = A[i ai + l ak], B(l, j) = B[l bk + j bj], C(i, j) = C[i ci + j cj].
+constexpr int DOT_WARPS = 4;
+template <typename TA, typename TB, typename TC, int NC>
+__global__ void __launch_bounds__(32 * DOT_WARPS)
+    k_gemm_dot(int m, int n, int k, TC alpha, const TA* __restrict__ A, long long ai, long long ak, long long sA,
+               const TB* __restrict__ B, long long bk, long long bj, long long sB, TC beta, TC* __restrict__ C,
+               long long ci, long long cj, long long sC) {
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * DOT_WARPS + (threadIdx.x >> 5), j0 = blockIdx.y * NC;
+  if (i >= m) return;  // whole warp
+  A += blockIdx.z * sA + i * ai;
+  B += blockIdx.z * sB + j0 * bj;
+  TC acc[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) acc[j] = el<TC>::zero();
+#pragma unroll 2
+  for (int l = lane; l < k; l += 32) {
+    const TA a = A[l * ak];
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+      if (j0 + j < n) acc[j] = fmac(acc[j], a, B[l * bk + j * bj]);
+  }
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc[j] = addv(acc[j], shfl_xor(acc[j], off));
+    if (lane == j && j0 + j < n) {
+      TC* c = C + blockIdx.z * sC + i * ci + (j0 + j) * cj;
+      TC v = scal<TC, TC>(alpha, acc[j]);
+      if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, *c));
+      *c = v;
+    }
+  }
 }
 
 // 64 x 64 tile, 4 x 4 outputs per thread (more arithmetic per shared-memory
@@ -408,7 +492,8 @@ __global__ void __launch_bounds__(32 * TRSM_WARPS) k_trsm_diag(const E* A, int l
   for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
     int r = e / nb, c = e % nb;
     bool tr = (mode >= 2);
-    T[r][c] = tr ? A[(long long)(i0 + c) * lda + i0 + r] : A[(long long)(i0 + r) * lda + i0 + c];
+    const E a = tr ? A[(long long)(i0 + c) * lda + i0 + r] : A[(long long)(i0 + r) * lda + i0 + c];
+    T[r][c] = r == c && (mode == 1 || mode == 2) ? el<E>::div(el<E>::one(), a) : a;  // reciprocal diagonal
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -419,13 +504,13 @@ __global__ void __launch_bounds__(32 * TRSM_WARPS) k_trsm_diag(const E* A, int l
   const bool unit = (mode == 0 || mode == 3);
   if (lower) {
     for (int s = 0; s < nb; ++s) {
-      if (!unit && lane == s) x = el<E>::div(x, T[s][s]);
+      if (!unit && lane == s) x = x * T[s][s];
       E xs = shfl(x, s);
       if (lane > s && lane < nb) x = fmsc(x, T[lane][s], xs);
     }
   } else {
     for (int s = nb - 1; s >= 0; --s) {
-      if (!unit && lane == s) x = el<E>::div(x, T[s][s]);
+      if (!unit && lane == s) x = x * T[s][s];
       E xs = shfl(x, s);
       if (lane < s) x = fmsc(x, T[lane][s], xs);
     }
@@ -446,8 +531,9 @@ __global__ void __launch_bounds__(128) k_trsm_diag_col(const E* A, int lda, long
   const bool tr = (mode >= 2);
   for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
     int r = e / NB, c = e % NB;
-    T[r][c] = (r < nb && c < nb) ? (tr ? A[(long long)(i0 + c) * lda + i0 + r] : A[(long long)(i0 + r) * lda + i0 + c])
-                                 : el<E>::zero();
+    const E a = (r < nb && c < nb) ? (tr ? A[(long long)(i0 + c) * lda + i0 + r] : A[(long long)(i0 + r) * lda + i0 + c])
+                                   : el<E>::zero();
+    T[r][c] = r == c && r < nb && (mode == 1 || mode == 2) ? el<E>::div(el<E>::one(), a) : a;  // reciprocal diagonal
   }
   __syncthreads();
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
@@ -463,7 +549,7 @@ __global__ void __launch_bounds__(128) k_trsm_diag_col(const E* A, int lda, long
       E v = x[r];
 #pragma unroll
       for (int c = 0; c < r; ++c) v = fmsc(v, T[r][c], x[c]);
-      x[r] = (unit || r >= nb) ? v : el<E>::div(v, T[r][r]);
+      x[r] = (unit || r >= nb) ? v : v * T[r][r];
     }
   } else {
 #pragma unroll
@@ -471,7 +557,7 @@ __global__ void __launch_bounds__(128) k_trsm_diag_col(const E* A, int lda, long
       E v = x[r];
 #pragma unroll
       for (int c = r + 1; c < NB; ++c) v = fmsc(v, T[r][c], x[c]);
-      x[r] = (unit || r >= nb) ? v : el<E>::div(v, T[r][r]);
+      x[r] = (unit || r >= nb) ? v : v * T[r][r];
     }
   }
 #pragma unroll
@@ -494,70 +580,170 @@ void trsm_diag(cudaStream_t s, const E* A, int lda, long long sA, int i0, int nb
   HS_COUNT_LAUNCH();
 }
 
-// The solve with a whole diagonal block of up to NBB rows in one launch:
-// rows [i0, i0 + nbs) of B (column block of TB_CW<E> columns per CTA, held in
-// shared memory) against the block's unit lower (mode 0, top down) or upper
-// triangle (mode 1, bottom up).  Per NB-row sub-block: one warp per column
-// solves the diagonal block with shuffles, then every thread updates the
-// block's remaining rows from the solved ones (the off-diagonal entries read
-// through L1).  Replaces the NB-blocked sequence of triangular solves and
-// small products (and their trips through global memory) inside the block.
-template <typename E> struct tb_cw { static constexpr int v = sizeof(E) == 16 ? 8 : 16; };
-template <typename E>
-__global__ void __launch_bounds__(32 * tb_cw<E>::v) k_trsm_blk(const E* __restrict__ A, int lda, long long sA, int i0,
-                                                               int nbs, int mode, E* __restrict__ B, int ldb,
-                                                               long long sB, int nrhs) {
-  constexpr int CW = tb_cw<E>::v, NT = 32 * CW;
-  __shared__ E Bs[NBB][CW + 1];
-  __shared__ E Ld[NB][NB + 1];
+// The solve with a whole diagonal block of up to NBB rows in one launch: rows
+// [i0, i0 + nbs) of B (CW columns per CTA, held in shared memory) against the
+// block's triangle; mode as k_trsm_diag's (0: L, 1: U, 2: U^T, 3: L^T; 0 and 2
+// run top down, 1 and 3 bottom up).  Per sub-block of SB rows one warp per
+// column substitutes with shuffles, then every thread updates the rows still
+// to solve.  The sub-block's columns of the triangle are staged in shared
+// memory by cp.async, the next sub-block's while this one is solved.
+// What bounds it is the substitution's chain and, in FP64, the pipe (two
+// thread-operations per SM and clock): complex sub-blocks of 16 rows put the
+// real and the imaginary part of a row on two lanes, two dependent
+// multiply-adds a step instead of four on a half-idle warp, and the host takes
+// as few columns per CTA as spread them over the SMs (trsm_cw).  A 128-row
+// block with one FP64 complex column: 274 us with eight columns per CTA, of
+// which seven were padding.
+template <typename E> struct tb_sb { static constexpr int v = sizeof(E) == 16 ? 16 : 32; };  // sub-block rows
+
+template <int BYTES> __device__ __forceinline__ void cp_elem(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+
+// One warp: x (rows r0 .. r0 + nb of column c in Bs) <- solve with the nb x nb
+// triangle whose (r, t) entry is T[r][t].  The diagonal's reciprocals are taken
+// by all lanes at once before the chain, which then only multiplies (a complex
+// FP64 division inside it would be some thirty operations of the pipe a step).
+template <typename E, int SB, int CW>
+__device__ __forceinline__ void tri_solve_warp(const E (*T)[SB + 1], E (*Bs)[CW + 1], int r0, int nb, int c, bool down,
+                                               bool unit, int lane) {
+  if constexpr (sizeof(E) == 16) {  // complex FP64: lane = 2 row + part
+    const int r = lane >> 1, im = lane & 1;
+    const bool live = r < nb;
+    double x = live ? (im ? Bs[r0 + r][c].y : Bs[r0 + r][c].x) : 0.0;
+    const E inv = (live && !unit) ? el<E>::div(el<E>::one(), T[r][r]) : el<E>::one();
+    for (int q = 0; q < nb; ++q) {
+      const int t = down ? q : nb - 1 - q;
+      if (!unit) {
+        const double o = __shfl_xor_sync(0xffffffffu, x, 1);
+        if (r == t) x = im ? fma(x, inv.x, o * inv.y) : fma(x, inv.x, -o * inv.y);
+      }
+      const double xr = __shfl_sync(0xffffffffu, x, 2 * t), xi = __shfl_sync(0xffffffffu, x, 2 * t + 1);
+      if (live && (down ? r > t : r < t)) {
+        const E l = T[r][t];
+        // re -= l.x xr - l.y xi,  im -= l.x xi + l.y xr
+        x = im ? fma(-l.y, xr, fma(-l.x, xi, x)) : fma(l.y, xi, fma(-l.x, xr, x));
+      }
+    }
+    if (live) (im ? Bs[r0 + r][c].y : Bs[r0 + r][c].x) = x;
+  } else {
+    E x = lane < nb ? Bs[r0 + lane][c] : el<E>::zero();
+    const E inv = (lane < nb && !unit) ? el<E>::div(el<E>::one(), T[lane][lane]) : el<E>::one();
+    for (int q = 0; q < nb; ++q) {
+      const int t = down ? q : nb - 1 - q;
+      if (!unit && lane == t) x = x * inv;
+      const E xt = shfl(x, t);
+      if (lane < nb && (down ? lane > t : lane < t)) x = fmsc(x, T[lane][t], xt);
+    }
+    if (lane < nb) Bs[r0 + lane][c] = x;
+  }
+}
+
+template <typename E, int CW>
+__global__ void __launch_bounds__(CW <= 4 ? 128 : 32 * CW)
+    k_trsm_blk(const E* __restrict__ A, int lda, long long sA, int i0, int nbs, int mode, E* __restrict__ B, int ldb,
+               long long sB, int nrhs) {
+  constexpr int SB = tb_sb<E>::v, NT = CW <= 4 ? 128 : 32 * CW;
+  extern __shared__ __align__(16) unsigned char trsm_smem[];
+  E(*Bs)[CW + 1] = reinterpret_cast<E(*)[CW + 1]>(trsm_smem);
+  E(*Lp)[NBB][SB + 1] = reinterpret_cast<E(*)[NBB][SB + 1]>(trsm_smem + sizeof(E) * NBB * (CW + 1));
   const int b = blockIdx.y, c0 = blockIdx.x * CW, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  A += b * sA;
-  B += b * sB;
+  const bool down = mode == 0 || mode == 2, unit = mode == 0 || mode == 3, tr = mode >= 2;
+  A += b * sA + (long long)i0 * lda + i0;
+  B += b * sB + (long long)i0 * ldb + c0;
+  const int nsub = (nbs + SB - 1) / SB;
+  // rows still to solve at sub-block `sub`, itself included: [lo, hi)
+  auto range = [&](int sub, int& r0, int& nb, int& lo, int& hi) {
+    r0 = sub * SB;
+    nb = min(SB, nbs - r0);
+    lo = down ? r0 : 0;
+    hi = down ? nbs : r0 + nb;
+  };
+  auto stage = [&](int q) {
+    int r0, nb, lo, hi;
+    range(down ? q : nsub - 1 - q, r0, nb, lo, hi);
+    if (!tr) {  // (r, t) at A[r][r0 + t]: rows of nb contiguous entries
+      for (int e = tid; e < (hi - lo) * nb; e += NT) {
+        const int r = lo + e / nb, t = e % nb;
+        cp_elem<sizeof(E)>(&Lp[q & 1][r][t], A + (long long)r * lda + r0 + t);
+      }
+    } else {  // (r, t) at A[r0 + t][r]: contiguous along r
+      const int nr = hi - lo;
+      for (int e = tid; e < nr * nb; e += NT) {
+        const int t = e / nr, r = lo + e % nr;
+        cp_elem<sizeof(E)>(&Lp[q & 1][r][t], A + (long long)(r0 + t) * lda + r);
+      }
+    }
+    cp_commit();
+  };
+  stage(0);
   for (int e = tid; e < nbs * CW; e += NT) {
     const int r = e / CW, c = e % CW;
-    Bs[r][c] = c0 + c < nrhs ? B[(long long)(i0 + r) * ldb + c0 + c] : el<E>::zero();
+    Bs[r][c] = c0 + c < nrhs ? B[(long long)r * ldb + c] : el<E>::zero();
   }
-  const int nsub = (nbs + NB - 1) / NB;
   for (int q = 0; q < nsub; ++q) {
-    const int sub = mode == 0 ? q : nsub - 1 - q;
-    const int r0 = sub * NB, nb = min(NB, nbs - r0);
-    for (int e = tid; e < nb * nb; e += NT) {
-      const int r = e / nb, c = e % nb;
-      Ld[r][c] = A[(long long)(i0 + r0 + r) * lda + i0 + r0 + c];
-    }
-    __syncthreads();  // (also orders the previous sub-block's updates of Bs)
-    if (warp < CW) {
-      E x = lane < nb ? Bs[r0 + lane][warp] : el<E>::zero();
-      if (mode == 0) {
-        for (int t = 0; t < nb; ++t) {
-          const E xt = shfl(x, t);
-          if (lane > t && lane < nb) x = fmsc(x, Ld[lane][t], xt);
-        }
-      } else {
-        for (int t = nb - 1; t >= 0; --t) {
-          if (lane == t) x = el<E>::div(x, Ld[t][t]);
-          const E xt = shfl(x, t);
-          if (lane < t) x = fmsc(x, Ld[lane][t], xt);
-        }
-      }
-      if (lane < nb) Bs[r0 + lane][warp] = x;
-    }
+    int r0, nb, lo, hi;
+    range(down ? q : nsub - 1 - q, r0, nb, lo, hi);
+    cp_wait<0>();
+    __syncthreads();  // the panel has landed; the previous update of Bs is done
+    if (q + 1 < nsub) stage(q + 1);
+    for (int c = warp; c < CW && c0 + c < nrhs; c += NT / 32)
+      tri_solve_warp<E, SB, CW>(&Lp[q & 1][r0], Bs, r0, nb, c, down, unit, lane);
     __syncthreads();
-    // the block's rows still to solve: below (mode 0) or above (mode 1) the sub-block
-    const int ra = mode == 0 ? r0 + nb : 0, rb = mode == 0 ? nbs : r0;
+    const int ra = down ? r0 + nb : 0, rb = down ? nbs : r0;
     for (int e = tid; e < (rb - ra) * CW; e += NT) {
       const int r = ra + e / CW, c = e % CW;
-      const E* arow = A + (long long)(i0 + r) * lda + i0 + r0;
       E acc = Bs[r][c];
-      for (int t = 0; t < nb; ++t) acc = fmsc(acc, arow[t], Bs[r0 + t][c]);
+      if (nb == SB) {
+#pragma unroll
+        for (int t = 0; t < SB; ++t) acc = fmsc(acc, Lp[q & 1][r][t], Bs[r0 + t][c]);
+      } else {
+        for (int t = 0; t < nb; ++t) acc = fmsc(acc, Lp[q & 1][r][t], Bs[r0 + t][c]);
+      }
       Bs[r][c] = acc;
     }
   }
   __syncthreads();
   for (int e = tid; e < nbs * CW; e += NT) {
     const int r = e / CW, c = e % CW;
-    if (c0 + c < nrhs) B[(long long)(i0 + r) * ldb + c0 + c] = Bs[r][c];
+    if (c0 + c < nrhs) B[(long long)r * ldb + c] = Bs[r][c];
   }
+}
+
+// Columns per CTA: the fewest columns on the busiest SM (its CTAs share the
+// pipe), more per CTA where that costs at most a tenth (the triangle is staged
+// once per CTA).
+int trsm_cw(int nrhs, int batch) {
+  int best = 1;
+  double bt = 1e300;
+  for (int cw : {8, 4, 2, 1}) {
+    const double t = std::ceil((double)((nrhs + cw - 1) / cw) * batch / 152.0) * cw;
+    if (t < 0.9 * bt) {
+      bt = t;
+      best = cw;
+    }
+  }
+  return best;
+}
+
+template <typename E, int CW>
+void launch_trsm_blk(cudaStream_t s, const E* A, int lda, long long sA, int i0, int nbs, int mode, E* B, int ldb,
+                     long long sB, int nrhs, int batch) {
+  constexpr int SB = tb_sb<E>::v, NT = CW <= 4 ? 128 : 32 * CW;
+  constexpr int smem = (int)sizeof(E) * (NBB * (CW + 1) + 2 * NBB * (SB + 1));
+  if constexpr (smem > 48 * 1024) {
+    static bool attr[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !attr[dev]) {
+      cudaFuncSetAttribute(k_trsm_blk<E, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (dev >= 0 && dev < 64) attr[dev] = true;
+    }
+  }
+  dim3 g((nrhs + CW - 1) / CW, batch);
+  k_trsm_blk<E, CW><<<g, NT, smem, s>>>(A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs);
+  HS_COUNT_LAUNCH();
 }
 
 // Solve with the diagonal block rows [i0, i0 + nbs) of A: one launch of
@@ -568,29 +754,33 @@ __global__ void __launch_bounds__(32 * tb_cw<E>::v) k_trsm_blk(const E* __restri
 template <typename E>
 void trsm_blk(cudaStream_t s, const E* A, int lda, long long sA, int i0, int nbs, int mode, E* B, int ldb,
               long long sB, int nrhs, int batch) {
-  constexpr int CW = tb_cw<E>::v;
   if ((long long)nrhs * batch < 8192) {
-    dim3 g((nrhs + CW - 1) / CW, batch);
-    k_trsm_blk<E><<<g, 32 * CW, 0, s>>>(A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs);
-    HS_COUNT_LAUNCH();
-    return;
+    switch (trsm_cw(nrhs, batch)) {
+      case 8: launch_trsm_blk<E, 8>(s, A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs, batch); return;
+      case 4: launch_trsm_blk<E, 4>(s, A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs, batch); return;
+      case 2: launch_trsm_blk<E, 2>(s, A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs, batch); return;
+      default: launch_trsm_blk<E, 1>(s, A, lda, sA, i0, nbs, mode, B, ldb, sB, nrhs, batch); return;
+    }
   }
   const E m1 = -el<E>::one(), one = el<E>::one();
   const int I1 = i0 + nbs;
-  if (mode == 0) {
+  const bool tr = mode >= 2;
+  if (mode == 0 || mode == 2) {
     for (int j = i0; j < I1; j += NB) {
       const int nb = std::min(NB, I1 - j);
-      trsm_diag<E>(s, A, lda, sA, j, nb, 0, B, ldb, sB, nrhs, batch);
+      trsm_diag<E>(s, A, lda, sA, j, nb, mode, B, ldb, sB, nrhs, batch);
       if (I1 - j - nb > 0)
-        gemm<E, E, E>(s, OP_N, OP_N, I1 - j - nb, nrhs, nb, m1, A + (long long)(j + nb) * lda + j, lda, sA,
+        gemm<E, E, E>(s, tr ? OP_T : OP_N, OP_N, I1 - j - nb, nrhs, nb, m1,
+                      tr ? A + (long long)j * lda + j + nb : A + (long long)(j + nb) * lda + j, lda, sA,
                       B + (long long)j * ldb, ldb, sB, one, B + (long long)(j + nb) * ldb, ldb, sB, batch);
     }
   } else {
     for (int j = i0 + ((nbs - 1) / NB) * NB; j >= i0; j -= NB) {
       const int nb = std::min(NB, I1 - j);
-      trsm_diag<E>(s, A, lda, sA, j, nb, 1, B, ldb, sB, nrhs, batch);
+      trsm_diag<E>(s, A, lda, sA, j, nb, mode, B, ldb, sB, nrhs, batch);
       if (j > i0)
-        gemm<E, E, E>(s, OP_N, OP_N, j - i0, nrhs, nb, m1, A + (long long)i0 * lda + j, lda, sA,
+        gemm<E, E, E>(s, tr ? OP_T : OP_N, OP_N, j - i0, nrhs, nb, m1,
+                      tr ? A + (long long)j * lda + i0 : A + (long long)i0 * lda + j, lda, sA,
                       B + (long long)j * ldb, ldb, sB, one, B + (long long)i0 * ldb, ldb, sB, batch);
     }
   }
@@ -626,6 +816,71 @@ __global__ void k_swaps(const int* piv, long long sP, int n, int reverse, E* B, 
 }  // namespace
 
 namespace {
+// Launch a small-tile product, k split over a cluster when splits > 1.
+template <typename TA, typename TB, typename TC, int TM, int TN>
+void launch_gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
+                 const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch, int splits) {
+  dim3 grid((n + TN - 1) / TN, (m + TM - 1) / TM, batch * splits);
+  if (splits == 1) {
+    k_gemm<TA, TB, TC, TM, TN><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
+                                                    sC, 1);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = splits;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_gemm<TA, TB, TC, TM, TN>, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C,
+                       ldc, sC, splits);
+  }
+  HS_COUNT_LAUNCH();
+}
+
+template <typename TA, typename TB, typename TC>
+void launch_dot(cudaStream_t s, int m, int n, int k, TC alpha, const TA* A, long long ai, long long ak, long long sA,
+                const TB* B, long long bk, long long bj, long long sB, TC beta, TC* C, long long ci, long long cj,
+                long long sC, int batch) {
+  const int nc = n >= 8 ? 8 : n >= 4 ? 4 : n >= 2 ? 2 : 1;
+  dim3 grid((m + DOT_WARPS - 1) / DOT_WARPS, (n + nc - 1) / nc, batch);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, 32 * DOT_WARPS, 0, s>>>(m, n, k, alpha, A, ai, ak, sA, B, bk, bj, sB, beta, C, ci, cj, sC);
+  };
+  if (nc == 8) go(k_gemm_dot<TA, TB, TC, 8>);
+  else if (nc == 4) go(k_gemm_dot<TA, TB, TC, 4>);
+  else if (nc == 2) go(k_gemm_dot<TA, TB, TC, 2>);
+  else go(k_gemm_dot<TA, TB, TC, 1>);
+  HS_COUNT_LAUNCH();
+}
+
+// FP64 tile edge and k splits: the pipe's time of the busiest SM (the SM's
+// CTAs share it, two thread-operations per clock) plus a latency per CTA.
+struct Fp64Tile { int t, splits; };
+Fp64Tile fp64_tile(int m, int n, int k, int batch, double fma) {
+  Fp64Tile best{64, 1};
+  double bt = 1e300;
+  for (int t : {64, 32, 16})
+    for (int sp = 1; sp <= (t == 64 ? 1 : kMaxCluster); ++sp) {
+      if (sp > 1 && (k / sp < 2 * BK || (long long)batch * sp > 65535)) break;
+      const double ctas = (double)((m + t - 1) / t) * ((n + t - 1) / t) * batch * sp;
+      const int kc = ((k + sp - 1) / sp + BK - 1) / BK * BK;
+      // the 64-wide tile has no such padding of k and better reuse when it fills the chip
+      const double one = (double)t * t * fma * (t == 64 ? (k + 7) / 8 * 8 : kc) / 2.0 + (sp > 1 ? 3000.0 : 1500.0);
+      if ((m + t - 1) / t > 65535) continue;  // grid.y
+      const double time = std::ceil(ctas / 152.0) * one * (t == 64 ? 1.0 : t == 32 ? 1.02 : 1.06);
+      if (time < bt) {
+        bt = time;
+        best = Fp64Tile{t, sp};
+      }
+    }
+  return best;
+}
+
 // SIMT product (FP64, or FP32 where the tensor-core path is not taken).
 template <typename TA, typename TB, typename TC>
 void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
@@ -633,9 +888,39 @@ void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, 
   const bool prof = prof_active(is_fp64<TC>::v ? 1 : 2);
   cudaEvent_t ev = nullptr;
   if (prof) prof_begin(s, &ev);
+  const double fl = flops_per_mac<TA, TB>() * (double)m * n * k * batch;
+  // few columns or rows: dot products (grid limits: rows / 4 in x, batch in z)
+  if (std::min(m, n) <= 8 && batch <= 65535) {
+    const long long ai = opA == OP_N ? lda : 1, ak = opA == OP_N ? 1 : lda;
+    const long long bk = opB == OP_N ? ldb : 1, bj = opB == OP_N ? 1 : ldb;
+    if (n <= m)
+      launch_dot<TA, TB, TC>(s, m, n, k, alpha, A, ai, ak, sA, B, bk, bj, sB, beta, C, ldc, 1, sC, batch);
+    else
+      launch_dot<TB, TA, TC>(s, n, m, k, alpha, B, bj, bk, sB, A, ak, ai, sA, beta, C, 1, ldc, sC, batch);
+    if (prof) prof_end(s, ev, fl);
+    return;
+  }
+  if constexpr (is_fp64<TC>::v) {
+    const Fp64Tile t = fp64_tile(m, n, k, batch, flops_per_mac<TA, TB>() / 2.0);
+    if (t.t != 64) {
+      if (t.t == 32)
+        launch_gemm<TA, TB, TC, 32, 32>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
+                                        t.splits);
+      else
+        launch_gemm<TA, TB, TC, 16, 16>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
+                                        t.splits);
+      if (prof) prof_end(s, ev, fl);
+      return;
+    }
+    dim3 grid((n + GB - 1) / GB, (m + GB - 1) / GB, batch);
+    k_gemm_big<TA, TB, TC><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, 1);
+    HS_COUNT_LAUNCH();
+    if (prof) prof_end(s, ev, fl);
+    return;
+  }
   constexpr long long kFill = 2 * 152;  // tiles that keep every SM of the chip busy
   const long long t64 = (long long)((m + GB - 1) / GB) * ((n + GB - 1) / GB) * batch;
-  const long long t32 = (long long)((m + BM - 1) / BM) * ((n + BN - 1) / BN) * batch;
+  const long long t32 = (long long)((m + 31) / 32) * ((n + 31) / 32) * batch;
   // 64 x 64 tiles (twice the arithmetic per shared-memory load) when they fill the
   // chip, for matrices of at least one tile each way or with at least 60% of
   // the tiles' outputs inside the matrix (e.g. 56-row blocks)
@@ -685,7 +970,7 @@ void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, 
                              sC, splits64);
         }
         HS_COUNT_LAUNCH();
-        if (prof) prof_end(s, ev, flops_per_mac<TA, TB>() * (double)m * n * k * batch);
+        if (prof) prof_end(s, ev, fl);
         return;
       }
     }
@@ -715,27 +1000,10 @@ void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, 
       splits = std::max(1, std::min(splits, kMaxCluster));
       if ((long long)batch * splits > 65535) splits = 1;
     }
-    dim3 grid((n + BN - 1) / BN, (m + BM - 1) / BM, batch * splits);
-    if (splits == 1) {
-      k_gemm<TA, TB, TC><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, 1);
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid;
-      cfg.blockDim = dim3(256);
-      cfg.stream = s;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 1;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = splits;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      cudaLaunchKernelEx(&cfg, k_gemm<TA, TB, TC>, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC,
-                         splits);
-    }
-    HS_COUNT_LAUNCH();
+    launch_gemm<TA, TB, TC, 32, 32>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
+                                    splits);
   }
-  if (prof) prof_end(s, ev, flops_per_mac<TA, TB>() * (double)m * n * k * batch);
+  if (prof) prof_end(s, ev, fl);
 }
 
 // Products the split-TF32 tensor-core path takes (t32_gemm modes): complex x
@@ -937,21 +1205,20 @@ void lu_solve(cudaStream_t s, int trans, const E* A, int lda, long long sA, int 
                       ldb, sB, batch);
     }
   } else {
-    for (int i0 = 0; i0 < n; i0 += NB) {  // U^T y = b
-      int nb = n - i0 < NB ? n - i0 : NB;
-      trsm_diag<E>(s, A, lda, sA, i0, nb, 2, B, ldb, sB, nrhs, batch);
-      int rest = n - i0 - nb;
-      if (rest > 0)
-        gemm<E, E, E>(s, OP_T, OP_N, rest, nrhs, nb, m1, A + (long long)i0 * lda + i0 + nb, lda, sA,
-                      B + (long long)i0 * ldb, ldb, sB, one, B + (long long)(i0 + nb) * ldb, ldb, sB, batch);
+    for (int I0 = 0; I0 < n; I0 += NBB) {  // U^T y = b
+      const int I1 = std::min(n, I0 + NBB);
+      trsm_blk<E>(s, A, lda, sA, I0, I1 - I0, 2, B, ldb, sB, nrhs, batch);
+      if (n - I1 > 0)
+        gemm<E, E, E>(s, OP_T, OP_N, n - I1, nrhs, I1 - I0, m1, A + (long long)I0 * lda + I1, lda, sA,
+                      B + (long long)I0 * ldb, ldb, sB, one, B + (long long)I1 * ldb, ldb, sB, batch);
     }
-    int last = ((n - 1) / NB) * NB;
-    for (int i0 = last; i0 >= 0; i0 -= NB) {  // L^T w = y
-      int nb = n - i0 < NB ? n - i0 : NB;
-      trsm_diag<E>(s, A, lda, sA, i0, nb, 3, B, ldb, sB, nrhs, batch);
-      if (i0 > 0)
-        gemm<E, E, E>(s, OP_T, OP_N, i0, nrhs, nb, m1, A + (long long)i0 * lda, lda, sA, B + (long long)i0 * ldb, ldb,
-                      sB, one, B, ldb, sB, batch);
+    const int lastB = ((n - 1) / NBB) * NBB;
+    for (int I0 = lastB; I0 >= 0; I0 -= NBB) {  // L^T w = y
+      const int I1 = std::min(n, I0 + NBB);
+      trsm_blk<E>(s, A, lda, sA, I0, I1 - I0, 3, B, ldb, sB, nrhs, batch);
+      if (I0 > 0)
+        gemm<E, E, E>(s, OP_T, OP_N, I0, nrhs, I1 - I0, m1, A + (long long)I0 * lda, lda, sA, B + (long long)I0 * ldb,
+                      ldb, sB, one, B, ldb, sB, batch);
     }
     k_swaps<E><<<gs, 128, 0, s>>>(piv, sP, n, 1, B, ldb, sB, nrhs);
     HS_COUNT_LAUNCH();
