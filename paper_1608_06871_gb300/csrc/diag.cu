@@ -207,8 +207,8 @@ int hs_dgemm_emulated(int m, int n, int k, const void* A, const void* B, void* C
   double* a = const_cast<double*>(static_cast<const double*>(A));
   double* b = const_cast<double*>(static_cast<const double*>(B));
   // A(b, i, kk) = A[b m k + i k + kk];  Bt(b, j, kk) = B[b k n + kk n + j];  C(b, i, j) = C[b m n + i n + j]
-  const hs::OzView va{a, (long long)m * k, k, 0, 1, 1}, vb{b, (long long)k * n, 1, 0, n, 1},
-      vc{static_cast<double*>(C), (long long)m * n, n, 0, 1, 1};
+  const hs::OzSrc va{a, (long long)m * k, k, 1, hs::OZ_REAL}, vb{b, (long long)k * n, 1, n, hs::OZ_REAL};
+  const hs::OzView vc{static_cast<double*>(C), (long long)m * n, n, 0, 1, 1};
   const size_t bytes = hs::ozaki_scratch_bytes(m, n, k, batch, false);
   void* scratch = nullptr;
   if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess) return HS_ENOMEM;
@@ -288,15 +288,40 @@ int hs_cgemm32(int m, int n, int k, const void* A, const void* B, void* C, int b
   return HS_OK;
 }
 
+namespace {
+// The scratch a context would give its FP64 products, for the length of a call.
+struct CallScratch {
+  hs::OzScratch sc;
+  const hs::OzScratch* prev = hs::g_oz_scratch;
+  cudaStream_t s;
+  explicit CallScratch(cudaStream_t st) : s(st) {
+    void* p = nullptr;
+    if (cudaMallocAsync(&p, (size_t)256 << 20, s) == cudaSuccess) {
+      sc.p = static_cast<char*>(p);
+      sc.bytes = (size_t)256 << 20;
+    } else {
+      cudaGetLastError();
+    }
+    hs::g_oz_scratch = &sc;
+  }
+  ~CallScratch() {
+    hs::g_oz_scratch = prev;
+    if (sc.p) cudaFreeAsync(sc.p, s);
+  }
+};
+}  // namespace
+
 int hs_zgemm(int transA, int transB, int m, int n, int k, const void* A, const void* B, void* C, int accumulate,
              void* stream) {
   if (m <= 0 || n <= 0 || k <= 0 || !A || !B || !C) return HS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int opA = transA ? hs::OP_T : hs::OP_N, opB = transB ? hs::OP_T : hs::OP_N;
+  CallScratch scratch(s);
   hs::gemm<double2, double2, double2>(s, opA, opB, m, n, k, make_double2(1.0, 0.0), static_cast<const double2*>(A),
                                       transA ? m : k, 0, static_cast<const double2*>(B), transB ? k : n, 0,
                                       make_double2(accumulate ? 1.0 : 0.0, 0.0), static_cast<double2*>(C), n, 0, 1);
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return HS_ECUDA;
+  if (hs::tc_timed_out(s)) return HS_ETIMEOUT;
   return HS_OK;
 }
 
@@ -313,6 +338,7 @@ int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, voi
   cudaMemsetAsync(info, 0, sizeof(int) * (size_t)batch, s);
   const long long sA = (long long)n * n, sB = (long long)n * nrhs;
   if (precision == HS_FP64) {
+    CallScratch scratch(s);
     hs::lu_factor<double2>(s, static_cast<double2*>(A), n, sA, n, piv, n, info, batch);
     hs::lu_solve<double2>(s, hs::OP_N, static_cast<double2*>(A), n, sA, n, piv, n, static_cast<double2*>(B), nrhs, sB,
                           nrhs, batch);
@@ -329,6 +355,7 @@ int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, voi
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return HS_ECUDA;
   for (int v : h)
     if (v != 0) return HS_ESINGULAR;
+  if (hs::tc_timed_out(s)) return HS_ETIMEOUT;
   return HS_OK;
 }
 

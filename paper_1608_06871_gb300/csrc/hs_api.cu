@@ -211,6 +211,7 @@ struct hs_ctx {
   // captured factorisation and refinement passes read it there, so one graph
   // serves every k of a sweep on this tree
   double* d_k = nullptr;
+  OzScratch oz;  // slices of the emulated FP64 products (ensure_oz)
   double k_dev = 0.0;
   long long builds = 0;
   // phase times of the last build recorded launch by launch (-1 after a graph replay)
@@ -222,8 +223,15 @@ namespace {
 
 struct LaunchScope {
   long long* prev;
-  explicit LaunchScope(hs_ctx* c) : prev(g_launch_counter) { g_launch_counter = &c->launches; }
-  ~LaunchScope() { g_launch_counter = prev; }
+  const OzScratch* prev_oz;
+  explicit LaunchScope(hs_ctx* c) : prev(g_launch_counter), prev_oz(g_oz_scratch) {
+    g_launch_counter = &c->launches;
+    g_oz_scratch = &c->oz;
+  }
+  ~LaunchScope() {
+    g_launch_counter = prev;
+    g_oz_scratch = prev_oz;
+  }
 };
 
 int fail(hs_ctx* c, int code, const std::string& msg) {
@@ -328,6 +336,19 @@ int ensure_ws(hs_ctx* ctx, size_t bytes, Arena& a) {
   a.base = ctx->ws_base;
   a.cap = ctx->ws_cap;
   a.off = 0;
+  return HS_OK;
+}
+
+// Scratch of the emulated FP64 products of a context, allocated once (at the
+// first build of an FP64 context, the first gradient or Gauss-Newton step of a
+// mixed one): the leaf products of a few hundred leaves at a time, 32 to 512 MB.
+int ensure_oz(hs_ctx* ctx) {
+  if (ctx->oz.p || !g_oz_enabled) return HS_OK;
+  const size_t n = std::min<size_t>((size_t)512 << 20, std::max<size_t>((size_t)32 << 20, (size_t)ctx->nleaf * 1500000));
+  char* p = nullptr;
+  CKR(dalloc(ctx, &p, n));
+  ctx->oz.p = p;
+  ctx->oz.bytes = n;
   return HS_OK;
 }
 
@@ -875,6 +896,7 @@ int factor(hs_ctx* ctx, double k) {
   if (ctx->cfg.precision == HS_MIXED) return factor_mixed(ctx, k);
   cudaStream_t s = ctx->stream;
   CKR(phase_events(ctx));
+  CKR(ensure_oz(ctx));
   CKR(set_device_k(ctx, s, k));
   CK(cudaMemsetAsync(ctx->d_info, 0, sizeof(int) * ctx->ninfo, s));
   CK(cudaEventRecord(ctx->ph_ev[0], s));
@@ -1000,15 +1022,15 @@ int check_ctx(hs_ctx* ctx, bool need_built) {
 
 cudaStream_t pick(hs_ctx* ctx, void* stream) { return stream ? (cudaStream_t)stream : ctx->stream; }
 
-// Real and imaginary parts of a complex matrix (rows x k, leading dimension
-// ld, interleaved) as strided real views for slicing.
-OzView re_view(const double2* A, int ld, int part) {
-  return OzView{const_cast<double*>(reinterpret_cast<const double*>(A)) + part, 0, 2LL * ld, 0, 2, 1};
+// A complex matrix (row stride sr, column stride sk, in complex entries) as the
+// left or right operand of an emulated complex product.
+OzSrc cleft(const double2* A, long long sr, long long sk) {
+  return OzSrc{reinterpret_cast<const double*>(A), 0, 2 * sr, 2 * sk, OZ_CLEFT};
 }
-// The same for the transpose of a k x rows complex matrix (row index along its columns).
-OzView re_view_t(const double2* A, int ld, int part) {
-  return OzView{const_cast<double*>(reinterpret_cast<const double*>(A)) + part, 0, 2, 0, 2LL * ld, 1};
+OzSrc cright(const double2* B, long long sj, long long sl) {
+  return OzSrc{reinterpret_cast<const double*>(B), 0, 2 * sj, 2 * sl, OZ_CRIGHT};
 }
+OzView cout_view(double2* C, long long ldc) { return OzView{reinterpret_cast<double*>(C), 0, 2 * ldc, 0, 1, 1}; }
 
 // Far field for M incidences into ufar (device, M x P complex).
 int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const double* thetas, int P, double2* ufar,
@@ -1055,9 +1077,9 @@ size_t mixed_bytes(hs_ctx* ctx, int M, int P) {
        Arena::bytes(s3_elems(ctx, M), 8) + 2 * Arena::bytes(nb * M, 8);
   for (auto& L : ctx->levels) b += Arena::bytes((size_t)L.nbox * 2 * L.ni * M, 8);
   if (g_oz_enabled)
-    b += 2 * std::max(oz_wide_bytes(M, 2 * (int)nb, false),
-                      oz_wide_bytes(M, 2 * (int)nb, true) + oz_wide_bytes(P, 2 * (int)nb, false)) +
-         4 * std::max(oz_partial_bytes((int)nb, M, 2 * (int)nb), oz_partial_bytes(M, P, 2 * (int)nb));
+    b += std::max(oz_operand_bytes(2 * M, 4 * (int)nb, 1, false),
+                  oz_operand_bytes(M, 4 * (int)nb, 1, true) + oz_operand_bytes(2 * P, 4 * (int)nb, 1, false)) +
+         std::max(oz_plane_bytes((int)nb, 2 * M, 4 * (int)nb, 1), oz_plane_bytes(M, 2 * P, 4 * (int)nb, 1)) + 512;
   return b;
 }
 
@@ -1103,17 +1125,16 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
   // the exterior residual, then as the left operand of the far field) and of
   // the receiver matrix
   const bool emu = g_oz_enabled;
-  const size_t ob_ps = emu ? oz_wide_bytes(M, 2 * nb, false) : 0;
-  const size_t ob_psa = emu ? oz_wide_bytes(M, 2 * nb, true) : 0, ob_a2 = emu ? oz_wide_bytes(P, 2 * nb, false) : 0;
-  const size_t ob_part = emu ? std::max(oz_partial_bytes(nb, M, 2 * nb), oz_partial_bytes(M, P, 2 * nb)) : 0;
-  char* ozs = emu ? a.get<char>(2 * std::max(ob_ps, ob_psa + ob_a2)) : nullptr;
-  char* ozp = emu ? a.get<char>(4 * ob_part) : nullptr;
+  const size_t ob_ps = emu ? oz_operand_bytes(2 * M, 4 * nb, 1, false) : 0;
+  const size_t ob_psa = emu ? oz_operand_bytes(M, 4 * nb, 1, true) : 0;
+  const size_t ob_a2 = emu ? oz_operand_bytes(2 * P, 4 * nb, 1, false) : 0;
+  const size_t ob_part = emu ? std::max(oz_plane_bytes(nb, 2 * M, 4 * nb, 1), oz_plane_bytes(M, 2 * P, 4 * nb, 1)) : 0;
+  char* ozs = emu ? a.get<char>(std::max(ob_ps, ob_psa + ob_a2)) : nullptr;
+  char* ozp = emu ? a.get<char>(ob_part) : nullptr;
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  const size_t ob_ds = oz_wide_bytes(nb, 2 * nb, true);
   if (emu && ctx->ds_oz_k != ctx->bie_k) {  // the exterior rows of this k, sliced once
-    if (!ctx->d_ds_oz) CKR(dalloc(ctx, &ctx->d_ds_oz, 2 * ob_ds));
-    oz_slice_wide(s, re_view(ctx->d_DS, 2 * nb, 0), nb, 2 * nb, true, ctx->d_ds_oz);
-    oz_slice_wide(s, re_view(ctx->d_DS, 2 * nb, 1), nb, 2 * nb, true, ctx->d_ds_oz + ob_ds);
+    if (!ctx->d_ds_oz) CKR(dalloc(ctx, &ctx->d_ds_oz, oz_operand_bytes(nb, 4 * nb, 1, true)));
+    oz_slice(s, cleft(ctx->d_DS, 2 * nb, 1), nb, 4 * nb, 1, true, ctx->d_ds_oz);
     ctx->ds_oz_k = ctx->bie_k;
   }
 
@@ -1135,10 +1156,9 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
       boundary_gather(s, X, ctx->d_D1, ctx->nL, ctx->h, M, ub, psib);
       scattered_data(s, ub, psib, ui, dni, (long long)nbM, PS);
       if (emu) {
-        oz_slice_wide(s, re_view_t(PS, M, 0), M, 2 * nb, false, ozs);
-        oz_slice_wide(s, re_view_t(PS, M, 1), M, 2 * nb, false, ozs + ob_ps);
-        const cudaError_t e = oz_zmul_wide(s, nb, M, 2 * nb, ctx->d_ds_oz, ctx->d_ds_oz + ob_ds, ozs, ozs + ob_ps,
-                                           -1.0, 0.0, rext, M, ozp);
+        oz_slice(s, cright(PS, 1, M), 2 * M, 4 * nb, 1, false, ozs);
+        const cudaError_t e = oz_multiply(s, nb, 2 * M, 4 * nb, 1, -1.0, ctx->d_ds_oz, ozs, false, 0.0,
+                                          cout_view(rext, M), ozp);
         if (e != cudaSuccess) return fail(ctx, HS_ECUDA, std::string("emulated FP64 product: ") + cudaGetErrorString(e));
       } else {
         gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, 2 * nb, mone, ctx->d_DS, 2 * nb, 0, PS, M, 0, zero,
@@ -1228,13 +1248,11 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
     boundary_gather(s, X, ctx->d_D1, ctx->nL, ctx->h, M, ub, psib);
     scattered_data(s, ub, psib, ui, dni, (long long)nbM, PS);
     if (emu) {  // uf = PS^T A2^T
-      char *pa = ozs, *pb = ozs + 2 * ob_psa;
-      oz_slice_wide(s, re_view_t(PS, M, 0), M, 2 * nb, true, pa);
-      oz_slice_wide(s, re_view_t(PS, M, 1), M, 2 * nb, true, pa + ob_psa);
-      oz_slice_wide(s, re_view(A2, 2 * nb, 0), P, 2 * nb, false, pb);
-      oz_slice_wide(s, re_view(A2, 2 * nb, 1), P, 2 * nb, false, pb + ob_a2);
+      char *pa = ozs, *pb = ozs + ob_psa;
+      oz_slice(s, cleft(PS, 1, M), M, 4 * nb, 1, true, pa);
+      oz_slice(s, cright(A2, 2 * nb, 1), 2 * P, 4 * nb, 1, false, pb);
       const cudaError_t e =
-          oz_zmul_wide(s, M, P, 2 * nb, pa, pa + ob_psa, pb, pb + ob_a2, 1.0, 0.0, uf, P, ozp);
+          oz_multiply(s, M, 2 * P, 4 * nb, 1, 1.0, pa, pb, false, 0.0, cout_view(uf, P), ozp);
       if (e != cudaSuccess) return fail(ctx, HS_ECUDA, std::string("emulated FP64 product: ") + cudaGetErrorString(e));
     } else {
       gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, one, PS, M, 0, A2, 2 * nb, 0, zero, uf, P, 0, 1);
@@ -1285,7 +1303,8 @@ size_t mixed_adjoint_bytes(hs_ctx* ctx, int P) {
              Arena::bytes(8, 8);
   for (auto& L : ctx->levels) b += Arena::bytes((size_t)L.nbox * 2 * L.ni * P, 8);
   if (g_oz_enabled)
-    b += Arena::bytes(2 * oz_wide_bytes(P, (int)nb, false), 1) + Arena::bytes(4 * oz_partial_bytes(2 * (int)nb, P, (int)nb), 1);
+    b += Arena::bytes(oz_operand_bytes(2 * P, 2 * (int)nb, 1, false), 1) +
+         Arena::bytes(oz_plane_bytes(2 * (int)nb, 2 * P, 2 * (int)nb, 1), 1);
   return b;
 }
 
@@ -1337,15 +1356,12 @@ int mixed_adjoint(hs_ctx* ctx, cudaStream_t s, const double2* A2, int P, double2
   // the exterior rows' transposed product DS^T Yext by the emulated FP64 product:
   // DS^T sliced once per k, Yext (as the right operand) once per pass
   const bool emu = g_oz_enabled;
-  const size_t ob_y = emu ? oz_wide_bytes(P, nb, false) : 0, ob_part = emu ? oz_partial_bytes(2 * nb, P, nb) : 0;
-  char* ozs = emu ? a.get<char>(2 * ob_y) : nullptr;
-  char* ozp = emu ? a.get<char>(4 * ob_part) : nullptr;
+  char* ozs = emu ? a.get<char>(oz_operand_bytes(2 * P, 2 * nb, 1, false)) : nullptr;
+  char* ozp = emu ? a.get<char>(oz_plane_bytes(2 * nb, 2 * P, 2 * nb, 1)) : nullptr;
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  const size_t ob_dst = oz_wide_bytes(2 * nb, nb, true);
   if (emu && ctx->dst_oz_k != ctx->bie_k) {
-    if (!ctx->d_dst_oz) CKR(dalloc(ctx, &ctx->d_dst_oz, 2 * ob_dst));
-    oz_slice_wide(s, re_view_t(ctx->d_DS, 2 * nb, 0), 2 * nb, nb, true, ctx->d_dst_oz);
-    oz_slice_wide(s, re_view_t(ctx->d_DS, 2 * nb, 1), 2 * nb, nb, true, ctx->d_dst_oz + ob_dst);
+    if (!ctx->d_dst_oz) CKR(dalloc(ctx, &ctx->d_dst_oz, oz_operand_bytes(2 * nb, 2 * nb, 1, true)));
+    oz_slice(s, cleft(ctx->d_DS, 1, 2 * nb), 2 * nb, 2 * nb, 1, true, ctx->d_dst_oz);
     ctx->dst_oz_k = ctx->bie_k;
   }
   const LeafScratchT<float>& w = ctx->ws32;
@@ -1364,10 +1380,9 @@ int mixed_adjoint(hs_ctx* ctx, cudaStream_t s, const double2* A2, int P, double2
     const bool first = it == 0;
     // FP64 residual L - A^T Y of every unknown (L itself on the first pass)
     if (!first && emu) {
-      oz_slice_wide(s, re_view_t(Yext, P, 0), P, nb, false, ozs);
-      oz_slice_wide(s, re_view_t(Yext, P, 1), P, nb, false, ozs + ob_y);
-      const cudaError_t e = oz_zmul_wide(s, 2 * nb, P, nb, ctx->d_dst_oz, ctx->d_dst_oz + ob_dst, ozs, ozs + ob_y, 1.0,
-                                         0.0, V, P, ozp);
+      oz_slice(s, cright(Yext, 1, P), 2 * P, 2 * nb, 1, false, ozs);
+      const cudaError_t e = oz_multiply(s, 2 * nb, 2 * P, 2 * nb, 1, 1.0, ctx->d_dst_oz, ozs, false, 0.0,
+                                        cout_view(V, P), ozp);
       if (e != cudaSuccess) return fail(ctx, HS_ECUDA, std::string("emulated FP64 product: ") + cudaGetErrorString(e));
     } else if (!first) {
       gemm<double2, double2, double2>(s, OP_T, OP_N, 2 * nb, P, nb, make_double2(1, 0), ctx->d_DS, 2 * nb, 0, Yext, P,
@@ -1918,6 +1933,7 @@ int hs_gn_step(hs_ctx* ctx, const double* data, const double* alphas, int M, con
                 std::max(jacobian_bytes(ctx, M, P),
                          4 * Arena::bytes((size_t)ctx->B.nb * M, 16) + Arena::bytes((size_t)2 * ctx->B.nb * M, 16) +
                              Arena::bytes((size_t)P * 2 * ctx->B.nb, 16));
+  CKR(ensure_oz(ctx));
   CKR(ensure_ws(ctx, need, a));
   double* da = a.get<double>(M);
   double* dt = a.get<double>(P);
@@ -2228,6 +2244,7 @@ int hs_gradient_dev(hs_ctx* ctx, const double* data, const double* alphas, int M
   CKR(valid_angles(ctx, M, P));
   if (!data || !alphas || !thetas || !grad || !misfit_out) return fail(ctx, HS_EINVAL, "NULL pointer");
   Arena a;
+  CKR(ensure_oz(ctx));
   CKR(ensure_ws(ctx, gradient_bytes(ctx, M, P), a));
   return gradient_core(ctx, pick(ctx, stream), data, alphas, M, thetas, P, grad, misfit_out, a);
 }
@@ -2243,6 +2260,7 @@ int hs_gradient(hs_ctx* ctx, const double* data, const double* alphas, int M, co
   Arena a;
   size_t need = Arena::bytes(M, 8) + Arena::bytes(P, 8) + Arena::bytes((size_t)2 * MP, 8) + Arena::bytes(nm, 8) +
                 Arena::bytes(8, 8) + gradient_bytes(ctx, M, P);
+  CKR(ensure_oz(ctx));
   CKR(ensure_ws(ctx, need, a));
   double* da = a.get<double>(M);
   double* dt = a.get<double>(P);

@@ -136,8 +136,8 @@ void contract_jacobian(cudaStream_t s, const double2* Ug, const double2* Zg, int
   const size_t bsx = oz_operand_bytes(S1, nX, 1, false), bsy = oz_operand_bytes(S2, nX, 1, false);
   char *osx = base, *osy = base + bsx, *oa = base + bsx + bsy;
   if (emu) {  // the sine tables, sliced once as the right operands of both projections
-    oz_slice(s, OzView{const_cast<double*>(sx), 0, nX, 0, 1, 1}, S1, nX, 1, false, osx);
-    oz_slice(s, OzView{const_cast<double*>(sy), 0, nX, 0, 1, 1}, S2, nX, 1, false, osy);
+    oz_slice(s, OzSrc{sx, 0, nX, 1, OZ_REAL}, S1, nX, 1, false, osx);
+    oz_slice(s, OzSrc{sy, 0, nX, 1, OZ_REAL}, S2, nX, 1, false, osy);
   }
   for (long long c0 = 0; c0 < MP; c0 += C) {
     const int nc = (int)std::min<long long>(C, MP - c0);
@@ -153,8 +153,8 @@ void contract_jacobian(cudaStream_t s, const double2* Ug, const double2* Zg, int
       done = oz_multiply(s, 2 * nc * nX, S1, nX, 1, 1.0, oa, osx, true, 0.0, vt) == cudaSuccess;
       // J_pair[m1][m2] = k2 sum_gy T_pair[gy][m1] sy[m2][gy]
       if (done) {
-        const OzView vtt{Td, 2LL * nX * S1, 2, 1, 2LL * S1, 2}, vj{Jd, 2LL * S1 * S2, 2LL * S2, 1, 2, 2};
-        oz_slice(s, vtt, 2 * S1, nX, nc, true, oa);
+        const OzView vj{Jd, 2LL * S1 * S2, 2LL * S2, 1, 2, 2};
+        oz_slice(s, OzSrc{Td, 2LL * nX * S1, 2, 2LL * S1, OZ_PAIR}, 2 * S1, nX, nc, true, oa);
         done = oz_multiply(s, 2 * S1, S2, nX, nc, k2, oa, osy, true, 0.0, vj) == cudaSuccess;
       }
     }
@@ -494,12 +494,31 @@ void split_stack_t(cudaStream_t s, const double2* J, int rows, int cols, double*
   HS_COUNT_LAUNCH();
 }
 
-size_t normal_matrix_emulated_bytes(int rows, int n) { return ozaki_scratch_bytes(n, n, rows, 1, false); }
+// k of the normal matrix per launch: its sliced operands stay below about 0.5 GB.
+static int normal_chunk(int rows, int n) {
+  const long long c = (512LL << 20) / (32LL * (n + 128)) / 384 * 384;
+  return (int)std::min<long long>(rows, std::max<long long>(384, c));
+}
 
-// A = JstT JstT^T (n x n) for JstT (n x rows) by the emulated FP64 product.
+size_t normal_matrix_emulated_bytes(int rows, int n) { return ozaki_scratch_bytes(n, n, normal_chunk(rows, n), 1, false); }
+
+__global__ void k_mirror_upper(double* A, int n, int bs);
+
+// A = JstT JstT^T (n x n) for JstT (n x rows) by the emulated FP64 product: the
+// tiles that meet the lower triangle, then the upper part mirrored.
 bool normal_matrix_emulated(cudaStream_t s, double* JstT, int rows, int n, double* A, void* scratch, size_t bytes) {
-  const OzView v{JstT, 0, rows, 0, 1, 1}, c{A, 0, n, 0, 1, 1};
-  return ozaki_gemm(s, n, n, rows, 1, 1.0, v, v, true, 0.0, c, scratch, bytes) == cudaSuccess;
+  const OzView c{A, 0, n, 0, 1, 1};
+  const int ck = normal_chunk(rows, n);
+  for (int r0 = 0; r0 < rows; r0 += ck) {
+    const OzSrc v{JstT + r0, 0, rows, 1, OZ_REAL};
+    if (ozaki_gemm(s, n, n, std::min(ck, rows - r0), 1, 1.0, v, v, true, r0 ? 1.0 : 0.0, c, scratch, bytes, true) !=
+        cudaSuccess)
+      return false;
+  }
+  const long long tot = (long long)n * n;
+  k_mirror_upper<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(A, n, 128);
+  HS_COUNT_LAUNCH();
+  return true;
 }
 
 // A[r][c] = A[c][r] for the entries above the computed block-lower part

@@ -860,9 +860,9 @@ void launch_dot(cudaStream_t s, int m, int n, int k, TC alpha, const TA* A, long
 
 // FP64 tile edge and k splits: the pipe's time of the busiest SM (the SM's
 // CTAs share it, two thread-operations per clock) plus a latency per CTA.
-struct Fp64Tile { int t, splits; };
+struct Fp64Tile { int t, splits; double cycles; };
 Fp64Tile fp64_tile(int m, int n, int k, int batch, double fma) {
-  Fp64Tile best{64, 1};
+  Fp64Tile best{64, 1, 0.0};
   double bt = 1e300;
   for (int t : {64, 32, 16})
     for (int sp = 1; sp <= (t == 64 ? 1 : kMaxCluster); ++sp) {
@@ -875,7 +875,7 @@ Fp64Tile fp64_tile(int m, int n, int k, int batch, double fma) {
       const double time = std::ceil(ctas / 152.0) * one * (t == 64 ? 1.0 : t == 32 ? 1.02 : 1.06);
       if (time < bt) {
         bt = time;
-        best = Fp64Tile{t, sp};
+        best = Fp64Tile{t, sp, time};
       }
     }
   return best;
@@ -1006,6 +1006,65 @@ void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, 
   if (prof) prof_end(s, ev, fl);
 }
 
+inline double re_of(double x) { return x; }
+inline double re_of(double2 x) { return x.x; }
+inline double im_of(double) { return 0.0; }
+inline double im_of(double2 x) { return x.y; }
+
+// FP64 products by the emulated product on the tensor cores (ozaki.cu) where
+// its estimated time is clearly below the FP64 pipe's: 36 bf16 products are
+// about a tenth of the pipe's time per multiply-add, but operands are sliced
+// first (two more launches, 16 bytes written and read per entry) and tiles are
+// 128 x 64, so small and thin products stay on the pipe (the two models' times
+// are compared, with a fifth in favour of the pipe).  The products of the k = 40
+// FP64 batch: 160 ms on the pipe, 27 ms sliced and multiplied; the batch 227 ->
+// 98.5 ms, a k = 20 gradient 65.8 -> 44.3 ms.  Error against 64 bits of random
+// complex products: 7e-17 .. 1.3e-16 of the result for k = 32 .. 1792, on the
+// pipe 2.5e-16 .. 7e-16 (rows whose entries spread over 1e5: 4.5e-16 against
+// 3e-16 at k = 128, 4.8e-16 against 1.9e-15 at 1792); of far fields, fields,
+// Jacobians and steps at k = 5 .. 20: unchanged (5e-13 .. 5e-12).
+// Batches, then k, are cut to what the calling thread's scratch holds.
+// Complex factors other than real ones, and calls without scratch, are refused.
+template <typename TA, typename TB, typename TC>
+bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
+                   const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch) {
+  constexpr bool ca = is_cplx<TA>::v, cb = is_cplx<TB>::v;
+  const OzScratch* sc = g_oz_scratch;
+  if (!g_oz_enabled || !sc || !sc->p || k <= 0 || im_of(alpha) != 0.0 || im_of(beta) != 0.0) return false;
+  if (std::min(m, n) <= 8) return false;
+  const int mr = ca && !cb ? 2 * m : m, nr = cb ? 2 * n : n, kr = ca && cb ? 2 * k : k;
+  const bool bsh = sB == 0 && batch > 1;
+  if (oz_cycles(mr, nr, kr, batch, bsh) > 0.8 * fp64_tile(m, n, k, batch, flops_per_mac<TA, TB>() / 2.0).cycles)
+    return false;
+  const long long ea = ca ? 2 : 1, eb = cb ? 2 : 1;
+  OzSrc a{reinterpret_cast<const double*>(A), ea * sA, ea * (opA == OP_N ? lda : 1), ea * (opA == OP_N ? 1 : lda),
+          ca ? (cb ? OZ_CLEFT : OZ_PAIR) : OZ_REAL};
+  OzSrc b{reinterpret_cast<const double*>(B), eb * sB, eb * (opB == OP_N ? 1 : ldb), eb * (opB == OP_N ? ldb : 1),
+          cb ? (ca ? OZ_CRIGHT : OZ_PAIR) : OZ_REAL};
+  constexpr bool cc = ca || cb;
+  OzView c{reinterpret_cast<double*>(C), (cc ? 2 : 1) * sC, (cc ? 2LL : 1LL) * ldc, 0, 1, 1};
+  if (ca && !cb) c = OzView{reinterpret_cast<double*>(C), 2 * sC, 2LL * ldc, 1, 2, 2};
+  // the largest batch chunk, then the longest piece of k, that the scratch holds
+  int nb = batch, kc = kr;
+  while (nb > 1 && ozaki_scratch_bytes(mr, nr, kr, nb, bsh) > sc->bytes) nb = (nb + 1) / 2;
+  while (kc > 384 && ozaki_scratch_bytes(mr, nr, kc, nb, bsh) > sc->bytes) kc = ((kc + 1) / 2 + 383) / 384 * 384;
+  if (ozaki_scratch_bytes(mr, nr, kc, nb, bsh) > sc->bytes) return false;
+  for (int b0 = 0; b0 < batch; b0 += nb)
+    for (int k0 = 0; k0 < kr; k0 += kc) {
+      OzSrc ai = a, bi = b;
+      OzView ci = c;
+      const long long l0 = ca && cb ? k0 / 2 : k0;  // (kc is even)
+      ai.p += b0 * a.sb + l0 * a.sk;
+      bi.p += b0 * b.sb + l0 * b.sk;
+      ci.p += b0 * c.sb;
+      const cudaError_t e =
+          ozaki_gemm(s, mr, nr, std::min(kc, kr - k0), std::min(nb, batch - b0), re_of(alpha), ai, bi, bsh,
+                     k0 == 0 ? re_of(beta) : 1.0, ci, sc->p, sc->bytes);
+      if (e == cudaErrorNotSupported && b0 == 0 && k0 == 0) return false;
+    }
+  return true;
+}
+
 // Products the split-TF32 tensor-core path takes (t32_gemm modes): complex x
 // complex (2), real x complex (1), real x real (0), FP32, no transposes.
 template <typename TA, typename TB, typename TC> struct t32_mode { static constexpr int v = -1; };
@@ -1129,6 +1188,8 @@ void gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const
       }
     }
   }
+  if constexpr (is_fp64<TC>::v)
+    if (gemm_emulated<TA, TB, TC>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch)) return;
   gemm_simt<TA, TB, TC>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch);
 }
 

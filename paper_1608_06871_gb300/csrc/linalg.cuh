@@ -76,42 +76,54 @@ bool tc_timed_out(cudaStream_t s);
 bool oz_timed_out(cudaStream_t s);
 cudaError_t tc_raise_timeout_flag();
 
-// FP64 products on the tensor cores by exact BF16 slices (ozaki.cu).  A strided
-// FP64 view: element (b, i, k) at p[b sb + (i / ig) si + (i % ig) sg + k sk]
-// (ig = 2 reads the real and imaginary parts of complex rows as two real rows).
+// FP64 products on the tensor cores by exact BF16 slices (ozaki.cu).
+// Output view: element (b, i, j) at p[b sb + (i / ig) si + (i % ig) sg + j sk]
+// (ig = 2 writes real rows 2 r, 2 r + 1 as the parts of complex rows).
 struct OzView {
   double* p;
   long long sb, si, sg, sk;
   int ig;
 };
+// Source of an operand's rows (A's rows, or B's columns): entry (b, i, k), strides in doubles.
+//   OZ_REAL    p[i sr + k sk]
+//   OZ_PAIR    rows 2 r + q are the parts q of complex rows r: p[r sr + k sk + q]
+//   OZ_CLEFT   k = 2 l + q runs over the parts of a complex row: p[i sr + l sk + q]
+//   OZ_CRIGHT  the right operand to OZ_CLEFT: rows 2 j, 2 j + 1 are (re, -im), (im, re)
+//              of complex column j along k = 2 l + q, p[j sr + l sk + ...]
+enum { OZ_REAL = 0, OZ_PAIR = 1, OZ_CLEFT = 2, OZ_CRIGHT = 3 };
+struct OzSrc {
+  const double* p;
+  long long sb, sr, sk;
+  int kind;
+};
 extern bool g_oz_enabled;
 // Scratch bytes of ozaki_gemm for these sizes.
 size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared);
-// C[b] = alpha A[b] B[b] + beta C[b] (m x n, k inner; beta = 0 never reads C)
-// with A given row-wise (A(b, i, kk)) and B by its transpose Bt(b, j, kk);
-// b_shared: one B for every batch.  Returns cudaErrorNotSupported when the
-// tensor-map encoder is unavailable, cudaErrorInvalidValue on bad sizes.
-cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzView A, OzView Bt,
-                       bool b_shared, double beta, OzView C, void* scratch, size_t scratch_bytes);
+// C[b] = alpha A[b] B[b] + beta C[b] (m x n, k inner; beta = 0 never reads C), sizes of the
+// real product; b_shared: one B for every batch; sym: only the 128 x 64 tiles that meet the
+// lower triangle are computed.  Returns cudaErrorNotSupported when the tensor-map encoder is
+// unavailable, cudaErrorInvalidValue on bad sizes.
+cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
+                       double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym = false);
 // The same in two steps, for an operand used by many products: oz_slice cuts
-// the rows of a view (A's rows with is_a, or B's columns through Bt) into
-// oz_operand_bytes of slices, once; oz_multiply multiplies two sliced operands.
+// an operand into oz_operand_bytes of slices, once; oz_multiply multiplies two
+// sliced operands.  planes (oz_plane_bytes, may be NULL): with fewer tiles than
+// SMs the pieces of k run as separate tiles into FP64 planes summed in order.
 size_t oz_operand_bytes(int rows, int k, int batch, bool is_a);
-void oz_slice(cudaStream_t s, OzView v, int rows, int k, int batch, bool is_a, void* buf);
+size_t oz_plane_bytes(int m, int n, int k, int batch);
+void oz_slice(cudaStream_t s, OzSrc v, int rows, int k, int batch, bool is_a, void* buf);
 cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double alpha, const void* Aop, const void* Bop,
-                        bool b_shared, double beta, OzView C);
-// Split-k form for products with few output tiles and a long k: an operand
-// sliced "wide" (every piece of k side by side in one row, oz_wide_bytes) is
-// multiplied by one launch with the pieces along grid.z into per-piece FP64
-// planes (oz_partial_bytes), which oz_zmul_wide sums in order for a complex
-// product C (m x n, ldc) = alpha A B + beta C from the real and imaginary
-// parts of A (rows) and of B^T (rows); partials: 4 oz_partial_bytes.
-size_t oz_wide_bytes(int rows, int k, bool is_a);
-size_t oz_partial_bytes(int m, int n, int k);
-void oz_slice_wide(cudaStream_t s, OzView v, int rows, int k, bool is_a, void* buf);
-cudaError_t oz_multiply_wide(cudaStream_t s, int m, int n, int k, const void* Aop, const void* Bop, double* partial);
-cudaError_t oz_zmul_wide(cudaStream_t s, int m, int n, int k, const void* Are, const void* Aim, const void* Bre,
-                         const void* Bim, double alpha, double beta, double2* C, int ldc, void* partials);
+                        bool b_shared, double beta, OzView C, void* planes = nullptr, bool sym = false);
+// Device scratch for the emulated products behind gemm<FP64>: set for the
+// calling thread by whoever owns the stream's work (a context for the length
+// of a call); without it FP64 products stay on the FP64 pipe.
+struct OzScratch {
+  char* p = nullptr;
+  size_t bytes = 0;
+};
+extern thread_local const OzScratch* g_oz_scratch;
+// Estimated clocks of an emulated product on the whole chip (sizes of the real product).
+double oz_cycles(int m, int n, int k, int batch, bool b_shared);
 // The left operand of the Jacobian's x-projection for the pairs c0 .. c0 + nc - 1
 // of d * P + p, sliced straight from the fields: rows 2 (c nX + gy) + part of
 // u_d z_p over gx (2 nc nX rows, k = nX; oz_operand_bytes(2 nc nX, nX, 1, true)).

@@ -14,18 +14,20 @@
 // (s + t <= 7: 36 pairs) carries the weight 2^(-7 (d + 2)), so the pairs of one
 // diagonal accumulate into one FP32 accumulator in tensor memory:
 //   |partial sum| <= K 4096 (d + 3) < 2^24  for K <= 384,
-// which bounds the k extent of one launch (the host splits longer products
-// and accumulates the pieces in FP64).  The epilogue recombines the 8 diagonal
-// sums exactly in 64-bit integers (two groups of four, < 2^46 each) and rounds
-// once to FP64.  What is dropped is the pairs with s + t >= 8, below
-// 2^-55 k max|A_i.| max|B_.j| per entry, and one FP64 rounding per piece: the
-// result stays within the FP64 product's own bound 2 k u |A| |B|.
+// which bounds the k extent of one piece (longer products sum their pieces in
+// FP64).  The epilogue recombines the 8 diagonal sums in 64-bit integers (the
+// last bits rounded at 2^-53 of the row times column scale for k = 384, 2^-56 for 32) and forms
+// the double from its bits.  What is dropped is the pairs with s + t >= 8,
+// below 2^-55 k max|A_i.| max|B_.j| per entry, and one FP64 rounding per piece:
+// the result stays within the FP64 product's own bound 2 k u |A| |B|.
+// A complex product is one real product: rows of A as (re, im) pairs along k,
+// columns of B as the pairs (re, -im) and (im, re).
 //
-// Kernel: one CTA per 128 x 64 output tile; warp 0 loads slice tiles with TMA
+// Kernel: one persistent CTA per SM, 128 x 64 output tiles; warp 0 loads slice tiles with TMA
 // (cp.async.bulk.tensor, three-dimensional maps over [slice][row][k], 32-wide
 // k slices of 64-byte rows with the 64-byte swizzle) into a two-stage ring, warp 1 issues the tcgen05 BF16 MMAs (M = 128, N = 64 to 256,
 // K = 16; 28 per stage of 32 k) into the eight diagonal accumulators (all
-// 512 TMEM columns), warps 2..5 read them back.  Every mbarrier wait is
+// 512 TMEM columns), warps 2..9 read them back.  Every mbarrier wait is
 // bounded; a timeout sets the library's tensor-core timeout flag.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -54,13 +56,15 @@ constexpr int OZ_ND = 8;         // anti-diagonals kept (s + t <= 7)
 constexpr int OZ_TM = 128;       // rows per tile
 constexpr int OZ_TN = 64;        // columns per tile
 constexpr int OZ_KS = 32;        // k per stage
-constexpr int OZ_KMAX = 384;     // k per launch keeping every diagonal sum below 2^24 (a multiple of 32)
-constexpr int OZ_THREADS = 192;  // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+constexpr int OZ_KMAX = 384;     // k per piece keeping every diagonal sum below 2^24 (a multiple of 32)
+constexpr int OZ_THREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 constexpr int OZ_A_SL = OZ_TM * 2 * OZ_KS;  // one slice of the A tile: 128 rows x 64 bytes (8 KB)
 constexpr int OZ_B_SL = OZ_TN * 2 * OZ_KS;  // same for B (4 KB)
 constexpr int OZ_STAGE = OZ_S * (OZ_A_SL + OZ_B_SL);  // 96 KB
 constexpr int OZ_SMEM = 2 * OZ_STAGE + 1024;
 constexpr long long OZ_WAIT = 1LL << 26;
+constexpr int OZ_NAN = 1 << 20;  // exponent of a row with an infinity or a NaN: its outputs are NaN
+constexpr int OZ_SR = 16;        // rows per CTA of the slicing kernel
 // instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = n
 __host__ __device__ constexpr uint32_t oz_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_TM >> 4) << 24);
@@ -105,11 +109,6 @@ __device__ __forceinline__ void oz_ld16(uint32_t ta, uint32_t (&v)[16]) {
       : "r"(ta));
 }
 
-// Element (b, i, k) of a strided FP64 view.
-__device__ __forceinline__ long long vaddr(const OzView& v, long long b, long long i, long long k) {
-  return b * v.sb + (i / v.ig) * v.si + (i % v.ig) * v.sg + k * v.sk;
-}
-
 // |x| as ordered 64-bit integers (the bit pattern of a non-negative double).
 __device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL; }
 
@@ -137,154 +136,217 @@ __device__ __forceinline__ unsigned short small_bf16(int a) {
   return (unsigned short)(__float_as_uint(f) >> 16);
 }
 
-// The 8 balanced base-128 digits of a 56-bit fixed-point N (|N| < 2^56),
-// written to o[s * plane]: N = H 2^28 + L with L in [-2^27, 2^27), then four
-// digits from each 32-bit half (weights 2^21, 2^14, 2^7, 1 within it), each
-// rounded to nearest: |a_0| <= 128, |a_s| <= 64 after, sum_s a_s 2^(49 - 7 s) = N.
-__device__ __forceinline__ void put_digits(long long n, unsigned short* o, long long plane) {
+// The 8 balanced base-128 digits of a 56-bit fixed-point N (|N| < 2^56) as
+// integers: N = H 2^28 + L with L in [-2^27, 2^27), then four digits from each
+// 32-bit half (weights 2^21, 2^14, 2^7, 1 within it), each rounded to nearest:
+// |a_0| <= 128, |a_s| <= 64 after, sum_s a_s 2^(49 - 7 s) = N.
+__device__ __forceinline__ void digits(long long n, int (&a)[OZ_S]) {
   const long long hq = (n + (1LL << 27)) >> 28;
   int h = (int)hq, l = (int)(n - (hq << 28));
-  int a;
-  a = (h + (1 << 20)) >> 21; h -= a << 21; o[0] = small_bf16(a);
-  a = (h + (1 << 13)) >> 14; h -= a << 14; o[plane] = small_bf16(a);
-  a = (h + (1 << 6)) >> 7;   h -= a << 7;  o[2 * plane] = small_bf16(a);
-  o[3 * plane] = small_bf16(h);
-  a = (l + (1 << 20)) >> 21; l -= a << 21; o[4 * plane] = small_bf16(a);
-  a = (l + (1 << 13)) >> 14; l -= a << 14; o[5 * plane] = small_bf16(a);
-  a = (l + (1 << 6)) >> 7;   l -= a << 7;  o[6 * plane] = small_bf16(a);
-  o[7 * plane] = small_bf16(l);
+  a[0] = (h + (1 << 20)) >> 21; h -= a[0] << 21;
+  a[1] = (h + (1 << 13)) >> 14; h -= a[1] << 14;
+  a[2] = (h + (1 << 6)) >> 7;   a[3] = h - (a[2] << 7);
+  a[4] = (l + (1 << 20)) >> 21; l -= a[4] << 21;
+  a[5] = (l + (1 << 13)) >> 14; l -= a[5] << 14;
+  a[6] = (l + (1 << 6)) >> 7;   a[7] = l - (a[6] << 7);
 }
 
-// Slices of the rows of a view (rows = A's rows, or B's columns): one warp
-// per row, lanes along k; slices written to out[s][b * rpad + i][kk] (BF16,
-// kpad wide, zero padded), the row's exponent to e[b * rpad + i].  Padding
-// rows get zero slices.  All in integer arithmetic (the FP64 pipe is the
-// scarce unit): the row's largest magnitude fixes e with max 2^-e in
-// [1/2, 1); each entry becomes the 56-bit fixed-point integer
-// N = round(x 2^(56 - e)), |N| < 2^56, whose balanced base-128 digits are the
-// slices (put_digits), which represent N exactly.
-__global__ void k_oz_slice(OzView v, int rows, int k, int rpad, int kpad, int batch, __nv_bfloat16* __restrict__ out,
-                           int* __restrict__ e, int ldo, int col0) {
-  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const long long total = (long long)batch * rpad;
-  if (r >= total) return;
-  const long long b = r / rpad;
-  const int i = (int)(r % rpad);
-  const long long plane = total * ldo;
-  unsigned short* o = reinterpret_cast<unsigned short*>(out) + r * ldo + col0;
-  const bool live = i < rows;
-  // the row's piece (k <= OZ_KMAX) is read once into registers
-  constexpr int KPL = OZ_KMAX / 32;
-  double x[KPL];
-  long long mx = 0;
+// The slices of two k-neighbours, one 32-bit store per slice.
+__device__ __forceinline__ void put2(double x0, double x1, int ex, uint32_t* o, long long plane2) {
+  int a[OZ_S], b[OZ_S];
+  digits(fixed56(x0, ex), a);
+  digits(fixed56(x1, ex), b);
 #pragma unroll
-  for (int q = 0; q < KPL; ++q) {
-    const int kk = lane + 32 * q;
-    x[q] = (live && kk < k) ? v.p[vaddr(v, b, i, kk)] : 0.0;
-    mx = max(mx, abs_bits(x[q]));
+  for (int s = 0; s < OZ_S; ++s) o[s * plane2] = (uint32_t)small_bf16(a[s]) | ((uint32_t)small_bf16(b[s]) << 16);
+}
+
+// Exponent of a row from its largest |x| (bit pattern): max in [2^(ex-1), 2^ex).
+__device__ __forceinline__ int row_exp(long long mx) {
+  const int e = (int)(mx >> 52);
+  return mx == 0 ? 0 : e == 0x7FF ? OZ_NAN : e - 1022;
+}
+
+__device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long i, long long k) {
+  const double* p = v.p + b * v.sb;
+  switch (v.kind) {
+    case OZ_REAL: return p[i * v.sr + k * v.sk];
+    case OZ_PAIR: return p[(i >> 1) * v.sr + k * v.sk + (i & 1)];
+    case OZ_CLEFT: return p[i * v.sr + (k >> 1) * v.sk + (k & 1)];
+    default: {  // OZ_CRIGHT: [re, -im; im, re]
+      const double x = p[(i >> 1) * v.sr + (k >> 1) * v.sk + ((i ^ k) & 1)];
+      return (k & 1) && !(i & 1) ? -x : x;
+    }
   }
-  for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  const int Emax = (int)(mx >> 52);
-  const int ex = mx == 0 ? 0 : Emax - 1022;  // largest |x| in [2^(ex-1), 2^ex)
-  if (lane == 0) e[r] = ex;
-#pragma unroll
-  for (int q = 0; q < KPL; ++q) {
-    const int kk = lane + 32 * q;
-    if (kk >= kpad) break;
-    put_digits(fixed56(x[q], ex), o + kk, plane);
+}
+
+// Slices of the rows of an operand (A's rows, or B's columns), one CTA per 16
+// rows and piece of k, written to out[s][b * rpad + i][k] (BF16, kt wide, zero
+// padded), the piece's row exponents to e[piece][b * rpad + i].  The block is
+// read once through shared memory (along k, or along the rows where those are
+// the contiguous direction), the row's largest magnitude fixes e with
+// max 2^-e in [1/2, 1), and each entry becomes the 56-bit fixed-point integer
+// N = round(x 2^(56 - e)), |N| < 2^56, whose balanced base-128 digits are the
+// slices and represent N exactly.  Integer arithmetic throughout (the FP64 pipe
+// is the scarce unit).  Padding rows get zero slices.
+__global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int pl, int rpad, int kt, long long total,
+                                                  __nv_bfloat16* __restrict__ out, int* __restrict__ e) {
+  extern __shared__ double tile[];
+  const int k0 = blockIdx.y * pl, kc = min(pl, k - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
+  const long long r0 = (long long)blockIdx.x * OZ_SR;
+  const int pitch = pl + 1;
+  auto get = [&](int r, int kk) {
+    const long long g = r0 + r, b = g / rpad, i = g % rpad;
+    tile[r * pitch + kk] = (g < total && i < rows && kk < kc) ? src_at(v, b, i, k0 + kk) : 0.0;
+  };
+  if (v.sk <= 2)
+    for (int q = threadIdx.x; q < OZ_SR * kp; q += 256) get(q / kp, q % kp);
+  else
+    for (int q = threadIdx.x; q < OZ_SR * kp; q += 256) get(q % OZ_SR, q / OZ_SR);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long plane2 = total * kt / 2;
+  for (int r = warp; r < OZ_SR && r0 + r < total; r += 8) {
+    const double* x = tile + r * pitch;
+    long long mx = 0;
+    for (int kk = lane; kk < kp; kk += 32) mx = max(mx, abs_bits(x[kk]));
+    for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    const int ex = row_exp(mx);
+    if (lane == 0) e[blockIdx.y * total + r0 + r] = ex;
+    uint32_t* o = reinterpret_cast<uint32_t*>(out) + ((r0 + r) * kt + k0) / 2;
+    for (int kk = 2 * lane; kk < kp; kk += 64) put2(x[kk], x[kk + 1], ex, o + kk / 2, plane2);
   }
 }
 
 // Slices of the Khatri-Rao rows of a chunk of (incidence, receiver) pairs, for
 // the x-projection of the Jacobian: complex row (pair c, gy) of w = u_d z_p
 // (d = (c0 + c) / P, p = (c0 + c) % P, fields on the interior grid,
-// [rhs][gy][gx]) over gx in [k0, k0 + kc), split into its real part (row
+// [rhs][gy][gx]) over the piece's gx, split into its real part (row
 // 2 (c nX + gy)) and imaginary part (row 2 (c nX + gy) + 1).  One warp per
-// complex row; the product is formed in FP64 in registers and never stored.
-__global__ void k_oz_slice_kr(const double2* __restrict__ Ug, const double2* __restrict__ Zg, int P, int nX,
-                              long long c0, int nc, int k0, int kc, int rpad, int kpad, __nv_bfloat16* __restrict__ out,
-                              int* __restrict__ e) {
+// complex row and piece, two neighbouring gx per lane (32-bit stores, a whole
+// 128-byte line per warp and slice: with 2-byte stores the kernel was bound by
+// the store instructions, 101 ms for the 25,600 pairs of the k = 40 Jacobian).
+// The product is formed in FP64 in registers and never stored.
+__global__ void __launch_bounds__(256) k_oz_slice_kr(const double2* __restrict__ Ug, const double2* __restrict__ Zg,
+                                                     int P, int nX, long long c0, int nc, int pl, long long rpad,
+                                                     int kt, __nv_bfloat16* __restrict__ out, int* __restrict__ e) {
   const long long r2 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r2 >= (long long)nc * nX) return;
+  const int k0 = blockIdx.y * pl, kc = min(pl, nX - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
   const long long c = c0 + r2 / nX, gy = r2 % nX, plane = (long long)nX * nX;
   const double2* u = Ug + (c / P) * plane + gy * nX + k0;
   const double2* z = Zg + (c % P) * plane + gy * nX + k0;
-  constexpr int KPL = OZ_KMAX / 32;
-  double wr[KPL], wi[KPL];
+  constexpr int KPL = OZ_KMAX / 64;
+  double2 w[KPL][2];
   long long mr = 0, mi = 0;
 #pragma unroll
-  for (int q = 0; q < KPL; ++q) {
-    const int kk = lane + 32 * q;
-    double2 w = make_double2(0.0, 0.0);
-    if (kk < kc) {
-      const double2 a = u[kk], b = z[kk];
-      w = make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  for (int q = 0; q < KPL; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int kk = 2 * lane + 64 * q + h;
+      w[q][h] = make_double2(0.0, 0.0);
+      if (kk < kc) {
+        const double2 a = u[kk], b = z[kk];
+        w[q][h] = make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+      }
+      mr = max(mr, abs_bits(w[q][h].x));
+      mi = max(mi, abs_bits(w[q][h].y));
     }
-    wr[q] = w.x;
-    wi[q] = w.y;
-    mr = max(mr, abs_bits(w.x));
-    mi = max(mi, abs_bits(w.y));
-  }
   for (int off = 16; off > 0; off >>= 1) {
     mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, off));
     mi = max(mi, __shfl_xor_sync(0xffffffffu, mi, off));
   }
-  const int er = mr == 0 ? 0 : (int)(mr >> 52) - 1022, ei = mi == 0 ? 0 : (int)(mi >> 52) - 1022;
-  const long long plane_s = (long long)rpad * kpad;
-  unsigned short* o_re = reinterpret_cast<unsigned short*>(out) + (2 * r2) * kpad;
-  unsigned short* o_im = o_re + kpad;
+  const int er = row_exp(mr), ei = row_exp(mi);
   if (lane == 0) {
-    e[2 * r2] = er;
-    e[2 * r2 + 1] = ei;
+    e[blockIdx.y * rpad + 2 * r2] = er;
+    e[blockIdx.y * rpad + 2 * r2 + 1] = ei;
   }
+  const long long plane2 = rpad * kt / 2;
+  uint32_t* o_re = reinterpret_cast<uint32_t*>(out) + (2 * r2 * kt + k0) / 2;
+  uint32_t* o_im = o_re + kt / 2;
 #pragma unroll
   for (int q = 0; q < KPL; ++q) {
-    const int kk = lane + 32 * q;
-    if (kk >= kpad) break;
-    put_digits(fixed56(wr[q], er), o_re + kk, plane_s);
-    put_digits(fixed56(wi[q], ei), o_im + kk, plane_s);
+    const int kk = 2 * lane + 64 * q;
+    if (kk >= kp) break;
+    put2(w[q][0].x, w[q][1].x, er, o_re + kk / 2, plane2);
+    put2(w[q][0].y, w[q][1].y, ei, o_im + kk / 2, plane2);
   }
 }
 
 // Zero slices of the padding rows [first, rpad) of every slice plane.
-__global__ void k_oz_zero_rows(long long first, int rpad, int kpad, __nv_bfloat16* __restrict__ out, int* __restrict__ e) {
-  const long long n = (long long)(rpad - first) * kpad;
+__global__ void k_oz_zero_rows(long long first, long long rpad, int kt, int npc, __nv_bfloat16* __restrict__ out,
+                               int* __restrict__ e) {
+  const long long n = (rpad - first) * kt;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n * OZ_S) return;
   const int s = (int)(t / n);
   const long long j = t % n;
-  out[(long long)s * rpad * kpad + first * kpad + j] = __float2bfloat16_rn(0.f);
-  if (s == 0 && j % kpad == 0) e[first + j / kpad] = 0;
+  out[s * rpad * kt + first * kt + j] = __float2bfloat16_rn(0.f);
+  if (s == 0 && j < (rpad - first) * npc) e[(j / (rpad - first)) * rpad + first + j % (rpad - first)] = 0;
+}
+
+// V 2^e as a double (round to nearest even), in integer arithmetic: two 64-bit
+// conversions, a scaling and their sum would be half the epilogue's time on
+// the FP64 pipe.
+__device__ __forceinline__ double scaled(long long V, int e) {
+  if (e >= OZ_NAN / 2) return __longlong_as_double(0x7FF8000000000000LL);
+  unsigned long long a = V < 0 ? -(unsigned long long)V : (unsigned long long)V;
+  if (a == 0) return 0.0;
+  const int z = __clzll(a);
+  a <<= z;
+  const int E = 1023 + 63 - z + e;  // biased exponent of the leading bit
+  // 53 bits, rounded; a carry runs into the exponent field as it should
+  const unsigned long long q = (a >> 11) + ((a >> 10) & ((a & 0x3FF) != 0 || ((a >> 11) & 1)));
+  if (E < 1 || E > 2045) {  // subnormal or overflow
+    const double r = scalbn((double)q, E - 1075);
+    return V < 0 ? -r : r;
+  }
+  return __longlong_as_double((long long)((((unsigned long long)(E - 1)) << 52) + q) |
+                              (V < 0 ? (long long)0x8000000000000000ULL : 0LL));
 }
 
 struct OzParams {
-  int m, n, k, mpad, npad, kpad, nb_batch_b;  // nb_batch_b: 0 when B is shared by every batch
-  // zpieces: grid.z runs over the pieces of k (pl wide, k the whole extent) of one
-  // product instead of over a batch; piece z writes its own output plane z
-  int zpieces, pl;
+  int m, n, k, pl, npc;        // k in pieces of pl
+  int mpad, npad, tm, tn;      // padded rows of A and B, tiles
+  int batch, b_shared, sym;    // sym: only tiles that meet the lower triangle
+  int zs, ppz;                 // z groups of ppz pieces, each to its own plane of C (zs > 1: alpha 1, beta 0)
+  long long items, zplane;
   double alpha, beta;
-  const int* ea;
-  const int* eb;
+  const int *ea, *eb;          // exponents [piece][row]
+  long long ea_piece, eb_piece;
   OzView C;
 };
 
+struct OzItem { int z, b, tm, tn; };
+__device__ __forceinline__ bool oz_item(const OzParams& P, long long it, OzItem& o) {
+  o.tn = (int)(it % P.tn);
+  long long t = it / P.tn;
+  o.tm = (int)(t % P.tm);
+  t /= P.tm;
+  o.b = (int)(t % P.batch);
+  o.z = (int)(t / P.batch);
+  return !(P.sym && o.tn * OZ_TN >= (o.tm + 1) * OZ_TM);
+}
+
+// Persistent: each CTA takes every gridDim.x-th 128 x 64 tile (or piece group
+// of one) and runs all its pieces of k, summing them in registers.  What bounds
+// it: 36 slice products, 2304 tensor cycles per 32-k stage at the bf16 rate, and
+// the epilogue of each piece, which cannot overlap the next piece's products
+// (the eight diagonals fill TMEM).  So the epilogue is integer arithmetic on
+// eight warps (one conversion per diagonal, two diagonals per 32-bit
+// multiply-add, the double assembled from its bits), and the ring already
+// loads the next piece behind it.  Before, one launch per piece with an FP64
+// epilogue on four warps and C read back per piece kept the tensor pipe at 17%:
+// the products of a k = 40 Gauss-Newton step (Jacobian projections and normal
+// matrix, 3.2e12 flops) took 278 ms, now 110 ms (the normal matrix by its
+// lower tiles only).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_mma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzParams P) {
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   __shared__ uint32_t tslot;
-  __shared__ __align__(8) uint64_t full[2], empty[2], done;
+  __shared__ __align__(8) uint64_t full[2], empty[2], accf, acce, done;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.z;  // batch, or piece of k
-  const int tm = blockIdx.y, tn = blockIdx.x;
-  const bool zp = P.zpieces != 0;
-  const int rowA = (zp ? 0 : b * P.mpad) + tm * OZ_TM;
-  const int rowB = (zp ? 0 : (P.nb_batch_b ? b : 0) * P.npad) + tn * OZ_TN;
-  const int kbase = zp ? b * P.pl : 0;
-  const int nst = zp ? (min(P.pl, P.k - kbase) + OZ_KS - 1) / OZ_KS : P.kpad / OZ_KS;
-  const int bB = zp ? b : (P.nb_batch_b ? b : 0);  // exponent plane of B
 
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(512));
@@ -295,6 +357,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&full[i])), "r"(1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&empty[i])), "r"(1));
     }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&accf)), "r"(1));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce)), "r"(8));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&done)), "r"(1));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -303,60 +367,168 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tslot;
   bool ok = true;
+  auto stages = [&](int p) { return (min(P.pl, P.k - p * P.pl) + OZ_KS - 1) / OZ_KS; };
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer
-      for (int i = 0; i < nst && ok; ++i) {
-        const int st = i & 1;
-        if (i >= 2) ok = oz_wait(su32(&empty[st]), ((i >> 1) - 1) & 1);
-        if (!ok) break;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[st])), "r"(OZ_STAGE)
-                     : "memory");
-        const uint32_t base = su32(sm + st * OZ_STAGE);
-        const int kx = kbase + i * OZ_KS;
-        oz_tma3(base, &mapA, kx, rowA, 0, su32(&full[st]));
-        oz_tma3(base + OZ_S * OZ_A_SL, &mapB, kx, rowB, 0, su32(&full[st]));
+      int c = 0;      // stages issued
+      for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
+        OzItem o;
+        if (!oz_item(P, it, o)) continue;
+        const int rowA = o.b * P.mpad + o.tm * OZ_TM, rowB = (P.b_shared ? 0 : o.b) * P.npad + o.tn * OZ_TN;
+        for (int p = o.z * P.ppz; p < min(P.npc, (o.z + 1) * P.ppz) && ok; ++p) {
+          const int nst = stages(p);
+          for (int i = 0; i < nst; ++i, ++c) {
+            const int st = c & 1;
+            if (c >= 2) ok = oz_wait(su32(&empty[st]), ((c >> 1) - 1) & 1);
+            if (!ok) break;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[st])), "r"(OZ_STAGE)
+                         : "memory");
+            const uint32_t base = su32(sm + st * OZ_STAGE);
+            const int kx = p * P.pl + i * OZ_KS;
+            oz_tma3(base, &mapA, kx, rowA, 0, su32(&full[st]));
+            oz_tma3(base + OZ_S * OZ_A_SL, &mapB, kx, rowB, 0, su32(&full[st]));
+          }
+        }
       }
+      // every copy issued has landed before the CTA may leave
+      for (int q = max(0, c - 2); q < c; ++q) ok = oz_wait(su32(&full[q & 1]), (q >> 1) & 1) && ok;
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
-      for (int i = 0; i < nst && ok; ++i) {
-        const int st = i & 1;
-        ok = oz_wait(su32(&full[st]), (i >> 1) & 1);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t aB = su32(sm + st * OZ_STAGE), bB = aB + OZ_S * OZ_A_SL;
-        // The B slices of a k block lie back to back (slice t at rows 64 t .. 64 t + 63)
-        // and the diagonal accumulators are adjacent in TMEM (diagonal d at columns
-        // 64 d ..), so one MMA with N = 64 w multiplies A_s by B_t .. B_(t+w-1) into
-        // diagonals s + t .. s + t + w - 1: per slice s the 8 - s pairs take
-        // MMAs of N = 256, 128 and 64 (14 per 16 k instead of 36).
+      int c = 0, pc = 0;
+      for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
+        OzItem o;
+        if (!oz_item(P, it, o)) continue;
+        for (int p = o.z * P.ppz; p < min(P.npc, (o.z + 1) * P.ppz) && ok; ++p, ++pc) {
+          if (pc > 0) ok = oz_wait(su32(&acce), (pc - 1) & 1);  // the epilogue has read the accumulators
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const int nst = stages(p);
+          for (int i = 0; i < nst; ++i, ++c) {
+            const int st = c & 1;
+            ok = oz_wait(su32(&full[st]), (c >> 1) & 1);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t aB = su32(sm + st * OZ_STAGE), bB = aB + OZ_S * OZ_A_SL;
+            // The B slices of a k block lie back to back (slice t at rows 64 t .. 64 t + 63)
+            // and the diagonal accumulators are adjacent in TMEM (diagonal d at columns
+            // 64 d ..), so one MMA with N = 64 w multiplies A_s by B_t .. B_(t+w-1) into
+            // diagonals s + t .. s + t + w - 1: per slice s the 8 - s pairs take
+            // MMAs of N = 256, 128 and 64 (14 per 16 k instead of 36).
 #pragma unroll 1
-        for (int kh = 0; kh < OZ_KS / 16; ++kh) {
+            for (int kh = 0; kh < OZ_KS / 16; ++kh) {
 #pragma unroll 1
-          for (int s = 0; s < OZ_S; ++s) {
-            const uint64_t da = oz_desc(aB + s * OZ_A_SL + kh * 32);
-            const uint32_t acc = (i > 0 || kh > 0 || s > 0) ? 1u : 0u;
-            int t = 0;
+              for (int s = 0; s < OZ_S; ++s) {
+                const uint64_t da = oz_desc(aB + s * OZ_A_SL + kh * 32);
+                const uint32_t acc = (i > 0 || kh > 0 || s > 0) ? 1u : 0u;
+                int t = 0;
 #pragma unroll 1
-            while (t + s < OZ_ND) {
-              const int left = OZ_ND - s - t;
-              const int w = left >= 4 ? 4 : left >= 2 ? 2 : 1;
-              const uint64_t db = oz_desc(bB + t * OZ_B_SL + kh * 32);
-              const uint32_t idesc = oz_idesc(w * OZ_TN);
-              asm volatile(
-                  "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)((s + t) * OZ_TN)),
-                  "l"(da), "l"(db), "r"(idesc), "r"(acc));
-              t += w;
+                while (t + s < OZ_ND) {
+                  const int left = OZ_ND - s - t;
+                  const int w = left >= 4 ? 4 : left >= 2 ? 2 : 1;
+                  const uint64_t db = oz_desc(bB + t * OZ_B_SL + kh * 32);
+                  const uint32_t idesc = oz_idesc(w * OZ_TN);
+                  asm volatile(
+                      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+                          tmem + (uint32_t)((s + t) * OZ_TN)),
+                      "l"(da), "l"(db), "r"(idesc), "r"(acc));
+                  t += w;
+                }
+              }
             }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                su32(&empty[st])));
           }
+          if (ok)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                su32(&accf)));
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            su32(&empty[st])));
       }
       // one more commit tracks every MMA issued above
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done)));
+    }
+  } else {
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows (lane = row), 32 of the 64 columns
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(half * 32);
+    int pc = 0;
+    for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
+      OzItem o;
+      if (!oz_item(P, it, o)) continue;
+      const int r = o.tm * OZ_TM + quarter * 32 + lane, cb = o.tn * OZ_TN + half * 32;
+      const int p0 = o.z * P.ppz, p1 = min(P.npc, p0 + P.ppz);
+      double acc[32];
+      for (int p = p0; p < p1; ++p, ++pc) {
+        // (rows and columns of the padding have exponents too)
+        const int ea = P.ea[p * P.ea_piece + (long long)o.b * P.mpad + r];
+        const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + lane];
+        // |sum of the piece| <= 1.02 kc: V = sum 2^(63 - rs) stays below 2^62
+        const int rs = 33 - __clz(min(P.pl, P.k - p * P.pl));
+        ok = oz_wait(su32(&accf), pc & 1);
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+        for (int ch = 0; ch < 2; ++ch) {
+          // pairs of diagonals in 32 bits: |C_d| <= 384 4096 (d + 3) (6.3e6 for d = 0),
+          // 128 C_d + C_(d+1) <= 1.83e9 < 2^31
+          long long V[16];
+#pragma unroll
+          for (int g = 0; g < 2; ++g) {
+            uint32_t v[4][16];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) oz_ld16(ta + (uint32_t)((4 * g + d) * OZ_TN + ch * 16), v[d]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;");
+            if (ch == 1 && g == 1) {  // last read of this piece: the accumulators are free
+              asm volatile("tcgen05.fence::before_thread_sync;");
+              __syncwarp();
+              if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acce)) : "memory");
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int q0 = 128 * __float2int_rn(__uint_as_float(v[0][j])) + __float2int_rn(__uint_as_float(v[1][j]));
+              const int q1 = 128 * __float2int_rn(__uint_as_float(v[2][j])) + __float2int_rn(__uint_as_float(v[3][j]));
+              const long long w = ((long long)q0 << 14) + q1;
+              // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63
+              V[j] = g == 0 ? w << (28 - rs) : V[j] + ((w + (1LL << (rs - 1))) >> rs);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int eb = __shfl_sync(0xffffffffu, ebl, ch * 16 + j);
+            const double x = scaled(V[j], ea + eb + rs - 63);
+            acc[ch * 16 + j] = p == p0 ? x : acc[ch * 16 + j] + x;
+          }
+        }
+      }
+      if (!ok) break;
+      if (r < P.m) {
+        double* pr = P.C.p + o.z * P.zplane + o.b * P.C.sb + (r / P.C.ig) * P.C.si + (r % P.C.ig) * P.C.sg;
+        if (P.C.sk == 1 && (reinterpret_cast<uintptr_t>(pr + cb) & 15) == 0 && cb + 32 <= P.n) {
+          double2* p2 = reinterpret_cast<double2*>(pr + cb);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            double2 x = make_double2(P.alpha * acc[2 * j], P.alpha * acc[2 * j + 1]);
+            if (P.beta != 0.0) {
+              const double2 y = p2[j];
+              x = make_double2(fma(P.beta, y.x, x.x), fma(P.beta, y.y, x.y));
+            }
+            p2[j] = x;
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (cb + j < P.n) {
+              double* q = pr + (cb + j) * P.C.sk;
+              const double x = P.alpha * acc[j];
+              *q = P.beta == 0.0 ? x : fma(P.beta, *q, x);
+            }
+        }
+      }
     }
   }
   // everyone: wait until the tensor cores are done with TMEM and the stages
@@ -365,49 +537,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
   if (!all_ok && threadIdx.x == 0) atomicExch(&g_oz_timeout, 1);
-  if (all_ok && warp >= 2) {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows; lane = row
-    const int quarter = warp & 3;
-    const int r = tm * OZ_TM + quarter * 32 + lane;
-    const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16);
-    const bool row_ok = r < P.m;
-    const int ea = row_ok ? P.ea[(long long)b * P.mpad + r] : 0;
-    for (int c0 = 0; c0 < OZ_TN; c0 += 16) {
-      long long hi[16], lo[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
-#pragma unroll 1
-      for (int d = 0; d < OZ_ND; ++d) {
-        uint32_t v[16];
-        oz_ld16(ta + (uint32_t)(d * OZ_TN + c0), v);
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const long long x = (long long)__float2int_rn(__uint_as_float(v[j]));  // an exact integer
-          if (d < 4)
-            hi[j] = hi[j] * 128 + x;  // 2^7: one slice width
-          else
-            lo[j] = lo[j] * 128 + x;
-        }
-      }
-      if (row_ok) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int c = tn * OZ_TN + c0 + j;
-          if (c >= P.n) continue;
-          // sum_d C_d 2^(-7 (d + 2)) = hi 2^-35 + lo 2^-63, then the row and column scales
-          const double val = fma((double)lo[j], 0x1p-63, (double)hi[j] * 0x1p-35);
-          const int eb = P.eb[(long long)bB * P.npad + c];
-          double* pc = P.C.p + vaddr(P.C, b, r, c);
-          const double out = P.alpha * scalbn(val, ea + eb);
-          *pc = P.beta == 0.0 ? out : fma(P.beta, *pc, out);
-        }
-      }
-    }
-  }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// C = alpha sum_z plane_z + beta C, planes [z][b][i][j], in order.
+__global__ void k_oz_combine(const double* __restrict__ planes, int zs, long long zplane, int m, int n, double alpha,
+                             double beta, OzView C) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= zplane) return;
+  double v = 0.0;
+  for (int z = 0; z < zs; ++z) v += planes[z * zplane + e];
+  const long long j = e % n, t = e / n, i = t % m, b = t / m;
+  double* c = C.p + b * C.sb + (i / C.ig) * C.si + (i % C.ig) * C.sg + j * C.sk;
+  *c = beta == 0.0 ? alpha * v : fma(beta, *c, alpha * v);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -424,11 +568,11 @@ bool encode_fn() {
   return g_encode != nullptr;
 }
 
-// 3-D map over slices [OZ_S][rows][kpad] (BF16), box {32 k, box_rows, all
+// 3-D map over slices [OZ_S][rows][kt] (BF16), box {32 k, box_rows, all
 // slices} with the 64-byte swizzle of the MMA operand layout.
-bool make_map(CUtensorMap* map, void* base, long long rows, int kpad, int box_rows) {
-  const cuuint64_t dims[3] = {(cuuint64_t)kpad, (cuuint64_t)rows, (cuuint64_t)OZ_S};
-  const cuuint64_t strides[2] = {(cuuint64_t)kpad * 2, (cuuint64_t)rows * kpad * 2};
+bool make_map(CUtensorMap* map, void* base, long long rows, int kt, int box_rows) {
+  const cuuint64_t dims[3] = {(cuuint64_t)kt, (cuuint64_t)rows, (cuuint64_t)OZ_S};
+  const cuuint64_t strides[2] = {(cuuint64_t)kt * 2, (cuuint64_t)rows * kt * 2};
   const cuuint32_t box[3] = {(cuuint32_t)OZ_KS, (cuuint32_t)box_rows, (cuuint32_t)OZ_S};
   const cuuint32_t es[3] = {1, 1, 1};
   return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, es,
@@ -454,58 +598,7 @@ bool oz_timed_out(cudaStream_t s) {
   return v != 0;
 }
 
-size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared) {
-  const long long kp = rup(std::min(k, OZ_KMAX), OZ_KS), mp = rup(m, OZ_TM), np = rup(n, OZ_TN);
-  const long long nbB = b_shared ? 1 : batch;
-  const size_t a = ((size_t)OZ_S * batch * mp * kp * 2 + 1023) / 1024 * 1024 + ((size_t)batch * mp * 4 + 1023) / 1024 * 1024;
-  const size_t b = ((size_t)OZ_S * nbB * np * kp * 2 + 1023) / 1024 * 1024 + ((size_t)nbB * np * 4 + 1023) / 1024 * 1024;
-  return a + b;
-}
-
 namespace {
-
-void set_smem_attr() {
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    cudaFuncSetAttribute(k_oz_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-    if (dev >= 0 && dev < 64) attr_set[dev] = true;
-  }
-}
-
-// One launch of the tile kernel over a piece of k: sliced operands sa / sbt
-// (rows padded to mp / np, kp wide) and their exponents.
-cudaError_t launch_piece(cudaStream_t s, int m, int n, int kc, long long kp, long long mp, long long np, int batch,
-                         bool b_shared, double alpha, double beta, __nv_bfloat16* sa, const int* ea,
-                         __nv_bfloat16* sbt, const int* eb, OzView C) {
-  CUtensorMap ma, mb;
-  const long long ra = batch * mp, rb = (b_shared ? 1 : batch) * np;
-  if (!make_map(&ma, sa, ra, (int)kp, OZ_TM) || !make_map(&mb, sbt, rb, (int)kp, OZ_TN)) return cudaErrorInvalidValue;
-  OzParams P;
-  P.m = m;
-  P.n = n;
-  P.k = kc;
-  P.mpad = (int)mp;
-  P.npad = (int)np;
-  P.kpad = (int)kp;
-  P.nb_batch_b = b_shared ? 0 : 1;
-  P.zpieces = 0;
-  P.pl = 0;
-  P.alpha = alpha;
-  P.beta = beta;
-  P.ea = ea;
-  P.eb = eb;
-  P.C = C;
-  dim3 grid((unsigned)(np / OZ_TN), (unsigned)(mp / OZ_TM), (unsigned)batch);
-  const bool prof = prof_active(4);
-  cudaEvent_t ev = nullptr;
-  if (prof) prof_begin(s, &ev);
-  k_oz_mma<<<grid, OZ_THREADS, OZ_SMEM, s>>>(ma, mb, P);
-  HS_COUNT_LAUNCH();
-  if (prof) prof_end(s, ev, 2.0 * m * n * kc * batch);  // FP64-equivalent flops
-  return cudaSuccess;
-}
 
 size_t align_up(size_t b) { return (b + 1023) & ~size_t(1023); }
 
@@ -515,224 +608,150 @@ int piece_len(int k) {
   const int np = (k + OZ_KMAX - 1) / OZ_KMAX;
   return (int)std::min<long long>(OZ_KMAX, rup((k + np - 1) / np, OZ_KS));
 }
+int npieces(int k) { return (k + piece_len(k) - 1) / piece_len(k); }
+long long padded(int rows, bool is_a) { return rup(rows, is_a ? OZ_TM : OZ_TN); }
+size_t slice_bytes(long long total, int k) { return align_up((size_t)OZ_S * total * npieces(k) * piece_len(k) * 2); }
 
-// Byte layout of a sliced operand: piece after piece, each the slices
-// [OZ_S][batch * rpad][kp] and the exponents [batch * rpad].
-struct Piece {
-  size_t slices, exps, next;
-  long long kp;
-  int kc;
-};
-Piece piece_at(size_t off, int k0, int k, long long rows_total) {
-  Piece p;
-  p.kc = std::min(piece_len(k), k - k0);
-  p.kp = rup(p.kc, OZ_KS);
-  p.slices = off;
-  p.exps = off + align_up((size_t)OZ_S * rows_total * p.kp * 2);
-  p.next = p.exps + align_up((size_t)rows_total * 4);
-  return p;
+template <typename F> void once_per_device(bool (&done)[64], F&& f) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && done[dev]) return;
+  f();
+  if (dev >= 0 && dev < 64) done[dev] = true;
+}
+void set_smem_attr() {
+  static bool done[64] = {};
+  once_per_device(done, [] {
+    cudaFuncSetAttribute(k_oz_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
+    cudaFuncSetAttribute(k_oz_slice, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         OZ_SR * (OZ_KMAX + 1) * (int)sizeof(double));
+  });
+}
+
+// Groups of pieces that run as separate tiles where there are fewer tiles than SMs.
+int z_groups(int m, int n, int k, int batch) {
+  const long long tiles = padded(m, true) / OZ_TM * (padded(n, false) / OZ_TN) * batch;
+  return tiles >= 152 ? 1 : (int)std::min<long long>(npieces(k), (152 + tiles - 1) / tiles);
 }
 
 }  // namespace
 
 size_t oz_operand_bytes(int rows, int k, int batch, bool is_a) {
-  const long long rt = (long long)batch * rup(rows, is_a ? OZ_TM : OZ_TN);
-  size_t off = 0;
-  for (int k0 = 0; k0 < k; k0 += piece_len(k)) off = piece_at(off, k0, k, rt).next;
-  return off;
+  const long long total = batch * padded(rows, is_a);
+  return slice_bytes(total, k) + align_up((size_t)npieces(k) * total * 4);
 }
 
-void oz_slice(cudaStream_t s, OzView v, int rows, int k, int batch, bool is_a, void* buf) {
-  const long long rpad = rup(rows, is_a ? OZ_TM : OZ_TN), rt = batch * rpad;
+size_t oz_plane_bytes(int m, int n, int k, int batch) {
+  const int zs = z_groups(m, n, k, batch);
+  return zs == 1 ? 0 : align_up((size_t)zs * batch * m * n * 8);
+}
+
+void oz_slice(cudaStream_t s, OzSrc v, int rows, int k, int batch, bool is_a, void* buf) {
+  set_smem_attr();
+  const long long rpad = padded(rows, is_a), total = batch * rpad;
+  const int pl = piece_len(k), npc = npieces(k);
   char* base = reinterpret_cast<char*>(buf);
-  size_t off = 0;
-  for (int k0 = 0; k0 < k; k0 += piece_len(k)) {
-    const Piece p = piece_at(off, k0, k, rt);
-    OzView w = v;
-    w.p += k0 * v.sk;
-    k_oz_slice<<<(unsigned)((rt + 7) / 8), 256, 0, s>>>(w, rows, p.kc, (int)rpad, (int)p.kp, batch,
-                                                      reinterpret_cast<__nv_bfloat16*>(base + p.slices),
-                                                      reinterpret_cast<int*>(base + p.exps), (int)p.kp, 0);
-    HS_COUNT_LAUNCH();
-    off = p.next;
-  }
+  k_oz_slice<<<dim3((unsigned)((total + OZ_SR - 1) / OZ_SR), npc), 256, OZ_SR * (pl + 1) * sizeof(double), s>>>(
+      v, rows, k, pl, (int)rpad, npc * pl, total, reinterpret_cast<__nv_bfloat16*>(base),
+      reinterpret_cast<int*>(base + slice_bytes(total, k)));
+  HS_COUNT_LAUNCH();
 }
 
 void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, int P, int nX, long long c0, int nc,
                          void* buf) {
-  const int rows = 2 * nc * nX;
-  const long long rpad = rup(rows, OZ_TM);
-  char* base = reinterpret_cast<char*>(buf);
-  size_t off = 0;
-  for (int k0 = 0; k0 < nX; k0 += piece_len(nX)) {
-    const Piece p = piece_at(off, k0, nX, rpad);
-    __nv_bfloat16* sl = reinterpret_cast<__nv_bfloat16*>(base + p.slices);
-    int* ex = reinterpret_cast<int*>(base + p.exps);
-    const long long warps = (long long)nc * nX;
-    k_oz_slice_kr<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(Ug, Zg, P, nX, c0, nc, k0, p.kc, (int)rpad, (int)p.kp,
-                                                             sl, ex);
+  const int rows = 2 * nc * nX, pl = piece_len(nX), npc = npieces(nX), kt = npc * pl;
+  const long long rpad = padded(rows, true), warps = (long long)nc * nX;
+  __nv_bfloat16* sl = reinterpret_cast<__nv_bfloat16*>(buf);
+  int* ex = reinterpret_cast<int*>(reinterpret_cast<char*>(buf) + slice_bytes(rpad, nX));
+  k_oz_slice_kr<<<dim3((unsigned)((warps + 7) / 8), npc), 256, 0, s>>>(Ug, Zg, P, nX, c0, nc, pl, rpad, kt, sl, ex);
+  HS_COUNT_LAUNCH();
+  if (rpad > rows) {
+    const long long n = (rpad - rows) * kt * OZ_S;
+    k_oz_zero_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rows, rpad, kt, npc, sl, ex);
     HS_COUNT_LAUNCH();
-    if (rpad > rows) {
-      const long long n = (rpad - rows) * p.kp * OZ_S;
-      k_oz_zero_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rows, (int)rpad, (int)p.kp, sl, ex);
-      HS_COUNT_LAUNCH();
-    }
-    off = p.next;
   }
 }
 
 cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double alpha, const void* Aop, const void* Bop,
-                        bool b_shared, double beta, OzView C) {
-  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0 || batch > 65535) return cudaErrorInvalidValue;
+                        bool b_shared, double beta, OzView C, void* planes, bool sym) {
+  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
   if (!encode_fn()) return cudaErrorNotSupported;
   set_smem_attr();
-  const long long mp = rup(m, OZ_TM), np = rup(n, OZ_TN);
-  char* a = const_cast<char*>(reinterpret_cast<const char*>(Aop));
-  char* b = const_cast<char*>(reinterpret_cast<const char*>(Bop));
-  size_t oa = 0, ob = 0;
-  for (int k0 = 0; k0 < k; k0 += piece_len(k)) {
-    const Piece pa = piece_at(oa, k0, k, batch * mp), pb = piece_at(ob, k0, k, (b_shared ? 1 : batch) * np);
-    const cudaError_t e =
-        launch_piece(s, m, n, pa.kc, pa.kp, mp, np, batch, b_shared, alpha, k0 == 0 ? beta : 1.0,
-                     reinterpret_cast<__nv_bfloat16*>(a + pa.slices), reinterpret_cast<const int*>(a + pa.exps),
-                     reinterpret_cast<__nv_bfloat16*>(b + pb.slices), reinterpret_cast<const int*>(b + pb.exps), C);
-    if (e != cudaSuccess) return e;
-    oa = pa.next;
-    ob = pb.next;
-  }
-  return cudaGetLastError();
-}
-
-// ---- split-k products: one launch per real product, pieces of k along grid.z ----
-
-namespace {
-// C = alpha sum_p (P0 - P1) + i alpha sum_p (P2 + P3) (+ beta C), pieces summed in order.
-__global__ void k_oz_zcombine(const double* __restrict__ P0, const double* __restrict__ P1,
-                              const double* __restrict__ P2, const double* __restrict__ P3, int npc, int m, int n,
-                              double alpha, double beta, double2* __restrict__ C, int ldc) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long mn = (long long)m * n;
-  if (e >= mn) return;
-  double re = 0.0, im = 0.0;
-  for (int p = 0; p < npc; ++p) {
-    re += P0[p * mn + e] - P1[p * mn + e];
-    im += P2[p * mn + e] + P3[p * mn + e];
-  }
-  double2* c = C + (e / n) * ldc + (e % n);
-  const double2 v = make_double2(alpha * re, alpha * im);
-  *c = beta == 0.0 ? v : make_double2(v.x + beta * c->x, v.y + beta * c->y);
-}
-
-int npieces(int k) { return (k + piece_len(k) - 1) / piece_len(k); }
-}  // namespace
-
-size_t oz_wide_bytes(int rows, int k, bool is_a) {
-  const long long rpad = rup(rows, is_a ? OZ_TM : OZ_TN), kt = (long long)npieces(k) * piece_len(k);
-  return align_up((size_t)OZ_S * rpad * kt * 2) + align_up((size_t)npieces(k) * rpad * 4);
-}
-
-size_t oz_partial_bytes(int m, int n, int k) { return align_up((size_t)npieces(k) * m * n * 8); }
-
-void oz_slice_wide(cudaStream_t s, OzView v, int rows, int k, bool is_a, void* buf) {
-  const long long rpad = rup(rows, is_a ? OZ_TM : OZ_TN);
-  const int pl = piece_len(k), kt = npieces(k) * pl;
-  char* base = reinterpret_cast<char*>(buf);
-  __nv_bfloat16* sl = reinterpret_cast<__nv_bfloat16*>(base);
-  int* ex = reinterpret_cast<int*>(base + align_up((size_t)OZ_S * rpad * kt * 2));
-  for (int p = 0, k0 = 0; k0 < k; ++p, k0 += pl) {
-    const int kc = std::min(pl, k - k0);
-    OzView w = v;
-    w.p += k0 * v.sk;
-    k_oz_slice<<<(unsigned)((rpad + 7) / 8), 256, 0, s>>>(w, rows, kc, (int)rpad, (int)rup(kc, OZ_KS), 1, sl,
-                                                        ex + (long long)p * rpad, kt, k0);
-    HS_COUNT_LAUNCH();
-  }
-}
-
-cudaError_t oz_multiply_wide(cudaStream_t s, int m, int n, int k, const void* Aop, const void* Bop, double* partial) {
-  if (m <= 0 || n <= 0 || k <= 0) return cudaErrorInvalidValue;
-  if (!encode_fn()) return cudaErrorNotSupported;
-  set_smem_attr();
-  const long long mp = rup(m, OZ_TM), np = rup(n, OZ_TN);
-  const int pl = piece_len(k), npc = npieces(k), kt = npc * pl;
+  const long long mp = padded(m, true), np = padded(n, false), ta = batch * mp, tb = (b_shared ? 1 : batch) * np;
+  const int pl = piece_len(k), npc = npieces(k), zs = planes ? z_groups(m, n, k, batch) : 1;
   char* a = const_cast<char*>(reinterpret_cast<const char*>(Aop));
   char* b = const_cast<char*>(reinterpret_cast<const char*>(Bop));
   CUtensorMap ma, mb;
-  if (!make_map(&ma, a, mp, kt, OZ_TM) || !make_map(&mb, b, np, kt, OZ_TN)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, a, ta, npc * pl, OZ_TM) || !make_map(&mb, b, tb, npc * pl, OZ_TN)) return cudaErrorInvalidValue;
   OzParams P;
   P.m = m;
   P.n = n;
   P.k = k;
+  P.pl = pl;
+  P.npc = npc;
   P.mpad = (int)mp;
   P.npad = (int)np;
-  P.kpad = kt;
-  P.nb_batch_b = 1;
-  P.zpieces = 1;
-  P.pl = pl;
-  P.alpha = 1.0;
-  P.beta = 0.0;
-  P.ea = reinterpret_cast<const int*>(a + align_up((size_t)OZ_S * mp * kt * 2));
-  P.eb = reinterpret_cast<const int*>(b + align_up((size_t)OZ_S * np * kt * 2));
-  P.C = OzView{partial, (long long)m * n, n, 0, 1, 1};
-  dim3 grid((unsigned)(np / OZ_TN), (unsigned)(mp / OZ_TM), (unsigned)npc);
+  P.tm = (int)(mp / OZ_TM);
+  P.tn = (int)(np / OZ_TN);
+  P.batch = batch;
+  P.b_shared = b_shared ? 1 : 0;
+  P.sym = sym ? 1 : 0;
+  P.ppz = (npc + zs - 1) / zs;
+  P.zs = (npc + P.ppz - 1) / P.ppz;
+  P.items = (long long)P.tm * P.tn * batch * P.zs;
+  P.ea = reinterpret_cast<const int*>(a + slice_bytes(ta, k));
+  P.eb = reinterpret_cast<const int*>(b + slice_bytes(tb, k));
+  P.ea_piece = ta;
+  P.eb_piece = tb;
+  const bool split = P.zs > 1;
+  P.zplane = split ? (long long)batch * m * n : 0;
+  P.alpha = split ? 1.0 : alpha;
+  P.beta = split ? 0.0 : beta;
+  P.C = split ? OzView{reinterpret_cast<double*>(planes), (long long)m * n, n, 0, 1, 1} : C;
   const bool prof = prof_active(4);
   cudaEvent_t ev = nullptr;
   if (prof) prof_begin(s, &ev);
-  k_oz_mma<<<grid, OZ_THREADS, OZ_SMEM, s>>>(ma, mb, P);
+  k_oz_mma<<<(unsigned)std::min<long long>(P.items, 152), OZ_THREADS, OZ_SMEM, s>>>(ma, mb, P);
   HS_COUNT_LAUNCH();
-  if (prof) prof_end(s, ev, 2.0 * m * n * k);
+  if (split) {
+    k_oz_combine<<<(unsigned)((P.zplane + 255) / 256), 256, 0, s>>>(reinterpret_cast<double*>(planes), P.zs, P.zplane,
+                                                                    m, n, alpha, beta, C);
+    HS_COUNT_LAUNCH();
+  }
+  if (prof) prof_end(s, ev, 2.0 * m * n * k * batch);  // FP64-equivalent flops
   return cudaGetLastError();
 }
 
-cudaError_t oz_zmul_wide(cudaStream_t s, int m, int n, int k, const void* Are, const void* Aim, const void* Bre,
-                         const void* Bim, double alpha, double beta, double2* C, int ldc, void* partials) {
-  const size_t pb = oz_partial_bytes(m, n, k);
-  double* P[4];
-  for (int i = 0; i < 4; ++i) P[i] = reinterpret_cast<double*>(reinterpret_cast<char*>(partials) + i * pb);
-  cudaError_t e = oz_multiply_wide(s, m, n, k, Are, Bre, P[0]);
-  if (e == cudaSuccess) e = oz_multiply_wide(s, m, n, k, Aim, Bim, P[1]);
-  if (e == cudaSuccess) e = oz_multiply_wide(s, m, n, k, Are, Bim, P[2]);
-  if (e == cudaSuccess) e = oz_multiply_wide(s, m, n, k, Aim, Bre, P[3]);
-  if (e != cudaSuccess) return e;
-  const long long mn = (long long)m * n;
-  k_oz_zcombine<<<(unsigned)((mn + 255) / 256), 256, 0, s>>>(P[0], P[1], P[2], P[3], npieces(k), m, n, alpha, beta,
-                                                             C, ldc);
-  HS_COUNT_LAUNCH();
-  return cudaGetLastError();
+thread_local const OzScratch* g_oz_scratch = nullptr;
+
+// Per piece 2304 clocks a stage of products and about 9000 of epilogue on one
+// SM; slices written and read at about 2600 bytes a clock; launches.
+double oz_cycles(int m, int n, int k, int batch, bool b_shared) {
+  const double mp = (double)padded(m, true), np = (double)padded(n, false);
+  const int npc = npieces(k), zs = z_groups(m, n, k, batch);
+  const double tiles = mp / OZ_TM * (np / OZ_TN) * batch * zs, kt = (double)npc * piece_len(k);
+  const double tile = kt / OZ_KS * 2304.0 / zs + std::ceil((double)npc / zs) * 9000.0 + 1500.0;
+  const double slices = (batch * mp + (b_shared ? 1 : batch) * np) * kt * 40.0 / 2600.0;
+  return std::ceil(tiles / 152.0) * tile + slices + (zs > 1 ? 20000.0 : 14000.0);
 }
 
-cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzView A, OzView Bt, bool b_shared,
-                       double beta, OzView C, void* scratch, size_t scratch_bytes) {
-  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0 || batch > 65535) return cudaErrorInvalidValue;
+size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared) {
+  return oz_operand_bytes(m, k, batch, true) + oz_operand_bytes(n, k, b_shared ? 1 : batch, false) +
+         oz_plane_bytes(m, n, k, batch);
+}
+
+cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
+                       double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym) {
+  if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
   if (!encode_fn()) return cudaErrorNotSupported;
   if (ozaki_scratch_bytes(m, n, k, batch, b_shared) > scratch_bytes) return cudaErrorInvalidValue;
-  set_smem_attr();
-  const long long mp = rup(m, OZ_TM), np = rup(n, OZ_TN);
-  const long long nbB = b_shared ? 1 : batch;
-  // piece by piece, slicing each piece of both operands into the same scratch
-  for (int k0 = 0; k0 < k; k0 += piece_len(k)) {
-    const Piece pa = piece_at(0, k0, k, batch * mp), pb = piece_at(pa.next, k0, k, nbB * np);
-    char* base = reinterpret_cast<char*>(scratch);
-    OzView a = A, bt = Bt;
-    a.p += k0 * A.sk;
-    bt.p += k0 * Bt.sk;
-    const long long ra = batch * mp, rb = nbB * np;
-    k_oz_slice<<<(unsigned)((ra + 7) / 8), 256, 0, s>>>(a, m, pa.kc, (int)mp, (int)pa.kp, batch,
-                                                      reinterpret_cast<__nv_bfloat16*>(base + pa.slices),
-                                                      reinterpret_cast<int*>(base + pa.exps), (int)pa.kp, 0);
-    HS_COUNT_LAUNCH();
-    k_oz_slice<<<(unsigned)((rb + 7) / 8), 256, 0, s>>>(bt, n, pb.kc, (int)np, (int)pb.kp, (int)nbB,
-                                                      reinterpret_cast<__nv_bfloat16*>(base + pb.slices),
-                                                      reinterpret_cast<int*>(base + pb.exps), (int)pb.kp, 0);
-    HS_COUNT_LAUNCH();
-    const cudaError_t e =
-        launch_piece(s, m, n, pa.kc, pa.kp, mp, np, batch, b_shared, alpha, k0 == 0 ? beta : 1.0,
-                     reinterpret_cast<__nv_bfloat16*>(base + pa.slices), reinterpret_cast<const int*>(base + pa.exps),
-                     reinterpret_cast<__nv_bfloat16*>(base + pb.slices), reinterpret_cast<const int*>(base + pb.exps),
-                     C);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  char* a = reinterpret_cast<char*>(scratch);
+  char* b = a + oz_operand_bytes(m, k, batch, true);
+  char* pl = b + oz_operand_bytes(n, k, b_shared ? 1 : batch, false);
+  oz_slice(s, A, m, k, batch, true, a);
+  oz_slice(s, Bt, n, k, b_shared ? 1 : batch, false, b);
+  return oz_multiply(s, m, n, k, batch, alpha, a, b, b_shared, beta, C, oz_plane_bytes(m, n, k, batch) ? pl : nullptr,
+                     sym);
 }
 
 }  // namespace hs

@@ -1,8 +1,9 @@
 """FP64 and FP32 products and triangular solves at the edges of their kernels'
 ranges: dot-product kernel (up to eight rows or columns, one to several
 columns per warp, k below and above a warp's width), 16 x 16 and 32 x 32
-tiles with remainders and k splits, and the diagonal-block solves (one to
-eight columns per block, sub-block remainders, both sweeps).
+tiles with remainders and k splits, the diagonal-block solves (one to
+eight columns per block, sub-block remainders, both sweeps) and the panel
+clusters (32 to 256 rows per CTA, 1 to 16 CTAs, the tournament above).
 
 FP64 products: entry by entry against complex128 on the host within
 2 k u |A||B|; FP32: against the float64 product within 4 k u32 |A||B| (each
@@ -40,6 +41,31 @@ def test_zgemm_small(hs, m, n, k, tA, tB):
     assert bool(((C.cpu() - (a @ b + C0)).abs() <= bound).all())
 
 
+@pytest.mark.parametrize("m,n,k", [(700, 130, 260), (513, 300, 200), (200, 900, 1000)])
+@pytest.mark.parametrize("tA,tB", [(False, False), (True, False), (False, True), (True, True)])
+def test_zgemm_on_the_tensor_cores(hs, m, n, k, tA, tB):
+    """Sizes the emulated product takes: one and several pieces of k, remainders, both transposes."""
+    g = torch.Generator().manual_seed(m + n + k)
+    A, B, C0 = _rand((k, m) if tA else (m, k), g), _rand((n, k) if tB else (k, n), g), _rand((m, n), g)
+    A *= torch.logspace(-6, 6, A.shape[0], dtype=torch.float64)[:, None] if not tA else 1.0
+    a, b = A.T if tA else A, B.T if tB else B
+    C = C0.cuda().contiguous()
+    hs.hs_zgemm(A.cuda().contiguous(), B.cuda().contiguous(), C, tA, tB, True)
+    bound = 2 * k * 2.0 ** -53 * (a.abs() @ b.abs() + C0.abs())
+    assert bool(((C.cpu() - (a @ b + C0)).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_emulated_product_keeps_non_finite_rows(hs, bad):
+    g = torch.Generator().manual_seed(3)
+    A, B = _rand((1, 300, 500), g, False), _rand((1, 500, 70), g, False)
+    A[0, 17, 3] = bad
+    C = torch.empty((1, 300, 70), dtype=torch.float64, device="cuda")
+    hs.hs_dgemm_emulated(A.cuda(), B.cuda(), C)
+    finite = torch.isfinite(C.cpu()[0]).all(dim=1)
+    assert not bool(finite[17]) and int(finite.sum()) == 299
+
+
 @pytest.mark.parametrize("batch,m,n,k", [(1, 1, 1, 1), (3, 252, 5, 56), (2, 7, 200, 130), (1, 300, 8, 31),
                                          (2, 65, 9, 17), (1, 64, 64, 16), (3, 67, 130, 48), (1, 448, 81, 897)])
 @pytest.mark.parametrize("mode", [0, 1, 2])
@@ -61,7 +87,8 @@ def test_gemm32_small(hs, batch, m, n, k, mode):
 
 @pytest.mark.parametrize("dtype,u", [(torch.complex128, 2.0 ** -53), (torch.complex64, 2.0 ** -24)])
 @pytest.mark.parametrize("batch,n,nrhs", [(1, 1, 1), (1, 15, 1), (2, 129, 1), (1, 224, 2), (1, 144, 700), (3, 130, 160),
-                                          (1, 300, 1300)])
+                                          (1, 300, 1300), (9, 33, 2), (200, 31, 3), (20, 200, 2), (1, 513, 2),
+                                         (2, 1025, 1), (1, 2050, 1), (1, 4300, 2)])
 def test_block_solves(hs, dtype, u, batch, n, nrhs):
     g = torch.Generator().manual_seed(n * 7 + nrhs)
     A, B = _rand((batch, n, n), g).to(dtype), _rand((batch, n, nrhs), g).to(dtype)
