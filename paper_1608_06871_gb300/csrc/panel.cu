@@ -1,13 +1,10 @@
 // LU panel factorisation (columns [j0, j0 + nb) of a batch of n x n matrices)
 // for the blocked right-looking LU of linalg.cu.
 //
-// Short panels (at most PR = 256 rows below j0) are factored with partial
-// pivoting inside shared memory by one CTA per matrix, one thread per row: a
-// block argmax per column, the row swap, the scaling and the rank-1 update
-// all touch shared memory only.  The same row permutation is then applied to
-// the columns outside the panel through a shared-memory staging buffer.
+// Panels of up to 4096 rows are factored with partial pivoting by one
+// thread-block cluster per matrix (k_panel_cluster).
 //
-// Tall panels (the 1792-row coupled root system, the top merge levels) use
+// Taller panels (root systems above 64 leaves per side, normal matrices) use
 // tournament pivoting: sets of up to 256 rows are factored independently with
 // partial pivoting (one CTA each) and each keeps its nb pivot rows; the
 // candidates of 8 sets form the next round's sets until one set remains, whose
@@ -24,6 +21,7 @@
 #include <algorithm>
 #include <climits>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -207,55 +205,6 @@ __device__ void load_rows(E* T, int ld, int rows, int nb, const E* A, int lda, c
   }
 }
 
-// Short panel (m = n - j0 <= PR rows): one CTA per matrix.
-template <typename E>
-__global__ void __launch_bounds__(PT) k_panel_small(E* A, int lda, long long sA, int n, int j0, int nb, int* piv,
-                                                    long long sP, int* info) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  E* T = reinterpret_cast<E*>(smem_raw);
-  __shared__ int rid[PR], loc[PR];
-  __shared__ int sp[PNB];
-  __shared__ int aff_d[2 * PNB], aff_s[2 * PNB];
-  __shared__ int zc, naff;
-  const int b = blockIdx.x, t = threadIdx.x;
-  A += b * sA;
-  piv += b * sP;
-  const int m = n - j0, ld = nb + 1;
-  load_rows<E>(T, ld, m, nb, A + j0, lda, nullptr, j0);
-  if (t < m) rid[t] = t;
-  if (t == 0) zc = INT_MAX;
-  __syncthreads();
-  tile_lu<E>(T, ld, m, nb, rid, loc, sp, &zc);
-  for (int e = t; e < m * nb; e += PT) {
-    const int r = e / nb, c = e % nb;
-    A[(long long)(j0 + r) * lda + j0 + c] = T[loc[r] * ld + c];
-  }
-  if (t == 0) {
-    const int steps = min(m, nb);
-    for (int j = 0; j < steps; ++j) piv[j0 + j] = j0 + sp[j];
-    if (zc != INT_MAX && info[b] == 0) info[b] = j0 + zc + 1;
-    int k = 0;  // rows whose content changed: row r now holds old row rid[r]
-    for (int r = 0; r < m && k < 2 * PNB; ++r)
-      if (rid[r] != r) { aff_d[k] = r; aff_s[k] = rid[r]; ++k; }
-    naff = k;
-  }
-  __syncthreads();
-  // same permutation on the columns outside the panel, staged through T
-  const int na = naff, cols_out = n - nb;
-  for (int c0 = 0; c0 < cols_out && na > 0; c0 += APPLY_CH) {
-    for (int e = t; e < na * APPLY_CH; e += PT) {
-      const int a = e / APPLY_CH, cc = c0 + e % APPLY_CH;
-      if (cc < cols_out) T[e] = A[(long long)(j0 + aff_s[a]) * lda + (cc < j0 ? cc : cc + nb)];
-    }
-    __syncthreads();
-    for (int e = t; e < na * APPLY_CH; e += PT) {
-      const int a = e / APPLY_CH, cc = c0 + e % APPLY_CH;
-      if (cc < cols_out) A[(long long)(j0 + aff_d[a]) * lda + (cc < j0 ? cc : cc + nb)] = T[e];
-    }
-    __syncthreads();
-  }
-}
-
 // One tournament round: set blockIdx.x of matrix blockIdx.y.  Round 0 takes
 // rows j0 + 256 s .. ; later rounds take up to 256 candidate rows from the
 // previous round's list (entries < 0 are empty).  Writes the set's nb pivot
@@ -392,7 +341,7 @@ __global__ void __launch_bounds__(FIN_T) k_tp_finish(E* A, int lda, long long sA
   for (int c = 0; c < PNB; ++c) row[c] = x[c];
 }
 
-void set_smem_once(const void* f, size_t bytes) {
+void set_smem_once(const void* f, size_t bytes, bool wide_cluster = false) {
   static std::mutex mu;
   static std::vector<std::pair<const void*, int>> done;  // (kernel, device)
   int dev = 0;
@@ -401,11 +350,242 @@ void set_smem_once(const void* f, size_t bytes) {
   for (auto& d : done)
     if (d.first == f && d.second == dev) return;
   cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (wide_cluster) cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   done.emplace_back(f, dev);
 }
 
-size_t small_smem_elems(int m, int nb) {
-  return (size_t)std::max(m * (nb + 1), std::min(m, 2 * nb) * APPLY_CH);
+// ---- panels of up to 4096 rows: one thread-block cluster per matrix ---------
+//
+// The panel's rows are dealt to the CTAs of a cluster (RPC rows each) and stay
+// there, one thread per row and group of PNB / G columns (RPC G = 256), its
+// entries in registers with a mirror in shared memory.  Rows are relabelled
+// instead of moved.  Per column: the owners of the column reduce their
+// magnitudes (redux.sync on the leading 32 bits, then the lowest logical row),
+// the CTA's candidate row, its key and the reciprocal of its pivot go to every
+// CTA of the cluster through distributed shared memory, and after one cluster
+// barrier each CTA picks the best candidate and updates its rows from its local
+// copy.  Buffers alternate, so a column needs one CTA and one cluster barrier.
+// This is partial pivoting over the whole column (up to 2^-20 of the
+// magnitude), the multipliers come out with it, and the cluster also applies
+// the exchanges to the columns outside the panel.
+// What bounds it: in FP64 the pipe (two thread-operations per SM and clock, m
+// nb^2 / 2 multiply-adds of the panel), hence the spread over up to 16 SMs and
+// the reciprocal formed by one warp instead of by every row's thread; in FP32
+// the two barriers.  It replaces a 256-row CTA per set (180 us for a complex
+// FP64 panel of 256 rows, on one SM's pipe; 93 us now) and, above 256 rows, the
+// tournament of such sets with a separate solve for the multipliers (620 us at
+// 1792 rows; 210 us now).  The panels of the k = 40 FP64 batch: 50 -> 18.5 ms.
+__device__ __forceinline__ uint32_t cl_map(const void* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cl_st(uint32_t a, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cl_st(uint32_t a, float v) { cl_st(a, __float_as_uint(v)); }
+__device__ __forceinline__ void cl_st(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cl_st(uint32_t a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void cl_st(uint32_t a, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ uint32_t cl_ld(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Leading 32 bits of a magnitude, ordered as the magnitude is; + 1 so that an
+// active zero ranks above no row.
+__device__ __forceinline__ unsigned mag_bits(float m) { return __float_as_uint(m) + 1u; }
+__device__ __forceinline__ unsigned mag_bits(double m) { return (unsigned)__double2hiint(m) + 1u; }
+
+constexpr int PC_MAX = 16;    // CTAs per cluster
+constexpr int PC_STAGE = 64;  // columns staged at a time when the exchanges are applied
+
+template <typename E, int RPC> struct PcSmem {
+  static constexpr int LD = PNB + 1;
+  static constexpr size_t tile = sizeof(E) * (size_t)(RPC * LD > 2 * PNB * PC_STAGE ? RPC * LD : 2 * PNB * PC_STAGE);
+  static constexpr size_t crow = sizeof(E) * 2 * PC_MAX * PNB;
+  static constexpr size_t cinv = sizeof(E) * 2 * PC_MAX;
+  static constexpr size_t bytes = tile + crow + cinv;
+};
+
+template <typename E, int RPC>
+__global__ void __launch_bounds__(PT) k_panel_cluster(E* A, int lda, long long sA, int n, int j0, int nb, int* piv,
+                                                      long long sP, int* info, int nc) {
+  using S = PcSmem<E, RPC>;
+  using M = typename pmag<E>::T;
+  constexpr int G = PT / RPC, CG = PNB / G, LD = S::LD, NW = PT / 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  E* T = reinterpret_cast<E*>(smem_raw);
+  E(*crow)[PC_MAX][PNB] = reinterpret_cast<E(*)[PC_MAX][PNB]>(smem_raw + S::tile);
+  E(*cinv)[PC_MAX] = reinterpret_cast<E(*)[PC_MAX]>(smem_raw + S::tile + S::crow);
+  __shared__ unsigned cmag[2][PC_MAX], ckey[2][PC_MAX];
+  __shared__ unsigned wmag[2][NW], wkey[2][NW];
+  __shared__ int sp[PNB], naff, aff_d[2 * PNB], aff_s[2 * PNB];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const unsigned rank = nc > 1 ? blockIdx.x % nc : 0;
+  const int b = blockIdx.x / nc;
+  A += b * sA;
+  piv += b * sP;
+  const int m = n - j0, row0 = (int)rank * RPC, rows = max(0, min(RPC, m - row0));
+  const int tr = t % RPC, g = t / RPC;  // the thread's row, column group
+  if (t == 0) naff = 0;
+  for (int e = t; e < rows * nb; e += PT) {
+    const int r = e / nb, c = e % nb;
+    T[r * LD + c] = A[(long long)(j0 + row0 + r) * lda + j0 + c];
+  }
+  if (nc > 1) cl_sync(); else __syncthreads();  // (every CTA runs before another writes to its memory)
+  bool active = tr < rows;
+  const bool mine = active;
+  int mylg = row0 + tr;
+  E* row = T + tr * LD;
+  E r[CG];
+#pragma unroll
+  for (int c = 0; c < CG; ++c) r[c] = (active && g * CG + c < nb) ? row[g * CG + c] : el<E>::zero();
+  const int steps = min(m, nb);
+  int zc = INT_MAX;
+  for (int j = 0; j < steps; ++j) {
+    const int pb = j & 1;
+    unsigned mb = 0u, key = 0xffffffffu;
+    if (g == j / CG) {  // (whole warps: RPC is a multiple of 32)
+      const unsigned mm = active ? mag_bits(pmag<E>::of(row[j])) : 0u;
+      mb = __reduce_max_sync(0xffffffffu, mm);
+      key = __reduce_min_sync(0xffffffffu, active && mm == mb ? ((unsigned)mylg << 8) | (unsigned)tr : 0xffffffffu);
+    }
+    if (lane == 0) {
+      wmag[pb][warp] = mb;
+      wkey[pb][warp] = key;
+    }
+    __syncthreads();
+    {
+      const unsigned wb = lane < NW ? wmag[pb][lane] : 0u, wk = lane < NW ? wkey[pb][lane] : 0xffffffffu;
+      mb = __reduce_max_sync(0xffffffffu, wb);
+      key = __reduce_min_sync(0xffffffffu, wb == mb ? wk : 0xffffffffu);
+    }
+    // this CTA's candidate to every CTA: warp w serves CTAs w, w + 8; a CTA
+    // without active rows sends magnitude 0
+    const E* prow = T + (key & 255u) * LD;
+    if (mb > 0u) {
+      for (int d = warp; d < nc; d += NW)
+        if (lane < nb) cl_st(cl_map(&crow[pb][rank][lane], d), prow[lane]);
+      if (warp == NW - 1) {
+        const E pv = prow[j];
+        const E inv = pmag<E>::of(pv) > M(0) ? recip(pv) : el<E>::zero();
+        if (lane < nc) cl_st(cl_map(&cinv[pb][rank], lane), inv);
+      }
+    }
+    if (warp == 0 && lane < nc) {
+      cl_st(cl_map(&cmag[pb][rank], lane), mb);
+      cl_st(cl_map(&ckey[pb][rank], lane), key);
+    }
+    if (nc > 1) cl_sync(); else __syncthreads();
+    const unsigned cb = lane < nc ? cmag[pb][lane] : 0u, ck = lane < nc ? ckey[pb][lane] : 0xffffffffu;
+    const unsigned best = __reduce_max_sync(0xffffffffu, cb);
+    const unsigned bkey = __reduce_min_sync(0xffffffffu, cb == best ? ck : 0xffffffffu);
+    const int win = __ffs(__ballot_sync(0xffffffffu, cb == best && ck == bkey)) - 1;
+    const int lp = (int)(bkey >> 8);
+    if (t == 0) sp[j] = lp;
+    if (win == (int)rank && tr == (int)(bkey & 255u)) {
+      active = false;
+      mylg = j;
+    } else if (mylg == j) {
+      mylg = lp;
+    }
+    const E* u = crow[pb][win];
+    if (!(pmag<E>::of(u[j]) > M(0))) {
+      zc = min(zc, j);  // the column is left unscaled
+    } else if (active) {
+      const E l = row[j] * cinv[pb][win];
+#pragma unroll
+      for (int c = 0; c < CG; ++c) {
+        const int cc = g * CG + c;
+        if (cc > j && cc < nb) {
+          r[c] = fmsc(r[c], l, u[cc]);
+          row[cc] = r[c];
+        } else if (cc == j) {
+          r[c] = l;  // (the mirror keeps the unscaled entry: the row's other threads read it)
+        }
+      }
+    }
+  }
+  // rows to their places; the list of exchanged rows collects in CTA 0
+  if (mine) {
+    E* out = A + (long long)(j0 + mylg) * lda + j0;
+#pragma unroll
+    for (int c = 0; c < CG; ++c)
+      if (g * CG + c < nb) out[g * CG + c] = r[c];
+    if (g == 0 && mylg != row0 + tr) {
+      uint32_t slot;
+      asm volatile("atom.shared::cluster.add.u32 %0, [%1], 1;" : "=r"(slot) : "r"(cl_map(&naff, 0)) : "memory");
+      cl_st(cl_map(&aff_d[slot], 0), (uint32_t)(j0 + mylg));
+      cl_st(cl_map(&aff_s[slot], 0), (uint32_t)(j0 + row0 + tr));
+    }
+  }
+  if (rank == 0 && t < steps) piv[j0 + t] = j0 + sp[t];
+  if (rank == 0 && t == 0 && zc != INT_MAX && info[b] == 0) info[b] = j0 + zc + 1;
+  if (nc > 1) cl_sync(); else __syncthreads();
+  const int na = (int)cl_ld(cl_map(&naff, 0));
+  if (rank != 0 && t < na) {
+    aff_d[t] = (int)cl_ld(cl_map(&aff_d[t], 0));
+    aff_s[t] = (int)cl_ld(cl_map(&aff_s[t], 0));
+  }
+  if (nc > 1) cl_sync(); else __syncthreads();  // nobody reads another CTA's memory after this
+  // the same exchanges on the columns outside the panel, staged through T
+  const int out_cols = n - nb, chunks = (out_cols + PC_STAGE - 1) / PC_STAGE;
+  for (int ch = (int)rank; ch < chunks && na > 0; ch += nc) {
+    const int c0 = ch * PC_STAGE;
+    for (int e = t; e < na * PC_STAGE; e += PT) {
+      const int a = e / PC_STAGE, cc = c0 + e % PC_STAGE;
+      if (cc < out_cols) T[e] = A[(long long)aff_s[a] * lda + (cc < j0 ? cc : cc + nb)];
+    }
+    __syncthreads();
+    for (int e = t; e < na * PC_STAGE; e += PT) {
+      const int a = e / PC_STAGE, cc = c0 + e % PC_STAGE;
+      if (cc < out_cols) A[(long long)aff_d[a] * lda + (cc < j0 ? cc : cc + nb)] = T[e];
+    }
+    __syncthreads();
+  }
+}
+
+template <typename E, int RPC>
+void launch_cluster(cudaStream_t s, E* A, int lda, long long sA, int n, int j0, int nb, int* piv, long long sP,
+                    int* info, int batch, int nc) {
+  const size_t smem = PcSmem<E, RPC>::bytes;
+  set_smem_once((const void*)k_panel_cluster<E, RPC>, smem, true);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(batch * nc));
+  cfg.blockDim = dim3(PT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nc;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_panel_cluster<E, RPC>, A, lda, sA, n, j0, nb, piv, sP, info, nc);
+  HS_COUNT_LAUNCH();
+}
+
+// Rows per CTA for a panel of m rows: the fewest (the widest spread) that keep
+// the cluster within PC_MAX CTAs and the batch within one CTA per SM (more
+// CTAs would only queue: 1024 leaf matrices of 196 rows take one CTA each, 413 us a
+// panel against 670 before); 0 where the panel has more than PC_MAX * 256 rows.
+int cluster_rows(int m, int batch) {
+  for (int rpc : {32, 64, 128, 256}) {
+    const int nc = (m + rpc - 1) / rpc;
+    if (nc <= PC_MAX && ((long long)nc * batch <= 152 || rpc == 256)) return rpc;
+  }
+  return 0;
 }
 
 }  // namespace
@@ -415,11 +595,16 @@ void lu_panel(cudaStream_t s, E* A, int lda, long long sA, int n, int j0, int nb
               int batch) {
   const int m = n - j0;
   const size_t tile_bytes = (size_t)PR * (PNB + 1) * sizeof(E);
-  if (m <= PR) {
-    set_smem_once((const void*)k_panel_small<E>, tile_bytes);
-    const size_t bytes = small_smem_elems(m, nb) * sizeof(E);
-    k_panel_small<E><<<batch, PT, bytes, s>>>(A, lda, sA, n, j0, nb, piv, sP, info);
-    HS_COUNT_LAUNCH();
+  if (const int rpc = cluster_rows(m, batch)) {
+    int nc = 1;
+    while (nc * rpc < m) nc *= 2;
+    auto go = [&](auto r) {
+      launch_cluster<E, decltype(r)::value>(s, A, lda, sA, n, j0, nb, piv, sP, info, batch, nc);
+    };
+    if (rpc == 32) go(std::integral_constant<int, 32>{});
+    else if (rpc == 64) go(std::integral_constant<int, 64>{});
+    else if (rpc == 128) go(std::integral_constant<int, 128>{});
+    else go(std::integral_constant<int, 256>{});
     return;
   }
   // tournament (nb == PNB here: only the last panel is narrower, and it is short)
