@@ -1515,12 +1515,13 @@ int jacobian_into_mixed(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M
   if (F_out) CK(cudaMemcpyAsync(F_out, F, sizeof(double2) * MP, cudaMemcpyDeviceToDevice, s));
   double2* W = a.get<double2>(plane * C);
   double2* T = a.get<double2>((size_t)nX * S1 * C);
-  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, nX, S1, S2) : 0;
+  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, nX, S1, S2, M, P) : 0;
   char* oz = ozb ? a.get<char>(ozb) : nullptr;
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
   interior_sine_tables(s, ctx->d_xint, nX, S1, S2, ctx->d_sxi, ctx->d_syi);
   Phase ph("hs_jacobian_contract");
-  contract_jacobian(s, Ug, Zg, M, P, nX, ctx->d_sxi, ctx->d_syi, S1, S2, ctx->k * ctx->k, J, W, T, C, oz, ozb);
+  if (!contract_jacobian(s, Ug, Zg, M, P, nX, ctx->d_sxi, ctx->d_syi, S1, S2, ctx->k * ctx->k, J, W, T, C, oz, ozb))
+    return fail(ctx, HS_ECUDA, "emulated FP64 product of the Jacobian contraction");
   CK(cudaGetLastError());
   return HS_OK;
 }
@@ -1529,7 +1530,7 @@ size_t jacobian_bytes_mixed(hs_ctx* ctx, int M, int P) {
   const int nX = ctx->n14;
   const size_t plane = (size_t)nX * nX, MP = (size_t)M * P;
   const int C = contract_chunk(M, P, nX, ctx->S1, g_contract_budget);
-  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, nX, ctx->S1, ctx->S2) : 0;
+  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, nX, ctx->S1, ctx->S2, M, P) : 0;
   return Arena::bytes(plane * M, 16) + Arena::bytes(plane * P, 16) + Arena::bytes(MP, 16) +
          std::max(mixed_fields_bytes(ctx, M, P),
                   Arena::bytes(plane * C, 16) + Arena::bytes((size_t)nX * ctx->S1 * C, 16) + Arena::bytes(ozb, 1));
@@ -1549,13 +1550,14 @@ int jacobian_into(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, cons
   }
   double2* W = a.get<double2>(plane * C);
   double2* T = a.get<double2>((size_t)ctx->n14 * ctx->S1 * C);
-  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, ctx->n14, ctx->S1, ctx->S2) : 0;
+  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, ctx->n14, ctx->S1, ctx->S2, M, P) : 0;
   char* oz = ozb ? a.get<char>(ozb) : nullptr;
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
   interior_sine_tables(s, ctx->d_xint, ctx->n14, ctx->S1, ctx->S2, ctx->d_sxi, ctx->d_syi);
   Phase ph("hs_jacobian_contract");
-  contract_jacobian(s, Ug, Zg, M, P, ctx->n14, ctx->d_sxi, ctx->d_syi, ctx->S1, ctx->S2, ctx->k * ctx->k, J, W, T, C,
-                    oz, ozb);
+  if (!contract_jacobian(s, Ug, Zg, M, P, ctx->n14, ctx->d_sxi, ctx->d_syi, ctx->S1, ctx->S2, ctx->k * ctx->k, J, W, T, C,
+                    oz, ozb))
+    return fail(ctx, HS_ECUDA, "emulated FP64 product of the Jacobian contraction");
   CK(cudaGetLastError());
   return HS_OK;
 }
@@ -1564,7 +1566,7 @@ size_t jacobian_bytes(hs_ctx* ctx, int M, int P) {
   if (ctx->cfg.precision == HS_MIXED) return jacobian_bytes_mixed(ctx, M, P);
   const size_t plane = (size_t)ctx->n14 * ctx->n14;
   const int C = contract_chunk(M, P, ctx->n14, ctx->S1, g_contract_budget);
-  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, ctx->n14, ctx->S1, ctx->S2) : 0;
+  const size_t ozb = g_oz_enabled ? contract_emulated_bytes(C, ctx->n14, ctx->S1, ctx->S2, M, P) : 0;
   return Arena::bytes(plane * M, 16) + Arena::bytes(plane * P, 16) +
          std::max(Arena::bytes(plane * C, 16) + Arena::bytes((size_t)ctx->n14 * ctx->S1 * C, 16) +
                       Arena::bytes(ozb, 1),
@@ -2036,7 +2038,7 @@ int hs_gn_step_lsqr(hs_ctx* ctx, const double* data, const double* alphas, int M
                                  Arena::bytes((size_t)gemvT_parts(MP) * nm, 8)
                        : p64x ? Arena::bytes((size_t)MP * nm, 16) + Arena::bytes(N * C64, 16) +
                                     Arena::bytes((size_t)nX * S1 * C64, 16) +
-                                    Arena::bytes(contract_emulated_bytes(C64, nX, S1, S2), 1) +
+                                    Arena::bytes(contract_emulated_bytes(C64, nX, S1, S2, M, P), 1) +
                                     Arena::bytes((size_t)gemvT_parts(MP) * nm, 8)
                               : Arena::bytes((size_t)S2 * nX, 8) + Arena::bytes(N, 8) * 2 + Arena::bytes(N * M, 16) +
                                     Arena::bytes(MP, 16) + Arena::bytes((size_t)S1 * nX, 8));
@@ -2093,7 +2095,7 @@ int hs_gn_step_lsqr(hs_ctx* ctx, const double* data, const double* alphas, int M
   double* partT = nullptr;
   double2 *J64 = nullptr, *W64 = nullptr, *T64 = nullptr;
   char* oz = nullptr;
-  const size_t ozb = p64x ? contract_emulated_bytes(C64, nX, S1, S2) : 0;
+  const size_t ozb = p64x ? contract_emulated_bytes(C64, nX, S1, S2, M, P) : 0;
   if (p64x) {
     J64 = a.get<double2>((size_t)MP * nm);
     W64 = a.get<double2>(N * C64);
@@ -2122,7 +2124,8 @@ int hs_gn_step_lsqr(hs_ctx* ctx, const double* data, const double* alphas, int M
   }
   if (p64x) {
     Phase phj("hs_jacobian_contract");
-    contract_jacobian(s, Ug, Zg, M, P, nX, ctx->d_sxi, ctx->d_syi, S1, S2, k2, J64, W64, T64, C64, oz, ozb);
+    if (!contract_jacobian(s, Ug, Zg, M, P, nX, ctx->d_sxi, ctx->d_syi, S1, S2, k2, J64, W64, T64, C64, oz, ozb))
+    return fail(ctx, HS_ECUDA, "emulated FP64 product of the Jacobian contraction");
   }
   std::vector<unsigned char> keep(nm, 1);
   if (mask)

@@ -93,8 +93,8 @@ __global__ void k_khatri_rao(const double2* __restrict__ Ug, const double2* __re
 
 // Scratch of the emulated products of a chunk of C pairs (the slices of its
 // Khatri-Rao rows for the x-projection, then of its half-projected rows).
-size_t contract_emulated_bytes(int C, int nX, int S1, int S2) {
-  return oz_operand_bytes(S1, nX, 1, false) + oz_operand_bytes(S2, nX, 1, false) +
+size_t contract_emulated_bytes(int C, int nX, int S1, int S2, int M, int P) {
+  return oz_fix_bytes(M, nX) + oz_fix_bytes(P, nX) + oz_operand_bytes(S1, nX, 1, false) + oz_operand_bytes(S2, nX, 1, false) +
          std::max(oz_operand_bytes(2 * C * nX, nX, 1, true), oz_operand_bytes(2 * S1, nX, C, true));
 }
 
@@ -126,39 +126,41 @@ int contract_chunk32(int M, int P, int nX, int S1, size_t budget_bytes) {
 // With the emulated FP64 product (g_oz_enabled) both projections run on the
 // tensor cores: complex rows are read as pairs of real rows (re, im), and the
 // sine tables are the transposed right operands; scratch (after T) holds the
-// slices, contract_emulated_bytes(C, nX, S1, S2) bytes.
-void contract_jacobian(cudaStream_t s, const double2* Ug, const double2* Zg, int M, int P, int nX, const double* sx,
+// slices, contract_emulated_bytes(C, nX, S1, S2, M, P) bytes, and the fields are
+// overwritten by their fixed-point form.  False if a product could not be launched.
+bool contract_jacobian(cudaStream_t s, double2* Ug, double2* Zg, int M, int P, int nX, const double* sx,
                        const double* sy, int S1, int S2, double k2, double2* J, double2* W, double2* T, int C,
                        void* scratch, size_t scratch_bytes) {
   const long long plane = (long long)nX * nX, MP = (long long)M * P;
-  const bool emu = g_oz_enabled && scratch && scratch_bytes >= contract_emulated_bytes(C, nX, S1, S2);
-  char* base = reinterpret_cast<char*>(scratch);
+  char* eu = reinterpret_cast<char*>(scratch);
+  char* ez = eu + oz_fix_bytes(M, nX);
+  const bool emu = g_oz_enabled && scratch && scratch_bytes >= contract_emulated_bytes(C, nX, S1, S2, M, P);
+  char* base = ez + oz_fix_bytes(P, nX);
   const size_t bsx = oz_operand_bytes(S1, nX, 1, false), bsy = oz_operand_bytes(S2, nX, 1, false);
   char *osx = base, *osy = base + bsx, *oa = base + bsx + bsy;
-  if (emu) {  // the sine tables, sliced once as the right operands of both projections
+  if (emu) {
+    oz_fix_fields(s, Ug, M, nX, eu);
+    oz_fix_fields(s, Zg, P, nX, ez);
+    // the sine tables, sliced once as the right operands of both projections
     oz_slice(s, OzSrc{sx, 0, nX, 1, OZ_REAL}, S1, nX, 1, false, osx);
     oz_slice(s, OzSrc{sy, 0, nX, 1, OZ_REAL}, S2, nX, 1, false, osy);
   }
   for (long long c0 = 0; c0 < MP; c0 += C) {
     const int nc = (int)std::min<long long>(C, MP - c0);
     const long long n = nc * plane;
-    bool done = false;
     if (emu) {
       double* Td = reinterpret_cast<double*>(T);
       double* Jd = reinterpret_cast<double*>(J + c0 * S1 * S2);
       // T[(pair, gy)][m1] = sum_gx (u_d z_p)[gy][gx] sx[m1][gx]: the Khatri-Rao rows are
       // sliced straight from the fields (no W)
-      oz_slice_khatri_rao(s, Ug, Zg, P, nX, c0, nc, oa);
+      oz_slice_khatri_rao(s, Ug, Zg, eu, ez, P, nX, c0, nc, oa);
       const OzView vt{Td, 0, 2LL * S1, 1, 2, 2};
-      done = oz_multiply(s, 2 * nc * nX, S1, nX, 1, 1.0, oa, osx, true, 0.0, vt) == cudaSuccess;
+      if (oz_multiply(s, 2 * nc * nX, S1, nX, 1, 1.0, oa, osx, true, 0.0, vt) != cudaSuccess) return false;
       // J_pair[m1][m2] = k2 sum_gy T_pair[gy][m1] sy[m2][gy]
-      if (done) {
-        const OzView vj{Jd, 2LL * S1 * S2, 2LL * S2, 1, 2, 2};
-        oz_slice(s, OzSrc{Td, 2LL * nX * S1, 2, 2LL * S1, OZ_PAIR}, 2 * S1, nX, nc, true, oa);
-        done = oz_multiply(s, 2 * S1, S2, nX, nc, k2, oa, osy, true, 0.0, vj) == cudaSuccess;
-      }
-    }
-    if (!done) {
+      const OzView vj{Jd, 2LL * S1 * S2, 2LL * S2, 1, 2, 2};
+      oz_slice(s, OzSrc{Td, 2LL * nX * S1, 2, 2LL * S1, OZ_PAIR}, 2 * S1, nX, nc, true, oa);
+      if (oz_multiply(s, 2 * S1, S2, nX, nc, k2, oa, osy, true, 0.0, vj) != cudaSuccess) return false;
+    } else {
       k_khatri_rao<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(Ug, Zg, P, plane, c0, n, W);
       HS_COUNT_LAUNCH();
       gemm<double2, double, double2>(s, OP_N, OP_T, nc * nX, S1, nX, make_double2(1.0, 0.0), W, nX, 0, sx, nX, 0,
@@ -167,6 +169,7 @@ void contract_jacobian(cudaStream_t s, const double2* Ug, const double2* Zg, int
                                      nX, 0, make_double2(0.0, 0.0), J + c0 * S1 * S2, S2, (long long)S1 * S2, nc);
     }
   }
+  return true;
 }
 
 // Products with J without forming it, for iterative solves of the linearized

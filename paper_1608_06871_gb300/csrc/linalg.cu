@@ -175,43 +175,59 @@ __global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int m, int n, in
 }
 
 // Products with at most eight columns (or, with the roles of the operands
-// swapped by the host, rows): one warp per row i and NC columns, lanes along
-// k, one shuffle reduction per output.  Such a product is a few passes over
-// one operand; a square tile pads the columns to its width, and FP64 pays for
-// padding on the pipe (224 x 1 x 224 complex: 200 us with a 32 x 32 tile).
+// swapped by the host, rows): a warp takes RW rows and NC columns, lanes along
+// k.  Such a product is a few passes over one operand; a square tile pads the
+// columns to its width, and FP64 pays for padding on the pipe (224 x 1 x 224
+// complex: 200 us with a 32 x 32 tile).  The RW NC sums are reduced together,
+// each exchange halving the number of sums a lane carries (RW NC + log steps
+// instead of five per sum; in FP64 the additions are on the pipe).
 // Element strides, so that both transposes and the swap are the same code:
 // A(i, l) = A[i ai + l ak], B(l, j) = B[l bk + j bj], C(i, j) = C[i ci + j cj].
 constexpr int DOT_WARPS = 4;
-template <typename TA, typename TB, typename TC, int NC>
+template <typename TA, typename TB, typename TC, int NC, int RW>
 __global__ void __launch_bounds__(32 * DOT_WARPS)
     k_gemm_dot(int m, int n, int k, TC alpha, const TA* __restrict__ A, long long ai, long long ak, long long sA,
                const TB* __restrict__ B, long long bk, long long bj, long long sB, TC beta, TC* __restrict__ C,
                long long ci, long long cj, long long sC) {
+  constexpr int NV = NC * RW;  // sums, a power of two up to 32
   const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * DOT_WARPS + (threadIdx.x >> 5), j0 = blockIdx.y * NC;
-  if (i >= m) return;  // whole warp
-  A += blockIdx.z * sA + i * ai;
+  const int i0 = (blockIdx.x * DOT_WARPS + (threadIdx.x >> 5)) * RW, j0 = blockIdx.y * NC;
+  if (i0 >= m) return;  // whole warp
+  A += blockIdx.z * sA + i0 * ai;
   B += blockIdx.z * sB + j0 * bj;
-  TC acc[NC];
+  TC acc[NV];
 #pragma unroll
-  for (int j = 0; j < NC; ++j) acc[j] = el<TC>::zero();
+  for (int v = 0; v < NV; ++v) acc[v] = el<TC>::zero();
 #pragma unroll 2
   for (int l = lane; l < k; l += 32) {
-    const TA a = A[l * ak];
+    TA a[RW];
+    TB b[NC];
 #pragma unroll
-    for (int j = 0; j < NC; ++j)
-      if (j0 + j < n) acc[j] = fmac(acc[j], a, B[l * bk + j * bj]);
+    for (int r = 0; r < RW; ++r) a[r] = i0 + r < m ? A[r * ai + l * ak] : el<TA>::zero();
+#pragma unroll
+    for (int j = 0; j < NC; ++j) b[j] = j0 + j < n ? B[l * bk + j * bj] : el<TB>::zero();
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+      for (int j = 0; j < NC; ++j) acc[r * NC + j] = fmac(acc[r * NC + j], a[r], b[j]);
   }
+  int off = 16;
 #pragma unroll
-  for (int j = 0; j < NC; ++j) {
+  for (int nv = NV; nv > 1; nv >>= 1, off >>= 1) {
+    const bool up = lane & off;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[j] = addv(acc[j], shfl_xor(acc[j], off));
-    if (lane == j && j0 + j < n) {
-      TC* c = C + blockIdx.z * sC + i * ci + (j0 + j) * cj;
-      TC v = scal<TC, TC>(alpha, acc[j]);
-      if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, *c));
-      *c = v;
+    for (int v = 0; v < nv / 2; ++v) {
+      const TC keep = up ? acc[v + nv / 2] : acc[v], send = up ? acc[v] : acc[v + nv / 2];
+      acc[v] = addv(keep, shfl_xor(send, off));
     }
+  }
+  for (; off > 0; off >>= 1) acc[0] = addv(acc[0], shfl_xor(acc[0], off));
+  const int v = lane / (32 / NV), i = i0 + v / NC, j = j0 + v % NC;
+  if (lane % (32 / NV) == 0 && i < m && j < n) {
+    TC* c = C + blockIdx.z * sC + i * ci + j * cj;
+    TC x = scal<TC, TC>(alpha, acc[0]);
+    if (!is_zero(beta)) x = addv(x, scal<TC, TC>(beta, *c));
+    *c = x;
   }
 }
 
@@ -219,23 +235,18 @@ __global__ void __launch_bounds__(32 * DOT_WARPS)
 // load), k-step 8 with the next tile prefetched into registers.  For shapes
 // with enough tiles to fill the machine.
 constexpr int GB = 64, GK = 8;
-// With splits > 1 (8-byte output elements only: the partial tile must fit in
-// static shared memory) the kernel runs in clusters of `splits` CTAs along z,
-// each over a slice of k, and the partial tiles are summed in split order
-// through distributed shared memory, as in k_gemm.
 template <typename TA, typename TB, typename TC>
 __global__ void __launch_bounds__(256, 2) k_gemm_big(int opA, int opB, int m, int n, int k, TC alpha,
                                                   const TA* __restrict__ A, int lda, long long sA,
                                                   const TB* __restrict__ B, int ldb, long long sB, TC beta,
-                                                  TC* __restrict__ C, int ldc, long long sC, int splits) {
+                                                  TC* __restrict__ C, int ldc, long long sC) {
   __shared__ TA As[GK][GB];
   __shared__ TB Bs[GK][GB];
-  const int b = blockIdx.z / splits, sp = blockIdx.z % splits;
+  const int b = blockIdx.z;
   A += b * sA;
   B += b * sB;
   C += b * sC;
-  const int kc = ((k + splits - 1) / splits + GK - 1) / GK * GK;
-  const int kbeg = sp * kc, kend = min(k, kbeg + kc);
+  const int kbeg = 0, kend = k;
   const int row0 = blockIdx.y * GB, col0 = blockIdx.x * GB;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   TC acc[4][4];
@@ -292,32 +303,6 @@ __global__ void __launch_bounds__(256, 2) k_gemm_big(int opA, int opB, int m, in
     }
     __syncthreads();
   }
-  if constexpr (sizeof(TC) <= 8) {
-    if (splits > 1) {
-      __shared__ TC red[GB * GB];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) red[(ty + 16 * i) * GB + tx + 16 * j] = acc[i][j];
-      cg::cluster_group cl = cg::this_cluster();
-      cl.sync();
-      const int rows_per = (GB + splits - 1) / splits;
-      const int rb = sp * rows_per, re = min(GB, rb + rows_per);
-      for (int e = rb * GB + threadIdx.x; e < re * GB; e += 256) {
-        TC sum = el<TC>::zero();
-        for (int q = 0; q < splits; ++q) sum = addv(sum, cl.map_shared_rank(red, q)[e]);
-        const int r = row0 + e / GB, c = col0 + e % GB;
-        if (r < m && c < n) {
-          TC v = scal<TC, TC>(alpha, sum);
-          long long o = (long long)r * ldc + c;
-          if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, C[o]));
-          C[o] = v;
-        }
-      }
-      cl.sync();  // keep this CTA's partial tile alive until every rank has read it
-      return;
-    }
-  }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -333,21 +318,117 @@ __global__ void __launch_bounds__(256, 2) k_gemm_big(int opA, int opB, int m, in
 }
 
 
-// Untransposed FP32 products (real or complex, 4- or 8-byte elements): the
-// 64 x 64 tile and 4 x 4 outputs per thread of k_gemm_big, with the operand
-// tiles staged by cp.async 16-byte copies into a three-stage shared-memory
-// ring (k-step 16), so that the loads of the next two k-steps overlap the
-// products of the current one; zero-filled copies cover the edges.  Needs
-// 16-byte aligned operand rows (checked by the host).  splits > 1: k split
-// over a cluster, partial tiles summed in split order through distributed
-// shared memory.
-constexpr int PK = 16, PST = 3;
-template <typename TA, typename TB, typename TC>
-struct PipeCfg {
-  static constexpr int A_ST = GB * PK * (int)sizeof(TA);  // bytes of one A stage (64 rows x 16 k)
-  static constexpr int B_ST = PK * GB * (int)sizeof(TB);  // bytes of one B stage (16 k x 64 columns)
-  static constexpr int RING = PST * (A_ST + B_ST);
-  static constexpr int RED = GB * GB * (int)sizeof(TC);
+// FP32 products (real or complex operands): TM x TN tile, RM x RN outputs per
+// thread, operands staged by cp.async into a three-stage ring of 16-wide k-steps
+// (16-byte copies where the rows are aligned to them, one element each
+// otherwise; zero-filled at the edges), transposed operands in their own layout.
+// The arithmetic is packed: fma.rn.f32x2 does two multiply-adds in one issue
+// slot of two, so the loads and address work of the other slots no longer
+// compete with it (scalar FFMAs: one slot each, 40-55% of the rate).  The FP32
+// products of the k = 40 mixed batch: 15.7 -> 13.7 ms (batch 34.3 -> 32.6 ms),
+// of the 64 x 64 leaf one at k = 35: 76 -> 68 ms; 60 TFLOP/s of 78 on the tiles of
+// the largest leaf product (256 x 192 x 196 for 196 x 140 x 196: the rest is padding).
+//   complex x complex: P += (ar, ar)(br, bi), Q += (ai, ai)(br, bi), the product
+//     is (P.x - Q.y, P.y + Q.x); real x complex and complex x real: one; real:
+//     two columns at a time.
+// splits > 1: k split over a cluster, partial tiles summed in split order
+// through distributed shared memory.
+using u64 = unsigned long long;
+__device__ __forceinline__ u64 pk2(float x, float y) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 upk2(u64 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(u64& d, u64 a, u64 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+
+template <typename TA, typename TB> struct acc32;  // RN outputs of one row per thread
+template <> struct acc32<float2, float2> {
+  using TC = float2;
+  template <int RN> struct row {
+    u64 p[RN], q[RN];
+    __device__ void zero() {
+#pragma unroll
+      for (int j = 0; j < RN; ++j) p[j] = q[j] = 0ull;
+    }
+    __device__ void add(float2 a, const float2 (&b)[RN]) {
+      const u64 ar = pk2(a.x, a.x), ai = pk2(a.y, a.y);
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        const u64 bb = pk2(b[j].x, b[j].y);
+        fma2(p[j], ar, bb);
+        fma2(q[j], ai, bb);
+      }
+    }
+    __device__ float2 get(int j) const {
+      const float2 x = upk2(p[j]), y = upk2(q[j]);
+      return make_float2(x.x - y.y, x.y + y.x);
+    }
+  };
+};
+template <> struct acc32<float, float2> {
+  using TC = float2;
+  template <int RN> struct row {
+    u64 p[RN];
+    __device__ void zero() {
+#pragma unroll
+      for (int j = 0; j < RN; ++j) p[j] = 0ull;
+    }
+    __device__ void add(float a, const float2 (&b)[RN]) {
+      const u64 aa = pk2(a, a);
+#pragma unroll
+      for (int j = 0; j < RN; ++j) fma2(p[j], aa, pk2(b[j].x, b[j].y));
+    }
+    __device__ float2 get(int j) const { return upk2(p[j]); }
+  };
+};
+template <> struct acc32<float2, float> {
+  using TC = float2;
+  template <int RN> struct row {
+    u64 p[RN];
+    __device__ void zero() {
+#pragma unroll
+      for (int j = 0; j < RN; ++j) p[j] = 0ull;
+    }
+    __device__ void add(float2 a, const float (&b)[RN]) {
+      const u64 aa = pk2(a.x, a.y);
+#pragma unroll
+      for (int j = 0; j < RN; ++j) fma2(p[j], aa, pk2(b[j], b[j]));
+    }
+    __device__ float2 get(int j) const { return upk2(p[j]); }
+  };
+};
+template <> struct acc32<float, float> {
+  using TC = float;
+  template <int RN> struct row {
+    u64 p[RN / 2];
+    __device__ void zero() {
+#pragma unroll
+      for (int j = 0; j < RN / 2; ++j) p[j] = 0ull;
+    }
+    __device__ void add(float a, const float (&b)[RN]) {
+      const u64 aa = pk2(a, a);
+#pragma unroll
+      for (int j = 0; j < RN / 2; ++j) fma2(p[j], aa, pk2(b[2 * j], b[2 * j + 1]));
+    }
+    __device__ float get(int j) const { return j & 1 ? upk2(p[j / 2]).y : upk2(p[j / 2]).x; }
+  };
+};
+
+constexpr int PK = 16, PST = 3;  // k-step, stages
+template <typename TA, typename TB, int TM, int TN, int OPA, int OPB>
+struct Cfg32 {
+  using TC = typename acc32<TA, TB>::TC;
+  // k-major rows are padded (16 bytes) so that neighbouring rows start in other banks
+  static constexpr int AP = OPA == OP_N ? PK + 16 / (int)sizeof(TA) : TM;
+  static constexpr int BP = OPB == OP_N ? TN : PK + 16 / (int)sizeof(TB);
+  static constexpr int A_ST = (OPA == OP_N ? TM : PK) * AP * (int)sizeof(TA);
+  static constexpr int B_ST = (OPB == OP_N ? PK : TN) * BP * (int)sizeof(TB);
+  static constexpr int RING = PST * (A_ST + B_ST), RED = TM * TN * (int)sizeof(TC);
   static constexpr int SMEM = RING > RED ? RING : RED;
 };
 
@@ -358,13 +439,43 @@ __device__ __forceinline__ void cp16(void* dst, const void* src, int bytes) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename TA, typename TB, typename TC>
-__global__ void __launch_bounds__(256, 2) k_gemm_pipe(int m, int n, int k, TC alpha, const TA* __restrict__ A, int lda,
-                                                   long long sA, const TB* __restrict__ B, int ldb, long long sB,
-                                                   TC beta, TC* __restrict__ C, int ldc, long long sC, int splits) {
-  using Cf = PipeCfg<TA, TB, TC>;
+
+// One k-step of an operand: `lines` contiguous runs of `len` elements (rows
+// along k, or k lines along the rows / columns) into dst (pitch P).
+template <typename T, int LINES, int LEN, int P, int NT>
+__device__ __forceinline__ void stage32(T* dst, const T* src, long long ld, int line0, int nline, int e0, int nelem,
+                                        bool wide, int tid) {
+  constexpr int E = 16 / (int)sizeof(T);
+  if (wide) {
+#pragma unroll
+    for (int q = tid; q < LINES * (LEN / E); q += NT) {
+      const int l = q / (LEN / E), x = (q % (LEN / E)) * E;
+      const int valid = line0 + l < nline ? max(0, min(E, nelem - e0 - x)) : 0;
+      cp16(dst + l * P + x, valid ? src + (line0 + l) * ld + e0 + x : src, valid * (int)sizeof(T));
+    }
+  } else {
+#pragma unroll 4
+    for (int q = tid; q < LINES * LEN; q += NT) {
+      const int l = q / LEN, x = q % LEN;
+      const bool ok = line0 + l < nline && e0 + x < nelem;
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + l * P + x);
+      const T* p = ok ? src + (line0 + l) * ld + e0 + x : src;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(p), "n"((int)sizeof(T)),
+                   "r"(ok ? (int)sizeof(T) : 0)
+                   : "memory");
+    }
+  }
+}
+
+template <typename TA, typename TB, int TM, int TN, int RM, int RN, int OPA, int OPB>
+__global__ void __launch_bounds__((TM / RM) * (TN / RN), (TM / RM) * (TN / RN) > 128 ? 2 : 4)
+    k_gemm32(int m, int n, int k, typename acc32<TA, TB>::TC alpha, const TA* __restrict__ A, int lda, long long sA,
+             const TB* __restrict__ B, int ldb, long long sB, typename acc32<TA, TB>::TC beta,
+             typename acc32<TA, TB>::TC* __restrict__ C, int ldc, long long sC, int splits, int wideA, int wideB) {
+  using Cf = Cfg32<TA, TB, TM, TN, OPA, OPB>;
+  using TC = typename Cf::TC;
+  constexpr int TX = TN / RN, TY = TM / RM, NT = TX * TY;
   extern __shared__ __align__(16) unsigned char pipe_smem[];
-  constexpr int EA = 16 / (int)sizeof(TA), EB = 16 / (int)sizeof(TB);  // elements per 16-byte copy
   const int b = blockIdx.z / splits, sp = blockIdx.z % splits;
   A += b * sA;
   B += b * sB;
@@ -372,36 +483,25 @@ __global__ void __launch_bounds__(256, 2) k_gemm_pipe(int m, int n, int k, TC al
   const int kc = ((k + splits - 1) / splits + PK - 1) / PK * PK;
   const int kbeg = sp * kc, kend = min(k, kbeg + kc);
   const int nsteps = kend > kbeg ? (kend - kbeg + PK - 1) / PK : 0;
-  const int row0 = blockIdx.y * GB, col0 = blockIdx.x * GB;
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int row0 = blockIdx.y * TM, col0 = blockIdx.x * TN;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   auto As = [&](int st) { return reinterpret_cast<TA*>(pipe_smem + st * (Cf::A_ST + Cf::B_ST)); };
   auto Bs = [&](int st) { return reinterpret_cast<TB*>(pipe_smem + st * (Cf::A_ST + Cf::B_ST) + Cf::A_ST); };
-  // stage the k-step `step` into ring slot `st`
   auto issue = [&](int step, int st) {
     const int k0 = kbeg + step * PK;
-    TA* as = As(st);
-    TB* bs = Bs(st);
-    constexpr int CA = GB * PK / EA, CB = PK * GB / EB;  // 16-byte copies per stage
-    for (int q = tid; q < CA; q += 256) {
-      const int r = q / (PK / EA), kk = (q % (PK / EA)) * EA;
-      const int gr = row0 + r, gk = k0 + kk;
-      const int valid = (gr < m && gk < kend) ? min(EA, kend - gk) : 0;
-      const TA* src = valid ? A + (long long)gr * lda + gk : A;
-      cp16(as + r * PK + kk, src, valid * (int)sizeof(TA));
-    }
-    for (int q = tid; q < CB; q += 256) {
-      const int kk = q / (GB / EB), c = (q % (GB / EB)) * EB;
-      const int gk = k0 + kk, gc = col0 + c;
-      const int valid = (gk < kend && gc < n) ? min(EB, n - gc) : 0;
-      const TB* src = valid ? B + (long long)gk * ldb + gc : B;
-      cp16(bs + kk * GB + c, src, valid * (int)sizeof(TB));
-    }
+    if constexpr (OPA == OP_N)
+      stage32<TA, TM, PK, Cf::AP, NT>(As(st), A, lda, row0, m, k0, kend, wideA, tid);
+    else
+      stage32<TA, PK, TM, Cf::AP, NT>(As(st), A, lda, k0, kend, row0, m, wideA, tid);
+    if constexpr (OPB == OP_N)
+      stage32<TB, PK, TN, Cf::BP, NT>(Bs(st), B, ldb, k0, kend, col0, n, wideB, tid);
+    else
+      stage32<TB, TN, PK, Cf::BP, NT>(Bs(st), B, ldb, col0, n, k0, kend, wideB, tid);
   };
-  TC acc[4][4];
+  // the thread's rows ty + TY i and column pairs 2 tx + 2 TX (j / 2) + j % 2
+  typename acc32<TA, TB>::template row<RN> acc[RM];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = el<TC>::zero();
+  for (int i = 0; i < RM; ++i) acc[i].zero();
 #pragma unroll
   for (int st = 0; st < PST - 1; ++st) {
     if (st < nsteps) issue(st, st);
@@ -416,55 +516,58 @@ __global__ void __launch_bounds__(256, 2) k_gemm_pipe(int m, int n, int k, TC al
     const TB* bs = Bs(step % PST);
 #pragma unroll
     for (int kk = 0; kk < PK; ++kk) {
-      TA a[4];
-      TB bb[4];
+      TB bb[RN];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = as[(ty + 16 * i) * PK + kk];
+      for (int j = 0; j < RN; j += 2) {
+        const int c = 2 * tx + TX * j;
+        if constexpr (OPB == OP_N) {
+          struct alignas(2 * sizeof(TB)) two { TB x, y; };
+          const two v = *reinterpret_cast<const two*>(bs + kk * Cf::BP + c);
+          bb[j] = v.x;
+          bb[j + 1] = v.y;
+        } else {
+          bb[j] = bs[c * Cf::BP + kk];
+          bb[j + 1] = bs[(c + 1) * Cf::BP + kk];
+        }
+      }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = bs[kk * GB + tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmac(acc[i][j], a[i], bb[j]);
+      for (int i = 0; i < RM; ++i)
+        acc[i].add(OPA == OP_N ? as[(ty + TY * i) * Cf::AP + kk] : as[kk * Cf::AP + ty + TY * i], bb);
     }
   }
   cp_wait<0>();
   __syncthreads();
+  auto put = [&](int r, int c, TC v) {
+    v = scal<TC, TC>(alpha, v);
+    const long long o = (long long)r * ldc + c;
+    if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, C[o]));
+    C[o] = v;
+  };
   if (splits > 1) {
     TC* red = reinterpret_cast<TC*>(pipe_smem);  // the ring is free now
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) red[(ty + 16 * i) * GB + tx + 16 * j] = acc[i][j];
+      for (int j = 0; j < RN; ++j) red[(ty + TY * i) * TN + 2 * tx + TX * (j & ~1) + (j & 1)] = acc[i].get(j);
     cg::cluster_group cl = cg::this_cluster();
     cl.sync();
-    const int rows_per = (GB + splits - 1) / splits;
-    const int rb = sp * rows_per, re = min(GB, rb + rows_per);
-    for (int e = rb * GB + tid; e < re * GB; e += 256) {
+    const int rows_per = (TM + splits - 1) / splits;
+    const int rb = sp * rows_per, re = min(TM, rb + rows_per);
+    for (int e = rb * TN + tid; e < re * TN; e += NT) {
       TC sum = el<TC>::zero();
       for (int q = 0; q < splits; ++q) sum = addv(sum, cl.map_shared_rank(red, q)[e]);
-      const int r = row0 + e / GB, c = col0 + e % GB;
-      if (r < m && c < n) {
-        TC v = scal<TC, TC>(alpha, sum);
-        long long o = (long long)r * ldc + c;
-        if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, C[o]));
-        C[o] = v;
-      }
+      const int r = row0 + e / TN, c = col0 + e % TN;
+      if (r < m && c < n) put(r, c, sum);
     }
     cl.sync();  // keep this CTA's partial tile alive until every rank has read it
     return;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-      if (r < m && c < n) {
-        TC v = scal<TC, TC>(alpha, acc[i][j]);
-        long long o = (long long)r * ldc + c;
-        if (!is_zero(beta)) v = addv(v, scal<TC, TC>(beta, C[o]));
-        C[o] = v;
-      }
+    for (int j = 0; j < RN; ++j) {
+      const int r = row0 + ty + TY * i, c = col0 + 2 * tx + TX * (j & ~1) + (j & 1);
+      if (r < m && c < n) put(r, c, acc[i].get(j));
     }
 }
 
@@ -846,15 +949,25 @@ template <typename TA, typename TB, typename TC>
 void launch_dot(cudaStream_t s, int m, int n, int k, TC alpha, const TA* A, long long ai, long long ak, long long sA,
                 const TB* B, long long bk, long long bj, long long sB, TC beta, TC* C, long long ci, long long cj,
                 long long sC, int batch) {
-  const int nc = n >= 8 ? 8 : n >= 4 ? 4 : n >= 2 ? 2 : 1;
-  dim3 grid((m + DOT_WARPS - 1) / DOT_WARPS, (n + nc - 1) / nc, batch);
+  // columns of one pass over A; four rows per warp once that leaves enough warps
+  const int nc = n > 4 ? 8 : n > 2 ? 4 : n;
+  const int rw = (long long)m * batch < 152LL * 16 * 4 ? 1 : nc == 8 && sizeof(TC) == 16 ? 2 : 4;
+  dim3 grid((m + DOT_WARPS * rw - 1) / (DOT_WARPS * rw), (n + nc - 1) / nc, batch);
   auto go = [&](auto kernel) {
     kernel<<<grid, 32 * DOT_WARPS, 0, s>>>(m, n, k, alpha, A, ai, ak, sA, B, bk, bj, sB, beta, C, ci, cj, sC);
   };
-  if (nc == 8) go(k_gemm_dot<TA, TB, TC, 8>);
-  else if (nc == 4) go(k_gemm_dot<TA, TB, TC, 4>);
-  else if (nc == 2) go(k_gemm_dot<TA, TB, TC, 2>);
-  else go(k_gemm_dot<TA, TB, TC, 1>);
+  constexpr int RW = sizeof(TC) == 16 ? 2 : 4;  // of eight columns (registers)
+  if (rw == 1) {
+    if (nc == 8) go(k_gemm_dot<TA, TB, TC, 8, 1>);
+    else if (nc == 4) go(k_gemm_dot<TA, TB, TC, 4, 1>);
+    else if (nc == 2) go(k_gemm_dot<TA, TB, TC, 2, 1>);
+    else go(k_gemm_dot<TA, TB, TC, 1, 1>);
+  } else {
+    if (nc == 8) go(k_gemm_dot<TA, TB, TC, 8, RW>);
+    else if (nc == 4) go(k_gemm_dot<TA, TB, TC, 4, 4>);
+    else if (nc == 2) go(k_gemm_dot<TA, TB, TC, 2, 4>);
+    else go(k_gemm_dot<TA, TB, TC, 1, 4>);
+  }
   HS_COUNT_LAUNCH();
 }
 
@@ -879,6 +992,79 @@ Fp64Tile fp64_tile(int m, int n, int k, int batch, double fma) {
       }
     }
   return best;
+}
+
+template <typename TA, typename TB, int TM, int TN, int RM, int RN, int OPA, int OPB, typename TC>
+void launch_gemm32(cudaStream_t s, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA, const TB* B,
+                   int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch, int splits) {
+  constexpr int smem = Cfg32<TA, TB, TM, TN, OPA, OPB>::SMEM, NT = (TM / RM) * (TN / RN);
+  auto kernel = k_gemm32<TA, TB, TM, TN, RM, RN, OPA, OPB>;
+  if constexpr (smem > 48 * 1024) {
+    static bool attr[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !attr[dev]) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (dev >= 0 && dev < 64) attr[dev] = true;
+    }
+  }
+  constexpr int EA = 16 / (int)sizeof(TA), EB = 16 / (int)sizeof(TB);
+  const int wideA = lda % EA == 0 && sA % EA == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const int wideB = ldb % EB == 0 && sB % EB == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((n + TN - 1) / TN, (m + TM - 1) / TM, batch * splits);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = splits;
+  cfg.attrs = at;
+  cfg.numAttrs = splits > 1 ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits, wideA, wideB);
+  HS_COUNT_LAUNCH();
+}
+
+// FP32 tile (64 x 64 with 4 x 4 outputs per thread, or 32 x 32 with 4 x 2) and k
+// splits by the busiest SM's estimated clocks: 128 multiply-adds a clock at 3/4
+// (large tile) or half (small) of the rate, and a latency per CTA.
+template <typename TA, typename TB, typename TC>
+void gemm32(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
+            const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch) {
+  const double fma = flops_per_mac<TA, TB>() / 2.0;
+  int tile = 64, splits = 1;
+  double bt = 1e300;
+  for (int t : {64, 32})
+    for (int sp = 1; sp <= kMaxCluster; ++sp) {
+      if (sp > 1 && (k / sp < 64 || (long long)batch * sp > 65535)) break;
+      if ((m + t - 1) / t > 65535) continue;  // grid.y
+      const double ctas = (double)((m + t - 1) / t) * ((n + t - 1) / t) * batch * sp;
+      const double kc = ((k + sp - 1) / sp + PK - 1) / PK * PK;
+      const double one = t * t * fma * kc / 128.0 / (t == 64 ? 0.75 : 0.5);
+      const double time = std::ceil(ctas / 152.0) * one + 1500.0 * std::ceil(ctas / 608.0) + (sp > 1 ? 1500.0 : 0.0);
+      if (time < bt) {
+        bt = time;
+        tile = t;
+        splits = sp;
+      }
+    }
+  auto go = [&](auto oa, auto ob) {
+    constexpr int OA = decltype(oa)::value, OB = decltype(ob)::value;
+    if (tile == 64)
+      launch_gemm32<TA, TB, 64, 64, 4, 4, OA, OB>(s, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
+                                                  splits);
+    else
+      launch_gemm32<TA, TB, 32, 32, 4, 2, OA, OB>(s, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
+                                                  splits);
+  };
+  using N = std::integral_constant<int, OP_N>;
+  using T = std::integral_constant<int, OP_T>;
+  if (opA == OP_N && opB == OP_N) go(N{}, N{});
+  else if (opA == OP_T && opB == OP_N) go(T{}, N{});
+  else if (opA == OP_N) go(N{}, T{});
+  else go(T{}, T{});
 }
 
 // SIMT product (FP64, or FP32 where the tensor-core path is not taken).
@@ -913,97 +1099,15 @@ void gemm_simt(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, 
       return;
     }
     dim3 grid((n + GB - 1) / GB, (m + GB - 1) / GB, batch);
-    k_gemm_big<TA, TB, TC><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, 1);
+    k_gemm_big<TA, TB, TC><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC);
     HS_COUNT_LAUNCH();
     if (prof) prof_end(s, ev, fl);
     return;
   }
-  constexpr long long kFill = 2 * 152;  // tiles that keep every SM of the chip busy
-  const long long t64 = (long long)((m + GB - 1) / GB) * ((n + GB - 1) / GB) * batch;
-  const long long t32 = (long long)((m + 31) / 32) * ((n + 31) / 32) * batch;
-  // 64 x 64 tiles (twice the arithmetic per shared-memory load) when they fill the
-  // chip, for matrices of at least one tile each way or with at least 60% of
-  // the tiles' outputs inside the matrix (e.g. 56-row blocks)
-  const double fill64 = (double)m * n * batch / ((double)t64 * GB * GB);
-  // few big tiles with a long k: the same 64 x 64 tiles, k split over a cluster
-  int splits64 = 1;
-  constexpr bool pipe_types = !is_fp64<TC>::v && sizeof(TA) <= 8 && sizeof(TB) <= 8;
-  if (sizeof(TC) <= 8 && t64 < kFill && m >= GB && n >= GB && k >= 256) {
-    splits64 = (int)std::min<long long>((kFill + t64 - 1) / t64, k / 128);
-    splits64 = std::max(1, std::min(splits64, kMaxCluster));
-    if ((long long)batch * splits64 > 65535 || t64 * splits64 < 152) splits64 = 1;
+  if constexpr (!is_fp64<TC>::v) {
+    gemm32<TA, TB>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch);
+    if (prof) prof_end(s, ev, fl);
   }
-  if ((t64 >= kFill && ((m >= GB && n >= GB) || fill64 >= 0.6)) || splits64 > 1) {
-    dim3 grid((n + GB - 1) / GB, (m + GB - 1) / GB, batch * splits64);
-    // untransposed FP32 operands with 16-byte aligned rows: the cp.async pipeline
-    if constexpr (pipe_types) {
-      constexpr int EA = 16 / (int)sizeof(TA), EB = 16 / (int)sizeof(TB);
-      const bool aligned = opA == OP_N && opB == OP_N && lda % EA == 0 && ldb % EB == 0 && sA % EA == 0 &&
-                           sB % EB == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
-                           (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-      if (aligned) {
-        constexpr int smem = PipeCfg<TA, TB, TC>::SMEM;
-        static bool attr[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || !attr[dev]) {
-          cudaFuncSetAttribute(k_gemm_pipe<TA, TB, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-          if (dev >= 0 && dev < 64) attr[dev] = true;
-        }
-        if (splits64 == 1) {
-          k_gemm_pipe<TA, TB, TC><<<grid, 256, smem, s>>>(m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC,
-                                                          1);
-        } else {
-          cudaLaunchConfig_t cfg = {};
-          cfg.gridDim = grid;
-          cfg.blockDim = dim3(256);
-          cfg.dynamicSmemBytes = smem;
-          cfg.stream = s;
-          cudaLaunchAttribute at[1];
-          at[0].id = cudaLaunchAttributeClusterDimension;
-          at[0].val.clusterDim.x = 1;
-          at[0].val.clusterDim.y = 1;
-          at[0].val.clusterDim.z = splits64;
-          cfg.attrs = at;
-          cfg.numAttrs = 1;
-          cudaLaunchKernelEx(&cfg, k_gemm_pipe<TA, TB, TC>, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
-                             sC, splits64);
-        }
-        HS_COUNT_LAUNCH();
-        if (prof) prof_end(s, ev, fl);
-        return;
-      }
-    }
-    if (splits64 == 1) {
-      k_gemm_big<TA, TB, TC><<<grid, 256, 0, s>>>(opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC,
-                                                  1);
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid;
-      cfg.blockDim = dim3(256);
-      cfg.stream = s;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 1;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = splits64;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      cudaLaunchKernelEx(&cfg, k_gemm_big<TA, TB, TC>, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C,
-                         ldc, sC, splits64);
-    }
-    HS_COUNT_LAUNCH();
-  } else {
-    int splits = 1;
-    if (t32 < kFill && k >= 256) {
-      splits = (int)std::min<long long>((kFill + t32 - 1) / t32, k / 128);
-      splits = std::max(1, std::min(splits, kMaxCluster));
-      if ((long long)batch * splits > 65535) splits = 1;
-    }
-    launch_gemm<TA, TB, TC, 32, 32>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch,
-                                    splits);
-  }
-  if (prof) prof_end(s, ev, fl);
 }
 
 inline double re_of(double x) { return x; }
@@ -1057,10 +1161,8 @@ bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alp
       ai.p += b0 * a.sb + l0 * a.sk;
       bi.p += b0 * b.sb + l0 * b.sk;
       ci.p += b0 * c.sb;
-      const cudaError_t e =
-          ozaki_gemm(s, mr, nr, std::min(kc, kr - k0), std::min(nb, batch - b0), re_of(alpha), ai, bi, bsh,
-                     k0 == 0 ? re_of(beta) : 1.0, ci, sc->p, sc->bytes);
-      if (e == cudaErrorNotSupported && b0 == 0 && k0 == 0) return false;
+      ozaki_gemm(s, mr, nr, std::min(kc, kr - k0), std::min(nb, batch - b0), re_of(alpha), ai, bi, bsh,
+                 k0 == 0 ? re_of(beta) : 1.0, ci, sc->p, sc->bytes);
     }
   return true;
 }

@@ -101,8 +101,7 @@ extern bool g_oz_enabled;
 size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared);
 // C[b] = alpha A[b] B[b] + beta C[b] (m x n, k inner; beta = 0 never reads C), sizes of the
 // real product; b_shared: one B for every batch; sym: only the 128 x 64 tiles that meet the
-// lower triangle are computed.  Returns cudaErrorNotSupported when the tensor-map encoder is
-// unavailable, cudaErrorInvalidValue on bad sizes.
+// lower triangle are computed.  Returns cudaErrorInvalidValue on bad sizes.
 cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
                        double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym = false);
 // The same in two steps, for an operand used by many products: oz_slice cuts
@@ -124,10 +123,14 @@ struct OzScratch {
 extern thread_local const OzScratch* g_oz_scratch;
 // Estimated clocks of an emulated product on the whole chip (sizes of the real product).
 double oz_cycles(int m, int n, int k, int batch, bool b_shared);
+// Fields on the interior grid ([field][gy][gx], nX x nX) in the fixed point of
+// oz_slice_khatri_rao, in place; their row exponents to exps (oz_fix_bytes).
+size_t oz_fix_bytes(int fields, int nX);
+void oz_fix_fields(cudaStream_t s, double2* F, int fields, int nX, void* exps);
 // The left operand of the Jacobian's x-projection for the pairs c0 .. c0 + nc - 1
-// of d * P + p, sliced straight from the fields: rows 2 (c nX + gy) + part of
+// of d * P + p, sliced straight from the fixed-point fields: rows 2 (c nX + gy) + part of
 // u_d z_p over gx (2 nc nX rows, k = nX; oz_operand_bytes(2 nc nX, nX, 1, true)).
-void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, int P, int nX, long long c0, int nc,
-                         void* buf);
+void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, const void* eu, const void* ez, int P,
+                         int nX, long long c0, int nc, void* buf);
 
 }  // namespace hs

@@ -23,19 +23,18 @@
 // A complex product is one real product: rows of A as (re, im) pairs along k,
 // columns of B as the pairs (re, -im) and (im, re).
 //
-// Kernel: one persistent CTA per SM, 128 x 64 output tiles; warp 0 loads slice tiles with TMA
-// (cp.async.bulk.tensor, three-dimensional maps over [slice][row][k], 32-wide
-// k slices of 64-byte rows with the 64-byte swizzle) into a two-stage ring, warp 1 issues the tcgen05 BF16 MMAs (M = 128, N = 64 to 256,
+// Kernel: one persistent CTA per SM, 128 x 64 output tiles; warp 0 copies the
+// 32-wide k-steps of the tile's slices (stored by the slicing kernels in the
+// MMA operand layout, 64 + 32 KB in one piece each) into a two-stage ring with
+// cp.async.bulk, warp 1 issues the tcgen05 BF16 MMAs (M = 128, N = 64 to 256,
 // K = 16; 28 per stage of 32 k) into the eight diagonal accumulators (all
-// 512 TMEM columns), warps 2..9 read them back.  Every mbarrier wait is
+// 512 TMEM columns), sixteen warps read them back.  Every mbarrier wait is
 // bounded; a timeout sets the library's tensor-core timeout flag.
-#include <cuda.h>
-#include <cuda_bf16.h>
-#include <cudaTypedefs.h>
+#include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
-#include <mutex>
 
 #include "linalg.cuh"
 
@@ -57,7 +56,8 @@ constexpr int OZ_TM = 128;       // rows per tile
 constexpr int OZ_TN = 64;        // columns per tile
 constexpr int OZ_KS = 32;        // k per stage
 constexpr int OZ_KMAX = 384;     // k per piece keeping every diagonal sum below 2^24 (a multiple of 32)
-constexpr int OZ_THREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
+constexpr int OZ_EPI = 16;       // epilogue warps
+constexpr int OZ_THREADS = 64 + 32 * OZ_EPI;  // warp 0 TMA, warp 1 MMA, the others epilogue
 constexpr int OZ_A_SL = OZ_TM * 2 * OZ_KS;  // one slice of the A tile: 128 rows x 64 bytes (8 KB)
 constexpr int OZ_B_SL = OZ_TN * 2 * OZ_KS;  // same for B (4 KB)
 constexpr int OZ_STAGE = OZ_S * (OZ_A_SL + OZ_B_SL);  // 96 KB
@@ -72,7 +72,7 @@ __host__ __device__ constexpr uint32_t oz_idesc(int n) {
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// K-major, 64-byte swizzle (as TMA writes it): rows of 64 bytes (32 BF16),
+// K-major, 64-byte swizzle: rows of 64 bytes (32 BF16),
 // atoms of 8 rows (512 bytes, the 8-row group stride); the k offset inside the
 // row is added to the start address.
 __device__ __forceinline__ uint64_t oz_desc(uint32_t addr) {
@@ -93,20 +93,29 @@ __device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-__device__ __forceinline__ void oz_tma3(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+__device__ __forceinline__ void oz_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-      "[%5];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(bar)
       : "memory");
 }
 
-__device__ __forceinline__ void oz_ld16(uint32_t ta, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(ta));
+// Where the pair of entries (row r, k, k + 1) of slice 0 lies in a sliced operand,
+// in 32-bit words; slice s follows at s OZ_ROW TR.  The operand is stored as
+// the product reads it: blocks [row tile of TR rows][32-wide k-step][slice][row],
+// rows of 64 bytes with the 64-byte swizzle of the MMA operand layout (16-byte
+// chunk c of row r at c ^ ((r / 2) % 4)), so a stage is one contiguous copy.
+constexpr int OZ_ROW = 16;  // words per row
+template <int TR>
+__device__ __forceinline__ long long oz_at(long long r, int k, int nst) {
+  const int rr = (int)(r % TR), kk = k % OZ_KS;
+  return ((r / TR * nst + k / OZ_KS) * OZ_S * TR + rr) * OZ_ROW + ((((kk >> 3) ^ (rr >> 1)) & 3) << 2) + ((kk & 7) >> 1);
+}
+
+__device__ __forceinline__ void oz_ld8(uint32_t ta, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(ta));
 }
 
 // |x| as ordered 64-bit integers (the bit pattern of a non-negative double).
@@ -128,36 +137,28 @@ __device__ __forceinline__ long long fixed56(double x, int e) {
   return b < 0 ? -v : v;
 }
 
-// BF16 bits of a small integer |a| <= 2^8 (exact): the float from the magic
-// constant 1.5 * 2^23 (so that negative a stay in its binade), whose upper 16
-// bits are then the BF16 value.
-__device__ __forceinline__ unsigned short small_bf16(int a) {
-  const float f = __int_as_float(0x4B400000 + a) - 12582912.0f;
-  return (unsigned short)(__float_as_uint(f) >> 16);
-}
-
-// The 8 balanced base-128 digits of a 56-bit fixed-point N (|N| < 2^56) as
-// integers: N = H 2^28 + L with L in [-2^27, 2^27), then four digits from each
-// 32-bit half (weights 2^21, 2^14, 2^7, 1 within it), each rounded to nearest:
-// |a_0| <= 128, |a_s| <= 64 after, sum_s a_s 2^(49 - 7 s) = N.
-__device__ __forceinline__ void digits(long long n, int (&a)[OZ_S]) {
-  const long long hq = (n + (1LL << 27)) >> 28;
-  int h = (int)hq, l = (int)(n - (hq << 28));
-  a[0] = (h + (1 << 20)) >> 21; h -= a[0] << 21;
-  a[1] = (h + (1 << 13)) >> 14; h -= a[1] << 14;
-  a[2] = (h + (1 << 6)) >> 7;   a[3] = h - (a[2] << 7);
-  a[4] = (l + (1 << 20)) >> 21; l -= a[4] << 21;
-  a[5] = (l + (1 << 13)) >> 14; l -= a[5] << 14;
-  a[6] = (l + (1 << 6)) >> 7;   a[7] = l - (a[6] << 7);
-}
-
-// The slices of two k-neighbours, one 32-bit store per slice.
-__device__ __forceinline__ void put2(double x0, double x1, int ex, uint32_t* o, long long plane2) {
-  int a[OZ_S], b[OZ_S];
-  digits(fixed56(x0, ex), a);
-  digits(fixed56(x1, ex), b);
+// The slices of two k-neighbours N0, N1 (56-bit fixed point, |N| < 2^56), one
+// 32-bit store per slice: the 8 balanced base-128 digits a_s of N,
+// sum_s a_s 2^(49 - 7 s) = N, |a_0| <= 128, the others in [-64, 63].  With
+// B = sum_(s>0) 64 2^(49 - 7 s), the digits of N + B are its bit fields less 64
+// (the top one as it is): a field is a shift and a mask, its float comes from the
+// magic constant 2^23 or-ed under it (1.5 2^23 added, for the signed top one), and
+// the float's upper half is the exact BF16.
+__device__ __forceinline__ void put2(long long N0, long long N1, uint32_t* o, int plane) {
+  constexpr long long B = (64LL << 42) | (64LL << 35) | (64LL << 28) | (64LL << 21) | (64LL << 14) | (64LL << 7) | 64LL;
+  N0 += B;
+  N1 += B;
+  auto top = [](long long n) { return __float_as_uint(__int_as_float(0x4B400000 + (int)(n >> 49)) - 12582912.0f); };
+  o[0] = __byte_perm(top(N0), top(N1), 0x7632);
 #pragma unroll
-  for (int s = 0; s < OZ_S; ++s) o[s * plane2] = (uint32_t)small_bf16(a[s]) | ((uint32_t)small_bf16(b[s]) << 16);
+  for (int s = 1; s < OZ_S; ++s) {
+    const int sh = 49 - 7 * s;
+    const uint32_t f0 = ((uint32_t)((unsigned long long)N0 >> sh) & 127u) | 0x4B000000u;
+    const uint32_t f1 = ((uint32_t)((unsigned long long)N1 >> sh) & 127u) | 0x4B000000u;
+    const uint32_t b0 = __float_as_uint(__uint_as_float(f0) - 8388672.0f);
+    const uint32_t b1 = __float_as_uint(__uint_as_float(f1) - 8388672.0f);
+    o[s * plane] = __byte_perm(b0, b1, 0x7632);
+  }
 }
 
 // Exponent of a row from its largest |x| (bit pattern): max in [2^(ex-1), 2^ex).
@@ -180,7 +181,7 @@ __device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long 
 }
 
 // Slices of the rows of an operand (A's rows, or B's columns), one CTA per 16
-// rows and piece of k, written to out[s][b * rpad + i][k] (BF16, kt wide, zero
+// rows and piece of k, written in blocks (oz_at, row b * rpad + i; BF16, zero
 // padded), the piece's row exponents to e[piece][b * rpad + i].  The block is
 // read once through shared memory (along k, or along the rows where those are
 // the contiguous direction), the row's largest magnitude fixes e with
@@ -188,8 +189,9 @@ __device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long 
 // N = round(x 2^(56 - e)), |N| < 2^56, whose balanced base-128 digits are the
 // slices and represent N exactly.  Integer arithmetic throughout (the FP64 pipe
 // is the scarce unit).  Padding rows get zero slices.
-__global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int pl, int rpad, int kt, long long total,
-                                                  __nv_bfloat16* __restrict__ out, int* __restrict__ e) {
+template <int TR>
+__global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int pl, int rpad, int nst, long long total,
+                                                  uint32_t* __restrict__ out, int* __restrict__ e) {
   extern __shared__ double tile[];
   const int k0 = blockIdx.y * pl, kc = min(pl, k - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
   const long long r0 = (long long)blockIdx.x * OZ_SR;
@@ -204,7 +206,6 @@ __global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int 
     for (int q = threadIdx.x; q < OZ_SR * kp; q += 256) get(q % OZ_SR, q / OZ_SR);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long plane2 = total * kt / 2;
   for (int r = warp; r < OZ_SR && r0 + r < total; r += 8) {
     const double* x = tile + r * pitch;
     long long mx = 0;
@@ -212,77 +213,107 @@ __global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int 
     for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     const int ex = row_exp(mx);
     if (lane == 0) e[blockIdx.y * total + r0 + r] = ex;
-    uint32_t* o = reinterpret_cast<uint32_t*>(out) + ((r0 + r) * kt + k0) / 2;
-    for (int kk = 2 * lane; kk < kp; kk += 64) put2(x[kk], x[kk + 1], ex, o + kk / 2, plane2);
+    for (int kk = 2 * lane; kk < kp; kk += 64)
+      put2(fixed56(x[kk], ex), fixed56(x[kk + 1], ex), out + oz_at<TR>(r0 + r, k0 + kk, nst), OZ_ROW * TR);
+  }
+}
+
+// Fields in fixed point, in place: each row piece (gx in one piece of k) of a
+// field is scaled by 2^-e so that its largest part lies in [1/2, 1) and every
+// part becomes U = round(x 2^(55 - e)) = U1 2^28 + U0 with both halves signed
+// (|U1|, |U0| <= 2^27): (re1, re0, im1, im0) takes the place of the double2.
+// e[row npc + piece]; one warp per row piece.
+__global__ void __launch_bounds__(256) k_oz_fix(double2* __restrict__ F, long long nrows, int nX, int pl, int npc,
+                                                int* __restrict__ e) {
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= nrows * npc) return;
+  const long long row = w / npc;
+  const int k0 = (int)(w % npc) * pl, kc = min(pl, nX - k0);
+  double2* f = F + row * nX + k0;
+  long long mx = 0;
+  for (int kk = lane; kk < kc; kk += 32) mx = max(mx, max(abs_bits(f[kk].x), abs_bits(f[kk].y)));
+  for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  const int ex = row_exp(mx);
+  if (lane == 0) e[w] = ex;
+  for (int kk = lane; kk < kc; kk += 32) {
+    const double2 v = f[kk];
+    // (fixed56 scales by 2^(56 - e): one exponent up gives 2^(55 - e); a flagged row becomes zeros)
+    const long long a = fixed56(v.x, ex + 1), b = fixed56(v.y, ex + 1);
+    const int a1 = (int)((a + (1LL << 27)) >> 28), b1 = (int)((b + (1LL << 27)) >> 28);
+    const int4 o = make_int4(a1, (int)(a - ((long long)a1 << 28)), b1, (int)(b - ((long long)b1 << 28)));
+    reinterpret_cast<int4*>(f)[kk] = o;
   }
 }
 
 // Slices of the Khatri-Rao rows of a chunk of (incidence, receiver) pairs, for
 // the x-projection of the Jacobian: complex row (pair c, gy) of w = u_d z_p
-// (d = (c0 + c) / P, p = (c0 + c) % P, fields on the interior grid,
+// (d = (c0 + c) / P, p = (c0 + c) % P, fixed-point fields on the interior grid,
 // [rhs][gy][gx]) over the piece's gx, split into its real part (row
 // 2 (c nX + gy)) and imaginary part (row 2 (c nX + gy) + 1).  One warp per
-// complex row and piece, two neighbouring gx per lane (32-bit stores, a whole
-// 128-byte line per warp and slice: with 2-byte stores the kernel was bound by
-// the store instructions, 101 ms for the 25,600 pairs of the k = 40 Jacobian).
-// The product is formed in FP64 in registers and never stored.
-__global__ void __launch_bounds__(256) k_oz_slice_kr(const double2* __restrict__ Ug, const double2* __restrict__ Zg,
-                                                     int P, int nX, long long c0, int nc, int pl, long long rpad,
-                                                     int kt, __nv_bfloat16* __restrict__ out, int* __restrict__ e) {
+// complex row and piece, two neighbouring gx per lane, never stored.
+// The row's exponent is the fields' sum plus one (|re u re z| + |im u im z| < 2),
+// known before the products, so a row need not be held for its maximum; the
+// products are taken in integers, N = 2 (U1 Z1) + (U1 Z0 + U0 Z1) 2^-27 per
+// real product, six 32 x 32 + 64 multiply-adds per part (the U0 Z0 term is below
+// one unit of 2^-56).  Against FP64 products and the row's own maximum: no
+// operation on the FP64 pipe (60% busy then, with 145 instructions per real
+// entry), and an error of about one unit of 2^-56 of the fields' maxima where
+// FP64 rounds each product to 2^-53 of itself.  25,600 pairs at n = 448: 101 ms
+// with FP64 products and 2-byte stores, 95 with 32-bit stores, 54 now (164 GB
+// written, 82 GB of fields read: 4.5 TB/s).
+__global__ void __launch_bounds__(256) k_oz_slice_kr(const int4* __restrict__ Ug, const int4* __restrict__ Zg,
+                                                     const int* __restrict__ eu, const int* __restrict__ ez, int P,
+                                                     int nX, long long c0, int nc, int pl, int npc, long long rpad,
+                                                     int nst, uint32_t* __restrict__ out, int* __restrict__ e) {
   const long long r2 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r2 >= (long long)nc * nX) return;
   const int k0 = blockIdx.y * pl, kc = min(pl, nX - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
-  const long long c = c0 + r2 / nX, gy = r2 % nX, plane = (long long)nX * nX;
-  const double2* u = Ug + (c / P) * plane + gy * nX + k0;
-  const double2* z = Zg + (c % P) * plane + gy * nX + k0;
-  constexpr int KPL = OZ_KMAX / 64;
-  double2 w[KPL][2];
-  long long mr = 0, mi = 0;
-#pragma unroll
-  for (int q = 0; q < KPL; ++q)
+  const long long c = c0 + r2 / nX, gy = r2 % nX;
+  const long long ru = (c / P) * nX + gy, rz = (c % P) * nX + gy;
+  const int4* u = Ug + ru * nX + k0;
+  const int4* z = Zg + rz * nX + k0;
+  if (lane == 0) {
+    const int ex = min(eu[ru * npc + blockIdx.y] + ez[rz * npc + blockIdx.y] + 1, OZ_NAN);
+    e[blockIdx.y * rpad + 2 * r2] = ex;
+    e[blockIdx.y * rpad + 2 * r2 + 1] = ex;
+  }
+  auto mac = [](long long acc, int a, int b) { return acc + (long long)a * b; };
+#pragma unroll 2
+  for (int kk = 2 * lane; kk < kp; kk += 64) {
+    long long re[2], im[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int kk = 2 * lane + 64 * q + h;
-      w[q][h] = make_double2(0.0, 0.0);
-      if (kk < kc) {
-        const double2 a = u[kk], b = z[kk];
-        w[q][h] = make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+      int4 a = make_int4(0, 0, 0, 0), b = a;
+      if (kk + h < kc) {
+        a = u[kk + h];
+        b = z[kk + h];
       }
-      mr = max(mr, abs_bits(w[q][h].x));
-      mi = max(mi, abs_bits(w[q][h].y));
+      const long long rh = mac((long long)a.x * b.x, -a.z, b.z);
+      const long long rl = mac(mac(mac((long long)a.x * b.y, a.y, b.x), -a.z, b.w), -a.w, b.z);
+      const long long ih = mac((long long)a.x * b.z, a.z, b.x);
+      const long long il = mac(mac(mac((long long)a.x * b.w, a.y, b.z), a.z, b.y), a.w, b.x);
+      re[h] = 2 * rh + ((rl + (1LL << 26)) >> 27);
+      im[h] = 2 * ih + ((il + (1LL << 26)) >> 27);
     }
-  for (int off = 16; off > 0; off >>= 1) {
-    mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, off));
-    mi = max(mi, __shfl_xor_sync(0xffffffffu, mi, off));
-  }
-  const int er = row_exp(mr), ei = row_exp(mi);
-  if (lane == 0) {
-    e[blockIdx.y * rpad + 2 * r2] = er;
-    e[blockIdx.y * rpad + 2 * r2 + 1] = ei;
-  }
-  const long long plane2 = rpad * kt / 2;
-  uint32_t* o_re = reinterpret_cast<uint32_t*>(out) + (2 * r2 * kt + k0) / 2;
-  uint32_t* o_im = o_re + kt / 2;
-#pragma unroll
-  for (int q = 0; q < KPL; ++q) {
-    const int kk = 2 * lane + 64 * q;
-    if (kk >= kp) break;
-    put2(w[q][0].x, w[q][1].x, er, o_re + kk / 2, plane2);
-    put2(w[q][0].y, w[q][1].y, ei, o_im + kk / 2, plane2);
+    // (rows 2 r2 and 2 r2 + 1 lie in one tile, 64 bytes apart, with the same swizzle)
+    uint32_t* o = out + oz_at<OZ_TM>(2 * r2, k0 + kk, nst);
+    put2(re[0], re[1], o, OZ_ROW * OZ_TM);
+    put2(im[0], im[1], o + OZ_ROW, OZ_ROW * OZ_TM);
   }
 }
 
-// Zero slices of the padding rows [first, rpad) of every slice plane.
-__global__ void k_oz_zero_rows(long long first, long long rpad, int kt, int npc, __nv_bfloat16* __restrict__ out,
+// Zero slices and exponents of the padding rows [first, rpad) of the last tile.
+__global__ void k_oz_zero_rows(long long first, long long rpad, int nst, int npc, uint32_t* __restrict__ out,
                                int* __restrict__ e) {
-  const long long n = (rpad - first) * kt;
+  const int nr = (int)(rpad - first);
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * OZ_S) return;
-  const int s = (int)(t / n);
-  const long long j = t % n;
-  out[s * rpad * kt + first * kt + j] = __float2bfloat16_rn(0.f);
-  if (s == 0 && j < (rpad - first) * npc) e[(j / (rpad - first)) * rpad + first + j % (rpad - first)] = 0;
+  if (t >= (long long)nr * nst * OZ_S * OZ_ROW) return;
+  const int w = (int)(t % OZ_ROW), r = (int)(t / OZ_ROW % nr);
+  const long long blk = t / OZ_ROW / nr;  // k-step and slice
+  out[((rpad / OZ_TM - 1) * nst * OZ_S + blk) * OZ_TM * OZ_ROW + (first + r) % OZ_TM * OZ_ROW + w] = 0u;
+  if (t < (long long)nr * npc) e[(t / nr) * rpad + first + t % nr] = 0;
 }
 
 // V 2^e as a double (round to nearest even), in integer arithmetic: two 64-bit
@@ -312,6 +343,8 @@ struct OzParams {
   int zs, ppz;                 // z groups of ppz pieces, each to its own plane of C (zs > 1: alpha 1, beta 0)
   long long items, zplane;
   double alpha, beta;
+  const char *a, *b;           // sliced operands
+  int nst;                     // k-steps of a row tile
   const int *ea, *eb;          // exponents [piece][row]
   long long ea_piece, eb_piece;
   OzView C;
@@ -333,15 +366,17 @@ __device__ __forceinline__ bool oz_item(const OzParams& P, long long it, OzItem&
 // it: 36 slice products, 2304 tensor cycles per 32-k stage at the bf16 rate, and
 // the epilogue of each piece, which cannot overlap the next piece's products
 // (the eight diagonals fill TMEM).  So the epilogue is integer arithmetic on
-// eight warps (one conversion per diagonal, two diagonals per 32-bit
+// sixteen warps (one conversion per diagonal, two diagonals per 32-bit
 // multiply-add, the double assembled from its bits), and the ring already
 // loads the next piece behind it.  Before, one launch per piece with an FP64
 // epilogue on four warps and C read back per piece kept the tensor pipe at 17%:
 // the products of a k = 40 Gauss-Newton step (Jacobian projections and normal
-// matrix, 3.2e12 flops) took 278 ms, now 110 ms (the normal matrix by its
-// lower tiles only).
+// matrix, 3.2e12 flops) took 278 ms, now 102 ms (the normal matrix by its
+// lower tiles only).  Measured per tile: 4250 clocks (at 1.92 GHz) a stage and
+// 11,000 a piece; 30 TFLOP/s of FP64-equivalent work for long k, 1080 of the 1948
+// TFLOP/s bf16 peak issued (shared memory: 256 KB read and 96 KB written a stage).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_mma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, OzParams P) {
+    k_oz_mma(const __grid_constant__ OzParams P) {
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   __shared__ uint32_t tslot;
@@ -358,7 +393,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&empty[i])), "r"(1));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&accf)), "r"(1));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce)), "r"(8));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce)), "r"(OZ_EPI));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&done)), "r"(1));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -375,7 +410,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
         OzItem o;
         if (!oz_item(P, it, o)) continue;
-        const int rowA = o.b * P.mpad + o.tm * OZ_TM, rowB = (P.b_shared ? 0 : o.b) * P.npad + o.tn * OZ_TN;
+        const char* pa = P.a + (long long)(o.b * P.tm + o.tm) * P.nst * (OZ_S * OZ_A_SL);
+        const char* pb = P.b + (long long)((P.b_shared ? 0 : o.b) * P.tn + o.tn) * P.nst * (OZ_S * OZ_B_SL);
         for (int p = o.z * P.ppz; p < min(P.npc, (o.z + 1) * P.ppz) && ok; ++p) {
           const int nst = stages(p);
           for (int i = 0; i < nst; ++i, ++c) {
@@ -385,9 +421,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(&full[st])), "r"(OZ_STAGE)
                          : "memory");
             const uint32_t base = su32(sm + st * OZ_STAGE);
-            const int kx = p * P.pl + i * OZ_KS;
-            oz_tma3(base, &mapA, kx, rowA, 0, su32(&full[st]));
-            oz_tma3(base + OZ_S * OZ_A_SL, &mapB, kx, rowB, 0, su32(&full[st]));
+            const long long ks = p * (P.pl / OZ_KS) + i;
+            oz_copy(base, pa + ks * (OZ_S * OZ_A_SL), OZ_S * OZ_A_SL, su32(&full[st]));
+            oz_copy(base + OZ_S * OZ_A_SL, pb + ks * (OZ_S * OZ_B_SL), OZ_S * OZ_B_SL, su32(&full[st]));
           }
         }
       }
@@ -450,20 +486,20 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done)));
     }
   } else {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows (lane = row), 32 of the 64 columns
-    const int quarter = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(half * 32);
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows (lane = row), 16 of the 64 columns
+    const int quarter = warp & 3, part = (warp - 2) >> 2;
+    const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(part * 16);
     int pc = 0;
     for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
       OzItem o;
       if (!oz_item(P, it, o)) continue;
-      const int r = o.tm * OZ_TM + quarter * 32 + lane, cb = o.tn * OZ_TN + half * 32;
+      const int r = o.tm * OZ_TM + quarter * 32 + lane, cb = o.tn * OZ_TN + part * 16;
       const int p0 = o.z * P.ppz, p1 = min(P.npc, p0 + P.ppz);
-      double acc[32];
+      double acc[16];
       for (int p = p0; p < p1; ++p, ++pc) {
         // (rows and columns of the padding have exponents too)
         const int ea = P.ea[p * P.ea_piece + (long long)o.b * P.mpad + r];
-        const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + lane];
+        const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + (lane & 15)];
         // |sum of the piece| <= 1.02 kc: V = sum 2^(63 - rs) stays below 2^62
         const int rs = 33 - __clz(min(P.pl, P.k - p * P.pl));
         ok = oz_wait(su32(&accf), pc & 1);
@@ -472,46 +508,47 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
+        // pairs of diagonals in 32 bits: |C_d| <= 384 4096 (d + 3) (6.3e6 for d = 0),
+        // 128 C_d + C_(d+1) <= 1.83e9 < 2^31
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-          // pairs of diagonals in 32 bits: |C_d| <= 384 4096 (d + 3) (6.3e6 for d = 0),
-          // 128 C_d + C_(d+1) <= 1.83e9 < 2^31
-          long long V[16];
+        for (int h = 0; h < 2; ++h) {  // eight columns at a time (registers)
+          long long V[8];
+          int q0[8];
 #pragma unroll
-          for (int g = 0; g < 2; ++g) {
-            uint32_t v[4][16];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) oz_ld16(ta + (uint32_t)((4 * g + d) * OZ_TN + ch * 16), v[d]);
+          for (int g = 0; g < 4; ++g) {
+            uint32_t v[2][8];
+            oz_ld8(ta + (uint32_t)(2 * g * OZ_TN + 8 * h), v[0]);
+            oz_ld8(ta + (uint32_t)((2 * g + 1) * OZ_TN + 8 * h), v[1]);
             asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (ch == 1 && g == 1) {  // last read of this piece: the accumulators are free
+            if (h == 1 && g == 3) {  // last read of this piece: the accumulators are free
               asm volatile("tcgen05.fence::before_thread_sync;");
               __syncwarp();
               if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acce)) : "memory");
             }
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int q0 = 128 * __float2int_rn(__uint_as_float(v[0][j])) + __float2int_rn(__uint_as_float(v[1][j]));
-              const int q1 = 128 * __float2int_rn(__uint_as_float(v[2][j])) + __float2int_rn(__uint_as_float(v[3][j]));
-              const long long w = ((long long)q0 << 14) + q1;
-              // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63
-              V[j] = g == 0 ? w << (28 - rs) : V[j] + ((w + (1LL << (rs - 1))) >> rs);
+            for (int j = 0; j < 8; ++j) {
+              const int q = 128 * __float2int_rn(__uint_as_float(v[0][j])) + __float2int_rn(__uint_as_float(v[1][j]));
+              // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63, hi and lo = q 2^14 + the next q
+              if (g == 0 || g == 2) q0[j] = q;
+              else if (g == 1) V[j] = (((long long)q0[j] << 14) + q) << (28 - rs);
+              else V[j] += (((long long)q0[j] << 14) + q + (1LL << (rs - 1))) >> rs;
             }
           }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int eb = __shfl_sync(0xffffffffu, ebl, ch * 16 + j);
+          for (int j = 0; j < 8; ++j) {
+            const int eb = __shfl_sync(0xffffffffu, ebl, 8 * h + j);
             const double x = scaled(V[j], ea + eb + rs - 63);
-            acc[ch * 16 + j] = p == p0 ? x : acc[ch * 16 + j] + x;
+            acc[8 * h + j] = p == p0 ? x : acc[8 * h + j] + x;
           }
         }
       }
       if (!ok) break;
       if (r < P.m) {
         double* pr = P.C.p + o.z * P.zplane + o.b * P.C.sb + (r / P.C.ig) * P.C.si + (r % P.C.ig) * P.C.sg;
-        if (P.C.sk == 1 && (reinterpret_cast<uintptr_t>(pr + cb) & 15) == 0 && cb + 32 <= P.n) {
+        if (P.C.sk == 1 && (reinterpret_cast<uintptr_t>(pr + cb) & 15) == 0 && cb + 16 <= P.n) {
           double2* p2 = reinterpret_cast<double2*>(pr + cb);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
+          for (int j = 0; j < 8; ++j) {
             double2 x = make_double2(P.alpha * acc[2 * j], P.alpha * acc[2 * j + 1]);
             if (P.beta != 0.0) {
               const double2 y = p2[j];
@@ -521,7 +558,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
+          for (int j = 0; j < 16; ++j)
             if (cb + j < P.n) {
               double* q = pr + (cb + j) * P.C.sk;
               const double x = P.alpha * acc[j];
@@ -552,32 +589,6 @@ __global__ void k_oz_combine(const double* __restrict__ planes, int zs, long lon
   const long long j = e % n, t = e / n, i = t % m, b = t / m;
   double* c = C.p + b * C.sb + (i / C.ig) * C.si + (i % C.ig) * C.sg + j * C.sk;
   *c = beta == 0.0 ? alpha * v : fma(beta, *c, alpha * v);
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_encode_once;
-
-bool encode_fn() {
-  std::call_once(g_encode_once, [] {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  });
-  return g_encode != nullptr;
-}
-
-// 3-D map over slices [OZ_S][rows][kt] (BF16), box {32 k, box_rows, all
-// slices} with the 64-byte swizzle of the MMA operand layout.
-bool make_map(CUtensorMap* map, void* base, long long rows, int kt, int box_rows) {
-  const cuuint64_t dims[3] = {(cuuint64_t)kt, (cuuint64_t)rows, (cuuint64_t)OZ_S};
-  const cuuint64_t strides[2] = {(cuuint64_t)kt * 2, (cuuint64_t)rows * kt * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)OZ_KS, (cuuint32_t)box_rows, (cuuint32_t)OZ_S};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 inline long long rup(long long x, long long m) { return (x + m - 1) / m * m; }
@@ -623,7 +634,9 @@ void set_smem_attr() {
   static bool done[64] = {};
   once_per_device(done, [] {
     cudaFuncSetAttribute(k_oz_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-    cudaFuncSetAttribute(k_oz_slice, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_oz_slice<OZ_TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         OZ_SR * (OZ_KMAX + 1) * (int)sizeof(double));
+    cudaFuncSetAttribute(k_oz_slice<OZ_TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          OZ_SR * (OZ_KMAX + 1) * (int)sizeof(double));
   });
 }
@@ -651,23 +664,35 @@ void oz_slice(cudaStream_t s, OzSrc v, int rows, int k, int batch, bool is_a, vo
   const long long rpad = padded(rows, is_a), total = batch * rpad;
   const int pl = piece_len(k), npc = npieces(k);
   char* base = reinterpret_cast<char*>(buf);
-  k_oz_slice<<<dim3((unsigned)((total + OZ_SR - 1) / OZ_SR), npc), 256, OZ_SR * (pl + 1) * sizeof(double), s>>>(
-      v, rows, k, pl, (int)rpad, npc * pl, total, reinterpret_cast<__nv_bfloat16*>(base),
+  auto kernel = is_a ? k_oz_slice<OZ_TM> : k_oz_slice<OZ_TN>;
+  kernel<<<dim3((unsigned)((total + OZ_SR - 1) / OZ_SR), npc), 256, OZ_SR * (pl + 1) * sizeof(double), s>>>(
+      v, rows, k, pl, (int)rpad, npc * pl / OZ_KS, total, reinterpret_cast<uint32_t*>(base),
       reinterpret_cast<int*>(base + slice_bytes(total, k)));
   HS_COUNT_LAUNCH();
 }
 
-void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, int P, int nX, long long c0, int nc,
-                         void* buf) {
-  const int rows = 2 * nc * nX, pl = piece_len(nX), npc = npieces(nX), kt = npc * pl;
+size_t oz_fix_bytes(int fields, int nX) { return align_up((size_t)fields * nX * npieces(nX) * 4); }
+
+void oz_fix_fields(cudaStream_t s, double2* F, int fields, int nX, void* exps) {
+  const long long rows = (long long)fields * nX, warps = rows * npieces(nX);
+  k_oz_fix<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(F, rows, nX, piece_len(nX), npieces(nX),
+                                                      reinterpret_cast<int*>(exps));
+  HS_COUNT_LAUNCH();
+}
+
+void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, const void* eu, const void* ez, int P,
+                         int nX, long long c0, int nc, void* buf) {
+  const int rows = 2 * nc * nX, pl = piece_len(nX), npc = npieces(nX), nst = npc * pl / OZ_KS;
   const long long rpad = padded(rows, true), warps = (long long)nc * nX;
-  __nv_bfloat16* sl = reinterpret_cast<__nv_bfloat16*>(buf);
+  uint32_t* sl = reinterpret_cast<uint32_t*>(buf);
   int* ex = reinterpret_cast<int*>(reinterpret_cast<char*>(buf) + slice_bytes(rpad, nX));
-  k_oz_slice_kr<<<dim3((unsigned)((warps + 7) / 8), npc), 256, 0, s>>>(Ug, Zg, P, nX, c0, nc, pl, rpad, kt, sl, ex);
+  k_oz_slice_kr<<<dim3((unsigned)((warps + 7) / 8), npc), 256, 0, s>>>(
+      reinterpret_cast<const int4*>(Ug), reinterpret_cast<const int4*>(Zg), reinterpret_cast<const int*>(eu),
+      reinterpret_cast<const int*>(ez), P, nX, c0, nc, pl, npc, rpad, nst, sl, ex);
   HS_COUNT_LAUNCH();
   if (rpad > rows) {
-    const long long n = (rpad - rows) * kt * OZ_S;
-    k_oz_zero_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rows, rpad, kt, npc, sl, ex);
+    const long long n = (rpad - rows) * nst * OZ_S * OZ_ROW;
+    k_oz_zero_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rows, rpad, nst, npc, sl, ex);
     HS_COUNT_LAUNCH();
   }
 }
@@ -675,14 +700,11 @@ void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, i
 cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double alpha, const void* Aop, const void* Bop,
                         bool b_shared, double beta, OzView C, void* planes, bool sym) {
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
-  if (!encode_fn()) return cudaErrorNotSupported;
   set_smem_attr();
   const long long mp = padded(m, true), np = padded(n, false), ta = batch * mp, tb = (b_shared ? 1 : batch) * np;
   const int pl = piece_len(k), npc = npieces(k), zs = planes ? z_groups(m, n, k, batch) : 1;
   char* a = const_cast<char*>(reinterpret_cast<const char*>(Aop));
   char* b = const_cast<char*>(reinterpret_cast<const char*>(Bop));
-  CUtensorMap ma, mb;
-  if (!make_map(&ma, a, ta, npc * pl, OZ_TM) || !make_map(&mb, b, tb, npc * pl, OZ_TN)) return cudaErrorInvalidValue;
   OzParams P;
   P.m = m;
   P.n = n;
@@ -699,6 +721,9 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
   P.ppz = (npc + zs - 1) / zs;
   P.zs = (npc + P.ppz - 1) / P.ppz;
   P.items = (long long)P.tm * P.tn * batch * P.zs;
+  P.a = a;
+  P.b = b;
+  P.nst = npc * pl / OZ_KS;
   P.ea = reinterpret_cast<const int*>(a + slice_bytes(ta, k));
   P.eb = reinterpret_cast<const int*>(b + slice_bytes(tb, k));
   P.ea_piece = ta;
@@ -711,7 +736,7 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
   const bool prof = prof_active(4);
   cudaEvent_t ev = nullptr;
   if (prof) prof_begin(s, &ev);
-  k_oz_mma<<<(unsigned)std::min<long long>(P.items, 152), OZ_THREADS, OZ_SMEM, s>>>(ma, mb, P);
+  k_oz_mma<<<(unsigned)std::min<long long>(P.items, 152), OZ_THREADS, OZ_SMEM, s>>>(P);
   HS_COUNT_LAUNCH();
   if (split) {
     k_oz_combine<<<(unsigned)((P.zplane + 255) / 256), 256, 0, s>>>(reinterpret_cast<double*>(planes), P.zs, P.zplane,
@@ -743,7 +768,6 @@ size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared) {
 cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
                        double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym) {
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
-  if (!encode_fn()) return cudaErrorNotSupported;
   if (ozaki_scratch_bytes(m, n, k, batch, b_shared) > scratch_bytes) return cudaErrorInvalidValue;
   char* a = reinterpret_cast<char*>(scratch);
   char* b = a + oz_operand_bytes(m, k, batch, true);

@@ -145,10 +145,10 @@ void interior_sine_tables(cudaStream_t s, const double* xg_int, int n, int S1, i
 // Pairs per chunk of the contraction within budget_bytes of W and T (the
 // emulated FP64 product needs contract_emulated_bytes on top).
 int contract_chunk(int M, int P, int nX, int S1, size_t budget_bytes);
-size_t contract_emulated_bytes(int C, int nX, int S1, int S2);
+size_t contract_emulated_bytes(int C, int nX, int S1, int S2, int M, int P);
 // scratch: emulated-product slices (contract_emulated_bytes), or NULL for the
 // FP64 SIMT GEMMs.
-void contract_jacobian(cudaStream_t s, const double2* Ug, const double2* Zg, int M, int P, int nX, const double* sx,
+bool contract_jacobian(cudaStream_t s, double2* Ug, double2* Zg, int M, int P, int nX, const double* sx,
                        const double* sy, int S1, int S2, double k2, double2* J, double2* W, double2* T, int C,
                        void* scratch, size_t scratch_bytes);
 void split_stack(cudaStream_t s, const double2* J, int rows, int cols, double* Jst);
