@@ -88,18 +88,20 @@ __global__ void k_bie_plain(const double* __restrict__ x, const double* __restri
   Dl[e] = make_double2(d.x * w[j], d.y * w[j]);
 }
 
-// One block per (target node, near-panel slot): product-integration weights of
-// S and D against the 14 Lagrange basis polynomials of the source panel.
+// Product-integration weights of S and D against the 14 Lagrange basis
+// polynomials of the source panel, one block per target node of one panel pair
+// of each class.  The weights depend on the pair's relative position only, and
+// the panels of a square repeat a few dozen of them (Boundary::cls), so they are
+// integrated once per class and copied to every pair (k_bie_scatter): the 1824
+// Hankel evaluations of a node and panel are the cost (FP64): 1.9 ms for all
+// pairs of 8 x 8 leaves, 0.5 ms for the classes of any tree.
 __global__ void __launch_bounds__(128) k_bie_near(const double* __restrict__ x, const double* __restrict__ y,
-                                                  const int* __restrict__ panel, const double* __restrict__ p0x,
-                                                  const double* __restrict__ p0y, const double* __restrict__ tx,
-                                                  const double* __restrict__ ty, const double* __restrict__ pnx,
-                                                  const double* __restrict__ pny, const int* __restrict__ nearp,
-                                                  double h, double k, int nb, double2* __restrict__ S,
-                                                  double2* __restrict__ Dl) {
-  const int i = blockIdx.x;
-  const int q = nearp[panel[i] * NEAR + blockIdx.y];
-  if (q < 0) return;
+                                                  const double* __restrict__ p0x, const double* __restrict__ p0y,
+                                                  const double* __restrict__ tx, const double* __restrict__ ty,
+                                                  const double* __restrict__ pnx, const double* __restrict__ pny,
+                                                  const int* __restrict__ nearp, const int* __restrict__ rep, double h, double k, int ncls,
+                                                  double2* __restrict__ W) {
+  const int pair = rep[blockIdx.y], i = pair / NEAR * NPT + blockIdx.x, q = nearp[pair];
   const double ax = x[i] - p0x[q], ay = y[i] - p0y[q];
   const double at = ax * tx[q] + ay * ty[q];
   const double an = ax * pnx[q] + ay * pny[q];  // exactly 0 for a target on the source's side
@@ -162,18 +164,34 @@ __global__ void __launch_bounds__(128) k_bie_near(const double* __restrict__ x, 
       dr += red[wv][2 * NPT + 2 * j];
       di += red[wv][2 * NPT + 2 * j + 1];
     }
-    long long o = (long long)i * nb + q * NPT + j;
-    S[o] = make_double2(sr, si);
-    Dl[o] = make_double2(dr, di);
+    const int o = (blockIdx.y * NPT + blockIdx.x) * NPT + j;
+    W[o] = make_double2(sr, si);
+    W[ncls * NPT * NPT + o] = make_double2(dr, di);
   }
+}
+
+// The class weights W (two planes) into the rows of two matrices.
+__global__ void k_bie_scatter(const int* __restrict__ nearp, const int* __restrict__ cls, int ncls, int nb,
+                              const double2* __restrict__ W, double2* __restrict__ A, double2* __restrict__ B) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nb * NEAR * NPT) return;
+  const int j = e % NPT, slot = e / NPT % NEAR, i = e / NPT / NEAR;
+  const int pair = i / NPT * NEAR + slot, q = nearp[pair];
+  if (q < 0) return;
+  const int w = (cls[pair] * NPT + i % NPT) * NPT + j;
+  const long long o = (long long)i * nb + q * NPT + j;
+  A[o] = W[w];
+  B[o] = W[ncls * NPT * NPT + w];
 }
 
 void bie_matrices(cudaStream_t s, const Boundary& B, double k, double2* S, double2* Dl) {
   long long n = (long long)B.nb * B.nb;
   k_bie_plain<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(B.x, B.y, B.nx, B.ny, B.w, B.nb, k, S, Dl);
   HS_COUNT_LAUNCH();
-  k_bie_near<<<dim3(B.nb, NEAR), 128, 0, s>>>(B.x, B.y, B.panel, B.p0x, B.p0y, B.tx, B.ty, B.pnx, B.pny, B.near,
-                                              B.h, k, B.nb, S, Dl);
+  k_bie_near<<<dim3(NPT, B.ncls), 128, 0, s>>>(B.x, B.y, B.p0x, B.p0y, B.tx, B.ty, B.pnx, B.pny, B.near, B.rep, B.h,
+                                               k, B.ncls, B.wts);
+  HS_COUNT_LAUNCH();
+  k_bie_scatter<<<(unsigned)((B.nb * NEAR * NPT + 255) / 256), 256, 0, s>>>(B.near, B.cls, B.ncls, B.nb, B.wts, S, Dl);
   HS_COUNT_LAUNCH();
 }
 
@@ -203,7 +221,7 @@ __global__ void k_bie_plain_nt(const double* __restrict__ x, const double* __res
   H[e] = c * (sg * (dx * tx[p] + dy * ty[p]));
 }
 
-// One block per (target node, near-panel slot), as k_bie_near: product
+// One block per target node and class, as k_bie_near: product
 // integration of dG/dn_x and dG/dt_x against the source panel's Lagrange
 // basis.  With x - y = dt tau_q + an n_q in the source panel's frame, the
 // projections on the target's normal and tangent are dt (tau_q . n_x) +
@@ -211,15 +229,12 @@ __global__ void k_bie_plain_nt(const double* __restrict__ x, const double* __res
 // tau_q . n_x = 0, tau_q . t_x = sgn) K' vanishes and H is a principal value.
 __global__ void __launch_bounds__(128) k_bie_near_nt(const double* __restrict__ x, const double* __restrict__ y,
                                                      const double* __restrict__ nx, const double* __restrict__ ny,
-                                                     const int* __restrict__ panel, const double* __restrict__ p0x,
-                                                     const double* __restrict__ p0y, const double* __restrict__ tx,
-                                                     const double* __restrict__ ty, const double* __restrict__ pnx,
-                                                     const double* __restrict__ pny, const int* __restrict__ nearp,
-                                                     double h, double k, int nb, double2* __restrict__ Kp,
-                                                     double2* __restrict__ H) {
-  const int i = blockIdx.x, pi = panel[i];
-  const int q = nearp[pi * NEAR + blockIdx.y];
-  if (q < 0) return;
+                                                     const double* __restrict__ p0x, const double* __restrict__ p0y,
+                                                     const double* __restrict__ tx, const double* __restrict__ ty,
+                                                     const double* __restrict__ pnx, const double* __restrict__ pny,
+                                                     const int* __restrict__ nearp, const int* __restrict__ rep, double h, double k, int ncls,
+                                                     double2* __restrict__ W) {
+  const int pair = rep[blockIdx.y], pi = pair / NEAR, i = pi * NPT + blockIdx.x, q = nearp[pair];
   const bool self = q == pi;
   const double sg = ccw_sign(tx[pi], ty[pi], pnx[pi], pny[pi]);
   const double txx = sg * tx[pi], txy = sg * ty[pi], nxi = nx[i], nyi = ny[i];
@@ -307,9 +322,9 @@ __global__ void __launch_bounds__(128) k_bie_near_nt(const double* __restrict__ 
       }
       hr += sg * (-inv2pi) * pv;
     }
-    const long long o = (long long)i * nb + q * NPT + j;
-    Kp[o] = make_double2(kr, ki);
-    H[o] = make_double2(hr, hi2);
+    const int o = (blockIdx.y * NPT + blockIdx.x) * NPT + j;
+    W[o] = make_double2(kr, ki);
+    W[ncls * NPT * NPT + o] = make_double2(hr, hi2);
   }
 }
 
@@ -345,8 +360,10 @@ void bie_combined(cudaStream_t s, const Boundary& B, double k, double eta, doubl
   const unsigned g = (unsigned)((n + 255) / 256);
   k_bie_plain_nt<<<g, 256, 0, s>>>(B.x, B.y, B.nx, B.ny, B.w, B.panel, B.tx, B.ty, B.pnx, B.pny, B.nb, k, Kp, H);
   HS_COUNT_LAUNCH();
-  k_bie_near_nt<<<dim3(B.nb, NEAR), 128, 0, s>>>(B.x, B.y, B.nx, B.ny, B.panel, B.p0x, B.p0y, B.tx, B.ty, B.pnx,
-                                                 B.pny, B.near, B.h, k, B.nb, Kp, H);
+  k_bie_near_nt<<<dim3(NPT, B.ncls), 128, 0, s>>>(B.x, B.y, B.nx, B.ny, B.p0x, B.p0y, B.tx, B.ty, B.pnx, B.pny, B.near,
+                                                  B.rep, B.h, k, B.ncls, B.wts);
+  HS_COUNT_LAUNCH();
+  k_bie_scatter<<<(unsigned)((B.nb * NEAR * NPT + 255) / 256), 256, 0, s>>>(B.near, B.cls, B.ncls, B.nb, B.wts, Kp, H);
   HS_COUNT_LAUNCH();
   k_bie_combine<<<g, 256, 0, s>>>(B.nx, B.ny, B.tx, B.ty, B.pnx, B.pny, B.nb, B.h, k, eta, Kp, H, S, Dl);
   HS_COUNT_LAUNCH();

@@ -148,6 +148,50 @@ template <> __host__ __device__ inline float2 scal<float2, float2>(float2 s, flo
 
 }  // namespace hs
 
+// Fixed point of FP64 values, in integer arithmetic (the FP64 pipe is scarce).
+namespace hs {
+constexpr int OZ_NAN = 1 << 20;  // exponent of a row with an infinity or a NaN: its outputs are NaN
+// |x| as ordered 64-bit integers (the bit pattern of a non-negative double).
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL; }
+
+// round(x 2^(56 - e)) for |x| < 2^e, in integer arithmetic on the bit pattern
+// (mantissa shifted by the exponent difference, rounded to nearest); 0 for
+// zeros and subnormals, whose contribution is below the slices' resolution.
+__device__ __forceinline__ long long fixed56(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7FF);
+  if (E == 0) return 0;
+  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;  // 53-bit significand
+  const int sh = E - 1075 + 56 - e;                                     // x 2^(56-e) = m 2^sh, sh <= 3
+  long long v;
+  if (sh >= 0) v = m << sh;
+  else if (sh > -60) v = (m + (1LL << (-sh - 1))) >> (-sh);
+  else v = 0;
+  return b < 0 ? -v : v;
+}
+
+// Exponent of a row from its largest |x| (bit pattern): max in [2^(ex-1), 2^ex).
+__device__ __forceinline__ int row_exp(long long mx) {
+  const int e = (int)(mx >> 52);
+  return mx == 0 ? 0 : e == 0x7FF ? OZ_NAN : e - 1022;
+}
+}  // namespace hs
+
+// Asynchronous copies from global to shared memory: 16 bytes with zero fill past
+// `bytes`, or one element of 4, 8 or 16.
+namespace hs {
+__device__ __forceinline__ void cp16(void* dst, const void* src, int bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+template <int BYTES> __device__ __forceinline__ void cp_elem(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+}  // namespace hs
+
 // Launch bookkeeping: every kernel launch in the library goes through HS_LAUNCH
 // so that the context can report how many of its kernels ran.
 namespace hs {

@@ -1,6 +1,7 @@
 // C ABI of libhs (include/hs.h): host-side orchestration of the direct solver
 // of Sec. 2 and of the Jacobian / Gauss-Newton step of Sec. 3 on one GPU.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -156,6 +157,8 @@ struct hs_ctx {
   std::string err;
   long long launches = 0;
   std::vector<void*> allocs;  // persistent allocations
+  char* block = nullptr;      // the block small buffers are carved from (dalloc)
+  size_t block_left = 0;
   // geometry
   double *d_xg = nullptr, *d_xint = nullptr;
   double *d_q = nullptr, *d_c = nullptr, *d_sx16 = nullptr, *d_sy16 = nullptr, *d_T = nullptr, *d_Qg = nullptr;
@@ -307,15 +310,33 @@ bool injected_alloc_failure() {
   return true;
 }
 
+// A context's persistent buffers: those up to 4 MB are carved from 16 MB blocks
+// (a context has some 150 of them; a cudaMalloc and a cudaFree each made creating
+// and destroying a context a fifth of a low-frequency sweep), larger ones
+// are allocations of their own.
 template <typename T> int dalloc(hs_ctx* ctx, T** p, size_t n) {
   if (injected_alloc_failure()) return fail(ctx, HS_ENOMEM, "device allocation refused (injected failure)");
-  void* v = nullptr;
-  cudaError_t e = cudaMalloc(&v, std::max<size_t>(n, 1) * sizeof(T));
-  if (e != cudaSuccess)
-    return fail(ctx, HS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(n * sizeof(T)) + " bytes: " +
-                                    cudaGetErrorString(e));
-  ctx->allocs.push_back(v);
-  *p = reinterpret_cast<T*>(v);
+  constexpr size_t kSmall = (size_t)4 << 20, kBlock = (size_t)16 << 20;
+  const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~size_t(255);
+  const bool small = bytes <= kSmall;
+  if (!small || ctx->block_left < bytes) {
+    void* v = nullptr;
+    const size_t want = small ? kBlock : bytes;
+    cudaError_t e = cudaMalloc(&v, want);
+    if (e != cudaSuccess)
+      return fail(ctx, HS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(want) + " bytes: " +
+                                      cudaGetErrorString(e));
+    ctx->allocs.push_back(v);
+    if (!small) {
+      *p = reinterpret_cast<T*>(v);
+      return HS_OK;
+    }
+    ctx->block = (char*)v;
+    ctx->block_left = kBlock;
+  }
+  *p = reinterpret_cast<T*>(ctx->block);
+  ctx->block += bytes;
+  ctx->block_left -= bytes;
   return HS_OK;
 }
 
@@ -662,7 +683,28 @@ int setup_boundary(hs_ctx* ctx) {
     for (int q = 0; q < npanel && c < 5; ++q)
       if (segdist(p, q) <= h * (1 + 1e-9)) nearp[p * 5 + c++] = q;
   }
+  // Classes of pairs: the target panel's start, tangent and normal in the source
+  // panel's frame, and the sense of its tangent (all that the product-integration
+  // weights of S, D, K' and the tangential derivative depend on).
+  std::vector<int> cls(npanel * 5, 0), rep;
+  std::vector<std::array<long, 7>> keys;
+  for (int pair = 0; pair < npanel * 5; ++pair) {
+    const int p = pair / 5, q = nearp[pair];
+    if (q < 0) continue;
+    const double ax = (p0x[p] - p0x[q]) / h, ay = (p0y[p] - p0y[q]) / h;
+    const std::array<long, 7> key{std::lround(ax * tx[q] + ay * ty[q]),           std::lround(ax * pnx[q] + ay * pny[q]),
+                                  std::lround(tx[p] * tx[q] + ty[p] * ty[q]),     std::lround(tx[p] * pnx[q] + ty[p] * pny[q]),
+                                  std::lround(pnx[p] * tx[q] + pny[p] * ty[q]),   std::lround(pnx[p] * pnx[q] + pny[p] * pny[q]),
+                                  std::lround(pnx[p] * ty[p] - pny[p] * tx[p])};
+    const size_t c = std::find(keys.begin(), keys.end(), key) - keys.begin();
+    if (c == keys.size()) {
+      keys.push_back(key);
+      rep.push_back(pair);
+    }
+    cls[pair] = (int)c;
+  }
   Boundary& B = ctx->B;
+  B.ncls = (int)rep.size();
   B.nb = nb;
   B.npanel = npanel;
   B.h = h;
@@ -671,6 +713,9 @@ int setup_boundary(hs_ctx* ctx) {
   CKR(dalloc(ctx, &B.p0x, npanel)); CKR(dalloc(ctx, &B.p0y, npanel)); CKR(dalloc(ctx, &B.tx, npanel));
   CKR(dalloc(ctx, &B.ty, npanel)); CKR(dalloc(ctx, &B.pnx, npanel)); CKR(dalloc(ctx, &B.pny, npanel));
   CKR(dalloc(ctx, &B.near, npanel * 5));
+  CKR(dalloc(ctx, &B.cls, npanel * 5));
+  CKR(dalloc(ctx, &B.rep, B.ncls));
+  CKR(dalloc(ctx, &B.wts, (size_t)2 * B.ncls * 14 * 14));
   CK(cudaMemcpy(B.x, x.data(), sizeof(double) * nb, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(B.y, y.data(), sizeof(double) * nb, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(B.nx, nx.data(), sizeof(double) * nb, cudaMemcpyHostToDevice));
@@ -684,6 +729,8 @@ int setup_boundary(hs_ctx* ctx) {
   CK(cudaMemcpy(B.pnx, pnx.data(), sizeof(double) * npanel, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(B.pny, pny.data(), sizeof(double) * npanel, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(B.near, nearp.data(), sizeof(int) * npanel * 5, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(B.cls, cls.data(), sizeof(int) * npanel * 5, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(B.rep, rep.data(), sizeof(int) * B.ncls, cudaMemcpyHostToDevice));
   // quadrature constants
   std::vector<double> glx, glw;
   gauss_legendre(16, glx, glw);
@@ -1071,7 +1118,8 @@ size_t mixed_bytes(hs_ctx* ctx, int M, int P) {
   const size_t nb = ctx->B.nb, nl = ctx->nleaf;
   size_t b = 6 * Arena::bytes(nb * M, 16) + Arena::bytes(2 * nb * M, 16) + Arena::bytes((size_t)P * 2 * nb, 16) +
              Arena::bytes((size_t)M * P, 16) + Arena::bytes(2 * nb * M, 8) + Arena::bytes((size_t)P * 2 * nb, 8) +
-             Arena::bytes((size_t)M * P, 8) + Arena::bytes(8, 8) + Arena::bytes(nl * NL * M, 16);
+             Arena::bytes((size_t)M * P, 8) + Arena::bytes(8, 8) + Arena::bytes(nl * NL * M, 16) +
+             Arena::bytes(nl * NE * M, 16);
   b += Arena::bytes(nl * NL * M, 8) + 2 * Arena::bytes(field_buf_elems(ctx, M), 8) + Arena::bytes(nl * NE * M, 8) +
        Arena::bytes(nl * NI * M, 8) +
        Arena::bytes(s3_elems(ctx, M), 8) + 2 * Arena::bytes(nb * M, 8);
@@ -1113,6 +1161,7 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
   float2* duf = a.get<float2>((size_t)M * P);
   double* nrm = a.get<double>(8);
   double2* X = a.get<double2>(nX);
+  double2* DN = a.get<double2>((size_t)nl * NE * M);  // outward normal derivatives at the leaf edges
   float2* Up = a.get<float2>(nX);
   float2 *B0 = a.get<float2>(field_buf_elems(ctx, M)), *B1 = a.get<float2>(field_buf_elems(ctx, M));
   float2* tmp = a.get<float2>((size_t)nl * NE * M);
@@ -1152,7 +1201,7 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
     if (it > 0) {
       // FP64 residual of every row for the current iterate X; the exterior
       // rows: (D - I/2)(u_inc - u) - S (d_n u_inc - d_n u) = -[D - I/2, -S] [u_s; d_n u_s]
-      residual_pde(s, X, ctx->d_q, ctx->d_D1, nl, ctx->k, ctx->h, M, Up);
+      residual_pde(s, X, ctx->d_q, ctx->d_D1, nl, ctx->k, ctx->h, M, Up, DN);
       boundary_gather(s, X, ctx->d_D1, ctx->nL, ctx->h, M, ub, psib);
       scattered_data(s, ub, psib, ui, dni, (long long)nbM, PS);
       if (emu) {
@@ -1182,7 +1231,7 @@ int mixed_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const 
         leaf_particular(s, ctx->ws32, nl, ctx->d_k, M, Up, B0, tmp, wtmp);
         float2 *Hc = B0, *Hp = B1;
         for (int li = 0; li < nlev; ++li) {
-          residual_iface(s, ctx->levels[li], X, ctx->d_D1, ctx->nL, ctx->h, ctx->d_k, M, S3);
+          residual_iface(s, ctx->levels[li], X, DN, ctx->nL, ctx->d_k, M, S3);
           sweep_up_level<float2>(s, ctx->levels[li], ctx->ops32[li], Hc, S3, TT[li], Hp, M);
           std::swap(Hc, Hp);
         }

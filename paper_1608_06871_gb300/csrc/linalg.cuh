@@ -20,6 +20,24 @@ void gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const
           long long sA, const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC,
           int batch);
 
+// The FP32 kernels behind gemm() (gemm32.cu), for the four operand forms.
+template <typename TA, typename TB, typename TC>
+void gemm_fp32(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
+               const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch);
+
+template <>
+void gemm_fp32<float2, float2, float2>(cudaStream_t, int, int, int, int, int, float2, const float2*, int, long long, const float2*, int, long long, float2, float2*,
+                    int, long long, int);
+template <>
+void gemm_fp32<float, float2, float2>(cudaStream_t, int, int, int, int, int, float2, const float*, int, long long, const float2*, int, long long, float2, float2*,
+                    int, long long, int);
+template <>
+void gemm_fp32<float2, float, float2>(cudaStream_t, int, int, int, int, int, float2, const float2*, int, long long, const float*, int, long long, float2, float2*,
+                    int, long long, int);
+template <>
+void gemm_fp32<float, float, float>(cudaStream_t, int, int, int, int, int, float, const float*, int, long long, const float*, int, long long, float, float*,
+                    int, long long, int);
+
 // In-place LU with partial pivoting P A = L U of a batch of n x n matrices.
 // piv[j] (0-based) is the row swapped with row j at step j.  info[b] is set to
 // j+1 at the first exactly-zero pivot of matrix b (it must be zeroed first).

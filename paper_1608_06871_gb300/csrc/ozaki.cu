@@ -63,7 +63,6 @@ constexpr int OZ_B_SL = OZ_TN * 2 * OZ_KS;  // same for B (4 KB)
 constexpr int OZ_STAGE = OZ_S * (OZ_A_SL + OZ_B_SL);  // 96 KB
 constexpr int OZ_SMEM = 2 * OZ_STAGE + 1024;
 constexpr long long OZ_WAIT = 1LL << 26;
-constexpr int OZ_NAN = 1 << 20;  // exponent of a row with an infinity or a NaN: its outputs are NaN
 constexpr int OZ_SR = 16;        // rows per CTA of the slicing kernel
 // instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = n
 __host__ __device__ constexpr uint32_t oz_idesc(int n) {
@@ -118,25 +117,6 @@ __device__ __forceinline__ void oz_ld8(uint32_t ta, uint32_t (&v)[8]) {
                : "r"(ta));
 }
 
-// |x| as ordered 64-bit integers (the bit pattern of a non-negative double).
-__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL; }
-
-// round(x 2^(56 - e)) for |x| < 2^e, in integer arithmetic on the bit pattern
-// (mantissa shifted by the exponent difference, rounded to nearest); 0 for
-// zeros and subnormals, whose contribution is below the slices' resolution.
-__device__ __forceinline__ long long fixed56(double x, int e) {
-  const long long b = __double_as_longlong(x);
-  const int E = (int)((b >> 52) & 0x7FF);
-  if (E == 0) return 0;
-  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;  // 53-bit significand
-  const int sh = E - 1075 + 56 - e;                                     // x 2^(56-e) = m 2^sh, sh <= 3
-  long long v;
-  if (sh >= 0) v = m << sh;
-  else if (sh > -60) v = (m + (1LL << (-sh - 1))) >> (-sh);
-  else v = 0;
-  return b < 0 ? -v : v;
-}
-
 // The slices of two k-neighbours N0, N1 (56-bit fixed point, |N| < 2^56), one
 // 32-bit store per slice: the 8 balanced base-128 digits a_s of N,
 // sum_s a_s 2^(49 - 7 s) = N, |a_0| <= 128, the others in [-64, 63].  With
@@ -159,12 +139,6 @@ __device__ __forceinline__ void put2(long long N0, long long N1, uint32_t* o, in
     const uint32_t b1 = __float_as_uint(__uint_as_float(f1) - 8388672.0f);
     o[s * plane] = __byte_perm(b0, b1, 0x7632);
   }
-}
-
-// Exponent of a row from its largest |x| (bit pattern): max in [2^(ex-1), 2^ex).
-__device__ __forceinline__ int row_exp(long long mx) {
-  const int e = (int)(mx >> 52);
-  return mx == 0 ? 0 : e == 0x7FF ? OZ_NAN : e - 1022;
 }
 
 __device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long i, long long k) {

@@ -121,7 +121,10 @@ struct Boundary {
   double *x, *y, *nx, *ny, *w;  // node coordinates, outward normals, ds weights
   int *panel;                   // panel of each node
   double *p0x, *p0y, *tx, *ty, *pnx, *pny;  // panel start, tangent, normal
-  int *near;                    // [npanel][5] near panels (-1 padded)
+  int* near;                    // [npanel][5] near panels (-1 padded)
+  int ncls;                     // classes of (panel, near panel) pairs by relative position
+  int *cls, *rep;               // [npanel][5] class of a pair, [ncls] one pair (panel * 5 + slot) of each
+  double2* wts;                 // [2][ncls][14][14] product-integration weights of the classes
 };
 void upload_quad_constants(const double* gl_x, const double* gl_w, const double* tnodes, const double* lagden,
                            const double* dref, cudaStream_t s);
@@ -191,8 +194,9 @@ void convert_d2f(cudaStream_t s, const double2* a, float2* b, long long n);
 void convert_f2d_add(cudaStream_t s, const float2* a, double2* b, long long n);  // b += a
 // D1: device copy of the 16 x 16 Chebyshev-Lobatto differentiation matrix on [-1, 1].
 void residual_pde(cudaStream_t s, const double2* X, const double* q, const double* D1, int nleaf, double k, double h,
-                  int nrhs, float2* RP);
-void residual_iface(cudaStream_t s, const LevelMaps& L, const double2* X, const double* D1, int nL, double h,
+                  int nrhs, float2* RP, double2* DN);
+// DN: the outward normal derivatives [leaf][56][nrhs] that residual_pde wrote for the same X.
+void residual_iface(cudaStream_t s, const LevelMaps& L, const double2* X, const double2* DN, int nL,
                     const double* d_k, int nrhs, float2* S3);
 void boundary_gather(cudaStream_t s, const double2* X, const double* D1, int nL, double h, int nrhs, double2* ub,
                      double2* psib);

@@ -67,7 +67,8 @@ def test_emulated_product_keeps_non_finite_rows(hs, bad):
 
 
 @pytest.mark.parametrize("batch,m,n,k", [(1, 1, 1, 1), (3, 252, 5, 56), (2, 7, 200, 130), (1, 300, 8, 31),
-                                         (2, 65, 9, 17), (1, 64, 64, 16), (3, 67, 130, 48), (1, 448, 81, 897)])
+                                         (2, 65, 9, 17), (1, 64, 64, 16), (3, 67, 130, 48), (1, 448, 81, 897),
+                                         (40, 196, 140, 196), (300, 56, 48, 40), (300, 112, 96, 64)])
 @pytest.mark.parametrize("mode", [0, 1, 2])
 def test_gemm32_small(hs, batch, m, n, k, mode):
     g = torch.Generator().manual_seed(m + n * 7 + k)
