@@ -788,7 +788,7 @@ inline double im_of(double2 x) { return x.y; }
 // its estimated time is clearly below the FP64 pipe's: 36 bf16 products are
 // about a tenth of the pipe's time per multiply-add, but operands are sliced
 // first (two more launches, 16 bytes written and read per entry) and tiles are
-// 128 x 64, so small and thin products stay on the pipe (the two models' times
+// 128 x 32, so small and thin products stay on the pipe (the two models' times
 // are compared, with a fifth in favour of the pipe).  The products of the k = 40
 // FP64 batch: 160 ms on the pipe, 27 ms sliced and multiplied; the batch 227 ->
 // 98.5 ms, a k = 20 gradient 65.8 -> 44.3 ms.  Error against 64 bits of random
@@ -796,14 +796,19 @@ inline double im_of(double2 x) { return x.y; }
 // pipe 2.5e-16 .. 7e-16 (rows whose entries spread over 1e5: 4.5e-16 against
 // 3e-16 at k = 128, 4.8e-16 against 1.9e-15 at 1792); of far fields, fields,
 // Jacobians and steps at k = 5 .. 20: unchanged (5e-13 .. 5e-12).
-// Batches, then k, are cut to what the calling thread's scratch holds.
-// Complex factors other than real ones, and calls without scratch, are refused.
+// Batches, then columns, then k, are cut to what the calling thread's scratch holds.
+// Factors that are neither real nor (real x complex) imaginary, and calls without
+// scratch, are refused.
 template <typename TA, typename TB, typename TC>
 bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
                    const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC, int batch) {
   constexpr bool ca = is_cplx<TA>::v, cb = is_cplx<TB>::v;
   const OzScratch* sc = g_oz_scratch;
-  if (!g_oz_enabled || !sc || !sc->p || k <= 0 || im_of(alpha) != 0.0 || im_of(beta) != 0.0) return false;
+  if (!g_oz_enabled || !sc || !sc->p || k <= 0 || im_of(beta) != 0.0) return false;
+  // an imaginary factor of a real x complex product goes into the right operand
+  const bool turn = !ca && cb && re_of(alpha) == 0.0;
+  if (im_of(alpha) != 0.0 && !turn) return false;
+  const double factor = turn ? im_of(alpha) : re_of(alpha);
   if (std::min(m, n) <= 8) return false;
   const int mr = ca && !cb ? 2 * m : m, nr = cb ? 2 * n : n, kr = ca && cb ? 2 * k : k;
   const bool bsh = sB == 0 && batch > 1;
@@ -813,26 +818,30 @@ bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alp
   OzSrc a{reinterpret_cast<const double*>(A), ea * sA, ea * (opA == OP_N ? lda : 1), ea * (opA == OP_N ? 1 : lda),
           ca ? (cb ? OZ_CLEFT : OZ_PAIR) : OZ_REAL};
   OzSrc b{reinterpret_cast<const double*>(B), eb * sB, eb * (opB == OP_N ? 1 : ldb), eb * (opB == OP_N ? ldb : 1),
-          cb ? (ca ? OZ_CRIGHT : OZ_PAIR) : OZ_REAL};
+          cb ? (ca ? OZ_CRIGHT : turn ? OZ_PAIR_I : OZ_PAIR) : OZ_REAL};
   constexpr bool cc = ca || cb;
   OzView c{reinterpret_cast<double*>(C), (cc ? 2 : 1) * sC, (cc ? 2LL : 1LL) * ldc, 0, 1, 1};
   if (ca && !cb) c = OzView{reinterpret_cast<double*>(C), 2 * sC, 2LL * ldc, 1, 2, 2};
-  // the largest batch chunk, then the longest piece of k, that the scratch holds
-  int nb = batch, kc = kr;
-  while (nb > 1 && ozaki_scratch_bytes(mr, nr, kr, nb, bsh) > sc->bytes) nb = (nb + 1) / 2;
-  while (kc > 384 && ozaki_scratch_bytes(mr, nr, kc, nb, bsh) > sc->bytes) kc = ((kc + 1) / 2 + 383) / 384 * 384;
-  if (ozaki_scratch_bytes(mr, nr, kc, nb, bsh) > sc->bytes) return false;
+  // the largest batch chunk, then the most columns, then the longest piece of k
+  // that the scratch holds
+  int nb = batch, nn = nr, kc = kr;
+  auto fits = [&] { return ozaki_scratch_bytes(mr, nn, kc, nb, bsh) <= sc->bytes; };
+  while (nb > 1 && !fits()) nb = (nb + 1) / 2;
+  while (nn > 2048 && !fits()) nn = ((nn + 1) / 2 + 63) / 64 * 64;
+  while (kc > 384 && !fits()) kc = ((kc + 1) / 2 + 383) / 384 * 384;
+  if (!fits()) return false;
   for (int b0 = 0; b0 < batch; b0 += nb)
-    for (int k0 = 0; k0 < kr; k0 += kc) {
-      OzSrc ai = a, bi = b;
-      OzView ci = c;
-      const long long l0 = ca && cb ? k0 / 2 : k0;  // (kc is even)
-      ai.p += b0 * a.sb + l0 * a.sk;
-      bi.p += b0 * b.sb + l0 * b.sk;
-      ci.p += b0 * c.sb;
-      ozaki_gemm(s, mr, nr, std::min(kc, kr - k0), std::min(nb, batch - b0), re_of(alpha), ai, bi, bsh,
-                 k0 == 0 ? re_of(beta) : 1.0, ci, sc->p, sc->bytes);
-    }
+    for (int n0 = 0; n0 < nr; n0 += nn)
+      for (int k0 = 0; k0 < kr; k0 += kc) {
+        OzSrc ai = a, bi = b;
+        OzView ci = c;
+        const long long l0 = ca && cb ? k0 / 2 : k0, j0 = cb ? n0 / 2 : n0;  // (kc and nn are even)
+        ai.p += b0 * a.sb + l0 * a.sk;
+        bi.p += b0 * b.sb + l0 * b.sk + j0 * b.sr;
+        ci.p += b0 * c.sb + n0 * c.sk;
+        ozaki_gemm(s, mr, std::min(nn, nr - n0), std::min(kc, kr - k0), std::min(nb, batch - b0), factor, ai, bi, bsh,
+                   k0 == 0 ? re_of(beta) : 1.0, ci, sc->p, sc->bytes);
+      }
   return true;
 }
 

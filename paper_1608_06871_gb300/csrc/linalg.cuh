@@ -105,10 +105,11 @@ struct OzView {
 // Source of an operand's rows (A's rows, or B's columns): entry (b, i, k), strides in doubles.
 //   OZ_REAL    p[i sr + k sk]
 //   OZ_PAIR    rows 2 r + q are the parts q of complex rows r: p[r sr + k sk + q]
+//   OZ_PAIR_I  the same of i times those rows: (-im, re)
 //   OZ_CLEFT   k = 2 l + q runs over the parts of a complex row: p[i sr + l sk + q]
 //   OZ_CRIGHT  the right operand to OZ_CLEFT: rows 2 j, 2 j + 1 are (re, -im), (im, re)
 //              of complex column j along k = 2 l + q, p[j sr + l sk + ...]
-enum { OZ_REAL = 0, OZ_PAIR = 1, OZ_CLEFT = 2, OZ_CRIGHT = 3 };
+enum { OZ_REAL = 0, OZ_PAIR = 1, OZ_CLEFT = 2, OZ_CRIGHT = 3, OZ_PAIR_I = 4 };
 struct OzSrc {
   const double* p;
   long long sb, sr, sk;
@@ -118,7 +119,7 @@ extern bool g_oz_enabled;
 // Scratch bytes of ozaki_gemm for these sizes.
 size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared);
 // C[b] = alpha A[b] B[b] + beta C[b] (m x n, k inner; beta = 0 never reads C), sizes of the
-// real product; b_shared: one B for every batch; sym: only the 128 x 64 tiles that meet the
+// real product; b_shared: one B for every batch; sym: only the 128 x 32 tiles that meet the
 // lower triangle are computed.  Returns cudaErrorInvalidValue on bad sizes.
 cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
                        double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym = false);

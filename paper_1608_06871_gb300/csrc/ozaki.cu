@@ -23,12 +23,12 @@
 // A complex product is one real product: rows of A as (re, im) pairs along k,
 // columns of B as the pairs (re, -im) and (im, re).
 //
-// Kernel: one persistent CTA per SM, 128 x 64 output tiles; warp 0 copies the
+// Kernel: one persistent CTA per SM, 128 x 32 output tiles; warp 0 copies the
 // 32-wide k-steps of the tile's slices (stored by the slicing kernels in the
-// MMA operand layout, 64 + 32 KB in one piece each) into a two-stage ring with
-// cp.async.bulk, warp 1 issues the tcgen05 BF16 MMAs (M = 128, N = 64 to 256,
-// K = 16; 28 per stage of 32 k) into the eight diagonal accumulators (all
-// 512 TMEM columns), sixteen warps read them back.  Every mbarrier wait is
+// MMA operand layout, 64 + 16 KB in one piece each) into a two-stage ring with
+// cp.async.bulk, warp 1 issues the tcgen05 BF16 MMAs (M = 128, N = 32 to 256,
+// K = 16; 16 per stage of 32 k) into the eight diagonal accumulators (two sets of
+// 256 TMEM columns), sixteen warps read them back.  Every mbarrier wait is
 // bounded; a timeout sets the library's tensor-core timeout flag.
 #include <cuda_runtime.h>
 
@@ -53,14 +53,15 @@ namespace {
 constexpr int OZ_S = 8;          // slices per operand
 constexpr int OZ_ND = 8;         // anti-diagonals kept (s + t <= 7)
 constexpr int OZ_TM = 128;       // rows per tile
-constexpr int OZ_TN = 64;        // columns per tile
+constexpr int OZ_TN = 32;        // columns per tile
+constexpr int OZ_ACC = OZ_ND * OZ_TN;  // TMEM columns of one set of diagonal accumulators (two sets)
 constexpr int OZ_KS = 32;        // k per stage
 constexpr int OZ_KMAX = 384;     // k per piece keeping every diagonal sum below 2^24 (a multiple of 32)
 constexpr int OZ_EPI = 16;       // epilogue warps
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI;  // warp 0 TMA, warp 1 MMA, the others epilogue
 constexpr int OZ_A_SL = OZ_TM * 2 * OZ_KS;  // one slice of the A tile: 128 rows x 64 bytes (8 KB)
-constexpr int OZ_B_SL = OZ_TN * 2 * OZ_KS;  // same for B (4 KB)
-constexpr int OZ_STAGE = OZ_S * (OZ_A_SL + OZ_B_SL);  // 96 KB
+constexpr int OZ_B_SL = OZ_TN * 2 * OZ_KS;  // same for B (2 KB)
+constexpr int OZ_STAGE = OZ_S * (OZ_A_SL + OZ_B_SL);  // 80 KB
 constexpr int OZ_SMEM = 2 * OZ_STAGE + 1024;
 constexpr long long OZ_WAIT = 1LL << 26;
 constexpr int OZ_SR = 16;        // rows per CTA of the slicing kernel
@@ -146,6 +147,10 @@ __device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long 
   switch (v.kind) {
     case OZ_REAL: return p[i * v.sr + k * v.sk];
     case OZ_PAIR: return p[(i >> 1) * v.sr + k * v.sk + (i & 1)];
+    case OZ_PAIR_I: {  // i times the column: (-im, re)
+      const double x = p[(i >> 1) * v.sr + k * v.sk + ((i & 1) ^ 1)];
+      return i & 1 ? x : -x;
+    }
     case OZ_CLEFT: return p[i * v.sr + (k >> 1) * v.sk + (k & 1)];
     default: {  // OZ_CRIGHT: [re, -im; im, re]
       const double x = p[(i >> 1) * v.sr + (k >> 1) * v.sk + ((i ^ k) & 1)];
@@ -335,26 +340,26 @@ __device__ __forceinline__ bool oz_item(const OzParams& P, long long it, OzItem&
   return !(P.sym && o.tn * OZ_TN >= (o.tm + 1) * OZ_TM);
 }
 
-// Persistent: each CTA takes every gridDim.x-th 128 x 64 tile (or piece group
-// of one) and runs all its pieces of k, summing them in registers.  What bounds
-// it: 36 slice products, 2304 tensor cycles per 32-k stage at the bf16 rate, and
-// the epilogue of each piece, which cannot overlap the next piece's products
-// (the eight diagonals fill TMEM).  So the epilogue is integer arithmetic on
-// sixteen warps (one conversion per diagonal, two diagonals per 32-bit
-// multiply-add, the double assembled from its bits), and the ring already
-// loads the next piece behind it.  Before, one launch per piece with an FP64
-// epilogue on four warps and C read back per piece kept the tensor pipe at 17%:
-// the products of a k = 40 Gauss-Newton step (Jacobian projections and normal
-// matrix, 3.2e12 flops) took 278 ms, now 102 ms (the normal matrix by its
-// lower tiles only).  Measured per tile: 4250 clocks (at 1.92 GHz) a stage and
-// 11,000 a piece; 30 TFLOP/s of FP64-equivalent work for long k, 1080 of the 1948
-// TFLOP/s bf16 peak issued (shared memory: 256 KB read and 96 KB written a stage).
+// Persistent: each CTA takes every gridDim.x-th 128 x 32 tile (or piece group
+// of one) and runs all its pieces of k, summing them in registers; the eight
+// diagonals take half of TMEM, so one piece's epilogue runs behind the next one's
+// products.  What bounds it: per 32-k stage the 36 slice products (1152 tensor
+// clocks) read 136 KB of shared memory while 80 KB are written (1690 clocks);
+// 2000 to 2200 clocks at 1.92 GHz measured.  The epilogue (9400 clocks a piece: the
+// conversions of eight diagonals, the doubles assembled from their bits in
+// integer arithmetic) bounds pieces below 160 k.
+// Before, one launch per piece with an FP64 epilogue on four warps and C read
+// back per piece kept the tensor pipe at 17%: the products of a k = 40
+// Gauss-Newton step (Jacobian projections and normal matrix, 3.2e12 flops) took
+// 278 ms; 102 ms with 128 x 64 tiles that fill TMEM, epilogue and products in
+// turn; 83 ms now.  4864 x 4096 x k: 29 TFLOP/s of FP64-equivalent work at k = 256,
+// 34 at 1536 (1217 of the 1948 TFLOP/s bf16 peak issued).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_mma(const __grid_constant__ OzParams P) {
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   __shared__ uint32_t tslot;
-  __shared__ __align__(8) uint64_t full[2], empty[2], accf, acce, done;
+  __shared__ __align__(8) uint64_t full[2], empty[2], accf[2], acce[2], done;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (warp == 1) {
@@ -365,9 +370,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     for (int i = 0; i < 2; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&full[i])), "r"(1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&empty[i])), "r"(1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&accf[i])), "r"(1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce[i])), "r"(OZ_EPI));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&accf)), "r"(1));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce)), "r"(OZ_EPI));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&done)), "r"(1));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -411,7 +416,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         OzItem o;
         if (!oz_item(P, it, o)) continue;
         for (int p = o.z * P.ppz; p < min(P.npc, (o.z + 1) * P.ppz) && ok; ++p, ++pc) {
-          if (pc > 0) ok = oz_wait(su32(&acce), (pc - 1) & 1);  // the epilogue has read the accumulators
+          const int buf = pc & 1;
+          const uint32_t acc0 = tmem + (uint32_t)(buf * OZ_ACC);
+          if (pc > 1) ok = oz_wait(su32(&acce[buf]), ((pc >> 1) - 1) & 1);  // the epilogue has read this set
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
           const int nst = stages(p);
@@ -421,31 +428,20 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t aB = su32(sm + st * OZ_STAGE), bB = aB + OZ_S * OZ_A_SL;
-            // The B slices of a k block lie back to back (slice t at rows 64 t .. 64 t + 63)
+            // The B slices of a k block lie back to back (slice t at rows 32 t .. 32 t + 31)
             // and the diagonal accumulators are adjacent in TMEM (diagonal d at columns
-            // 64 d ..), so one MMA with N = 64 w multiplies A_s by B_t .. B_(t+w-1) into
-            // diagonals s + t .. s + t + w - 1: per slice s the 8 - s pairs take
-            // MMAs of N = 256, 128 and 64 (14 per 16 k instead of 36).
+            // 32 d ..), so one MMA with N = 32 (8 - s) multiplies A_s by B_0 .. B_(7-s)
+            // into diagonals s .. 7: 8 MMAs per 16 k instead of 36.
 #pragma unroll 1
             for (int kh = 0; kh < OZ_KS / 16; ++kh) {
 #pragma unroll 1
               for (int s = 0; s < OZ_S; ++s) {
-                const uint64_t da = oz_desc(aB + s * OZ_A_SL + kh * 32);
-                const uint32_t acc = (i > 0 || kh > 0 || s > 0) ? 1u : 0u;
-                int t = 0;
-#pragma unroll 1
-                while (t + s < OZ_ND) {
-                  const int left = OZ_ND - s - t;
-                  const int w = left >= 4 ? 4 : left >= 2 ? 2 : 1;
-                  const uint64_t db = oz_desc(bB + t * OZ_B_SL + kh * 32);
-                  const uint32_t idesc = oz_idesc(w * OZ_TN);
-                  asm volatile(
-                      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
-                          tmem + (uint32_t)((s + t) * OZ_TN)),
-                      "l"(da), "l"(db), "r"(idesc), "r"(acc));
-                  t += w;
-                }
+                const uint64_t da = oz_desc(aB + s * OZ_A_SL + kh * 32), db = oz_desc(bB + kh * 32);
+                const uint32_t acc = (i > 0 || kh > 0 || s > 0) ? 1u : 0u, idesc = oz_idesc((OZ_ND - s) * OZ_TN);
+                asm volatile(
+                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(acc0 + (uint32_t)(s * OZ_TN)),
+                    "l"(da), "l"(db), "r"(idesc), "r"(acc));
               }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -453,30 +449,33 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           }
           if (ok)
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                su32(&accf)));
+                su32(&accf[buf])));
         }
       }
       // one more commit tracks every MMA issued above
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done)));
     }
   } else {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows (lane = row), 16 of the 64 columns
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows (lane = row), 8 of the 32 columns
     const int quarter = warp & 3, part = (warp - 2) >> 2;
-    const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(part * 16);
     int pc = 0;
     for (long long it = blockIdx.x; it < P.items && ok; it += gridDim.x) {
       OzItem o;
       if (!oz_item(P, it, o)) continue;
-      const int r = o.tm * OZ_TM + quarter * 32 + lane, cb = o.tn * OZ_TN + part * 16;
+      const int r = o.tm * OZ_TM + quarter * 32 + lane, cb = o.tn * OZ_TN + part * 8;
       const int p0 = o.z * P.ppz, p1 = min(P.npc, p0 + P.ppz);
-      double acc[16];
+      double acc[8];
+      // (a product with +-1 would cost the FP64 pipe as much as the tile's conversions)
+      auto times = [&](double x) { return P.alpha == 1.0 ? x : P.alpha == -1.0 ? -x : P.alpha * x; };
       for (int p = p0; p < p1; ++p, ++pc) {
+        const int buf = pc & 1;
+        const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(buf * OZ_ACC + part * 8);
         // (rows and columns of the padding have exponents too)
         const int ea = P.ea[p * P.ea_piece + (long long)o.b * P.mpad + r];
-        const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + (lane & 15)];
+        const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + (lane & 7)];
         // |sum of the piece| <= 1.02 kc: V = sum 2^(63 - rs) stays below 2^62
         const int rs = 33 - __clz(min(P.pl, P.k - p * P.pl));
-        ok = oz_wait(su32(&accf), pc & 1);
+        ok = oz_wait(su32(&accf[buf]), (pc >> 1) & 1);
         if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
           break;
@@ -484,46 +483,41 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         asm volatile("tcgen05.fence::after_thread_sync;");
         // pairs of diagonals in 32 bits: |C_d| <= 384 4096 (d + 3) (6.3e6 for d = 0),
         // 128 C_d + C_(d+1) <= 1.83e9 < 2^31
+        int q[4][8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // eight columns at a time (registers)
-          long long V[8];
-          int q0[8];
+        for (int g = 0; g < 2; ++g) {
+          uint32_t v[4][8];
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            uint32_t v[2][8];
-            oz_ld8(ta + (uint32_t)(2 * g * OZ_TN + 8 * h), v[0]);
-            oz_ld8(ta + (uint32_t)((2 * g + 1) * OZ_TN + 8 * h), v[1]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (h == 1 && g == 3) {  // last read of this piece: the accumulators are free
-              asm volatile("tcgen05.fence::before_thread_sync;");
-              __syncwarp();
-              if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acce)) : "memory");
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int q = 128 * __float2int_rn(__uint_as_float(v[0][j])) + __float2int_rn(__uint_as_float(v[1][j]));
-              // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63, hi and lo = q 2^14 + the next q
-              if (g == 0 || g == 2) q0[j] = q;
-              else if (g == 1) V[j] = (((long long)q0[j] << 14) + q) << (28 - rs);
-              else V[j] += (((long long)q0[j] << 14) + q + (1LL << (rs - 1))) >> rs;
-            }
+          for (int d = 0; d < 4; ++d) oz_ld8(ta + (uint32_t)((4 * g + d) * OZ_TN), v[d]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;");
+          if (g == 1) {  // last read of this piece: this set of accumulators is free
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&acce[buf])) : "memory");
           }
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int eb = __shfl_sync(0xffffffffu, ebl, 8 * h + j);
-            const double x = scaled(V[j], ea + eb + rs - 63);
-            acc[8 * h + j] = p == p0 ? x : acc[8 * h + j] + x;
+            q[2 * g][j] = 128 * __float2int_rn(__uint_as_float(v[0][j])) + __float2int_rn(__uint_as_float(v[1][j]));
+            q[2 * g + 1][j] = 128 * __float2int_rn(__uint_as_float(v[2][j])) + __float2int_rn(__uint_as_float(v[3][j]));
           }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63, hi and lo = q 2^14 + the next q
+          const long long V = ((((long long)q[0][j] << 14) + q[1][j]) << (28 - rs)) +
+                              ((((long long)q[2][j] << 14) + q[3][j] + (1LL << (rs - 1))) >> rs);
+          const double x = scaled(V, ea + __shfl_sync(0xffffffffu, ebl, j) + rs - 63);
+          acc[j] = p == p0 ? x : acc[j] + x;
         }
       }
       if (!ok) break;
       if (r < P.m) {
         double* pr = P.C.p + o.z * P.zplane + o.b * P.C.sb + (r / P.C.ig) * P.C.si + (r % P.C.ig) * P.C.sg;
-        if (P.C.sk == 1 && (reinterpret_cast<uintptr_t>(pr + cb) & 15) == 0 && cb + 16 <= P.n) {
+        if (P.C.sk == 1 && (reinterpret_cast<uintptr_t>(pr + cb) & 15) == 0 && cb + 8 <= P.n) {
           double2* p2 = reinterpret_cast<double2*>(pr + cb);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            double2 x = make_double2(P.alpha * acc[2 * j], P.alpha * acc[2 * j + 1]);
+          for (int j = 0; j < 4; ++j) {
+            double2 x = make_double2(times(acc[2 * j]), times(acc[2 * j + 1]));
             if (P.beta != 0.0) {
               const double2 y = p2[j];
               x = make_double2(fma(P.beta, y.x, x.x), fma(P.beta, y.y, x.y));
@@ -532,11 +526,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
+          for (int j = 0; j < 8; ++j)
             if (cb + j < P.n) {
-              double* q = pr + (cb + j) * P.C.sk;
-              const double x = P.alpha * acc[j];
-              *q = P.beta == 0.0 ? x : fma(P.beta, *q, x);
+              double* w = pr + (cb + j) * P.C.sk;
+              const double x = times(acc[j]);
+              *w = P.beta == 0.0 ? x : fma(P.beta, *w, x);
             }
         }
       }
@@ -723,15 +717,15 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
 
 thread_local const OzScratch* g_oz_scratch = nullptr;
 
-// Per piece 2304 clocks a stage of products and about 9000 of epilogue on one
-// SM; slices written and read at about 2600 bytes a clock; launches.
+// Per tile 2100 clocks a stage, or 9400 a piece where that is more; slices
+// written and read at about 2600 bytes a clock; launches.
 double oz_cycles(int m, int n, int k, int batch, bool b_shared) {
   const double mp = (double)padded(m, true), np = (double)padded(n, false);
   const int npc = npieces(k), zs = z_groups(m, n, k, batch);
   const double tiles = mp / OZ_TM * (np / OZ_TN) * batch * zs, kt = (double)npc * piece_len(k);
-  const double tile = kt / OZ_KS * 2304.0 / zs + std::ceil((double)npc / zs) * 9000.0 + 1500.0;
+  const double tile = std::max(kt / OZ_KS * 2100.0 / zs, std::ceil((double)npc / zs) * 9400.0);
   const double slices = (batch * mp + (b_shared ? 1 : batch) * np) * kt * 40.0 / 2600.0;
-  return std::ceil(tiles / 152.0) * tile + slices + (zs > 1 ? 20000.0 : 14000.0);
+  return std::ceil(tiles / 152.0) * tile + slices + (zs > 1 ? 24000.0 : 18000.0);
 }
 
 size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared) {
