@@ -173,6 +173,7 @@ struct hs_ctx {
   double2 *d_S = nullptr, *d_Dm = nullptr, *d_B1 = nullptr, *d_B2 = nullptr, *d_C = nullptr;
   double2 *d_Kp = nullptr, *d_Ht = nullptr;  // combined-field scratch (cfg.bm_eta > 0)
   int* d_Cpiv = nullptr;
+  LuInv<double2> Cinv;  // inverses of the diagonal blocks of C's factors
   const double2* Rroot = nullptr;
   double* d_D1 = nullptr;  // Chebyshev-Lobatto differentiation matrix (device copy)
   // mixed precision: FP32 factors (kept leaf scratch: LU(Aii), X, Ni, Kinv), FP64 refinement
@@ -338,6 +339,15 @@ template <typename T> int dalloc(hs_ctx* ctx, T** p, size_t n) {
   ctx->block += bytes;
   ctx->block_left -= bytes;
   return HS_OK;
+}
+
+// Room for the diagonal blocks' inverses of a batch of n x n LUs and for a copy of
+// up to `cols` right-hand sides at a time.
+int alloc_inv(hs_ctx* ctx, LuInv<double2>* inv, int n, int cols, int batch) {
+  inv->sd = (long long)lu_inv_elems(n);
+  inv->cols = cols;
+  CKR(dalloc(ctx, &inv->d, (size_t)inv->sd * batch));
+  return dalloc(ctx, &inv->tmp, (size_t)n * cols * batch);
 }
 
 int ensure_ws(hs_ctx* ctx, size_t bytes, Arena& a) {
@@ -526,6 +536,7 @@ int setup_tree(hs_ctx* ctx) {
       CKR(dalloc(ctx, &L.M, nb * L.ni * L.ni));
       CKR(dalloc(ctx, &L.Mpiv, nb * L.ni));
       CKR(dalloc(ctx, &L.R, nb * (size_t)L.np * L.np));
+      if (L.ni > 128 && nb <= 4) CKR(alloc_inv(ctx, &L.inv, L.ni, L.np, (int)nb));
     } else {
       LevelOps<float2> O{};
       CKR(dalloc(ctx, &O.XZ, nb * 2 * L.ni * L.np));
@@ -758,6 +769,7 @@ int setup_boundary(hs_ctx* ctx) {
   if (ctx->cfg.precision == HS_FP64) {
     CKR(dalloc(ctx, &ctx->d_C, nn));
     CKR(dalloc(ctx, &ctx->d_Cpiv, nb));
+    CKR(alloc_inv(ctx, &ctx->Cinv, nb, 512, 1));
     CKR(dalloc(ctx, &ctx->d_Rb, nn));
   } else {
     CKR(dalloc(ctx, &ctx->d_Rb32, nn));
@@ -981,7 +993,7 @@ int factor(hs_ctx* ctx, double k) {
   CK(cudaMemcpyAsync(ctx->d_C, ctx->d_B1, sizeof(double2) * nb * nb, cudaMemcpyDeviceToDevice, s));
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, nb, nb, make_double2(-1, 0), ctx->d_B2, nb, 0, ctx->Rroot, nb, 0,
                                   make_double2(1, 0), ctx->d_C, nb, 0, 1);
-  lu_factor<double2>(s, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, ctx->d_info, 1);
+  lu_factor<double2>(s, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, ctx->d_info, 1, ctx->Cinv);
   CK(cudaEventRecord(ctx->ph_ev[2], s));
   CK(cudaGetLastError());
   CKR(check_info(ctx));
@@ -1000,7 +1012,7 @@ int root_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, double2
   // rhs = (D - I/2) u_inc - S d_n u_inc
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, one, ctx->d_Dm, nb, 0, ui, M, 0, zero, f, M, 0, 1);
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, mone, ctx->d_S, nb, 0, dni, M, 0, one, f, M, 0, 1);
-  lu_solve<double2>(s, OP_N, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, f, M, 0, M, 1);
+  lu_solve<double2>(s, OP_N, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, f, M, 0, M, 1, ctx->Cinv);
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, one, ctx->Rroot, nb, 0, f, M, 0, zero, g, M, 0, 1);
   return HS_OK;
 }
@@ -1032,7 +1044,7 @@ int sweep_adjoint(hs_ctx* ctx, cudaStream_t s, const double2* A2, int P, double2
   Phase ph("hs_adjoint_sweep");
   adjoint_root_init(s, nb, P, ctx->k, A2, E, CP);
   gemm<double2, double2, double2>(s, OP_T, OP_N, nb, P, nb, one, ctx->Rroot, nb, 0, E, P, 0, one, CP, P, 0, 1);
-  lu_solve<double2>(s, OP_T, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, CP, P, 0, P, 1);
+  lu_solve<double2>(s, OP_T, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, CP, P, 0, P, 1, ctx->Cinv);
   gemm<double2, double2, double2>(s, OP_T, OP_N, nb, P, nb, one, ctx->d_B2, nb, 0, CP, P, 0, one, E, P, 0, 1);
   permute_rows<double2>(s, E, ctx->d_bie_of_root, nb, P, bufB);  // root box order
   const double2* Lp = bufB;

@@ -973,9 +973,36 @@ void gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const
   gemm_simt<TA, TB, TC>(s, opA, opB, m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch);
 }
 
+namespace {
+template <typename E> __global__ void k_identity(E* A, int n, int lda, long long sA) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (long long)n * n) return;
+  const int r = (int)(e / n), c = (int)(e % n);
+  A[blockIdx.y * sA + (long long)r * lda + c] = r == c ? el<E>::one() : el<E>::zero();
+}
+
+// D[b] (NBB wide, holding the identity) <- the inverse of the n x n triangle at A.
 template <typename E>
-void lu_factor(cudaStream_t s, E* A, int lda, long long sA, int n, int* piv, long long sP, int* info, int batch) {
+void tri_inverse(cudaStream_t s, const E* A, int lda, long long sA, int n, int mode, E* D, long long sD, int batch) {
+  switch (trsm_cw(n, batch)) {
+    case 8: launch_trsm_blk<E, 8>(s, A, lda, sA, 0, n, mode, D, NBB, sD, n, batch); return;
+    case 4: launch_trsm_blk<E, 4>(s, A, lda, sA, 0, n, mode, D, NBB, sD, n, batch); return;
+    case 2: launch_trsm_blk<E, 2>(s, A, lda, sA, 0, n, mode, D, NBB, sD, n, batch); return;
+    default: launch_trsm_blk<E, 1>(s, A, lda, sA, 0, n, mode, D, NBB, sD, n, batch); return;
+  }
+}
+}  // namespace
+
+template <typename E>
+void lu_factor(cudaStream_t s, E* A, int lda, long long sA, int n, int* piv, long long sP, int* info, int batch,
+               const LuInv<E>& inv) {
   const E m1 = -el<E>::one(), one = el<E>::one();
+  if (inv.d)
+    for (int b = 0; b < batch; ++b) {
+      const int blocks = 2 * ((n + NBB - 1) / NBB);
+      k_identity<E><<<dim3(NBB * NBB / 256, blocks), 256, 0, s>>>(inv.d + b * inv.sd, NBB, NBB, (long long)NBB * NBB);
+      HS_COUNT_LAUNCH();
+    }
   // Two-level right-looking blocking: super-panels of NBB columns, each
   // factored as NB-wide pivoted panels whose updates stay inside the
   // super-panel; then U12 = L11^-1 A12 for the super-panel's rows and one
@@ -994,22 +1021,34 @@ void lu_factor(cudaStream_t s, E* A, int lda, long long sA, int n, int* piv, lon
       }
     }
     const int rest = n - J1;
+    E* Li = inv.d ? inv.d + (long long)(J0 / NBB) * 2 * NBB * NBB : nullptr;
+    if (inv.d) tri_inverse<E>(s, A + (long long)J0 * (lda + 1), lda, sA, nbs, 0, Li, inv.sd, batch);
     if (rest > 0) {
-      trsm_blk<E>(s, A, lda, sA, J0, nbs, 0, A + J1, lda, sA, rest, batch);  // U12 = L11^-1 A12
+      // U12 = L11^-1 A12: on the tensor cores with the inverse (its operand is sliced
+      // before the result is written, so in place), or by substitution
+      bool done = false;
+      if constexpr (is_fp64<E>::v)
+        done = Li && gemm_emulated<E, E, E>(s, OP_N, OP_N, nbs, rest, nbs, one, Li, NBB, inv.sd,
+                                            A + (long long)J0 * lda + J1, lda, sA, el<E>::zero(),
+                                            A + (long long)J0 * lda + J1, lda, sA, batch);
+      if (!done) trsm_blk<E>(s, A, lda, sA, J0, nbs, 0, A + J1, lda, sA, rest, batch);
       gemm<E, E, E>(s, OP_N, OP_N, rest, rest, nbs, m1, A + (long long)J1 * lda + J0, lda, sA,
                     A + (long long)J0 * lda + J1, lda, sA, one, A + (long long)J1 * lda + J1, lda, sA, batch);
     }
   }
+  if (inv.d) {  // the inverses of the upper triangles: one launch for all whole blocks
+    const int full = n / NBB, tail = n - full * NBB;
+    E* Ui = inv.d + NBB * NBB;
+    if (batch == 1 && full > 0)
+      tri_inverse<E>(s, A, lda, (long long)NBB * (lda + 1), NBB, 1, Ui, 2LL * NBB * NBB, full);
+    else
+      for (int q = 0; q < full; ++q)
+        tri_inverse<E>(s, A + (long long)q * NBB * (lda + 1), lda, sA, NBB, 1, Ui + q * 2LL * NBB * NBB, inv.sd, batch);
+    if (tail > 0)
+      tri_inverse<E>(s, A + (long long)full * NBB * (lda + 1), lda, sA, tail, 1, Ui + full * 2LL * NBB * NBB, inv.sd,
+                     batch);
+  }
 }
-
-namespace {
-template <typename E> __global__ void k_identity(E* A, int n, int lda, long long sA) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)n * n) return;
-  const int r = (int)(e / n), c = (int)(e % n);
-  A[blockIdx.y * sA + (long long)r * lda + c] = r == c ? el<E>::one() : el<E>::zero();
-}
-}  // namespace
 
 template <typename E>
 void lu_inverse(cudaStream_t s, const E* A, int lda, long long sA, int n, const int* piv, long long sP, E* Inv,
@@ -1022,9 +1061,49 @@ void lu_inverse(cudaStream_t s, const E* A, int lda, long long sA, int n, const 
 
 template <typename E>
 void lu_solve(cudaStream_t s, int trans, const E* A, int lda, long long sA, int n, const int* piv, long long sP, E* B,
-              int ldb, long long sB, int nrhs, int batch) {
+              int ldb, long long sB, int nrhs, int batch, const LuInv<E>& inv) {
   dim3 gs((nrhs + 127) / 128, batch);
   const E m1 = -el<E>::one(), one = el<E>::one();
+  if (inv.d && inv.tmp) {
+    // With the diagonal blocks' inverses every step is a product: the first sweep
+    // leaves its solution in tmp, the second one in B.  (One FP64 complex column:
+    // 7 us a product, 53 us a block's substitution.)
+    if (trans == OP_N) {
+      k_swaps<E><<<gs, 128, 0, s>>>(piv, sP, n, 0, B, ldb, sB, nrhs);
+      HS_COUNT_LAUNCH();
+    }
+    const int opd = trans, first = trans == OP_N ? 0 : 1;  // L then U, or U^T then L^T
+    for (int c0 = 0; c0 < nrhs; c0 += inv.cols) {
+      const int nc = std::min(inv.cols, nrhs - c0), ldt = inv.cols;
+      const long long sT = (long long)n * ldt;
+      E* b = B + c0;
+      auto block = [&](int I0, int tri) { return inv.d + ((long long)(I0 / NBB) * 2 + tri) * NBB * NBB; };
+      for (int I0 = 0; I0 < n; I0 += NBB) {
+        const int I1 = std::min(n, I0 + NBB);
+        E* y = inv.tmp + (long long)I0 * ldt;
+        gemm<E, E, E>(s, opd, OP_N, I1 - I0, nc, I1 - I0, one, block(I0, first), NBB, inv.sd, b + (long long)I0 * ldb,
+                      ldb, sB, el<E>::zero(), y, ldt, sT, batch);
+        if (n - I1 > 0)
+          gemm<E, E, E>(s, opd, OP_N, n - I1, nc, I1 - I0, m1,
+                        trans == OP_N ? A + (long long)I1 * lda + I0 : A + (long long)I0 * lda + I1, lda, sA, y, ldt,
+                        sT, one, b + (long long)I1 * ldb, ldb, sB, batch);
+      }
+      for (int I0 = (n - 1) / NBB * NBB; I0 >= 0; I0 -= NBB) {
+        const int I1 = std::min(n, I0 + NBB);
+        E* x = b + (long long)I0 * ldb;
+        gemm<E, E, E>(s, opd, OP_N, I1 - I0, nc, I1 - I0, one, block(I0, 1 - first), NBB, inv.sd,
+                      inv.tmp + (long long)I0 * ldt, ldt, sT, el<E>::zero(), x, ldb, sB, batch);
+        if (I0 > 0)
+          gemm<E, E, E>(s, opd, OP_N, I0, nc, I1 - I0, m1, trans == OP_N ? A + I0 : A + (long long)I0 * lda, lda, sA, x,
+                        ldb, sB, one, inv.tmp, ldt, sT, batch);
+      }
+    }
+    if (trans != OP_N) {
+      k_swaps<E><<<gs, 128, 0, s>>>(piv, sP, n, 1, B, ldb, sB, nrhs);
+      HS_COUNT_LAUNCH();
+    }
+    return;
+  }
   if (trans == OP_N) {
     k_swaps<E><<<gs, 128, 0, s>>>(piv, sP, n, 0, B, ldb, sB, nrhs);
     HS_COUNT_LAUNCH();
@@ -1079,12 +1158,16 @@ template void gemm<double, double2, double2>(cudaStream_t, int, int, int, int, i
 template void gemm<double2, double, double2>(cudaStream_t, int, int, int, int, int, double2, const double2*, int,
                                              long long, const double*, int, long long, double2, double2*, int,
                                              long long, int);
-template void lu_factor<double>(cudaStream_t, double*, int, long long, int, int*, long long, int*, int);
-template void lu_factor<double2>(cudaStream_t, double2*, int, long long, int, int*, long long, int*, int);
+template void lu_factor<double>(cudaStream_t, double*, int, long long, int, int*, long long, int*, int,
+                             const LuInv<double>&);
+template void lu_factor<double2>(cudaStream_t, double2*, int, long long, int, int*, long long, int*, int,
+                             const LuInv<double2>&);
 template void lu_solve<double>(cudaStream_t, int, const double*, int, long long, int, const int*, long long, double*,
-                               int, long long, int, int);
+                               int, long long, int, int,
+                               const LuInv<double>&);
 template void lu_solve<double2>(cudaStream_t, int, const double2*, int, long long, int, const int*, long long,
-                                double2*, int, long long, int, int);
+                                double2*, int, long long, int, int,
+                               const LuInv<double2>&);
 
 template void gemm<float, float, float>(cudaStream_t, int, int, int, int, int, float, const float*, int, long long,
                                         const float*, int, long long, float, float*, int, long long, int);
@@ -1096,8 +1179,10 @@ template void gemm<float, float2, float2>(cudaStream_t, int, int, int, int, int,
 template void gemm<float2, float, float2>(cudaStream_t, int, int, int, int, int, float2, const float2*, int,
                                           long long, const float*, int, long long, float2, float2*, int, long long,
                                           int);
-template void lu_factor<float>(cudaStream_t, float*, int, long long, int, int*, long long, int*, int);
-template void lu_factor<float2>(cudaStream_t, float2*, int, long long, int, int*, long long, int*, int);
+template void lu_factor<float>(cudaStream_t, float*, int, long long, int, int*, long long, int*, int,
+                             const LuInv<float>&);
+template void lu_factor<float2>(cudaStream_t, float2*, int, long long, int, int*, long long, int*, int,
+                             const LuInv<float2>&);
 template void lu_inverse<double>(cudaStream_t, const double*, int, long long, int, const int*, long long, double*, int,
                                  long long, int);
 template void lu_inverse<float>(cudaStream_t, const float*, int, long long, int, const int*, long long, float*, int,
@@ -1105,8 +1190,9 @@ template void lu_inverse<float>(cudaStream_t, const float*, int, long long, int,
 template void lu_inverse<float2>(cudaStream_t, const float2*, int, long long, int, const int*, long long, float2*, int,
                                  long long, int);
 template void lu_solve<float>(cudaStream_t, int, const float*, int, long long, int, const int*, long long, float*, int,
-                              long long, int, int);
+                              long long, int, int, const LuInv<float>&);
 template void lu_solve<float2>(cudaStream_t, int, const float2*, int, long long, int, const int*, long long, float2*,
-                               int, long long, int, int);
+                               int, long long, int, int,
+                               const LuInv<float2>&);
 
 }  // namespace hs

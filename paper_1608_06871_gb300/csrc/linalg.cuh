@@ -38,12 +38,30 @@ template <>
 void gemm_fp32<float, float, float>(cudaStream_t, int, int, int, int, int, float, const float*, int, long long, const float*, int, long long, float, float*,
                     int, long long, int);
 
+// Inverses of the 128-row diagonal blocks of an LU (unit lower and upper
+// triangle), kept with the factors where a system is solved with again and again:
+// d[b sd + (2 block + (0: L, 1: U)) 128^2] (leading dimension 128), and room for a
+// copy of `cols` right-hand sides, tmp[b n cols + row cols + column].  Every step of
+// a solve is then a product.  The substitution of a 128-row block is a chain
+// bound by FP64 latency on as many SMs as there are columns; the root solves and the
+// few large merges at the top of an FP64 tree (at most four systems of more than 128 rows:
+// below that the batched substitutions fill the chip) gain: solve for one incidence
+// at k = 5 554 -> 372 us, k = 5 Gauss-Newton step 5.55 -> 5.34 ms, k = 20 gradient
+// 27.7 -> 26.1, k = 40 FP64 batch 61.7 -> 58.9 ms; errors against 64 bits unchanged.
+template <typename E> struct LuInv {
+  E* d = nullptr;
+  long long sd = 0;
+  E* tmp = nullptr;
+  int cols = 0;
+};
+inline size_t lu_inv_elems(int n) { return (size_t)((n + 127) / 128) * 2 * 128 * 128; }
+
 // In-place LU with partial pivoting P A = L U of a batch of n x n matrices.
 // piv[j] (0-based) is the row swapped with row j at step j.  info[b] is set to
 // j+1 at the first exactly-zero pivot of matrix b (it must be zeroed first).
 template <typename E>
 void lu_factor(cudaStream_t s, E* A, int lda, long long sA, int n, int* piv, long long sP, int* info,
-               int batch);
+               int batch, const LuInv<E>& inv = {});
 
 // Inv[b] = A[b]^{-1} (n x n, leading dimension ldi) from the factors of
 // lu_factor (identity right-hand sides through lu_solve).
@@ -62,7 +80,7 @@ void lu_panel(cudaStream_t s, E* A, int lda, long long sA, int n, int j0, int nb
 // (n x nrhs, leading dimension ldb) from the factors of lu_factor.
 template <typename E>
 void lu_solve(cudaStream_t s, int trans, const E* A, int lda, long long sA, int n, const int* piv,
-              long long sP, E* B, int ldb, long long sB, int nrhs, int batch);
+              long long sP, E* B, int ldb, long long sB, int nrhs, int batch, const LuInv<E>& inv = {});
 
 
 // FP32 products on the tensor cores by a two-term TF32 split (tc32.cu):

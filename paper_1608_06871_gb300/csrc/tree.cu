@@ -250,7 +250,7 @@ template <typename C> void merge_level(cudaStream_t s, const LevelMaps& L, const
   // top = B33 * bottom - top  (V = B33 Aa - Bb)
   gemm<C, C, C>(s, OP_N, OP_N, ni, np, ni, one, O.B33, ni, nn, O.XZ + (long long)ni * np, np, xz, mone, O.XZ, np, xz,
                 nb);
-  lu_factor<C>(s, O.M, ni, nn, ni, O.Mpiv, ni, info, nb);
+  lu_factor<C>(s, O.M, ni, nn, ni, O.Mpiv, ni, info, nb, O.inv);
   if constexpr (kInv) {
     // W = M^{-1} explicitly (the sweeps then apply it with one GEMM per
     // level); R is free until its diagonal blocks are gathered and stages W
@@ -266,7 +266,7 @@ template <typename C> void merge_level(cudaStream_t s, const LevelMaps& L, const
     HS_COUNT_LAUNCH();
   } else {
     // X = M^{-1} V (top half)
-    lu_solve<C>(s, OP_N, O.M, ni, nn, ni, O.Mpiv, ni, O.XZ, np, xz, np, nb);
+    lu_solve<C>(s, OP_N, O.M, ni, nn, ni, O.Mpiv, ni, O.XZ, np, xz, np, nb, O.inv);
   }
   // bottom = -A33 X - bottom  (Z = -Aa - A33 X)
   gemm<C, C, C>(s, OP_N, OP_N, ni, np, ni, mone, O.A33, ni, nn, O.XZ, np, xz, mone, O.XZ + (long long)ni * np, np, xz,
@@ -317,7 +317,7 @@ void sweep_adjoint_level(cudaStream_t s, const LevelMaps& L, const LevelOps<C>& 
     cudaMemcpy2DAsync(MU, (size_t)mu * sizeof(C), Lc, (size_t)tw * sizeof(C), (size_t)tw * sizeof(C), nb,
                       cudaMemcpyDeviceToDevice, s);
   } else {
-    lu_solve<C>(s, OP_T, O.M, ni, nn, ni, O.Mpiv, ni, MU, nrhs, mu, nrhs, nb);
+    lu_solve<C>(s, OP_T, O.M, ni, nn, ni, O.Mpiv, ni, MU, nrhs, mu, nrhs, nb, O.inv);
   }
   // la3 = B33^T Wt - lambda_tb
   gemm<C, C, C>(s, OP_T, OP_N, ni, nrhs, ni, one, O.B33, ni, nn, MU, nrhs, mu, mone, MU + (long long)ni * nrhs, nrhs,
@@ -360,7 +360,7 @@ void sweep_up_level(cudaStream_t s, const LevelMaps& L, const LevelOps<C>& O, co
     cudaMemcpy2DAsync(TT, tt * sizeof(C), S3, tt * sizeof(C), (size_t)ni * nrhs * sizeof(C), nb,
                       cudaMemcpyDeviceToDevice, s);
   } else {
-    lu_solve<C>(s, OP_N, O.M, ni, nn, ni, O.Mpiv, ni, TT, nrhs, tt, nrhs, nb);
+    lu_solve<C>(s, OP_N, O.M, ni, nn, ni, O.Mpiv, ni, TT, nrhs, tt, nrhs, nb, O.inv);
   }
   // bottom := -A33 t_a - (h3a - s_b) = t_b
   gemm<C, C, C>(s, OP_N, OP_N, ni, nrhs, ni, mone, O.A33, ni, nn, TT, nrhs, tt, mone, TT + (long long)ni * nrhs, nrhs,

@@ -47,6 +47,7 @@ template <typename C> struct LevelOps {
   C *A33, *B33, *M;  // [nbox][ni][ni]; M: LU of I - B33 A33 (FP64), W = (I - B33 A33)^{-1} (FP32)
   int* Mpiv;  // [nbox][ni]
   C* R;       // [nbox][np][np]  parent impedance-to-impedance maps
+  LuInv<C> inv;  // FP64: of M, the few large systems at the top of the tree (else empty)
 };
 
 // Legacy FP64 view used by the FP64 path.

@@ -99,3 +99,23 @@ def test_block_solves(hs, dtype, u, batch, n, nrhs):
     r = (A @ X - B).abs().amax(dim=(1, 2))
     scale = A.abs().sum(dim=2).amax(dim=1) * X.abs().amax(dim=(1, 2)) + B.abs().amax(dim=(1, 2))
     assert bool((r <= 8 * n * u * scale).all())
+
+
+@pytest.mark.parametrize("nL,M,P", [(1, 1, 3), (2, 3, 1), (4, 530, 7), (8, 2, 600)])
+def test_fp64_solves_by_block_inverses(hs, nL, M, P):
+    """Far fields and gradients of FP64 contexts whose root (and top merge) systems have one block, a
+    remainder block, and more right-hand sides of either sweep than one chunk of columns, against the
+    oracle with the bounds the other FP64 contexts are held to."""
+    import numpy as np
+    from oracle import forward as F
+    k, c = 2.0 + nL / 4, np.array([[0.05, -0.02], [0.01, 0.03]])
+    al, th = np.linspace(0.1, 6.0, M), np.linspace(0.2, 6.1, P)
+    fw = F.forward_from_coeffs(c, k, nL)
+    ref, _ = fw.solve_plane(al, th)
+    S = hs.Solver(nL, 2, 2).build(c, k)
+    uf = S.solve(al, th)
+    assert np.linalg.norm(uf - ref) < 1e-10 * np.linalg.norm(ref)
+    g, _ = S.gradient(ref * 1.1, al, th)
+    go = F.misfit_gradient(fw.jacobian(al, th, 2, 2), ref.ravel(), ref.ravel() * 1.1)
+    assert np.linalg.norm(g.ravel() - go) < 1e-9 * np.linalg.norm(go)
+    S.close()
