@@ -119,3 +119,18 @@ def test_fp64_solves_by_block_inverses(hs, nL, M, P):
     go = F.misfit_gradient(fw.jacobian(al, th, 2, 2), ref.ravel(), ref.ravel() * 1.1)
     assert np.linalg.norm(g.ravel() - go) < 1e-9 * np.linalg.norm(go)
     S.close()
+
+
+@pytest.mark.parametrize("nL,M,P,k", [(1, 2, 1, 0.7), (2, 1, 9, 3.0), (4, 3, 17, 6.0)])
+def test_mixed_adjoint_residuals(hs, nL, M, P, k):
+    """Jacobians of mixed contexts (adjoint residuals for one to seventeen receivers: part of a block's
+    eight, and one more than one or two blocks; leaves with one to four boundary sides) against the
+    oracle within the FP64 contexts' 1e-9."""
+    import numpy as np
+    from oracle import forward as F
+    c = np.array([[0.05, -0.02], [0.01, 0.03]])
+    al, th = np.linspace(0.1, 6.0, M), np.linspace(0.2, 6.1, P)
+    S = hs.Solver(nL, 2, 2, precision=hs.HS_MIXED).build(c, k)
+    J, Jo = S.jacobian(al, th), F.forward_from_coeffs(c, k, nL).jacobian(al, th, 2, 2)
+    assert np.linalg.norm(J - Jo) < 1e-9 * np.linalg.norm(Jo)
+    S.close()
