@@ -122,24 +122,35 @@ __device__ __forceinline__ void oz_ld8(uint32_t ta, uint32_t (&v)[8]) {
 // 32-bit store per slice: the 8 balanced base-128 digits a_s of N,
 // sum_s a_s 2^(49 - 7 s) = N, |a_0| <= 128, the others in [-64, 63].  With
 // B = sum_(s>0) 64 2^(49 - 7 s), the digits of N + B are its bit fields less 64
-// (the top one as it is): a field is a shift and a mask, its float comes from the
-// magic constant 2^23 or-ed under it (1.5 2^23 added, for the signed top one), and
-// the float's upper half is the exact BF16.
+// (the top one as it is).  Both numbers' fields are taken at once: a byte
+// permutation puts 16-bit windows of the two side by side, one shift and one
+// logical operation leave both fields under the BF16 128 (0x4300, unit 1), and a
+// packed subtraction of 192 gives the two exact BF16 digits.  The signed top digits get
+// their floats from 1.5 2^23 added below them.  (Field by field, with an FP32
+// subtraction each, the pair took 45 logical operations instead of 24, and the
+// slicing kernels were bound by them.)
 __device__ __forceinline__ void put2(long long N0, long long N1, uint32_t* o, int plane) {
   constexpr long long B = (64LL << 42) | (64LL << 35) | (64LL << 28) | (64LL << 21) | (64LL << 14) | (64LL << 7) | 64LL;
+  static_assert(OZ_S == 8, "seven fields and the top digit");
   N0 += B;
   N1 += B;
   auto top = [](long long n) { return __float_as_uint(__int_as_float(0x4B400000 + (int)(n >> 49)) - 12582912.0f); };
   o[0] = __byte_perm(top(N0), top(N1), 0x7632);
-#pragma unroll
-  for (int s = 1; s < OZ_S; ++s) {
-    const int sh = 49 - 7 * s;
-    const uint32_t f0 = ((uint32_t)((unsigned long long)N0 >> sh) & 127u) | 0x4B000000u;
-    const uint32_t f1 = ((uint32_t)((unsigned long long)N1 >> sh) & 127u) | 0x4B000000u;
-    const uint32_t b0 = __float_as_uint(__uint_as_float(f0) - 8388672.0f);
-    const uint32_t b1 = __float_as_uint(__uint_as_float(f1) - 8388672.0f);
-    o[s * plane] = __byte_perm(b0, b1, 0x7632);
-  }
+  auto digits = [](uint32_t w, int off) {
+    uint32_t d;
+    asm("sub.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(((w >> off) & 0x007F007Fu) | 0x43004300u), "r"(0x43404340u));
+    return d;
+  };
+  const uint32_t l0 = (uint32_t)N0, l1 = (uint32_t)N1, h0 = (uint32_t)((unsigned long long)N0 >> 28),
+                 h1 = (uint32_t)((unsigned long long)N1 >> 28);
+  const uint32_t h01 = __byte_perm(h0, h1, 0x5410), l01 = __byte_perm(l0, l1, 0x5410);
+  o[1 * plane] = digits(__byte_perm(h0, h1, 0x6521), 6);
+  o[2 * plane] = digits(h01, 7);
+  o[3 * plane] = digits(h01, 0);
+  o[4 * plane] = digits(__byte_perm(l0, l1, 0x7632), 5);
+  o[5 * plane] = digits(__byte_perm(l0, l1, 0x6521), 6);
+  o[6 * plane] = digits(l01, 7);
+  o[7 * plane] = digits(l01, 0);
 }
 
 __device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long i, long long k) {
@@ -239,24 +250,26 @@ __global__ void __launch_bounds__(256) k_oz_fix(double2* __restrict__ F, long lo
 // operation on the FP64 pipe (60% busy then, with 145 instructions per real
 // entry), and an error of about one unit of 2^-56 of the fields' maxima where
 // FP64 rounds each product to 2^-53 of itself.  25,600 pairs at n = 448: 101 ms
-// with FP64 products and 2-byte stores, 95 with 32-bit stores, 54 now (164 GB
-// written, 82 GB of fields read: 4.5 TB/s).
+// with FP64 products and 2-byte stores, 95 with 32-bit stores, 54 in integers, 47.7 with
+// the digits of two neighbours taken at once.
 __global__ void __launch_bounds__(256) k_oz_slice_kr(const int4* __restrict__ Ug, const int4* __restrict__ Zg,
-                                                     const int* __restrict__ eu, const int* __restrict__ ez, int P,
-                                                     int nX, long long c0, int nc, int pl, int npc, long long rpad,
-                                                     int nst, uint32_t* __restrict__ out, int* __restrict__ e) {
-  const long long r2 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+                                                     const int* __restrict__ eu, const int* __restrict__ ez,
+                                                     unsigned P, unsigned nX, unsigned d0, unsigned p0, unsigned nr,
+                                                     int pl, int npc, long long rpad, int nst,
+                                                     uint32_t* __restrict__ out, int* __restrict__ e) {
+  const unsigned r2 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (r2 >= (long long)nc * nX) return;
-  const int k0 = blockIdx.y * pl, kc = min(pl, nX - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
-  const long long c = c0 + r2 / nX, gy = r2 % nX;
-  const long long ru = (c / P) * nX + gy, rz = (c % P) * nX + gy;
+  if (r2 >= nr) return;
+  const int k0 = blockIdx.y * pl, kc = min(pl, (int)nX - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
+  // (32-bit divisions: the pair's incidence and receiver count from those of the chunk's first pair, d0 and p0)
+  const unsigned c = p0 + r2 / nX, gy = r2 % nX;
+  const long long ru = (long long)(d0 + c / P) * nX + gy, rz = (long long)(c % P) * nX + gy;
   const int4* u = Ug + ru * nX + k0;
   const int4* z = Zg + rz * nX + k0;
   if (lane == 0) {
     const int ex = min(eu[ru * npc + blockIdx.y] + ez[rz * npc + blockIdx.y] + 1, OZ_NAN);
-    e[blockIdx.y * rpad + 2 * r2] = ex;
-    e[blockIdx.y * rpad + 2 * r2 + 1] = ex;
+    e[blockIdx.y * rpad + 2LL * r2] = ex;
+    e[blockIdx.y * rpad + 2LL * r2 + 1] = ex;
   }
   auto mac = [](long long acc, int a, int b) { return acc + (long long)a * b; };
 #pragma unroll 2
@@ -277,7 +290,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_kr(const int4* __restrict__ Ug
       im[h] = 2 * ih + ((il + (1LL << 26)) >> 27);
     }
     // (rows 2 r2 and 2 r2 + 1 lie in one tile, 64 bytes apart, with the same swizzle)
-    uint32_t* o = out + oz_at<OZ_TM>(2 * r2, k0 + kk, nst);
+    uint32_t* o = out + oz_at<OZ_TM>(2LL * r2, k0 + kk, nst);
     put2(re[0], re[1], o, OZ_ROW * OZ_TM);
     put2(im[0], im[1], o + OZ_ROW, OZ_ROW * OZ_TM);
   }
@@ -656,7 +669,8 @@ void oz_slice_khatri_rao(cudaStream_t s, const double2* Ug, const double2* Zg, c
   int* ex = reinterpret_cast<int*>(reinterpret_cast<char*>(buf) + slice_bytes(rpad, nX));
   k_oz_slice_kr<<<dim3((unsigned)((warps + 7) / 8), npc), 256, 0, s>>>(
       reinterpret_cast<const int4*>(Ug), reinterpret_cast<const int4*>(Zg), reinterpret_cast<const int*>(eu),
-      reinterpret_cast<const int*>(ez), P, nX, c0, nc, pl, npc, rpad, nst, sl, ex);
+      reinterpret_cast<const int*>(ez), (unsigned)P, (unsigned)nX, (unsigned)(c0 / P), (unsigned)(c0 % P),
+      (unsigned)warps, pl, npc, rpad, nst, sl, ex);
   HS_COUNT_LAUNCH();
   if (rpad > rows) {
     const long long n = (rpad - rows) * nst * OZ_S * OZ_ROW;
