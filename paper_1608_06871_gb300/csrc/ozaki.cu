@@ -153,59 +153,96 @@ __device__ __forceinline__ void put2(long long N0, long long N1, uint32_t* o, in
   o[7 * plane] = digits(l01, 0);
 }
 
-__device__ __forceinline__ double src_at(const OzSrc& v, long long b, long long i, long long k) {
+// Row i of an operand's real form: entries 2 j and 2 j + 1 lie at p[j step + a0] and
+// p[j step + a1], negated where f0, f1 say so.
+struct OzRowAt {
+  const double* p;
+  long long step, a0, a1;
+  bool f0, f1;
+};
+__device__ __forceinline__ OzRowAt row_at(const OzSrc& v, long long b, int i) {
+  const int odd = i & 1;
   const double* p = v.p + b * v.sb;
   switch (v.kind) {
-    case OZ_REAL: return p[i * v.sr + k * v.sk];
-    case OZ_PAIR: return p[(i >> 1) * v.sr + k * v.sk + (i & 1)];
-    case OZ_PAIR_I: {  // i times the column: (-im, re)
-      const double x = p[(i >> 1) * v.sr + k * v.sk + ((i & 1) ^ 1)];
-      return i & 1 ? x : -x;
-    }
-    case OZ_CLEFT: return p[i * v.sr + (k >> 1) * v.sk + (k & 1)];
-    default: {  // OZ_CRIGHT: [re, -im; im, re]
-      const double x = p[(i >> 1) * v.sr + (k >> 1) * v.sk + ((i ^ k) & 1)];
-      return (k & 1) && !(i & 1) ? -x : x;
-    }
+    case OZ_REAL: return {p + i * v.sr, 2 * v.sk, 0, v.sk, false, false};
+    case OZ_PAIR: return {p + (i >> 1) * v.sr + odd, 2 * v.sk, 0, v.sk, false, false};
+    case OZ_PAIR_I: return {p + (i >> 1) * v.sr + 1 - odd, 2 * v.sk, 0, v.sk, !odd, !odd};  // i times it: (-im, re)
+    case OZ_CLEFT: return {p + i * v.sr, v.sk, 0, 1, false, false};
+    default: return {p + (i >> 1) * v.sr, v.sk, odd, 1 - odd, false, !odd};  // OZ_CRIGHT: [re, -im; im, re]
   }
 }
 
-// Slices of the rows of an operand (A's rows, or B's columns), one CTA per 16
-// rows and piece of k, written in blocks (oz_at, row b * rpad + i; BF16, zero
-// padded), the piece's row exponents to e[piece][b * rpad + i].  The block is
-// read once through shared memory (along k, or along the rows where those are
-// the contiguous direction), the row's largest magnitude fixes e with
-// max 2^-e in [1/2, 1), and each entry becomes the 56-bit fixed-point integer
-// N = round(x 2^(56 - e)), |N| < 2^56, whose balanced base-128 digits are the
-// slices and represent N exactly.  Integer arithmetic throughout (the FP64 pipe
-// is the scarce unit).  Padding rows get zero slices.
+struct OzSliced {  // an operand and where its slices go
+  OzSrc v;
+  int rows, rpad, k, pl, nst;
+  long long total;  // padded rows of all batches
+  uint32_t* out;
+  int* e;
+};
+
+// The slices of 16 rows and one piece of k, two rows a warp.
 template <int TR>
-__global__ void __launch_bounds__(256) k_oz_slice(OzSrc v, int rows, int k, int pl, int rpad, int nst, long long total,
-                                                  uint32_t* __restrict__ out, int* __restrict__ e) {
-  extern __shared__ double tile[];
-  const int k0 = blockIdx.y * pl, kc = min(pl, k - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
-  const long long r0 = (long long)blockIdx.x * OZ_SR;
-  const int pitch = pl + 1;
-  auto get = [&](int r, int kk) {
-    const long long g = r0 + r, b = g / rpad, i = g % rpad;
-    tile[r * pitch + kk] = (g < total && i < rows && kk < kc) ? src_at(v, b, i, k0 + kk) : 0.0;
+__device__ __forceinline__ void slice_rows(const OzSliced& o, int block, double* tile) {
+  const int k0 = blockIdx.y * o.pl, kc = min(o.pl, o.k - k0), kp = (kc + OZ_KS - 1) / OZ_KS * OZ_KS;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pitch = o.pl + 1;
+  const long long r0 = (long long)block * OZ_SR, b = r0 / o.rpad;  // (rpad is a multiple of the 16 rows)
+  const int i0 = (int)(r0 - b * o.rpad);
+  auto entry = [&](const OzRowAt& at, bool row, int kk) {
+    if (!row || kk >= kc) return 0.0;
+    const double x = at.p[(k0 + kk) / 2 * at.step + (kk & 1 ? at.a1 : at.a0)];
+    return (kk & 1 ? at.f1 : at.f0) ? -x : x;
   };
-  if (v.sk <= 2)
-    for (int q = threadIdx.x; q < OZ_SR * kp; q += 256) get(q / kp, q % kp);
-  else
-    for (int q = threadIdx.x; q < OZ_SR * kp; q += 256) get(q % OZ_SR, q / OZ_SR);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int r = warp; r < OZ_SR && r0 + r < total; r += 8) {
+  if (o.v.sk <= 2) {  // along k, each warp its own rows
+#pragma unroll
+    for (int r = warp; r < OZ_SR; r += 8) {
+      const OzRowAt at = row_at(o.v, b, min(i0 + r, o.rows - 1));
+#pragma unroll 4
+      for (int kk = lane; kk < kp; kk += 32) tile[r * pitch + kk] = entry(at, i0 + r < o.rows, kk);
+    }
+    __syncwarp();
+  } else {  // along the rows where those are the contiguous direction
+    const int r = threadIdx.x % OZ_SR;
+    const OzRowAt at = row_at(o.v, b, min(i0 + r, o.rows - 1));
+#pragma unroll 4
+    for (int kk = threadIdx.x / OZ_SR; kk < kp; kk += 256 / OZ_SR)
+      tile[r * pitch + kk] = entry(at, i0 + r < o.rows, kk);
+    __syncthreads();
+  }
+  for (int r = warp; r < OZ_SR; r += 8) {
     const double* x = tile + r * pitch;
     long long mx = 0;
     for (int kk = lane; kk < kp; kk += 32) mx = max(mx, abs_bits(x[kk]));
     for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     const int ex = row_exp(mx);
-    if (lane == 0) e[blockIdx.y * total + r0 + r] = ex;
+    if (lane == 0) o.e[blockIdx.y * o.total + r0 + r] = ex;
     for (int kk = 2 * lane; kk < kp; kk += 64)
-      put2(fixed56(x[kk], ex), fixed56(x[kk + 1], ex), out + oz_at<TR>(r0 + r, k0 + kk, nst), OZ_ROW * TR);
+      put2(fixed56(x[kk], ex), fixed56(x[kk + 1], ex), o.out + oz_at<TR>(r0 + r, k0 + kk, o.nst), OZ_ROW * TR);
   }
+}
+
+// Slices of the rows of one or both operands of a product (A's rows, or B's
+// columns), one CTA per 16 rows and piece of k (the first na CTAs: A),
+// written in blocks (oz_at, row b * rpad + i; BF16, zero padded), the piece's row
+// exponents to e[piece][b * rpad + i].  The block is read once through shared memory
+// (along k, or along the rows where those are the contiguous direction), the row's largest magnitude
+// fixes e with max 2^-e in [1/2, 1), and each entry becomes the 56-bit fixed-point integer
+// N = round(x 2^(56 - e)), |N| < 2^56, whose balanced base-128 digits are the
+// slices and represent N exactly.  Integer arithmetic throughout (the FP64 pipe
+// is the scarce unit).  Padding rows get zero slices.
+// Most launches are small (the products of one merge or panel update) and bound by
+// latency: with two launches a product, 64-bit divisions per entry and
+// a block barrier they took 15 to 17 us each.  One launch, one division a block, rows loaded
+// and sliced by the same warp: 10.2 -> 6.2 ms for the 209 products of a k = 40 FP64 batch
+// (58.3 -> 55.3 ms), k = 20 gradient 25.8 -> 23.8 ms, k = 5 Gauss-Newton step 5.3 -> 5.1.
+// (Pairs of k-neighbours loaded straight into registers: faster for the small launches, but the
+// strided loads cost the large ones more, 60.2 ms.)
+__global__ void __launch_bounds__(256) k_oz_slice(const __grid_constant__ OzSliced A, const __grid_constant__ OzSliced B,
+                                                  unsigned na) {
+  extern __shared__ double tile[];
+  if (blockIdx.x < na)
+    slice_rows<OZ_TM>(A, blockIdx.x, tile);
+  else
+    slice_rows<OZ_TN>(B, blockIdx.x - na, tile);
 }
 
 // Fields in fixed point, in place: each row piece (gx in one piece of k) of a
@@ -615,9 +652,7 @@ void set_smem_attr() {
   static bool done[64] = {};
   once_per_device(done, [] {
     cudaFuncSetAttribute(k_oz_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-    cudaFuncSetAttribute(k_oz_slice<OZ_TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         OZ_SR * (OZ_KMAX + 1) * (int)sizeof(double));
-    cudaFuncSetAttribute(k_oz_slice<OZ_TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_oz_slice, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          OZ_SR * (OZ_KMAX + 1) * (int)sizeof(double));
   });
 }
@@ -640,16 +675,28 @@ size_t oz_plane_bytes(int m, int n, int k, int batch) {
   return zs == 1 ? 0 : align_up((size_t)zs * batch * m * n * 8);
 }
 
-void oz_slice(cudaStream_t s, OzSrc v, int rows, int k, int batch, bool is_a, void* buf) {
-  set_smem_attr();
+namespace {
+OzSliced sliced(OzSrc v, int rows, int k, int batch, bool is_a, void* buf) {
   const long long rpad = padded(rows, is_a), total = batch * rpad;
-  const int pl = piece_len(k), npc = npieces(k);
   char* base = reinterpret_cast<char*>(buf);
-  auto kernel = is_a ? k_oz_slice<OZ_TM> : k_oz_slice<OZ_TN>;
-  kernel<<<dim3((unsigned)((total + OZ_SR - 1) / OZ_SR), npc), 256, OZ_SR * (pl + 1) * sizeof(double), s>>>(
-      v, rows, k, pl, (int)rpad, npc * pl / OZ_KS, total, reinterpret_cast<uint32_t*>(base),
-      reinterpret_cast<int*>(base + slice_bytes(total, k)));
+  return {v,     rows,
+          (int)rpad, k,
+          piece_len(k), npieces(k) * piece_len(k) / OZ_KS,
+          total, reinterpret_cast<uint32_t*>(base),
+          reinterpret_cast<int*>(base + slice_bytes(total, k))};
+}
+
+void launch_slice(cudaStream_t s, const OzSliced& a, const OzSliced& b, bool has_a, bool has_b) {
+  set_smem_attr();
+  const unsigned na = has_a ? (unsigned)(a.total / OZ_SR) : 0, nb = has_b ? (unsigned)(b.total / OZ_SR) : 0;
+  k_oz_slice<<<dim3(na + nb, npieces(a.k)), 256, OZ_SR * (a.pl + 1) * sizeof(double), s>>>(a, b, na);
   HS_COUNT_LAUNCH();
+}
+}  // namespace
+
+void oz_slice(cudaStream_t s, OzSrc v, int rows, int k, int batch, bool is_a, void* buf) {
+  const OzSliced o = sliced(v, rows, k, batch, is_a, buf);
+  launch_slice(s, o, o, is_a, !is_a);
 }
 
 size_t oz_fix_bytes(int fields, int nX) { return align_up((size_t)fields * nX * npieces(nX) * 4); }
@@ -754,8 +801,7 @@ cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double al
   char* a = reinterpret_cast<char*>(scratch);
   char* b = a + oz_operand_bytes(m, k, batch, true);
   char* pl = b + oz_operand_bytes(n, k, b_shared ? 1 : batch, false);
-  oz_slice(s, A, m, k, batch, true, a);
-  oz_slice(s, Bt, n, k, b_shared ? 1 : batch, false, b);
+  launch_slice(s, sliced(A, m, k, batch, true, a), sliced(Bt, n, k, b_shared ? 1 : batch, false, b), true, true);
   return oz_multiply(s, m, n, k, batch, alpha, a, b, b_shared, beta, C, oz_plane_bytes(m, n, k, batch) ? pl : nullptr,
                      sym);
 }
