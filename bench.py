@@ -498,7 +498,7 @@ def run_hs(args, world, rank, local):
                 "gpu_launches": main["launches"],
                 "roofline": {"bound": "alu",
                              "kernel": "k_gemm<FP64> (batched FP64 GEMM family)" if fp64_fam
-                             else "k_gemm / k_gemm_big <FP32> (SIMT FP32 GEMM family: merges, sweeps, LU "
+                             else "k_gemm32 / k_gemm_dot <FP32> (SIMT FP32 GEMM family: merges, sweeps, LU "
                                   "updates, leaf operators; the largest family of the mixed step)",
                              "achieved": achieved, "peak": fam_peak, "unit": "TFLOP/s",
                              "frac": (achieved / fam_peak) if (achieved and fam_peak) else None,
