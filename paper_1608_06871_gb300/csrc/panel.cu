@@ -529,9 +529,9 @@ __global__ void __launch_bounds__(PT) k_panel_cluster(E* A, int lda, long long s
       cl_st(cl_map(&aff_s[slot], 0), (uint32_t)(j0 + row0 + tr));
     }
   }
-  if (rank == 0 && t < steps) piv[j0 + t] = j0 + sp[t];
   if (rank == 0 && t == 0 && zc != INT_MAX && info[b] == 0) info[b] = j0 + zc + 1;
   if (nc > 1) cl_sync(); else __syncthreads();
+  if (rank == 0 && t < steps) piv[j0 + t] = j0 + sp[t];  // (thread 0 wrote sp, the last entry after the loop's barrier)
   const int na = (int)cl_ld(cl_map(&naff, 0));
   if (rank != 0 && t < na) {
     aff_d[t] = (int)cl_ld(cl_map(&aff_d[t], 0));
