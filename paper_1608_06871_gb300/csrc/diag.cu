@@ -214,7 +214,10 @@ int hs_dgemm_emulated(int m, int n, int k, const void* A, const void* B, void* C
   if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess) return HS_ENOMEM;
   const cudaError_t e = hs::ozaki_gemm(s, m, n, k, batch, 1.0, va, vb, false, 0.0, vc, scratch, bytes);
   cudaFreeAsync(scratch, s);
-  if (e != cudaSuccess) return e == cudaErrorInvalidValue ? HS_EINVAL : HS_ECUDA;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorInvalidValue ? HS_EINVAL : HS_ECUDA;
+  }
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return HS_ECUDA;
   if (hs::tc_timed_out(s)) return HS_ETIMEOUT;
   return HS_OK;

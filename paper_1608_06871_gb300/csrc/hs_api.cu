@@ -239,6 +239,7 @@ struct LaunchScope {
 };
 
 int fail(hs_ctx* c, int code, const std::string& msg) {
+  if (code == HS_ECUDA) cudaGetLastError();  // reported here, not by the next call too
   if (c) c->err = msg;
   return code;
 }

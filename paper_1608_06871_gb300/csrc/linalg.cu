@@ -830,6 +830,7 @@ bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alp
   while (nn > 2048 && !fits()) nn = ((nn + 1) / 2 + 63) / 64 * 64;
   while (kc > 384 && !fits()) kc = ((kc + 1) / 2 + 383) / 384 * 384;
   if (!fits()) return false;
+  // (what is left over for the last parts fits too; a launch that fails stays the last CUDA error)
   for (int b0 = 0; b0 < batch; b0 += nb)
     for (int n0 = 0; n0 < nr; n0 += nn)
       for (int k0 = 0; k0 < kr; k0 += kc) {

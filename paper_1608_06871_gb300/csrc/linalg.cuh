@@ -134,11 +134,13 @@ struct OzSrc {
   int kind;
 };
 extern bool g_oz_enabled;
-// Scratch bytes of ozaki_gemm for these sizes.
+// Scratch bytes of ozaki_gemm for these sizes; with the operands' bytes (oz_operand_bytes)
+// alone it runs too, without planes.
 size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared);
 // C[b] = alpha A[b] B[b] + beta C[b] (m x n, k inner; beta = 0 never reads C), sizes of the
 // real product; b_shared: one B for every batch; sym: only the 128 x 32 tiles that meet the
-// lower triangle are computed.  Returns cudaErrorInvalidValue on bad sizes.
+// lower triangle are computed.  Returns cudaErrorInvalidValue on bad sizes, or the error of a
+// launch, which also stays the CUDA runtime's last error.
 cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
                        double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym = false);
 // The same in two steps, for an operand used by many products: oz_slice cuts

@@ -773,7 +773,7 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
     HS_COUNT_LAUNCH();
   }
   if (prof) prof_end(s, ev, 2.0 * m * n * k * batch);  // FP64-equivalent flops
-  return cudaGetLastError();
+  return cudaPeekAtLastError();  // (left for the API call's own check: gemm() returns nothing)
 }
 
 thread_local const OzScratch* g_oz_scratch = nullptr;
@@ -794,16 +794,21 @@ size_t ozaki_scratch_bytes(int m, int n, int k, int batch, bool b_shared) {
          oz_plane_bytes(m, n, k, batch);
 }
 
+// The operands' bytes grow with every size; the planes' do not (fewer tiles than SMs
+// want some, more want none), so a part of a product that fits may want planes that do
+// not: its pieces of k then run one after the other in each tile.
+
 cudaError_t ozaki_gemm(cudaStream_t s, int m, int n, int k, int batch, double alpha, OzSrc A, OzSrc Bt, bool b_shared,
                        double beta, OzView C, void* scratch, size_t scratch_bytes, bool sym) {
   if (m <= 0 || n <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
-  if (ozaki_scratch_bytes(m, n, k, batch, b_shared) > scratch_bytes) return cudaErrorInvalidValue;
+  const size_t ab = oz_operand_bytes(m, k, batch, true), bb = oz_operand_bytes(n, k, b_shared ? 1 : batch, false),
+               pb = oz_plane_bytes(m, n, k, batch);
+  if (ab + bb > scratch_bytes) return cudaErrorInvalidValue;
   char* a = reinterpret_cast<char*>(scratch);
-  char* b = a + oz_operand_bytes(m, k, batch, true);
-  char* pl = b + oz_operand_bytes(n, k, b_shared ? 1 : batch, false);
+  char *b = a + ab, *pl = b + bb;
   launch_slice(s, sliced(A, m, k, batch, true, a), sliced(Bt, n, k, b_shared ? 1 : batch, false, b), true, true);
-  return oz_multiply(s, m, n, k, batch, alpha, a, b, b_shared, beta, C, oz_plane_bytes(m, n, k, batch) ? pl : nullptr,
-                     sym);
+  return oz_multiply(s, m, n, k, batch, alpha, a, b, b_shared, beta, C,
+                     pb && ab + bb + pb <= scratch_bytes ? pl : nullptr, sym);
 }
 
 }  // namespace hs
