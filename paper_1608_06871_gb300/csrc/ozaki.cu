@@ -15,9 +15,8 @@
 // diagonal accumulate into one FP32 accumulator in tensor memory:
 //   |partial sum| <= K 4096 (d + 3) < 2^24  for K <= 384,
 // which bounds the k extent of one piece (longer products sum their pieces in
-// FP64).  The epilogue recombines the 8 diagonal sums in 64-bit integers (the
-// last bits rounded at 2^-53 of the row times column scale for k = 384, 2^-56 for 32) and forms
-// the double from its bits.  What is dropped is the pairs with s + t >= 8,
+// FP64).  The epilogue recombines the 8 diagonal sums exactly in integers and
+// rounds them once to the double, formed from its bits.  What is dropped is the pairs with s + t >= 8,
 // below 2^-55 k max|A_i.| max|B_.j| per entry, and one FP64 rounding per piece:
 // the result stays within the FP64 product's own bound 2 k u |A| |B|.
 // A complex product is one real product: rows of A as (re, im) pairs along k,
@@ -345,13 +344,24 @@ __global__ void k_oz_zero_rows(long long first, long long rpad, int nst, int npc
   if (t < (long long)nr * npc) e[(t / nr) * rpad + first + t % nr] = 0;
 }
 
-// V 2^e as a double (round to nearest even), in integer arithmetic: two 64-bit
-// conversions, a scaling and their sum would be half the epilogue's time on
-// the FP64 pipe.
-__device__ __forceinline__ double scaled(long long V, int e) {
+// (hi 2^28 + lo) 2^e as a double (round to nearest even), |hi|, |lo| < 2^46, in
+// integer arithmetic: two 64-bit conversions, a scaling and their sum would be half
+// the epilogue's time on the FP64 pipe.
+__device__ __forceinline__ double scaled(long long hi, long long lo, int e) {
   if (e >= OZ_NAN / 2) return __longlong_as_double(0x7FF8000000000000LL);
-  unsigned long long a = V < 0 ? -(unsigned long long)V : (unsigned long long)V;
+  constexpr unsigned low = (1u << 28) - 1;
+  long long h = hi + (lo >> 28);  // h 2^28 + l with 0 <= l < 2^28
+  unsigned l = (unsigned)lo & low;
+  const bool neg = h < 0;
+  if (neg) {
+    h = -h - (l != 0);
+    l = (0u - l) & low;
+  }
+  // the leading 64 bits, what is cut off below them as a last bit (it only decides ties)
+  const int cut = max(28 - __clzll(h), 0);
+  unsigned long long a = ((unsigned long long)h << (28 - cut)) | (l >> cut) | ((l & ((1u << cut) - 1)) != 0);
   if (a == 0) return 0.0;
+  e += cut;
   const int z = __clzll(a);
   a <<= z;
   const int E = 1023 + 63 - z + e;  // biased exponent of the leading bit
@@ -359,10 +369,10 @@ __device__ __forceinline__ double scaled(long long V, int e) {
   const unsigned long long q = (a >> 11) + ((a >> 10) & ((a & 0x3FF) != 0 || ((a >> 11) & 1)));
   if (E < 1 || E > 2045) {  // subnormal or overflow
     const double r = scalbn((double)q, E - 1075);
-    return V < 0 ? -r : r;
+    return neg ? -r : r;
   }
   return __longlong_as_double((long long)((((unsigned long long)(E - 1)) << 52) + q) |
-                              (V < 0 ? (long long)0x8000000000000000ULL : 0LL));
+                              (neg ? (long long)0x8000000000000000ULL : 0LL));
 }
 
 struct OzParams {
@@ -523,8 +533,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // (rows and columns of the padding have exponents too)
         const int ea = P.ea[p * P.ea_piece + (long long)o.b * P.mpad + r];
         const int ebl = P.eb[p * P.eb_piece + (long long)(P.b_shared ? 0 : o.b) * P.npad + cb + (lane & 7)];
-        // |sum of the piece| <= 1.02 kc: V = sum 2^(63 - rs) stays below 2^62
-        const int rs = 33 - __clz(min(P.pl, P.k - p * P.pl));
         ok = oz_wait(su32(&accf[buf]), (pc >> 1) & 1);
         if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
@@ -554,9 +562,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           // sum_d C_d 2^(-7 (d + 2)) = (hi 2^28 + lo) 2^-63, hi and lo = q 2^14 + the next q
-          const long long V = ((((long long)q[0][j] << 14) + q[1][j]) << (28 - rs)) +
-                              ((((long long)q[2][j] << 14) + q[3][j] + (1LL << (rs - 1))) >> rs);
-          const double x = scaled(V, ea + __shfl_sync(0xffffffffu, ebl, j) + rs - 63);
+          const double x = scaled(((long long)q[0][j] << 14) + q[1][j], ((long long)q[2][j] << 14) + q[3][j],
+                                  ea + __shfl_sync(0xffffffffu, ebl, j) - 63);
           acc[j] = p == p0 ? x : acc[j] + x;
         }
       }
