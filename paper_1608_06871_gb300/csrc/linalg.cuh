@@ -160,6 +160,14 @@ struct OzScratch {
   size_t bytes = 0;
 };
 extern thread_local const OzScratch* g_oz_scratch;
+// Keeps the FP64 products enqueued in its scope on the FP64 pipe.
+struct PipeScope {
+  const OzScratch* const held = g_oz_scratch;
+  PipeScope() { g_oz_scratch = nullptr; }
+  ~PipeScope() { g_oz_scratch = held; }
+  PipeScope(const PipeScope&) = delete;
+  PipeScope& operator=(const PipeScope&) = delete;
+};
 // Estimated clocks of an emulated product on the whole chip (sizes of the real product).
 double oz_cycles(int m, int n, int k, int batch, bool b_shared);
 // Fields on the interior grid ([field][gy][gx], nX x nX) in the fixed point of
