@@ -123,7 +123,10 @@ int hs_solve_dev(hs_ctx* ctx, const double* alphas, int M, const double* thetas,
  * function again in that process.  All calls share the array and it keeps
  * the last call's contents (every region is written before it is read, so
  * nothing needs clearing): calls whose GPU work overlaps -- on different
- * streams or from different contexts -- race on it; serialise them. */
+ * streams or from different contexts -- race on it; serialise them.  The
+ * array is all that a call writes besides ufar, so it may run on one stream
+ * while other calls of ctx that only read the factors (solves, fields,
+ * Jacobians, gradients) run on another. */
 int hs_solve_noalloc(hs_ctx* ctx, const double* alphas, int M, const double* thetas, int P,
                      double* ufar, void* stream);
 

@@ -1004,16 +1004,17 @@ int factor(hs_ctx* ctx, double k) {
   return HS_OK;
 }
 
-// Root impedances f (nb x M) for plane waves; also returns ui, dni, g.
+// Root impedances f (nb x M) for plane waves; also returns ui, dni, g.  inv: the
+// blocks' inverses with the room its solve writes (the context's, or a caller's own).
 int root_solve(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, double2* ui, double2* dni, double2* f,
-               double2* g) {
+               double2* g, const LuInv<double2>& inv) {
   const int nb = ctx->B.nb;
   const double2 one = make_double2(1, 0), mone = make_double2(-1, 0), zero = make_double2(0, 0);
   incident_plane(s, ctx->B, ctx->k, alphas, M, ui, dni);
   // rhs = (D - I/2) u_inc - S d_n u_inc
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, one, ctx->d_Dm, nb, 0, ui, M, 0, zero, f, M, 0, 1);
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, mone, ctx->d_S, nb, 0, dni, M, 0, one, f, M, 0, 1);
-  lu_solve<double2>(s, OP_N, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, f, M, 0, M, 1, ctx->Cinv);
+  lu_solve<double2>(s, OP_N, ctx->d_C, nb, 0, nb, ctx->d_Cpiv, 0, f, M, 0, M, 1, inv);
   gemm<double2, double2, double2>(s, OP_N, OP_N, nb, M, nb, one, ctx->Rroot, nb, 0, f, M, 0, zero, g, M, 0, 1);
   return HS_OK;
 }
@@ -1112,7 +1113,7 @@ int solve_into(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M, const d
   double2* PS = a.get<double2>((size_t)2 * nb * M);
   double2* A2 = a.get<double2>((size_t)P * 2 * nb);
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g));
+  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g, ctx->Cinv));
   boundary_data(s, nb, M, ctx->k, f, g, ui, dni, PS);
   farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, thetas, P, A2);
   gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, make_double2(1, 0), PS, M, 0, A2, 2 * nb, 0,
@@ -1339,7 +1340,7 @@ int fields_and_adjoint(hs_ctx* ctx, cudaStream_t s, const double* alphas, int M,
   double2* A2 = a.get<double2>((size_t)P * 2 * nb);
   double2 *E = a.get<double2>((size_t)nb * P), *CP = a.get<double2>((size_t)nb * P);
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g));
+  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g, ctx->Cinv));
   CKR(sweep_down(ctx, s, f, M, bufA, bufB, T3, Uleaf));
   leaf_to_grid(s, Uleaf, NL, ctx->nL, M, Ug);
   farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, thetas, P, A2);
@@ -1669,7 +1670,7 @@ int gradient_core(hs_ctx* ctx, cudaStream_t s, const double* ddata, const double
     double2 *f = sub.get<double2>((size_t)nb * M), *g = sub.get<double2>((size_t)nb * M);
     double2* PS = sub.get<double2>((size_t)2 * nb * M);
     double2* A2 = sub.get<double2>((size_t)P * 2 * nb);
-    CKR(root_solve(ctx, s, da, M, ui, dni, f, g));
+    CKR(root_solve(ctx, s, da, M, ui, dni, f, g, ctx->Cinv));
     boundary_data(s, nb, M, ctx->k, f, g, ui, dni, PS);
     farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, dt, P, A2);
     gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, make_double2(1, 0), PS, M, 0, A2, 2 * nb, 0,
@@ -1718,6 +1719,9 @@ size_t far_solve_scratch_bytes(const hs_ctx* ctx, int M, int P) {
 
 // The far-field solve of solve_into with every temporary carved from the
 // caller's scratch (no allocation).  Used by the allocation-free entry point.
+// The scratch is all that it writes besides ufar: the root solve's copy of the right-hand
+// sides takes the room of g (written only after it), the emulated products' slices
+// what is left over, so it may run beside the context's other calls.
 int solve_far_in_scratch(hs_ctx* ctx, void* stream, const double* alphas, int M, const double* thetas, int P,
                          double* ufar, void* scratch, size_t scratch_bytes) {
   CKR(check_ctx(ctx, true));
@@ -1734,7 +1738,17 @@ int solve_far_in_scratch(hs_ctx* ctx, void* stream, const double* alphas, int M,
   double2* p = reinterpret_cast<double2*>(scratch);
   double2 *ui = p, *dni = ui + nb * M, *f = dni + nb * M, *g = f + nb * M;
   double2 *PS = g + nb * M, *A2 = PS + 2 * nb * M;
-  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g));
+  LuInv<double2> inv = ctx->Cinv;
+  inv.tmp = g;
+  inv.cols = M;
+  const size_t used = (far_solve_scratch_bytes(ctx, M, P) + 255) & ~size_t(255);
+  OzScratch rest;
+  if (used < scratch_bytes) {
+    rest.p = reinterpret_cast<char*>(scratch) + used;
+    rest.bytes = scratch_bytes - used;
+  }
+  g_oz_scratch = &rest;  // (for this call: the launch scope puts the former one back)
+  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g, inv));
   boundary_data(s, (int)nb, M, ctx->k, f, g, ui, dni, PS);
   farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, thetas, P, A2);
   gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * (int)nb, make_double2(1, 0), PS, M, 0, A2, 2 * (int)nb, 0,
@@ -1899,7 +1913,7 @@ int hs_fields_dev(hs_ctx* ctx, const double* alphas, int M, double* u, void* str
   double2* T3 = a.get<double2>(t3_elems(ctx, M));
   double2* Uleaf = a.get<double2>((size_t)ctx->nleaf * NL * M);
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g));
+  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g, ctx->Cinv));
   CKR(sweep_down(ctx, s, f, M, bufA, bufB, T3, Uleaf));
   leaf_to_nodes(s, Uleaf, ctx->nL, M, reinterpret_cast<double2*>(u));
   CK(cudaGetLastError());
@@ -1935,7 +1949,7 @@ int hs_forward_dev(hs_ctx* ctx, const double* alphas, int M, const double* theta
   double2* T3 = a.get<double2>(t3_elems(ctx, M));
   double2* Uleaf = a.get<double2>((size_t)ctx->nleaf * NL * M);
   if (a.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g));
+  CKR(root_solve(ctx, s, alphas, M, ui, dni, f, g, ctx->Cinv));
   boundary_data(s, nb, M, ctx->k, f, g, ui, dni, PS);
   farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, thetas, P, A2);
   gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, make_double2(1, 0), PS, M, 0, A2, 2 * nb, 0,
@@ -2028,7 +2042,7 @@ int hs_gn_step(hs_ctx* ctx, const double* data, const double* alphas, int M, con
     double2 *f = sub.get<double2>((size_t)nb * M), *g = sub.get<double2>((size_t)nb * M);
     double2* PS = sub.get<double2>((size_t)2 * nb * M);
     double2* A2 = sub.get<double2>((size_t)P * 2 * nb);
-    CKR(root_solve(ctx, s, da, M, ui, dni, f, g));
+    CKR(root_solve(ctx, s, da, M, ui, dni, f, g, ctx->Cinv));
     boundary_data(s, nb, M, ctx->k, f, g, ui, dni, PS);
     farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, dt, P, A2);
     gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, make_double2(1, 0), PS, M, 0, A2, 2 * nb, 0,
@@ -2135,7 +2149,7 @@ int hs_gn_step_lsqr(hs_ctx* ctx, const double* data, const double* alphas, int M
     double2* PS = sub.get<double2>((size_t)2 * nb * M);
     double2* A2 = sub.get<double2>((size_t)P * 2 * nb);
     if (sub.over) return fail(ctx, HS_ENOMEM, "workspace request beyond its sizing");
-    CKR(root_solve(ctx, s, da, M, ui, dni, f, g));
+    CKR(root_solve(ctx, s, da, M, ui, dni, f, g, ctx->Cinv));
     boundary_data(s, nb, M, ctx->k, f, g, ui, dni, PS);
     farfield_matrix(s, ctx->B, ctx->k, ctx->cfg.R, dt, P, A2);
     gemm<double2, double2, double2>(s, OP_T, OP_T, M, P, 2 * nb, make_double2(1, 0), PS, M, 0, A2, 2 * nb, 0,
