@@ -8,8 +8,6 @@
 //   each side by increasing coordinate:         e = side*14 + (t-1)        (56)
 //   S: (a, 0)   E: (15, b)   N: (a, 15)   W: (0, b)
 // The 4 corner nodes are not unknowns of the discretisation.
-#include <optional>
-
 #include "tree.cuh"
 
 namespace hs {
@@ -176,31 +174,33 @@ void leaf_build_chunk(cudaStream_t s, const double* q, int leaf0, int nleaf, dou
   const double eta = k;
   k_leaf_assemble<T><<<nleaf, 256, 0, s>>>(q, leaf0, d_k, h, w.Aii, w.Aie, w.Ni, w.NiT, w.Ne);
   HS_COUNT_LAUNCH();
-  // The spectral blocks are graded: their rows and columns spread over four decades, and
-  // the emulated product's error is relative to a row's and a column's largest entry.
-  // With it, far fields of FP64 contexts were up to 1.5 times as far from the dense
-  // solution of the same system (k = 3.1 on 4 x 4 leaves: 4.0e-13 on the pipe, 5.0e-13),
-  // the factor T = Ne - Ni X the largest part of it.  The products with K^{-1} below
-  // make no difference and stay emulated.
-  std::optional<PipeScope> pipe(std::in_place);
-  lu_factor<T>(s, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, info, nleaf);
-  // X = Aii^{-1} Aie (Dirichlet-to-interior map), W = Aii^{-T} Ni^T (adjoint)
-  if (w.Ainv && !Q) {
-    // keep Aii^{-1} (the mixed path's particular solves use it); X by one GEMM
-    // staged in NiT, whose transpose rows the path without adjoint never needs
-    lu_inverse<T>(s, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, w.Ainv + (long long)leaf0 * NI * NI, NI,
-                  (long long)NI * NI, nleaf);
-    gemm<T, T, T>(s, OP_N, OP_N, NI, NE, NI, T(1), w.Ainv + (long long)leaf0 * NI * NI, NI, (long long)NI * NI, w.Aie,
-                  NE, (long long)NI * NE, T(0), w.NiT, NE, (long long)NI * NE, nleaf);
-    cudaMemcpyAsync(w.Aie, w.NiT, sizeof(T) * (size_t)nleaf * NI * NE, cudaMemcpyDeviceToDevice, s);
-  } else {
-    lu_solve<T>(s, OP_N, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, w.Aie, NE, (long long)NI * NE, NE, nleaf);
+  {
+    // The spectral blocks are graded: their rows and columns spread over four decades,
+    // and the emulated product's error is relative to a row's and a column's largest
+    // entry.  With it, far fields of FP64 contexts were up to 1.5 times as far from the
+    // dense solution of the same system (k = 3.1 on 4 x 4 leaves: 4.0e-13 on the pipe,
+    // 5.0e-13), the factor T the largest part of it.  The adjoint's solve and the products
+    // with K^{-1} make no difference and stay emulated.
+    const PipeScope pipe;
+    lu_factor<T>(s, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, info, nleaf);
+    // X = Aii^{-1} Aie (Dirichlet-to-interior map)
+    if (w.Ainv && !Q) {
+      // keep Aii^{-1} (the mixed path's particular solves use it); X by one GEMM
+      // staged in NiT, whose transpose rows the path without adjoint never needs
+      lu_inverse<T>(s, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, w.Ainv + (long long)leaf0 * NI * NI, NI,
+                    (long long)NI * NI, nleaf);
+      gemm<T, T, T>(s, OP_N, OP_N, NI, NE, NI, T(1), w.Ainv + (long long)leaf0 * NI * NI, NI, (long long)NI * NI,
+                    w.Aie, NE, (long long)NI * NE, T(0), w.NiT, NE, (long long)NI * NE, nleaf);
+      cudaMemcpyAsync(w.Aie, w.NiT, sizeof(T) * (size_t)nleaf * NI * NE, cudaMemcpyDeviceToDevice, s);
+    } else {
+      lu_solve<T>(s, OP_N, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, w.Aie, NE, (long long)NI * NE, NE, nleaf);
+    }
+    // T = Ne - Ni X  (leaf Dirichlet-to-Neumann map), stored in Ne
+    gemm<T, T, T>(s, OP_N, OP_N, NE, NE, NI, T(-1), w.Ni, NI, (long long)NE * NI, w.Aie, NE, (long long)NI * NE, T(1),
+                  w.Ne, NE, (long long)NE * NE, nleaf);
   }
-  if (Q)  // W is needed only by the adjoint operator
+  if (Q)  // W = Aii^{-T} Ni^T, needed only by the adjoint operator
     lu_solve<T>(s, OP_T, w.Aii, NI, (long long)NI * NI, NI, w.piv, NI, w.NiT, NE, (long long)NI * NE, NE, nleaf);
-  // T = Ne - Ni X  (leaf Dirichlet-to-Neumann map), stored in Ne
-  gemm<T, T, T>(s, OP_N, OP_N, NE, NE, NI, T(-1), w.Ni, NI, (long long)NE * NI, w.Aie, NE, (long long)NI * NE, T(1),
-                w.Ne, NE, (long long)NE * NE, nleaf);
   {
     long long n = (long long)nleaf * NE * NE;
     k_make_K<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.Ne, d_k, w.K, w.Kinv, nleaf);
@@ -213,7 +213,6 @@ void leaf_build_chunk(cudaStream_t s, const double* q, int leaf0, int nleaf, dou
     k_leaf_R<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w.Kinv, d_k, R, Y, nleaf);
     HS_COUNT_LAUNCH();
   }
-  pipe.reset();
   C m1 = el<C>::zero(), z0 = el<C>::zero(), ieta2 = el<C>::zero();
   m1.x = T(-1);
   ieta2.y = T(2.0 * eta);
