@@ -43,6 +43,14 @@ extern "C" {
 #define HS_ENOCONV (-6)     /* iterative refinement did not converge          */
 #define HS_ETIMEOUT (-7)    /* a bounded device wait gave up                  */
 
+/* HS_ETIMEOUT: the tensor-core products (of every kind of context) bound their
+ * device waits; one that gives up leaves its results unspecified and sets a
+ * flag of the device.  hs_build, hs_build_nodes, hs_solve, hs_jacobian,
+ * hs_gradient, hs_gn_step and hs_gn_step_lsqr, which wait for the GPU, read
+ * and clear it before they return.  The calls that only enqueue work (the
+ * _dev ones, hs_solve_noalloc) cannot: a timeout in one of them is returned by
+ * the next of the calls above on the same context. */
+
 #define HS_FP64 0   /* every step in complex FP64                            */
 #define HS_MIXED 1  /* FP32 factors and sweep, FP64 residual refinement       */
 

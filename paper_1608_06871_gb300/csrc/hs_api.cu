@@ -216,6 +216,7 @@ struct hs_ctx {
   // serves every k of a sweep on this tree
   double* d_k = nullptr;
   OzScratch oz;  // slices of the emulated FP64 products (ensure_oz)
+  bool tc_pending = false;  // some of them ran since the timeout flags were last read
   double k_dev = 0.0;
   long long builds = 0;
   // phase times of the last build recorded launch by launch (-1 after a graph replay)
@@ -228,13 +229,16 @@ namespace {
 struct LaunchScope {
   long long* prev;
   const OzScratch* prev_oz;
-  explicit LaunchScope(hs_ctx* c) : prev(g_launch_counter), prev_oz(g_oz_scratch) {
+  bool* prev_pending;
+  explicit LaunchScope(hs_ctx* c) : prev(g_launch_counter), prev_oz(g_oz_scratch), prev_pending(g_tc_pending) {
     g_launch_counter = &c->launches;
     g_oz_scratch = &c->oz;
+    g_tc_pending = &c->tc_pending;
   }
   ~LaunchScope() {
     g_launch_counter = prev;
     g_oz_scratch = prev_oz;
+    g_tc_pending = prev_pending;
   }
 };
 
@@ -384,14 +388,22 @@ int ensure_oz(hs_ctx* ctx) {
   return HS_OK;
 }
 
+// HS_ETIMEOUT if a tensor-core wait of the context's work gave up; waits for s.  Reading
+// the flags takes some 25 us, so calls that launched no such product leave them.
+int check_tc(hs_ctx* ctx, cudaStream_t s) {
+  if (!ctx->tc_pending && !tc_timeout_raised()) return HS_OK;
+  ctx->tc_pending = false;
+  return tc_timed_out(s) ? fail(ctx, HS_ETIMEOUT, "a tensor-core GEMM wait gave up") : HS_OK;
+}
+
 int check_info(hs_ctx* ctx) {
   std::vector<int> info(ctx->ninfo);
   CK(cudaMemcpyAsync(info.data(), ctx->d_info, sizeof(int) * ctx->ninfo, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   for (int v : info)
     if (v != 0) return fail(ctx, HS_ESINGULAR, "zero pivot in a factorisation (column " + std::to_string(v) + ")");
-  if (tc_timed_out(ctx->stream)) return fail(ctx, HS_ETIMEOUT, "a tensor-core GEMM wait gave up");
-  return HS_OK;
+  ctx->tc_pending = true;  // (a build reads the flags whatever ran)
+  return check_tc(ctx, ctx->stream);
 }
 
 // Events bracketing the interior factorisation (leaves and merges) and the
@@ -1883,7 +1895,8 @@ int hs_solve(hs_ctx* ctx, const double* alphas, int M, const double* thetas, int
   cudaFreeAsync(dt, s);
   cudaFreeAsync(du, s);
   CK(cudaStreamSynchronize(s));
-  return r;
+  CKR(r);
+  return check_tc(ctx, s);
 }
 
 int hs_fields_dev(hs_ctx* ctx, const double* alphas, int M, double* u, void* stream) {
@@ -1989,7 +2002,7 @@ int hs_jacobian(hs_ctx* ctx, const double* alphas, int M, const double* thetas, 
   CKR(jacobian_into(ctx, s, da, M, dt, P, dJ, a));
   CK(cudaMemcpyAsync(J, dJ, sizeof(double2) * nJ, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  return HS_OK;
+  return check_tc(ctx, s);
 }
 
 int hs_gn_step(hs_ctx* ctx, const double* data, const double* alphas, int M, const double* thetas, int P,
@@ -2355,6 +2368,7 @@ int hs_gradient(hs_ctx* ctx, const double* data, const double* alphas, int M, co
   CK(cudaMemcpyAsync(grad, dg, sizeof(double) * nm, cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&mis, dm, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  CKR(check_tc(ctx, s));
   if (misfit_out) *misfit_out = mis;
   return HS_OK;
 }

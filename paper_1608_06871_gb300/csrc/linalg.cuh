@@ -92,7 +92,6 @@ void lu_solve(cudaStream_t s, int trans, const E* A, int lda, long long sA, int 
 bool t32_gemm(cudaStream_t s, int mode, int m, int n, int k, float2 alpha, const float* A, long long lda,
               long long sA, const float* B, long long ldb, long long sB, float2 beta, void* C, int ldc, long long sC,
               int batch);
-bool t32_timed_out(cudaStream_t s);
 // gemm() measures, once per shape, the tensor-core and the SIMT product and
 // keeps the faster (g_autotune; off: a fixed size rule); g_last_gemm_tc is 1
 // when the calling thread's last gemm() ran on the tensor cores.
@@ -109,8 +108,15 @@ extern thread_local int g_last_gemm_tc;
 // tensor-core wait gave up (the split-TF32 product's, the emulated-FP64 one's,
 // and the one the host raises in tests; tcgemm.cu).
 bool tc_timed_out(cudaStream_t s);
-bool oz_timed_out(cudaStream_t s);
+// One kernel family's flag: enqueues a copy of it to *v or (clear) of *v, a zero, to it.
+void oz_timeout_flag(cudaStream_t s, int* v, bool clear);
+void t32_timeout_flag(cudaStream_t s, int* v, bool clear);
 cudaError_t tc_raise_timeout_flag();
+// The host raised a flag that no check has read yet.
+bool tc_timeout_raised();
+// Set by the emulated FP64 products that the calling thread launches, where it points
+// somewhere: the owner of the work then reads the flags once it has waited for it.
+extern thread_local bool* g_tc_pending;
 
 // FP64 products on the tensor cores by exact BF16 slices (ozaki.cu).
 // Output view: element (b, i, j) at p[b sb + (i / ig) si + (i % ig) sg + j sk]

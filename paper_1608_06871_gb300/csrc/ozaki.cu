@@ -622,16 +622,11 @@ inline long long rup(long long x, long long m) { return (x + m - 1) / m * m; }
 
 bool g_oz_enabled = true;  // process-wide switch (hs_set_fp64_emulation)
 
-bool oz_timed_out(cudaStream_t s) {
-  int v = 0, z = 0;
-  cudaStreamSynchronize(s);
-  cudaMemcpyFromSymbolAsync(&v, g_oz_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  if (v) {
-    cudaMemcpyToSymbolAsync(g_oz_timeout, &z, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  }
-  return v != 0;
+void oz_timeout_flag(cudaStream_t s, int* v, bool clear) {
+  if (clear)
+    cudaMemcpyToSymbolAsync(g_oz_timeout, v, sizeof(int), 0, cudaMemcpyHostToDevice, s);
+  else
+    cudaMemcpyFromSymbolAsync(v, g_oz_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
 }
 
 namespace {
@@ -772,6 +767,7 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
   const bool prof = prof_active(4);
   cudaEvent_t ev = nullptr;
   if (prof) prof_begin(s, &ev);
+  if (g_tc_pending) *g_tc_pending = true;
   k_oz_mma<<<(unsigned)std::min<long long>(P.items, 152), OZ_THREADS, OZ_SMEM, s>>>(P);
   HS_COUNT_LAUNCH();
   if (split) {
@@ -784,6 +780,7 @@ cudaError_t oz_multiply(cudaStream_t s, int m, int n, int k, int batch, double a
 }
 
 thread_local const OzScratch* g_oz_scratch = nullptr;
+thread_local bool* g_tc_pending = nullptr;
 
 // Per tile 2100 clocks a stage, or 9400 a piece where that is more; slices
 // written and read at about 2600 bytes a clock; launches.

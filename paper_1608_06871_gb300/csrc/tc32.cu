@@ -476,16 +476,11 @@ void launch_mma(cudaStream_t s, dim3 grid, const CUtensorMap& ma, const CUtensor
 
 }  // namespace
 
-bool t32_timed_out(cudaStream_t s) {
-  int v = 0, z = 0;
-  cudaStreamSynchronize(s);
-  cudaMemcpyFromSymbolAsync(&v, g_t32_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  if (v) {
-    cudaMemcpyToSymbolAsync(g_t32_timeout, &z, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  }
-  return v != 0;
+void t32_timeout_flag(cudaStream_t s, int* v, bool clear) {
+  if (clear)
+    cudaMemcpyToSymbolAsync(g_t32_timeout, v, sizeof(int), 0, cudaMemcpyHostToDevice, s);
+  else
+    cudaMemcpyFromSymbolAsync(v, g_t32_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
 }
 
 bool t32_gemm(cudaStream_t s, int mode, int m, int n, int k, float2 alpha, const float* A, long long lda,
