@@ -377,15 +377,21 @@ int ensure_ws(hs_ctx* ctx, size_t bytes, Arena& a) {
 
 // Scratch of the emulated FP64 products of a context, allocated once (at the
 // first build of an FP64 context, the first gradient or Gauss-Newton step of a
-// mixed one): the leaf products of a few hundred leaves at a time, 32 to 512 MB.
-int ensure_oz(hs_ctx* ctx) {
-  if (ctx->oz.p || !g_oz_enabled) return HS_OK;
+// mixed one): the leaf products of a few hundred leaves at a time, 32 to 512 MB;
+// where the device has no room for it the products stay on the FP64 pipe.
+void ensure_oz(hs_ctx* ctx) {
+  if (!g_oz_enabled) return;
+  if (ctx->oz.p) return;
   const size_t n = std::min<size_t>((size_t)512 << 20, std::max<size_t>((size_t)32 << 20, (size_t)ctx->nleaf * 1500000));
+  const std::string err = ctx->err;
   char* p = nullptr;
-  CKR(dalloc(ctx, &p, n));
+  if (dalloc(ctx, &p, n) != HS_OK) {
+    cudaGetLastError();
+    ctx->err = err;
+    return;
+  }
   ctx->oz.p = p;
   ctx->oz.bytes = n;
-  return HS_OK;
 }
 
 // HS_ETIMEOUT if a tensor-core wait of the context's work gave up; waits for s.  Reading
@@ -968,7 +974,7 @@ int factor(hs_ctx* ctx, double k) {
   if (ctx->cfg.precision == HS_MIXED) return factor_mixed(ctx, k);
   cudaStream_t s = ctx->stream;
   CKR(phase_events(ctx));
-  CKR(ensure_oz(ctx));
+  ensure_oz(ctx);
   CKR(set_device_k(ctx, s, k));
   CK(cudaMemsetAsync(ctx->d_info, 0, sizeof(int) * ctx->ninfo, s));
   CK(cudaEventRecord(ctx->ph_ev[0], s));
@@ -2024,7 +2030,7 @@ int hs_gn_step(hs_ctx* ctx, const double* data, const double* alphas, int M, con
                 std::max(jacobian_bytes(ctx, M, P),
                          4 * Arena::bytes((size_t)ctx->B.nb * M, 16) + Arena::bytes((size_t)2 * ctx->B.nb * M, 16) +
                              Arena::bytes((size_t)P * 2 * ctx->B.nb, 16));
-  CKR(ensure_oz(ctx));
+  ensure_oz(ctx);
   CKR(ensure_ws(ctx, need, a));
   double* da = a.get<double>(M);
   double* dt = a.get<double>(P);
@@ -2336,7 +2342,7 @@ int hs_gradient_dev(hs_ctx* ctx, const double* data, const double* alphas, int M
   CKR(valid_angles(ctx, M, P));
   if (!data || !alphas || !thetas || !grad || !misfit_out) return fail(ctx, HS_EINVAL, "NULL pointer");
   Arena a;
-  CKR(ensure_oz(ctx));
+  ensure_oz(ctx);
   CKR(ensure_ws(ctx, gradient_bytes(ctx, M, P), a));
   return gradient_core(ctx, pick(ctx, stream), data, alphas, M, thetas, P, grad, misfit_out, a);
 }
@@ -2352,7 +2358,7 @@ int hs_gradient(hs_ctx* ctx, const double* data, const double* alphas, int M, co
   Arena a;
   size_t need = Arena::bytes(M, 8) + Arena::bytes(P, 8) + Arena::bytes((size_t)2 * MP, 8) + Arena::bytes(nm, 8) +
                 Arena::bytes(8, 8) + gradient_bytes(ctx, M, P);
-  CKR(ensure_oz(ctx));
+  ensure_oz(ctx);
   CKR(ensure_ws(ctx, need, a));
   double* da = a.get<double>(M);
   double* dt = a.get<double>(P);

@@ -1,6 +1,7 @@
 """Failures on FP64 contexts, made on the host as in test_gpu_failures.py: a
 tensor-core wait that gave up (the flag that it would set, set from the host)
-is reported by every call that synchronises, and once."""
+is reported by every call that synchronises, and once; scratch that only
+speeds the FP64 products up and cannot be had is not an error."""
 import numpy as np
 import pytest
 
@@ -59,3 +60,23 @@ def test_timeout_of_a_device_call_is_reported_by_the_next_that_synchronises(hs):
     other.build(c, 3.0)  # nothing is left over for another context
     s.close()
     other.close()
+
+
+def test_build_and_gradient_without_the_product_scratch(hs):
+    c, al, th = _problem()
+    ref = hs.Solver(4, 4, 4).build(c, 5.0)
+    far = ref.solve(al, th)
+    grad = ref.gradient(1.1 * far, al, th)[0]
+    s, m = hs.Solver(4, 4, 4), hs.Solver(4, 4, 4, precision=hs.HS_MIXED).build(c, 5.0)
+    try:
+        hs.hs_fail_next_allocs(1)  # the first allocation of each is the scratch
+        s.build(c, 5.0)
+        hs.hs_fail_next_allocs(1)
+        gm = m.gradient(1.1 * far, al, th)[0]
+    finally:
+        hs.hs_fail_next_allocs(0)
+    assert rel(s.solve(al, th), far) < 1e-10
+    assert rel(s.gradient(1.1 * far, al, th)[0], grad) < 1e-9
+    assert rel(gm, grad) < 1e-8
+    for x in (ref, s, m):
+        x.close()
