@@ -232,7 +232,9 @@ struct LaunchScope {
   bool* prev_pending;
   explicit LaunchScope(hs_ctx* c) : prev(g_launch_counter), prev_oz(g_oz_scratch), prev_pending(g_tc_pending) {
     g_launch_counter = &c->launches;
-    g_oz_scratch = &c->oz;
+    // a mixed context's only in the calls that allocate it (ensure_oz): what another call
+    // computes does not depend on whether one of them came before
+    g_oz_scratch = c->cfg.precision == HS_FP64 ? &c->oz : nullptr;
     g_tc_pending = &c->tc_pending;
   }
   ~LaunchScope() {
@@ -378,9 +380,11 @@ int ensure_ws(hs_ctx* ctx, size_t bytes, Arena& a) {
 // Scratch of the emulated FP64 products of a context, allocated once (at the
 // first build of an FP64 context, the first gradient or Gauss-Newton step of a
 // mixed one): the leaf products of a few hundred leaves at a time, 32 to 512 MB;
-// where the device has no room for it the products stay on the FP64 pipe.
+// where the device has no room for it the products stay on the FP64 pipe.  In use
+// from here to the end of the call.
 void ensure_oz(hs_ctx* ctx) {
   if (!g_oz_enabled) return;
+  g_oz_scratch = &ctx->oz;
   if (ctx->oz.p) return;
   const size_t n = std::min<size_t>((size_t)512 << 20, std::max<size_t>((size_t)32 << 20, (size_t)ctx->nleaf * 1500000));
   const std::string err = ctx->err;

@@ -344,6 +344,7 @@ void sine_eval_grid(cudaStream_t s, const double* c, int S1, int S2, const doubl
   k_sine_table<<<g2, 128, 0, s>>>(xg, n16, S2, sy);
   HS_COUNT_LAUNCH();
   // T[m1][gy] = sum_m2 c[m1][m2] sy[m2][gy];   Qg[gx][gy] = sum_m1 sx[m1][gx] T[m1][gy]
+  const PipeScope pipe;  // (an FP64 context has its scratch from the first build on: the same bits in every build)
   gemm<double, double, double>(s, OP_N, OP_N, S1, n16, S2, 1.0, c, S2, 0, sy, n16, 0, 0.0, T, n16, 0, 1);
   gemm<double, double, double>(s, OP_T, OP_N, n16, n16, S1, 1.0, sx, n16, 0, T, n16, 0, 0.0, Qg, n16, 0, 1);
   long long n = (long long)n16 * n16;

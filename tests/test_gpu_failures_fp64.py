@@ -1,7 +1,8 @@
 """Failures on FP64 contexts, made on the host as in test_gpu_failures.py: a
 tensor-core wait that gave up (the flag that it would set, set from the host)
 is reported by every call that synchronises, and once; scratch that only
-speeds the FP64 products up and cannot be had is not an error."""
+speeds the FP64 products up and cannot be had is not an error, and results do
+not depend on whether an earlier call allocated it."""
 import numpy as np
 import pytest
 
@@ -80,3 +81,16 @@ def test_build_and_gradient_without_the_product_scratch(hs):
     assert rel(gm, grad) < 1e-8
     for x in (ref, s, m):
         x.close()
+
+
+@pytest.mark.parametrize("precision", ["HS_FP64", "HS_MIXED"])
+def test_results_do_not_depend_on_earlier_calls(hs, precision):
+    # (32 x 32 leaves, 64 x 64 modes: q on the leaf grid is a product worth the tensor cores)
+    c, al, th = synth.random_coeffs(64, 64, seed=12, scale=0.004), synth.directions(24), synth.receivers(32)
+    s = hs.Solver(32, 64, 64, precision=getattr(hs, precision)).build(c, 16.0)
+    first = s.solve(al, th)
+    s.gradient(1.1 * first, al, th)
+    s.gn_step(1.1 * first, al, th, 1e-3, c)
+    s.build(c, 16.0)
+    assert np.array_equal(s.solve(al, th), first)
+    s.close()
