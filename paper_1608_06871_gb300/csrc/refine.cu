@@ -50,7 +50,6 @@ struct FixSum {
     m += (long long)a.x * x0;
     m += (long long)a.y * x1;
   }
-  __device__ __forceinline__ long long value() const { return h + (m >> 28); }
   // 2^-n of the value, rounded
   __device__ __forceinline__ long long down(int n) const {
     const long long v = h + ((m + (1LL << 27)) >> 28);
@@ -84,9 +83,11 @@ __device__ __forceinline__ double fix_double(long long v, int e) {
 // FP64 multiply-adds (two thread-operations per SM and clock) bounded this
 // kernel; the integer ones run seven times as fast: 2.49 -> 1.2 ms for 1024 leaves
 // and 128 right-hand sides, the normal derivatives included that the interface
-// residuals formed by FP64 sums of their own before (0.8 ms a pass).  Rounding of Lap_h u for plane
-// waves (k = 17 .. 40, h = 1/16), root mean square over the nodes: 1.49e-10,
-// 1.67e-10 and 1.55e-10 against 1.54e-10, 1.84e-10 and 1.66e-10 of the FP64 sums.
+// residuals formed by FP64 sums of their own before (0.8 ms a pass).  Rounding of Lap_h u +
+// k^2 (1 - q) u for plane waves (k = 17, 25, 40, h = 1/16; root mean square over the nodes,
+// from the exact sums with the same coefficients): 3.0e-11, 2.9e-11 and 2.7e-11, of the FP64
+// sums 7.1e-11, 8.1e-11 and 7.6e-11 (truncated shifts gave 3.8e-11, 4.0e-11 and 3.0e-11, half
+// of it a bias).
 __global__ void __launch_bounds__(RP_THREADS, 2) k_res_pde(const double2* __restrict__ X, const double* __restrict__ q,
                                                         const double* __restrict__ D1, double k, double h, int nrhs,
                                                         float2* __restrict__ RP, double2* __restrict__ DN) {
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(RP_THREADS, 2) k_res_pde(const double2* __rest
         const FixSum fy = mb ? ye[ma] - yo[ma] : ye[ma] + yo[ma];
         FixSum fq;
         fq.mac(cq[r], uv.x, uv.y);
-        const float o = -fix_float((fx.value() >> sa) + (fy.value() >> sb) + (fq.value() >> sq), ex + em - 56);
+        const float o = -fix_float(fx.down(sa) + fy.down(sb) + fq.down(sq), ex + em - 56);
         reinterpret_cast<float*>(RP + ((long long)leaf * NL + r) * nrhs + j0 + j)[p] = bad ? nanf_ : o;
       }
     }
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(RP_THREADS, 2) k_res_pde(const double2* __rest
       f[1].mac(d, v.z, v.w);
     }
     const double sg = side == 1 || side == 2 ? 1.0 : -1.0;
-    const double2 dn = make_double2(sg * fix_double(f[0].value(), ex + en - 56), sg * fix_double(f[1].value(), ex + en - 56));
+    const double2 dn = make_double2(sg * fix_double(f[0].down(0), ex + en - 56), sg * fix_double(f[1].down(0), ex + en - 56));
     DN[((long long)leaf * NE + r) * nrhs + j0 + j] =
         bad ? make_double2((double)nanf_, (double)nanf_) : dn;
   }
