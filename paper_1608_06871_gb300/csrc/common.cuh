@@ -155,14 +155,12 @@ constexpr int OZ_NAN = 1 << 20;  // exponent of a row with an infinity or a NaN:
 __device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL; }
 
 // round(x 2^(56 - e)) for |x| < 2^e, in integer arithmetic on the bit pattern
-// (mantissa shifted by the exponent difference, rounded to nearest); 0 for
-// zeros and subnormals, whose contribution is below the slices' resolution.
+// (mantissa shifted by the exponent difference, rounded to nearest).
 __device__ __forceinline__ long long fixed56(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7FF);
-  if (E == 0) return 0;
-  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;  // 53-bit significand
-  const int sh = E - 1075 + 56 - e;                                     // x 2^(56-e) = m 2^sh, sh <= 3
+  const long long m = (b & 0xFFFFFFFFFFFFFLL) | (E ? 0x10000000000000LL : 0LL);  // significand: x = m 2^(max(E, 1) - 1075)
+  const int sh = max(E, 1) - 1075 + 56 - e;  // x 2^(56-e) = m 2^sh, below 2^56
   long long v;
   if (sh >= 0) v = m << sh;
   else if (sh > -60) v = (m + (1LL << (-sh - 1))) >> (-sh);
@@ -173,7 +171,7 @@ __device__ __forceinline__ long long fixed56(double x, int e) {
 // Exponent of a row from its largest |x| (bit pattern): max in [2^(ex-1), 2^ex).
 __device__ __forceinline__ int row_exp(long long mx) {
   const int e = (int)(mx >> 52);
-  return mx == 0 ? 0 : e == 0x7FF ? OZ_NAN : e - 1022;
+  return mx == 0 ? 0 : e == 0x7FF ? OZ_NAN : e == 0 ? -1010 - __clzll(mx) : e - 1022;
 }
 }  // namespace hs
 
