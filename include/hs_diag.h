@@ -141,8 +141,11 @@ int hs_set_tc_margin(double margin);
  * DEVICE pointers on the current device, enqueued on `stream` (a
  * cudaStream_t, NULL for the legacy default stream) and synchronised before
  * return.  Runs the library's FP64 GEMM dispatch (the kernels of the FP64
- * solver and of the mixed path's FP64 refinement).  Errors: HS_EINVAL
- * (non-positive size, NULL pointer), HS_ECUDA. */
+ * solver and of the mixed path's FP64 refinement; large ones run as the
+ * emulated product below, with scratch allocated and freed on `stream`, or on
+ * the FP64 pipe where there is no room for it).  Errors: HS_EINVAL
+ * (non-positive size, NULL pointer), HS_ETIMEOUT (a bounded tensor-core wait
+ * gave up; C is then unspecified), HS_ECUDA. */
 int hs_zgemm(int transA, int transB, int m, int n, int k, const void* A, const void* B, void* C, int accumulate,
              void* stream);
 
@@ -185,7 +188,8 @@ int hs_jacobian32_products(long long rows, int n, const void* J, const double* v
  * for the legacy default stream) and synchronised before return.  precision
  * HS_FP64: complex128; HS_MIXED: complex64.  Allocates and frees its pivot
  * and status arrays.  Errors: HS_EINVAL (bad size or precision, NULL
- * pointer), HS_ESINGULAR (an exactly zero pivot), HS_ENOMEM, HS_ECUDA. */
+ * pointer), HS_ESINGULAR (an exactly zero pivot), HS_ENOMEM, HS_ETIMEOUT (a
+ * bounded tensor-core wait gave up; X is then unspecified), HS_ECUDA. */
 int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, void* stream);
 
 #ifdef __cplusplus

@@ -1,5 +1,6 @@
 // Measurement hooks (include/hs_diag.h): per-launch timing of the FP64 GEMM
 // family and an FP64 DFMA peak kernel.
+#include <algorithm>
 #include <vector>
 
 #include "../../include/hs.h"
@@ -291,25 +292,34 @@ int hs_cgemm32(int m, int n, int k, const void* A, const void* B, void* C, int b
 }
 
 namespace {
-// The scratch a context would give its FP64 products, for the length of a call.
+// Scratch for the FP64 products of a call as a context would give them, at most 256 MB
+// and none where they all run on the FP64 pipe: mapping it costs more than a small
+// product or system (64 unknowns: 1131 us with 256 MB a call, 504 us without).
 struct CallScratch {
   hs::OzScratch sc;
   const hs::OzScratch* prev = hs::g_oz_scratch;
+  bool* prev_pending = hs::g_tc_pending;
+  bool pending = false;  // a product ran on the tensor cores
   cudaStream_t s;
-  explicit CallScratch(cudaStream_t st) : s(st) {
+  CallScratch(cudaStream_t st, size_t want) : s(st) {
+    hs::g_tc_pending = &pending;
+    const size_t bytes = std::min(want, (size_t)256 << 20);
     void* p = nullptr;
-    if (cudaMallocAsync(&p, (size_t)256 << 20, s) == cudaSuccess) {
+    if (bytes && cudaMallocAsync(&p, bytes, s) == cudaSuccess) {
       sc.p = static_cast<char*>(p);
-      sc.bytes = (size_t)256 << 20;
-    } else {
+      sc.bytes = bytes;
+    } else if (bytes) {
       cudaGetLastError();
     }
     hs::g_oz_scratch = &sc;
   }
   ~CallScratch() {
     hs::g_oz_scratch = prev;
+    hs::g_tc_pending = prev_pending;
     if (sc.p) cudaFreeAsync(sc.p, s);
   }
+  // (reading the flags takes longer than a small product)
+  bool timed_out() const { return (pending || hs::tc_timeout_raised()) && hs::tc_timed_out(s); }
 };
 }  // namespace
 
@@ -318,13 +328,12 @@ int hs_zgemm(int transA, int transB, int m, int n, int k, const void* A, const v
   if (m <= 0 || n <= 0 || k <= 0 || !A || !B || !C) return HS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int opA = transA ? hs::OP_T : hs::OP_N, opB = transB ? hs::OP_T : hs::OP_N;
-  CallScratch scratch(s);
+  CallScratch scratch(s, hs::zgemm_scratch_bytes(m, n, k, 1));
   hs::gemm<double2, double2, double2>(s, opA, opB, m, n, k, make_double2(1.0, 0.0), static_cast<const double2*>(A),
                                       transA ? m : k, 0, static_cast<const double2*>(B), transB ? k : n, 0,
                                       make_double2(accumulate ? 1.0 : 0.0, 0.0), static_cast<double2*>(C), n, 0, 1);
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return HS_ECUDA;
-  if (hs::tc_timed_out(s)) return HS_ETIMEOUT;
-  return HS_OK;
+  return scratch.timed_out() ? HS_ETIMEOUT : HS_OK;
 }
 
 int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, void* stream) {
@@ -339,8 +348,10 @@ int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, voi
   }
   cudaMemsetAsync(info, 0, sizeof(int) * (size_t)batch, s);
   const long long sA = (long long)n * n, sB = (long long)n * nrhs;
+  // (the first trailing update, and the solve's)
+  const size_t want = std::max(hs::zgemm_scratch_bytes(n, n, 128, batch), hs::zgemm_scratch_bytes(n, nrhs, 128, batch));
+  CallScratch scratch(s, precision == HS_FP64 ? want : 0);
   if (precision == HS_FP64) {
-    CallScratch scratch(s);
     hs::lu_factor<double2>(s, static_cast<double2*>(A), n, sA, n, piv, n, info, batch);
     hs::lu_solve<double2>(s, hs::OP_N, static_cast<double2*>(A), n, sA, n, piv, n, static_cast<double2*>(B), nrhs, sB,
                           nrhs, batch);
@@ -357,8 +368,7 @@ int hs_lu_solve(int precision, int n, int nrhs, void* A, void* B, int batch, voi
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return HS_ECUDA;
   for (int v : h)
     if (v != 0) return HS_ESINGULAR;
-  if (hs::tc_timed_out(s)) return HS_ETIMEOUT;
-  return HS_OK;
+  return scratch.timed_out() ? HS_ETIMEOUT : HS_OK;
 }
 
 int hs_jacobian32_products(long long rows, int n, const void* J, const double* v, void* y, const void* u, double* g,

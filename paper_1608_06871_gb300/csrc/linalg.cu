@@ -784,6 +784,11 @@ inline double re_of(double2 x) { return x.x; }
 inline double im_of(double) { return 0.0; }
 inline double im_of(double2 x) { return x.y; }
 
+// mr x nr x kr: the sizes of the real product behind m x n x k.
+bool emulation_pays(int mr, int nr, int kr, int m, int n, int k, int batch, bool b_shared, double fma) {
+  return std::min(m, n) > 8 && oz_cycles(mr, nr, kr, batch, b_shared) <= 0.8 * fp64_tile(m, n, k, batch, fma).cycles;
+}
+
 // FP64 products by the emulated product on the tensor cores (ozaki.cu) where
 // its estimated time is clearly below the FP64 pipe's: 36 bf16 products are
 // about a tenth of the pipe's time per multiply-add, but operands are sliced
@@ -809,11 +814,9 @@ bool gemm_emulated(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alp
   const bool turn = !ca && cb && re_of(alpha) == 0.0;
   if (im_of(alpha) != 0.0 && !turn) return false;
   const double factor = turn ? im_of(alpha) : re_of(alpha);
-  if (std::min(m, n) <= 8) return false;
   const int mr = ca && !cb ? 2 * m : m, nr = cb ? 2 * n : n, kr = ca && cb ? 2 * k : k;
   const bool bsh = sB == 0 && batch > 1;
-  if (oz_cycles(mr, nr, kr, batch, bsh) > 0.8 * fp64_tile(m, n, k, batch, flops_per_mac<TA, TB>() / 2.0).cycles)
-    return false;
+  if (!emulation_pays(mr, nr, kr, m, n, k, batch, bsh, flops_per_mac<TA, TB>() / 2.0)) return false;
   const long long ea = ca ? 2 : 1, eb = cb ? 2 : 1;
   OzSrc a{reinterpret_cast<const double*>(A), ea * sA, ea * (opA == OP_N ? lda : 1), ea * (opA == OP_N ? 1 : lda),
           ca ? (cb ? OZ_CLEFT : OZ_PAIR) : OZ_REAL};
@@ -895,6 +898,12 @@ float g_tc_margin = 0.5f;
 int g_t32_mode = 1;                 // hs_set_tensor_cores: 0 off, 1 per-shape choice, 2 forced
 thread_local bool g_prof_suspended = false;
 thread_local int g_last_gemm_tc = 0;
+
+size_t zgemm_scratch_bytes(int m, int n, int k, int batch) {
+  return g_oz_enabled && emulation_pays(m, 2 * n, 2 * k, m, n, k, batch, false, 4.0)
+             ? ozaki_scratch_bytes(m, 2 * n, 2 * k, batch, false)
+             : 0;
+}
 
 template <typename TA, typename TB, typename TC>
 void gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,

@@ -20,6 +20,10 @@ void gemm(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const
           long long sA, const TB* B, int ldb, long long sB, TC beta, TC* C, int ldc, long long sC,
           int batch);
 
+// Scratch (OzScratch) with which gemm() takes such a complex FP64 product to the tensor
+// cores in one go; 0 where it runs on the FP64 pipe.
+size_t zgemm_scratch_bytes(int m, int n, int k, int batch);
+
 // The FP32 kernels behind gemm() (gemm32.cu), for the four operand forms.
 template <typename TA, typename TB, typename TC>
 void gemm_fp32(cudaStream_t s, int opA, int opB, int m, int n, int k, TC alpha, const TA* A, int lda, long long sA,
@@ -114,7 +118,7 @@ void t32_timeout_flag(cudaStream_t s, int* v, bool clear);
 cudaError_t tc_raise_timeout_flag();
 // The host raised a flag that no check has read yet.
 bool tc_timeout_raised();
-// Set by the emulated FP64 products that the calling thread launches, where it points
+// Set by the tensor-core products that the calling thread launches, where it points
 // somewhere: the owner of the work then reads the flags once it has waited for it.
 extern thread_local bool* g_tc_pending;
 

@@ -470,6 +470,7 @@ void set_attr() {
 template <int NT>
 void launch_mma(cudaStream_t s, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb, const TParams& P) {
   set_attr<NT>();
+  if (g_tc_pending) *g_tc_pending = true;
   k_t32_mma<NT><<<grid, TTHREADS, TCfg<NT>::SMEM, s>>>(ma, mb, P);
   HS_COUNT_LAUNCH();
 }
