@@ -51,7 +51,10 @@ extern "C" {
  * _dev ones, hs_solve_noalloc) cannot: a timeout in one of them is returned by
  * the next of the calls above on the same context. */
 
-#define HS_FP64 0   /* every step in complex FP64                            */
+#define HS_FP64 0   /* FP64 operands and results throughout; large products are
+                       summed from exact BF16 slices on the tensor cores, errors
+                       relative to the largest entries of rows and columns, or on
+                       the FP64 pipe (hs_set_fp64_emulation in hs_diag.h)      */
 #define HS_MIXED 1  /* FP32 factors and sweep, FP64 residual refinement       */
 
 typedef struct hs_ctx hs_ctx;

@@ -156,15 +156,22 @@ int hs_zgemm(int transA, int transB, int m, int n, int k, const void* A, const v
  * scaled by powers of two and split into eight exact 7-bit BF16 slices, the
  * 36 slice pairs of weight >= 2^-63 multiplied exactly in FP32 accumulators,
  * recombined exactly in integers and rounded once per piece of at most 384 of
- * k (within the FP64 product's bound 2 k u |A||B|).  Allocates and frees
- * its scratch on `stream`.  Errors: HS_EINVAL (bad size, NULL), HS_ENOMEM,
- * HS_ETIMEOUT (a bounded tensor-core wait gave up), HS_ECUDA (also when the
- * driver offers no tensor-map encoder). */
+ * k.  Each entry is within 1.25 k u max|A_i.| max|B_.j| (u = 2^-53, the largest
+ * entries of its row and column) of the exact one, besides the roundings of the
+ * result and of the sum of the pieces: about an FP64 product's error where the
+ * entries of a row are of one size, more where they are graded.  A row of A or
+ * a column of B with an infinity or a NaN gives NaN throughout.  Allocates and
+ * frees its scratch on `stream`.  Errors: HS_EINVAL (bad size, NULL),
+ * HS_ENOMEM, HS_ETIMEOUT (a bounded tensor-core wait gave up), HS_ECUDA. */
 int hs_dgemm_emulated(int m, int n, int k, const void* A, const void* B, void* C, int batch, void* stream);
 
-/* Use the emulated FP64 product above for the FP64 Jacobian contraction
- * (enable != 0, the default) or the FP64 SIMT GEMM (enable == 0).
- * Process-wide; takes effect at the next Jacobian.  Never fails. */
+/* Use the emulated FP64 product above (enable != 0, the default) or the FP64
+ * pipe (enable == 0) for the library's large FP64 products: the Jacobian
+ * contraction and the normal matrix, the exterior rows and far field of mixed
+ * contexts, and on FP64 contexts the merges, the root system, the sweeps and
+ * the adjoint (the elimination of the leaves is on the pipe either way).  The
+ * mixed path's residuals are summed in 56-bit fixed point either way.
+ * Process-wide; takes effect at the next call.  Never fails. */
 int hs_set_fp64_emulation(int enable);
 
 /* The two products LSQR applies to the explicit FP32 Jacobian (Sec. 3.3,
@@ -181,8 +188,8 @@ int hs_jacobian32_products(long long rows, int n, const void* J, const double* v
                            void* stream);
 
 /* Solve A[b] X[b] = B[b] in place in B for b < batch with the library's
- * batched LU (partial pivoting; tournament pivoting for panels taller than 256
- * rows) and triangular solves: complex (interleaved re, im), row-major,
+ * batched LU (partial pivoting; tournament pivoting for panels taller than
+ * 4096 rows) and triangular solves: complex (interleaved re, im), row-major,
  * A n x n (overwritten by its factors), B n x nrhs, contiguous batches, DEVICE
  * pointers on the current device, enqueued on `stream` (a cudaStream_t, NULL
  * for the legacy default stream) and synchronised before return.  precision

@@ -799,8 +799,10 @@ bool emulation_pays(int mr, int nr, int kr, int m, int n, int k, int batch, bool
 // 98.5 ms, a k = 20 gradient 65.8 -> 44.3 ms.  Error against 64 bits of random
 // complex products: 7e-17 .. 1.3e-16 of the result for k = 32 .. 1792, on the
 // pipe 2.5e-16 .. 7e-16 (rows whose entries spread over 1e5: 4.5e-16 against
-// 3e-16 at k = 128, 4.8e-16 against 1.9e-15 at 1792); of far fields, fields,
-// Jacobians and steps at k = 5 .. 20: unchanged (5e-13 .. 5e-12).
+// 3e-16 at k = 128, 4.8e-16 against 1.9e-15 at 1792).  It grows with the grading inside
+// rows and columns (the bound in ozaki.cu), so a caller with graded operands keeps them on the
+// pipe (PipeScope; the leaf elimination); far fields, fields, Jacobians and steps at k = 3 .. 20 are
+// as close to the dense solution as on the pipe, within 2%.
 // Batches, then columns, then k, are cut to what the calling thread's scratch holds.
 // Factors that are neither real nor (real x complex) imaginary, and calls without
 // scratch, are refused.

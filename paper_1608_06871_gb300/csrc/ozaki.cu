@@ -1,7 +1,8 @@
 // FP64 matrix products on the 5th-generation tensor cores by exact integer
 // slices (error-free splitting in the manner of Ozaki, Ogita, Oishi and Rump,
 // 2012, with row / column scaling as in Ozaki, Uchino and Imamura's later
-// variants), for the FP64 contractions of the Jacobian.
+// variants), for the FP64 contractions of the Jacobian, the exterior rows of the mixed
+// solver and the larger products of the FP64 one (gemm_emulated).
 //
 // C = alpha A B (+ beta C), A m x k and B k x n real FP64.  Every row i of A
 // is scaled by 2^-ea_i so that its largest entry lies in [1/2, 1), every
@@ -16,9 +17,14 @@
 //   |partial sum| <= K 4096 (d + 3) < 2^24  for K <= 384,
 // which bounds the k extent of one piece (longer products sum their pieces in
 // FP64).  The epilogue recombines the 8 diagonal sums exactly in integers and
-// rounds them once to the double, formed from its bits.  What is dropped is the pairs with s + t >= 8,
-// below 2^-55 k max|A_i.| max|B_.j| per entry, and one FP64 rounding per piece:
-// the result stays within the FP64 product's own bound 2 k u |A| |B|.
+// rounds them once to the double, formed from its bits.  What an entry of C can be
+// off by is set by the largest entries of its row and column: 2^-56 of each from the
+// 56-bit fixed point, and the pairs with s + t >= 8 left out, at most 3.6 2^-55 a term:
+//   below 1.25 k u max|A_i.| max|B_.j|   (u = 2^-53),
+// besides one rounding per piece and those of the sum of the pieces.  An FP64 product's
+// bound is k u |A_i.| |B_.j|: about the same where the entries of a row are of one size,
+// far smaller where they are graded against the column's (there this product loses
+// bits that FP64 keeps; the leaf elimination stays on the FP64 pipe for that reason).
 // A complex product is one real product: rows of A as (re, im) pairs along k,
 // columns of B as the pairs (re, -im) and (im, re).
 //
@@ -284,10 +290,12 @@ __global__ void __launch_bounds__(256) k_oz_fix(double2* __restrict__ F, long lo
 // real product, six 32 x 32 + 64 multiply-adds per part (the U0 Z0 term is below
 // one unit of 2^-56).  Against FP64 products and the row's own maximum: no
 // operation on the FP64 pipe (60% busy then, with 145 instructions per real
-// entry), and an error of about one unit of 2^-56 of the fields' maxima where
-// FP64 rounds each product to 2^-53 of itself.  25,600 pairs at n = 448: 101 ms
-// with FP64 products and 2-byte stores, 95 with 32-bit stores, 54 in integers, 47.7 with
-// the digits of two neighbours taken at once.
+// entry), and an error within 3.5 u of the product of the two fields' maxima over the
+// row piece, where FP64 rounds each product to u of itself (a row in which u is small
+// where z is large has that many bits fewer; the fields of this problem vary little
+// within a row: Jacobians are as close to the dense solution as before).  25,600 pairs at
+// n = 448: 101 ms with FP64 products and 2-byte stores, 95 with 32-bit stores, 54 in
+// integers, 47.7 with the digits of two neighbours taken at once.
 __global__ void __launch_bounds__(256) k_oz_slice_kr(const int4* __restrict__ Ug, const int4* __restrict__ Zg,
                                                      const int* __restrict__ eu, const int* __restrict__ ez,
                                                      unsigned P, unsigned nX, unsigned d0, unsigned p0, unsigned nr,
