@@ -84,11 +84,10 @@ __device__ __forceinline__ double2 recip(double2 x) {
 // the per-column latency is the point here); the thread keeps its row in
 // registers and mirrors every updated entry to the tile.
 // On return, loc[r] is the tile row holding logical row r, rid[] is permuted
-// into logical order, sp[j] (if not NULL) receives the logical row swapped
-// with row j at step j, and *zc is lowered to the first column whose pivot is
+// into logical order, and *zc is lowered to the first column whose pivot is
 // exactly zero (that column is then left unscaled).
 template <typename E>
-__device__ void tile_lu(E* T, int ld, int rows, int nb, int* rid, int* loc, int* sp, int* zc) {
+__device__ void tile_lu(E* T, int ld, int rows, int nb, int* rid, int* loc, int* zc) {
   using M = typename pmag<E>::T;
   constexpr int NW = PT / 32;
   __shared__ M wbest[2][NW];
@@ -142,7 +141,6 @@ __device__ void tile_lu(E* T, int ld, int rows, int nb, int* rid, int* loc, int*
       }
     }
     const int p = key & 255, lp = key >> 8;
-    if (sp && t == 0) sp[j] = lp;
     if (t == p) {
       active = false;
       mylg = j;
@@ -186,10 +184,10 @@ __device__ void tile_lu(E* T, int ld, int rows, int nb, int* rid, int* loc, int*
 }
 
 // Stage rows x nb elements into the tile T (row stride ld): tile row r is
-// source row ids[r] (or row0 + r without ids) of A (row stride lda).  One warp
-// per row, lanes along the columns, eight rows in flight per warp.
+// source row ids[r] of A (row stride lda).  One warp per row, lanes along the
+// columns, eight rows in flight per warp.
 template <typename E>
-__device__ void load_rows(E* T, int ld, int rows, int nb, const E* A, int lda, const int* ids, int row0) {
+__device__ void load_rows(E* T, int ld, int rows, int nb, const E* A, int lda, const int* ids) {
   constexpr int NW = PT / 32, RF = 8;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int r0 = warp * RF; r0 < rows; r0 += NW * RF) {
@@ -197,7 +195,7 @@ __device__ void load_rows(E* T, int ld, int rows, int nb, const E* A, int lda, c
 #pragma unroll
     for (int q = 0; q < RF; ++q) {
       const int r = r0 + q;
-      v[q] = (r < rows && lane < nb) ? A[(long long)(ids ? ids[r] : row0 + r) * lda + lane] : el<E>::zero();
+      v[q] = (r < rows && lane < nb) ? A[(long long)ids[r] * lda + lane] : el<E>::zero();
     }
 #pragma unroll
     for (int q = 0; q < RF; ++q)
@@ -246,9 +244,9 @@ __global__ void __launch_bounds__(PT) k_tp_select(E* A, int lda, long long sA, i
   if (myrow >= 0) rid[off + __popc(bal & ((1u << lane) - 1u))] = myrow;
   __syncthreads();
   const int ld = nb + 1;
-  load_rows<E>(T, ld, rows, nb, A + j0, lda, rid, 0);
+  load_rows<E>(T, ld, rows, nb, A + j0, lda, rid);
   __syncthreads();
-  tile_lu<E>(T, ld, rows, nb, rid, loc, nullptr, &zc);
+  tile_lu<E>(T, ld, rows, nb, rid, loc, &zc);
   if (!final_round) {
     if (t < nb) W[out_off + set * nb + t] = t < rows ? rid[t] : -1;
     return;
