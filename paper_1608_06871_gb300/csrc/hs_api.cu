@@ -267,6 +267,7 @@ int run_captured(hs_ctx* ctx, cudaStream_t s, GraphSlot& slot, bool capture, con
       slot.seen_k = k;
       return enqueue();
     }
+    if (s == cudaStreamLegacy) return enqueue();  // (cannot be captured; a graph captured elsewhere replays there)
     long long* counter = g_launch_counter;
     const long long before = counter ? *counter : 0;
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
