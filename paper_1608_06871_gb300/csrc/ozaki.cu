@@ -413,14 +413,14 @@ __device__ __forceinline__ bool oz_item(const OzParams& P, long long it, OzItem&
 // diagonals take half of TMEM, so one piece's epilogue runs behind the next one's
 // products.  What bounds it: per 32-k stage the 36 slice products (1152 tensor
 // clocks) read 136 KB of shared memory while 80 KB are written (1690 clocks);
-// 2000 to 2200 clocks at 1.92 GHz measured.  The epilogue (9400 clocks a piece: the
+// 2000 to 2200 clocks at 1.92 GHz measured.  The epilogue (9700 clocks a piece: the
 // conversions of eight diagonals, the doubles assembled from their bits in
 // integer arithmetic) bounds pieces below 160 k.
 // Before, one launch per piece with an FP64 epilogue on four warps and C read
 // back per piece kept the tensor pipe at 17%: the products of a k = 40
 // Gauss-Newton step (Jacobian projections and normal matrix, 3.2e12 flops) took
 // 278 ms; 102 ms with 128 x 64 tiles that fill TMEM, epilogue and products in
-// turn; 83 ms now.  4864 x 4096 x k: 29 TFLOP/s of FP64-equivalent work at k = 256,
+// turn; 88 ms now.  4864 x 4096 x k: 29 TFLOP/s of FP64-equivalent work at k = 256,
 // 34 at 1536 (1217 of the 1948 TFLOP/s bf16 peak issued).
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_mma(const __grid_constant__ OzParams P) {
