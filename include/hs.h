@@ -47,9 +47,12 @@ extern "C" {
  * device waits; one that gives up leaves its results unspecified and sets a
  * flag of the device.  hs_build, hs_build_nodes, hs_solve, hs_jacobian,
  * hs_gradient, hs_gn_step and hs_gn_step_lsqr, which wait for the GPU, read
- * and clear it before they return.  The calls that only enqueue work (the
- * _dev ones, hs_solve_noalloc) cannot: a timeout in one of them is returned by
- * the next of the calls above on the same context. */
+ * and clear it before they return (the solves, Jacobians and gradients where
+ * such a product ran on the context since the last reading, or a call ran on a
+ * stream of its own; the others always).
+ * The calls that only enqueue work (the _dev ones, hs_solve_noalloc) cannot: a
+ * timeout in one of them is returned by the first of the calls above on the same
+ * context that comes after its work has finished. */
 
 #define HS_FP64 0   /* FP64 operands and results throughout; large products are
                        summed from exact BF16 slices on the tensor cores, errors

@@ -217,6 +217,7 @@ struct hs_ctx {
   double* d_k = nullptr;
   OzScratch oz;  // slices of the emulated FP64 products (ensure_oz)
   bool tc_pending = false;  // some of them ran since the timeout flags were last read
+  bool tc_elsewhere = false;  // some calls ran on a stream of their own, which no reading waits for
   double k_dev = 0.0;
   long long builds = 0;
   // phase times of the last build recorded launch by launch (-1 after a graph replay)
@@ -403,7 +404,7 @@ void ensure_oz(hs_ctx* ctx) {
 // the flags takes some 25 us, so calls that launched no such product leave them.
 int check_tc(hs_ctx* ctx, cudaStream_t s) {
   if (!ctx->tc_pending && !tc_timeout_raised()) return HS_OK;
-  ctx->tc_pending = false;
+  ctx->tc_pending = ctx->tc_elsewhere;
   return tc_timed_out(s) ? fail(ctx, HS_ETIMEOUT, "a tensor-core GEMM wait gave up") : HS_OK;
 }
 
@@ -1104,7 +1105,11 @@ int check_ctx(hs_ctx* ctx, bool need_built) {
   return HS_OK;
 }
 
-cudaStream_t pick(hs_ctx* ctx, void* stream) { return stream ? (cudaStream_t)stream : ctx->stream; }
+cudaStream_t pick(hs_ctx* ctx, void* stream) {
+  if (!stream || (cudaStream_t)stream == ctx->stream) return ctx->stream;
+  ctx->tc_elsewhere = true;
+  return (cudaStream_t)stream;
+}
 
 // A complex matrix (row stride sr, column stride sk, in complex entries) as the
 // left or right operand of an emulated complex product.
